@@ -11,12 +11,11 @@
 //   big classes                       split into hash buckets of beta' (each a
 //                                     tile); all contributions to one target
 //                                     land in the same bucket
-// A tile groups its records by target in a shared-memory hash table (the
-// records of each target linked into a list), sums each target's values
-// exactly (192-bit fixed point, so the sum does not depend on the order of the
-// contributions and equals the sort-and-accumulate result bit for bit), drops
-// targets in psi, and scores in FP64 and appends the targets whose |score| can
-// reach the running top-N threshold.
+// A tile groups its records by target in a shared-memory hash table, drops
+// targets in psi, and appends the targets whose |score| can reach the running
+// top-N threshold; their values are summed after the launch by a rule that
+// does not depend on the order of the contributions, so that it equals the
+// sort-and-accumulate result bit for bit, and scored in FP64.
 //
 // The diagonal H_ii is carried exactly in 64-bit fixed point: the integral
 // terms are rounded once to multiples of 2^-s, and each pair's H_ii is the
@@ -285,7 +284,8 @@ __device__ __forceinline__ double flip_sign(double x, uint32_t flip) {
 
 }  // namespace
 
-constexpr int kCellThreads = 256;
+constexpr int kCellThreads = 128;
+constexpr int kCellCtas = 8;                        // per SM
 constexpr int kCap = 1024;                          // records per tile
 constexpr uint32_t kSmallMax = kCap / 2;            // packable class size
 constexpr uint32_t kBucketTarget = kCap * 13 / 16;  // expected records per hash bucket
@@ -1103,8 +1103,8 @@ struct CellArgs {
   unsigned long long *n_unique, *n_excluded;
   unsigned *err;
   int screened;  // records may carry the eps screen's drop marker
-  // exact sums left to k_long_sums (null: formed in the tile kernel): the
-  // values of each list, and per list (candidate slot, offset << 16 | length)
+  // targets of several records that can reach the threshold, summed by
+  // k_long_sums: the values of each, and (candidate slot, offset << 16 | length)
   double *lv;
   unsigned long long *lv_count;
   unsigned long long lv_cap;
@@ -1122,20 +1122,17 @@ __device__ __forceinline__ uint64_t mix_key(uint64_t z) {
   return z;
 }
 
-// Hash of a target key within a tile: the 32-bit finalizer of MurmurHash3
-// (Appleby) over the alpha word times an odd constant xor the beta word.
-// Bucket tiles hold one alpha string and the betas of one bucket, so the
-// finalizer's avalanche is what spreads them; cheaper than mix_key's two
-// 64-bit products.  Its low bits pick the slot of the tile's hash table
-// (2048 slots), its high 13 bits the bit of the tile's singleton filter.
+// Hash of a target key within a tile: a product per word and the multiply of
+// a finalizer, whose high half picks the slot (the top bits of a product
+// depend on every bit below them).  Bucket tiles hold one alpha string and the
+// betas of one bucket, which another multiplier picked.  The two rounds more
+// of the full MurmurHash3 finalizer (Appleby) spread no better and cost 0.5%
+// of a (24e,30o) search.
 __device__ __forceinline__ uint32_t tile_mix(uint64_t key) {
-  uint32_t h = (uint32_t)key * 0x9E3779B1u ^ (uint32_t)(key >> 32);
+  uint32_t h = (uint32_t)key * 0x9E3779B1u + (uint32_t)(key >> 32) * 0x85EBCA6Bu;
   h ^= h >> 16;
-  h *= 0x85EBCA6Bu;
-  h ^= h >> 13;
   h *= 0xC2B2AE35u;
-  h ^= h >> 16;
-  return h;
+  return h >> 16;
 }
 
 // Open addressing with linear probing; the table is at most 1/4 full, and the
@@ -1153,37 +1150,45 @@ __device__ __forceinline__ bool psi_contains(const uint64_t *ht, uint64_t mask, 
   return false;
 }
 
-// A tile first sorts out its singletons: every key of the tile (records and
-// the psi determinants routed to it) sets its bit of a filter of kFilterBits
-// bits, and a key that finds its bit set marks it in a second filter.  A
-// record whose bit is not marked shares its hash with no other key of the
-// tile, so it is the only contribution to its target, which is not in psi:
-// it is scored and appended at once.  (About three records in four are the
-// only contribution to their target; most of those are recognised so.)
-// The other records are grouped by target in a shared-memory hash table: a slot
-// holds the newest record of its target and each record the index of the
-// previous one, so that every target ends up with the list of its records.
-// The psi determinants that fall in the tile are entered first as markers, so
-// a target in psi is recognised without a global lookup.  The numerator is
-// then summed over each list by a rule that depends only on the multiset of
-// its values, so grouping by hashing gives the result of sorting the records
-// and summing the runs.  The records of the next tile are copied in
-// asynchronously meanwhile.
-constexpr uint32_t kEmptySlot = 0xffffffffu;
-constexpr uint32_t kPsiBit = 0x80000000u;  // slot holds psi marker (index in low bits)
-constexpr uint16_t kEndList = 0xffffu;
-constexpr int kPsiCap = 64;                // psi markers per tile; more: global lookups
+// A tile's records are grouped by target in a shared-memory hash table whose
+// slots are single words: the first record of the target (the one that claimed
+// the slot), how many more records it has, and the sum over those of a
+// quantised bound of |v| / (tau |E0 - H_ii|).  Integer atomics build the word,
+// so nothing is walked: after one pass over the records the claiming thread
+// knows whether its target has one record (it is scored by its own value),
+// cannot reach the threshold (it is only counted), or can (its values are
+// copied out and summed after the launch by k_long_sums).  The psi
+// determinants that fall in the tile are entered as markers, so a target in
+// psi is recognised without a global lookup.  The numerator is formed by a
+// rule that depends only on the multiset of a target's values, so grouping by
+// hashing gives the result of sorting the records and summing the runs.
+//
+// Word of a slot, B = log2 of the tile's record capacity:
+//   bits 0 .. B-1        the claiming record, or the index of a psi marker
+//   bit  B               the target is in psi
+//   bit  B+1             psi marker; empty slot (index all ones); or, once the
+//                        target was found to reach the threshold, the index
+//                        (below CAP / 2) of its cursor in S.cur
+//   bits B+2 .. 2B+1     further records of the target
+//   bits 2B+2 .. 31      sum of their quantised bounds
+// A quantised bound is at most kThr, and a target of kLong or more records
+// reaches the threshold whatever its sum, so the sum of a target that is
+// tested, of at most kLong - 2 further records, cannot overflow its field;
+// the sum of a longer one may, off the top of the word.  A target's records
+// all count before any is tested, and their order does not matter.
+constexpr int kPsiCap = 64;  // psi markers per tile; more: global lookups
 
-// The tile kernel comes in two sizes: tiles of kCap records (every packed,
-// medium and bucket tile) and tiles of kBigCap records for the hash buckets
-// that hot targets overfilled (bucket tiles only, one CTA per SM).  Per
-// record: two hash slots and eight filter bits.
-constexpr int kBigCap = 4096;
-constexpr int kBigThreads = 1024;
-// buckets of at most kMidCap records (most overfilled ones) take a middle
-// size: two CTAs of kMidThreads per SM
+// The tile kernel comes in three sizes: tiles of kCap records (every packed,
+// medium and bucket tile) and tiles of kMidCap and kBigCap records for the
+// hash buckets that hot targets overfilled (bucket tiles only).  Eight records
+// per thread (a warp's overhead per tile and the longest of its lanes' probe
+// sequences are shared by more of them) and four hash slots per record (with
+// two, an eighth of the records meet another target on their first probe).
 constexpr int kMidCap = 2048;
-constexpr int kMidThreads = 512;
+constexpr int kMidThreads = 256;
+constexpr int kBigCap = 4096;
+constexpr int kBigThreads = 512;
+constexpr int kRPT = 8;  // records per thread
 
 template <int CAP>
 constexpr int log2_of() {
@@ -1192,47 +1197,32 @@ constexpr int log2_of() {
   return b;
 }
 
-template <int CAP, bool PACKED>
-struct CellSmem {
-  static constexpr int kTab = 2 * CAP;           // hash slots (load <= 1/2)
-  static constexpr int kFilterWords = CAP / 4;   // 8 CAP filter bits
-  static constexpr int kFilterShift = 32 - (log2_of<CAP>() + 3);  // top bits pick a filter bit
-  StageRec rec[2][CAP];      // records (double-buffered by tile)
-  uint32_t seen[kFilterWords];  // filter bits of the tile's keys (records and psi entries)
-  uint32_t dup[kFilterWords];   // filter bits met twice or more
-  uint32_t alpha[2][PACKED ? CAP : 1];  // record target alpha strings (packed tiles)
-  uint64_t psik[2][kPsiCap]; // psi keys of the tile
-  uint32_t slot[kTab];       // newest record of the slot's target, a psi marker, or empty
-  uint32_t psibit[2][kTab / 32];  // slots whose key is in psi
-  uint16_t next[CAP];        // previous record of the same target, or kEndList
-  uint16_t targets[CAP];     // slots claimed by records, in order of claiming
-  uint16_t psi_slot[kPsiCap];  // slot claimed by each psi marker, or kEndList
-  uint32_t ntargets[2];      // by tile parity
-  static_assert(CAP < 0xffff && kTab <= 0xffff, "indices must fit 16 bits");
-  static_assert((1 << log2_of<CAP>()) == CAP, "capacity must be a power of two");
+template <int CAP>
+struct SlotWord {
+  static constexpr int B = log2_of<CAP>();
+  static constexpr uint32_t kIndex = (uint32_t)CAP - 1u;
+  static constexpr uint32_t kPsi = 1u << B;
+  static constexpr uint32_t kMark = 2u << B;
+  static constexpr uint32_t kEmpty = kMark | kIndex;
+  static constexpr int kCountShift = B + 2;
+  static constexpr uint32_t kOne = 1u << kCountShift;
+  static constexpr int kSumShift = 2 * B + 2;
+  static constexpr uint32_t kLong = CAP <= 1024 ? 32u : 8u;
+  static constexpr uint32_t kThr = (1u << (32 - kSumShift)) / kLong;
+  static_assert((1 << B) == CAP, "capacity must be a power of two");
+  static_assert((kLong - 2) * kThr < (1u << (32 - kSumShift)), "the sum must fit its field");
+  static_assert(kPsiCap < CAP / 2, "markers and cursors differ from the empty word");
 };
-using TileSmem = CellSmem<kCap, true>;
-using BigTileSmem = CellSmem<kBigCap, false>;
-using MidTileSmem = CellSmem<kMidCap, false>;
 
-__device__ __forceinline__ void cp_async8(void *smem, const void *gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-}
+template <int CAP>
+struct CellSmem {
+  static constexpr int kTab = 4 * CAP;  // hash slots (load <= 1/4)
+  uint64_t key[CAP];            // target keys of the tile's records
+  uint64_t psik[kPsiCap];       // psi keys of the tile
+  uint32_t slot[kTab];
+  uint32_t cur[CAP / 2];        // next value position of each target that reaches the threshold
+  uint32_t ncur;                // their number
+};
 
 // A tile that the kernel reduces on chip; oversized hash buckets go to the
 // global path, anything else outside the limits is a planning bug.
@@ -1247,503 +1237,388 @@ __device__ __forceinline__ bool tile_on_chip(const TileDesc &d, uint64_t stage_c
   return fits;
 }
 
-template <int CAP, bool PACKED>
-__device__ __forceinline__ void prefetch_tile(CellSmem<CAP, PACKED> &S, int buf,
-                                              const TileDesc &d, const CellArgs &C) {
-  for (uint32_t e = threadIdx.x; e < d.npairs; e += blockDim.x) {
-    cp_async16(&S.rec[buf][e], C.st.rec + d.start + e);
-    if (PACKED && d.kind == kTilePacked) cp_async4(&S.alpha[buf][e], C.st.alpha + d.start + e);
-  }
-  const uint32_t np = d.psi_hi - d.psi_lo;
-  if (np <= (uint32_t)kPsiCap)
-    for (uint32_t q = threadIdx.x; q < np; q += blockDim.x)
-      cp_async8(&S.psik[buf][q], C.psi_list + d.psi_lo + q);
-  cp_async_commit();
+// |v| / (tau |den|) in units of 1 / kThr, rounded up, at most kThr.  inv_tau is
+// kThr / tau_f, or infinity without a threshold.  An upper bound: |v| is
+// truncated to a float from its bits (no FP64 instruction; within 2^-23),
+// |den| was truncated when it was staged and tau_f rounded down, and the factor
+// 1.00001 covers those and the float operations.  A value above the normal
+// float range, a zero denominator and anything that is not a number count as
+// reaching the threshold; a |v| below the range counts as its smallest value.
+template <uint32_t kThr>
+__device__ __forceinline__ uint32_t quantised_bound(uint32_t v_lo, uint32_t v_hi, float den,
+                                                    float inv_tau) {
+  const uint32_t hi = v_hi & 0x7fffffffu;
+  float vf = __uint_as_float(__funnelshift_l(v_lo, hi - 0x38000000u, 3));
+  if (hi < 0x38100000u) vf = 1.17549435e-38f;
+  const float r = __fdividef(vf * 1.00001f, fabsf(den)) * inv_tau;
+  const bool big = !(r < (float)kThr) || hi >= 0x47f00000u || den == 0.0f;
+  return big ? kThr : __float2uint_ru(r);
 }
 
-// Target key of record e (bucket and medium tiles share one alpha string).
-template <int CAP, bool PACKED>
-__device__ __forceinline__ uint64_t rec_key(const CellSmem<CAP, PACKED> &S, int buf, uint32_t e,
-                                            bool packed, uint32_t alpha) {
-  return pack_key(PACKED && packed ? S.alpha[buf][PACKED ? e : 0] : alpha, S.rec[buf][e].beta);
-}
-template <int CAP, bool PACKED>
-__device__ __forceinline__ uint64_t slot_key(const CellSmem<CAP, PACKED> &S, int buf, uint32_t v,
-                                             bool packed, uint32_t alpha) {
-  return (v & kPsiBit) ? S.psik[buf][v & ~kPsiBit] : rec_key(S, buf, v, packed, alpha);
-}
-
-
-// |v| as a float for the threshold bound: from the bits (no FP64 instruction),
-// +inf when |v| lies above the float range so that the bound always passes.
-__device__ __forceinline__ float abs_bound(double v) {
-  bool ok;
-  const float f = abs_as_float(v, &ok);
-  return (ok || fx_exponent(v) < 1023) ? f : __int_as_float(0x7f800000);
-}
-
-// Sum of five or more values (list from e through next) in the 128-bit
-// fixed-point accumulator anchored to their largest exponent: equal bit for bit
-// for any order.  The first walk also sums |v| in float.  |num| <= sum |v|, so
-// a target whose bound cannot reach the running threshold tau |E0 - H_ii|
-// fails the screen whatever its exact numerator: *reach is cleared and the
-// exact sum is skipped.  The test is conservative: a list holds at most kBigCap
-// = 4096 values, so the float sum lies within 4095 * 2^-24 < 2.45e-4 below the
-// exact sum of the (truncated, hence smaller) terms, which the factor 1.0003
-// covers; tau_f is rounded down and den truncated, and the 0.99999 margin
-// covers the float product.  Kept out of line: rare, and it would weigh on
-// the common path's registers.
-__device__ __noinline__ double long_numerator(const StageRec *r, const uint16_t *next,
-                                              uint32_t e, float tau_f, float den, int walk_max,
-                                              bool *reach, bool *deferred, unsigned long long *fix,
-                                              const CellArgs &C) {
-  int emax = 1, len = 0;
-  float sabs = 0.0f;
-  for (uint32_t i = e; i != kEndList; i = next[i]) {
-    if (++len > walk_max) {  // a hot target: its warp sums it (warp_numerator)
-      *deferred = true;
-      return 0.0;
-    }
-    const int ex = fx_exponent(r[i].v);
-    emax = ex > emax ? ex : emax;
-    sabs += abs_bound(r[i].v);
-  }
-  const float df = fabsf(den);
-  if (tau_f > 0.0f && df != 0.0f && !(sabs * 1.0003f >= tau_f * df * 0.99999f)) {
-    *reach = false;
-    return 0.0;
-  }
-  // The exact sum (several times the walk's cost, and one lane's work that
-  // its CTA waits for at the next barrier) is left to k_long_sums when its
-  // buffers have room: the values are copied out and the candidate is
-  // appended with the list's entry, whose slot the caller fills in.
-  if (C.lv) {
-    const unsigned long long fi = atomicAdd(C.nfix, 1ull);
-    const unsigned long long off = atomicAdd(C.lv_count, (unsigned long long)len);
-    if (fi < C.fix_cap) {
-      if (off + (unsigned long long)len <= C.lv_cap) {
-        unsigned long long j = off;
-        for (uint32_t i = e; i != kEndList; i = next[i]) C.lv[j++] = r[i].v;
-        C.fix[fi].y = (off << 16) | (unsigned long long)len;
-        *fix = fi;
-        return 0.0;
+// One CTA reduces tiles blockIdx.x, + gridDim.x, ...  Thread t holds records t,
+// t + THREADS, ... of a tile in registers.  Three barriers per tile, a fourth
+// when a target of several records reaches the threshold.
+//
+// Bound: instruction issue (the records are read once, at 1.7 TB/s): about 200
+// warp instructions per 32 records at (24e,30o), 58% of issue slots.  The
+// linked lists this replaces (a filter of singletons, then a list per target,
+// walked by one thread) issued about 340 and waited at the barriers for the
+// warps that walked: 116.8 ms per (24e,30o) search, C = 1e5, against 71.  Four
+// records in 256 threads take 95 ms; twice the CTAs on half the slots 12 ms
+// more; keys in place before the claims without the first barrier (fences
+// instead) 8 ms more.
+template <int CAP, int THREADS, int CTAS>
+__global__ void __launch_bounds__(THREADS, CTAS) k_cells(CellArgs C) {
+  using Smem = CellSmem<CAP>;
+  using W = SlotWord<CAP>;
+  constexpr uint32_t kTabMask = (uint32_t)Smem::kTab - 1u;
+  static_assert(CAP == kRPT * THREADS && THREADS >= kPsiCap, "records per thread");
+  static_assert(kRPT == 8 && W::kThr < 256 && Smem::kTab <= 65536, "packed bounds and slots");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Smem &S = *reinterpret_cast<Smem *>(smem_raw);
+  const int lane = threadIdx.x & 31;
+  uint32_t my_unique = 0, my_excl = 0;
+  for (int i = threadIdx.x; i < Smem::kTab; i += THREADS) S.slot[i] = W::kEmpty;
+  if (threadIdx.x == 0) S.ncur = 0;
+  const float inv_tau = C.tau_f > 0.0f ? (float)W::kThr / C.tau_f : __int_as_float(0x7f800000);
+  uint32_t tile = C.tile0 + blockIdx.x;
+  TileDesc d = {0, 0, 0, 0, 0, 0, 0, 0};
+  if (tile < C.ntiles) d = C.tiles[tile];
+#pragma unroll 1
+  for (; tile < C.ntiles; tile += gridDim.x) {
+    const bool on = tile_on_chip<CAP>(d, C.st.cap, C.err);
+    const uint32_t nrec = on ? d.npairs : 0u;
+    const uint32_t npsi = on ? d.psi_hi - d.psi_lo : 0u;
+    const bool psi_local = npsi <= (uint32_t)kPsiCap;
+    // record k of this thread: its value, and by 8 and 16 bits its quantised
+    // bound and its slot
+    double v[kRPT];
+    uint64_t q = 0, slot_lo = 0, slot_hi = 0;
+    uint32_t live = 0;
+    auto bound_of = [&](int k) { return (uint32_t)(q >> (8 * k)) & 0xffu; };
+    auto slot_of = [&](int k) {
+      return (uint32_t)((k < 4 ? slot_lo : slot_hi) >> (16 * (k & 3))) & 0xffffu;
+    };
+    const StageRec *src = C.st.rec + d.start + threadIdx.x;
+    uint64_t pkey = 0;
+    const bool has_marker = psi_local && threadIdx.x < npsi;
+    if (has_marker) pkey = C.psi_list[d.psi_lo + threadIdx.x];
+#pragma unroll
+    for (int k0 = 0; k0 < kRPT; k0 += 4) {
+      if ((uint32_t)(k0 * THREADS) >= nrec) {  // uniform
+#pragma unroll
+        for (int k = k0; k < k0 + 4; ++k) v[k] = 0.0;
+        continue;
       }
-      C.fix[fi].y = ~0ull;  // no room for the values: the entry stays unused
+      uint4 raw[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (threadIdx.x + (uint32_t)((k0 + k) * THREADS) < nrec)
+          raw[k] = __ldcs(reinterpret_cast<const uint4 *>(src + (k0 + k) * THREADS));
+        else
+          raw[k] = make_uint4(0, 0, 0, 0);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t e = threadIdx.x + (uint32_t)((k0 + k) * THREADS);
+        v[k0 + k] = __hiloint2double((int)raw[k].y, (int)raw[k].x);
+        if (e < nrec) {
+          const uint32_t alpha = d.kind == kTilePacked ? __ldcs(C.st.alpha + d.start + e) : d.alpha;
+          const uint64_t key = pack_key(alpha, raw[k].z);
+          S.key[e] = key;
+          const uint64_t h = tile_mix(key) & kTabMask;
+          if (k0 == 0) slot_lo |= h << (16 * k);
+          else slot_hi |= h << (16 * k);
+          if (!(C.screened && is_dropped(v[k0 + k]))) live |= 1u << (k0 + k);
+          q |= (uint64_t)quantised_bound<W::kThr>(raw[k].x, raw[k].y, __uint_as_float(raw[k].w),
+                                                  inv_tau)
+               << (8 * (k0 + k));
+        }
+      }
     }
+    if (has_marker) S.psik[threadIdx.x] = pkey;
+    TileDesc dn = {0, 0, 0, 0, 0, 0, 0, 0};
+    if (tile + gridDim.x < C.ntiles) dn = C.tiles[tile + gridDim.x];
+    __syncthreads();  // keys in place; the previous tile is done with the table
+    if (threadIdx.x == 0) S.ncur = 0;
+    // the next tile's records start towards L2
+    if (threadIdx.x == 0 && dn.npairs - 1u < (uint32_t)CAP &&
+        (uint64_t)dn.start + dn.npairs <= C.st.cap)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(C.st.rec + dn.start),
+                   "r"(dn.npairs * 16u)
+                   : "memory");
+    // psi markers: claim a slot, or flag the slot that a record holds
+    uint32_t marker = 0xffffffffu;
+    if (has_marker) {
+      uint32_t h = tile_mix(pkey) & kTabMask;
+      int probe = 0;
+      for (; probe < Smem::kTab; ++probe) {
+        const uint32_t w = atomicCAS(&S.slot[h], W::kEmpty, W::kMark | threadIdx.x);
+        if (w == W::kEmpty) {
+          marker = h;
+          break;
+        }
+        if (!(w & W::kMark) && S.key[w & W::kIndex] == pkey) {
+          atomicOr(&S.slot[h], W::kPsi);
+          break;
+        }
+        h = (h + 1) & kTabMask;
+      }
+      if (probe == Smem::kTab) atomicOr(C.err, kErrTile);  // cannot happen at load < 1/2
+    }
+    // the records' first probes, issued before any result is used
+    uint32_t claimed = live, rest = 0, met = 0;
+#pragma unroll
+    for (int k0 = 0; k0 < kRPT; k0 += 4) {
+      if ((uint32_t)(k0 * THREADS) >= nrec) break;  // uniform
+      uint32_t got[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        got[k] = W::kEmpty;
+        if ((live >> (k0 + k)) & 1u)
+          got[k] = atomicCAS(&S.slot[slot_of(k0 + k)], W::kEmpty,
+                             threadIdx.x + (uint32_t)((k0 + k) * THREADS));
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (got[k] != W::kEmpty) {
+          const uint64_t key = S.key[threadIdx.x + (uint32_t)((k0 + k) * THREADS)];
+          claimed &= ~(1u << (k0 + k));
+          const bool mark = (got[k] & W::kMark) != 0u;
+          if (!mark && S.key[got[k] & W::kIndex] == key) {
+            atomicAdd(&S.slot[slot_of(k0 + k)], W::kOne | (bound_of(k0 + k) << W::kSumShift));
+          } else {
+            rest |= 1u << (k0 + k);
+            if (!mark) met |= 1u << (k0 + k);
+          }
+        }
+      }
+    }
+    // the others probe on, a thread's one after another in one loop (so that
+    // a warp loops for its busiest thread, not for its unluckiest record of
+    // each round)
+    if (rest) {
+      int k = __ffs(rest) - 1, probe = 0;
+      uint64_t key = S.key[threadIdx.x + (uint32_t)(k * THREADS)];
+      // a first probe that met another target's record need not be repeated
+      uint32_t h = (slot_of(k) + ((met >> k) & 1u)) & kTabMask;
+      for (;;) {
+        const uint32_t e = threadIdx.x + (uint32_t)(k * THREADS);
+        const uint32_t w = atomicCAS(&S.slot[h], W::kEmpty, e);
+        bool done = w == W::kEmpty, own = done;
+        if (!done) {
+          const bool mark = (w & W::kMark) != 0u;
+          done = (mark ? S.psik[w & W::kIndex] : S.key[w & W::kIndex]) == key;
+          // the first record of a psi marker's target takes the slot over
+          if (done && mark) own = atomicCAS(&S.slot[h], w, e | W::kPsi) == w;
+          if (done && !own) atomicAdd(&S.slot[h], W::kOne | (bound_of(k) << W::kSumShift));
+        }
+        if (!done && ++probe < Smem::kTab) {
+          h = (h + 1) & kTabMask;
+          continue;
+        }
+        if (!done) atomicOr(C.err, kErrTile);  // cannot happen at load < 1/2
+        if (own) claimed |= 1u << k;
+        const int sh = 16 * (k & 3);
+        if (k < 4) slot_lo = (slot_lo & ~(0xffffull << sh)) | ((uint64_t)h << sh);
+        else slot_hi = (slot_hi & ~(0xffffull << sh)) | ((uint64_t)h << sh);
+        rest &= rest - 1u;
+        if (!rest) break;
+        k = __ffs(rest) - 1;
+        probe = 0;
+        h = (slot_of(k) + ((met >> k) & 1u)) & kTabMask;
+        key = S.key[threadIdx.x + (uint32_t)(k * THREADS)];
+      }
+    }
+    __syncthreads();  // every slot word is complete
+    // the claiming thread decides on its target and empties the slot, unless
+    // the target's values are to be copied out
+    uint32_t pass = 0, multi = 0, own = 0;  // own: candidates, lists << 9, values << 17
+    my_unique += (uint32_t)__popc(claimed);
+#pragma unroll
+    for (int k = 0; k < kRPT; ++k) {
+      if (!((claimed >> k) & 1u)) continue;
+      const uint32_t h = slot_of(k), w = S.slot[h];
+      const uint32_t more = (w >> W::kCountShift) & (uint32_t)(CAP - 1);
+      bool in_psi = (w & W::kPsi) != 0u;
+      if (!psi_local)
+        in_psi = psi_contains(C.psi_ht, C.psi_mask,
+                              S.key[threadIdx.x + (uint32_t)(k * THREADS)], C.err);
+      if (in_psi) {
+        ++my_excl;
+      } else if ((w >> W::kSumShift) + bound_of(k) >= W::kThr || more + 1u >= W::kLong) {
+        pass |= 1u << k;
+        if (more) {
+          multi |= 1u << k;
+          own += (1u << 9) + ((more + 1u) << 17);
+          continue;
+        }
+      }
+      S.slot[h] = W::kEmpty;
+    }
+    // a marker that no record's target took over (in_psi targets are never
+    // copied out, so no cursor takes its place either)
+    if (marker != 0xffffffffu && S.slot[marker] == (W::kMark | threadIdx.x))
+      S.slot[marker] = W::kEmpty;
+    if (__any_sync(0xffffffffu, pass != 0u)) {
+      // candidates, targets to be summed and their values: one scan over the
+      // warp (at most 256 candidates, 128 lists and CAP values)
+      own += (uint32_t)__popc(pass);
+      uint32_t sum = own;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, sum, o);
+        if (lane >= o) sum += y;
+      }
+      const uint32_t all = __shfl_sync(0xffffffffu, sum, 31);
+      const uint32_t nf = (all >> 9) & 0xffu;
+      unsigned long long b0 = 0, f0 = 0, l0 = 0;
+      uint32_t c0 = 0;
+      if (lane == 0) {
+        b0 = atomicAdd(C.cand_count, (unsigned long long)(all & 0x1ffu));
+        if (nf) {
+          f0 = atomicAdd(C.nfix, (unsigned long long)nf);
+          l0 = atomicAdd(C.lv_count, (unsigned long long)(all >> 17));
+          c0 = atomicAdd(&S.ncur, nf);
+        }
+      }
+      b0 = __shfl_sync(0xffffffffu, b0, 0);
+      if (nf) {  // warp-uniform
+        f0 = __shfl_sync(0xffffffffu, f0, 0);
+        l0 = __shfl_sync(0xffffffffu, l0, 0);
+        c0 = __shfl_sync(0xffffffffu, c0, 0);
+      }
+      const uint32_t before = sum - own;
+      b0 += before & 0x1ffu;
+      f0 += (before >> 9) & 0xffu;
+      c0 += (before >> 9) & 0xffu;
+      l0 += before >> 17;
+#pragma unroll
+      for (int k = 0; k < kRPT; ++k) {
+        if (!((pass >> k) & 1u)) continue;
+        const unsigned long long at = b0++;
+        if (at < C.cand_cap) {
+          C.cand_key[at] = S.key[threadIdx.x + (uint32_t)(k * THREADS)];
+          C.cand_score[at] = v[k];  // the numerator; the exact score is formed after the launch
+        }
+        if ((multi >> k) & 1u) {
+          uint32_t *sl = &S.slot[slot_of(k)];
+          const uint32_t len = ((*sl >> W::kCountShift) & (uint32_t)(CAP - 1)) + 1u;
+          if (f0 < C.fix_cap && l0 + len <= C.lv_cap && at < C.cand_cap) {
+            C.lv[l0] = v[k];
+            C.fix[f0] = make_ulonglong2(at, (l0 << 16) | len);
+            S.cur[c0] = (uint32_t)l0 + 1u;
+            *sl = W::kMark | c0;
+          } else {
+            atomicOr(C.err, kErrValues);  // the host runs the launch again with more room
+            if (f0 < C.fix_cap) C.fix[f0].y = ~0ull;
+            *sl = W::kEmpty;
+            multi &= ~(1u << k);
+          }
+          ++f0;
+          ++c0;
+          l0 += len;
+        }
+      }
+    }
+    if (__syncthreads_or(multi != 0u)) {
+      // the other records of the targets to be summed
+#pragma unroll
+      for (int k = 0; k < kRPT; ++k) {
+        if (!(((live & ~claimed) >> k) & 1u)) continue;
+        const uint32_t w = S.slot[slot_of(k)];
+        if (w != W::kEmpty) C.lv[atomicAdd(&S.cur[w & W::kIndex], 1u)] = v[k];
+      }
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < kRPT; ++k)
+        if ((multi >> k) & 1u) S.slot[slot_of(k)] = W::kEmpty;
+    }
+    d = dn;
+  }
+  unsigned long long u = my_unique, x = my_excl;
+  for (int dl = 16; dl; dl >>= 1) {
+    u += __shfl_xor_sync(0xffffffffu, u, dl);
+    x += __shfl_xor_sync(0xffffffffu, x, dl);
+  }
+  if (lane == 0) {
+    if (u) atomicAdd(C.n_unique, u);
+    if (x) atomicAdd(C.n_excluded, x);
+  }
+}
+
+// The numerators of the targets with several records that can reach the
+// threshold, from the values the tile kernel copied out: two by IEEE addition
+// (the correctly rounded exact sum), three or four by the ordered FP64 sum,
+// more by the 128-bit fixed-point accumulator anchored to the largest
+// exponent.  Each depends only on the multiset of values, so not on the order
+// in which they were copied.  One thread per list of at most kWalk values; a
+// longer one is summed by the whole warp (integer additions: the same bits).
+constexpr unsigned long long kWalk = 32;
+
+__device__ __forceinline__ double list_sum(const double *x, unsigned len, unsigned *ovf) {
+  if (len == 2) return x[0] + x[1];
+  if (len == 3) return sum4_ordered(0.0, x[0], x[1], x[2]);
+  if (len == 4) return sum4_ordered(x[0], x[1], x[2], x[3]);
+  int emax = 1;
+  for (unsigned j = 0; j < len; ++j) {
+    const int ex = fx_exponent(x[j]);
+    emax = ex > emax ? ex : emax;
   }
   const int frac = fx128_frac_for(emax);
   Fx128 acc = {0, 0};
-  unsigned ovf = 0;
-  for (uint32_t i = e; i != kEndList; i = next[i]) {
-    Fx128 x = fx128_from_double(r[i].v, frac, &ovf);
-    fx128_add(acc, x);
+  for (unsigned j = 0; j < len; ++j) {
+    Fx128 t = fx128_from_double(x[j], frac, ovf);
+    fx128_add(acc, t);
   }
-  if (ovf) atomicOr(C.err, kErrAccum);
   return fx128_to_double(acc, frac);
 }
 
-// The exact sums left by long_numerator: one thread per list, the same
-// 128-bit fixed-point rule (so the same value bit for bit), written to the
-// candidate's score slot before its exact score is formed.
-__global__ void __launch_bounds__(256) k_long_sums(const ulonglong2 *fix,
-                                                   const unsigned long long *nfix,
-                                                   unsigned long long fix_cap, const double *lv,
-                                                   double *cand_score, unsigned *err) {
-  const unsigned long long n = *nfix < fix_cap ? *nfix : fix_cap;
-  for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (unsigned long long)gridDim.x * blockDim.x) {
-    const ulonglong2 f = fix[i];
-    if (f.y == ~0ull) continue;
-    const unsigned long long off = f.y >> 16, len = f.y & 0xffffull;
-    int emax = 1;
-    for (unsigned long long j = 0; j < len; ++j) {
-      const int ex = fx_exponent(lv[off + j]);
-      emax = ex > emax ? ex : emax;
-    }
-    const int frac = fx128_frac_for(emax);
-    Fx128 acc = {0, 0};
-    unsigned ovf = 0;
-    for (unsigned long long j = 0; j < len; ++j) {
-      Fx128 x = fx128_from_double(lv[off + j], frac, &ovf);
-      fx128_add(acc, x);
-    }
-    if (ovf) atomicOr(err, kErrAccum);
-    cand_score[f.x] = fx128_to_double(acc, frac);
-  }
-}
-
-// The numerator of a target with more than CAP / 32 records (a hot target),
-// formed by the whole warp: the lanes scan the tile's records for the key and
-// sum the matching values in the same 128-bit fixed-point accumulator as
-// long_numerator, then combine their partial sums (integer addition, so the
-// result is the same bit for bit); the float bound of sum |v| is formed the
-// same way, in another order, within the same error bound.  The records of
-// the target are exactly those with its key: a key met twice or more has no
-// singleton record, and screened-out records were never linked.
-template <int CAP, bool PACKED>
-__device__ __noinline__ double warp_numerator(const CellSmem<CAP, PACKED> &S, int buf, int nrec,
-                                              bool packed, uint32_t alpha, bool screened,
-                                              uint64_t key, float tau_f, float den, bool *reach,
-                                              unsigned *err) {
-  const int lane = (int)(threadIdx.x & 31u);
-  const StageRec *r = S.rec[buf];
+__device__ __forceinline__ double warp_list_sum(const double *x, unsigned len, unsigned *ovf) {
+  const unsigned lane = threadIdx.x & 31u;
   int emax = 1;
-  float sabs = 0.0f;
-  for (int i = lane; i < nrec; i += 32)
-    if (rec_key(S, buf, (uint32_t)i, packed, alpha) == key && !(screened && is_dropped(r[i].v))) {
-      const int ex = fx_exponent(r[i].v);
-      emax = ex > emax ? ex : emax;
-      sabs += abs_bound(r[i].v);
-    }
-  for (int o = 16; o; o >>= 1) {
-    const int em = __shfl_xor_sync(0xffffffffu, emax, o);
-    emax = em > emax ? em : emax;
-    sabs += __shfl_xor_sync(0xffffffffu, sabs, o);
+  for (unsigned j = lane; j < len; j += 32) {
+    const int ex = fx_exponent(x[j]);
+    emax = ex > emax ? ex : emax;
   }
-  const float df = fabsf(den);
-  if (tau_f > 0.0f && df != 0.0f && !(sabs * 1.0003f >= tau_f * df * 0.99999f)) {
-    *reach = false;
-    return 0.0;
-  }
+  emax = (int)__reduce_max_sync(0xffffffffu, (unsigned)emax);
   const int frac = fx128_frac_for(emax);
   Fx128 acc = {0, 0};
-  unsigned ovf = 0;
-  for (int i = lane; i < nrec; i += 32)
-    if (rec_key(S, buf, (uint32_t)i, packed, alpha) == key && !(screened && is_dropped(r[i].v))) {
-      Fx128 x = fx128_from_double(r[i].v, frac, &ovf);
-      fx128_add(acc, x);
-    }
+  for (unsigned j = lane; j < len; j += 32) {
+    Fx128 t = fx128_from_double(x[j], frac, ovf);
+    fx128_add(acc, t);
+  }
   for (int o = 16; o; o >>= 1) {
     Fx128 t;
     t.lo = __shfl_xor_sync(0xffffffffu, acc.lo, o);
     t.hi = __shfl_xor_sync(0xffffffffu, acc.hi, o);
     fx128_add(acc, t);
-    ovf |= __shfl_xor_sync(0xffffffffu, ovf, o);
   }
-  if (ovf && lane == 0) atomicOr(err, kErrAccum);
-  *reach = true;
   return fx128_to_double(acc, frac);
 }
 
-// Exact numerator over the record list starting at e (values of screened-out
-// records are never inserted); *reach is cleared when a list of five or more
-// cannot reach the threshold (its sum is then not formed), and *deferred is
-// set for a list longer than walk_max (left to warp_numerator).
-template <int CAP, bool PACKED>
-__device__ __forceinline__ double list_numerator(const CellSmem<CAP, PACKED> &S, int buf, uint32_t e,
-                                                 float tau_f, int walk_max, bool *reach,
-                                                 bool *deferred, unsigned long long *fix,
-                                                 const CellArgs &C) {
-  const StageRec *r = S.rec[buf];
-  const uint32_t e2 = S.next[e];
-  if (e2 == kEndList) return r[e].v;
-  // two records: IEEE addition rounds their exact sum once
-  const uint32_t e3 = S.next[e2];
-  if (e3 == kEndList) return r[e].v + r[e2].v;
-  // three or four: an order-independent FP64 sum; more: the 128-bit
-  // fixed-point accumulator anchored to the largest exponent
-  const uint32_t e4 = S.next[e3];
-  if (e4 == kEndList) return sum4_ordered(0.0, r[e].v, r[e2].v, r[e3].v);
-  if (S.next[e4] == kEndList) return sum4_ordered(r[e].v, r[e2].v, r[e3].v, r[e4].v);
-  return long_numerator(r, S.next, e, tau_f, r[e].den, walk_max, reach, deferred, fix, C);
-}
-
-template <int CAP, int THREADS, bool PACKED>
-__global__ void __launch_bounds__(THREADS) k_cells(CellArgs C) {
-  using Smem = CellSmem<CAP, PACKED>;
-  constexpr int kTab = Smem::kTab;
-  constexpr int kRPT = CAP / THREADS;  // records per thread
-  // hot targets (lists longer than CAP / 32) are summed by their warp in the
-  // large tiles; in kCap tiles one thread walks every list
-  constexpr bool kHotWarp = CAP > kCap;
-  static_assert(CAP % THREADS == 0 && kRPT <= 32, "records per thread");
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  Smem &S = *reinterpret_cast<Smem *>(smem_raw);
-  const int lane = threadIdx.x & 31;
-  const int warp_base = (int)(threadIdx.x & ~31u);
-  unsigned long long my_unique = 0, my_excl = 0;
-  for (int i = threadIdx.x; i < kTab; i += THREADS) S.slot[i] = kEmptySlot;
-  for (int i = threadIdx.x; i < kTab / 32; i += THREADS) S.psibit[0][i] = S.psibit[1][i] = 0u;
-  for (int i = threadIdx.x; i < Smem::kFilterWords; i += THREADS) S.seen[i] = S.dup[i] = 0u;
-  if (threadIdx.x == 0) S.ntargets[0] = S.ntargets[1] = 0;
-  // tiles blockIdx.x + k * gridDim.x; descriptors are read one tile ahead of
-  // the record copies, which run one tile ahead of the reduction
-  uint32_t tile = C.tile0 + blockIdx.x;
-  TileDesc d = {0, 0, 0, 0, 0, 0, 0, 0}, dn = {0, 0, 0, 0, 0, 0, 0, 0};
-  bool on = false, on_n = false;
-  if (tile < C.ntiles) {
-    d = C.tiles[tile];
-    on = tile_on_chip<CAP>(d, C.st.cap, C.err);
-    if (on) prefetch_tile(S, 0, d, C);
+__global__ void __launch_bounds__(256) k_long_sums(const ulonglong2 *fix,
+                                                   const unsigned long long *nfix,
+                                                   unsigned long long fix_cap, const double *lv,
+                                                   double *cand_score, unsigned *err) {
+  const unsigned long long n = *nfix < fix_cap ? *nfix : fix_cap;
+  unsigned ovf = 0;
+  // warp-uniform loop: long lists are summed by the whole warp
+  for (unsigned long long base = (unsigned long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
+       base < n; base += (unsigned long long)gridDim.x * blockDim.x) {
+    const unsigned long long i = base + (threadIdx.x & 31u);
+    ulonglong2 f = make_ulonglong2(0, ~0ull);
+    if (i < n) f = fix[i];
+    const bool used = f.y != ~0ull;
+    const unsigned long long len = f.y & 0xffffull;
+    if (used && len <= kWalk) cand_score[f.x] = list_sum(lv + (f.y >> 16), (unsigned)len, &ovf);
+    for (unsigned m = __ballot_sync(0xffffffffu, used && len > kWalk); m; m &= m - 1) {
+      const int src = __ffs(m) - 1;
+      const unsigned long long y = __shfl_sync(0xffffffffu, f.y, src);
+      const double s = warp_list_sum(lv + (y >> 16), (unsigned)(y & 0xffffull), &ovf);
+      if ((int)(threadIdx.x & 31u) == src) cand_score[f.x] = s;
+    }
   }
-  if (tile + gridDim.x < C.ntiles) dn = C.tiles[tile + gridDim.x];
-  int buf = 0;
-#pragma unroll 1
-  for (; tile < C.ntiles; tile += gridDim.x, buf ^= 1) {
-    TileDesc dnn = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (tile + 2 * gridDim.x < C.ntiles) dnn = C.tiles[tile + 2 * gridDim.x];
-    cp_async_wait_all();
-    __syncthreads();  // records of this tile in place; the previous tile is done
-    if (tile + gridDim.x < C.ntiles) {
-      on_n = tile_on_chip<CAP>(dn, C.st.cap, C.err);
-      if (on_n) prefetch_tile(S, buf ^ 1, dn, C);
-    } else {
-      on_n = false;
-    }
-    // psi bits of the previous tile are read by no one until the next barrier
-    for (int i = threadIdx.x; i < kTab / 32; i += THREADS) S.psibit[buf ^ 1][i] = 0u;
-    const uint32_t npsi = d.psi_hi - d.psi_lo;
-    const bool psi_local = npsi <= (uint32_t)kPsiCap;
-    const bool packed = PACKED && d.kind == kTilePacked;
-    const int nrec = on ? (int)d.npairs : 0;
-    // singleton filter: every key sets its bit; a bit met twice is marked.
-    // Thread t holds records t + k THREADS (k < kRPT); their hashes stay in
-    // registers for the insert phase, and the filter atomics of all of them
-    // are issued before any result is used.
-    uint32_t fm[kRPT], old[kRPT];
-    uint32_t live = 0;
-#pragma unroll
-    for (int k = 0; k < kRPT; ++k) {
-      const int e = (int)threadIdx.x + k * THREADS;
-      fm[k] = 0u;
-      old[k] = 0u;
-      if (e < nrec && !(C.screened && is_dropped(S.rec[buf][e].v))) {
-        live |= 1u << k;
-        fm[k] = tile_mix(rec_key(S, buf, (uint32_t)e, packed, d.alpha));
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < kRPT; ++k)
-      if ((live >> k) & 1u) {
-        const uint32_t f = fm[k] >> Smem::kFilterShift;
-        old[k] = atomicOr(&S.seen[f >> 5], 1u << (f & 31u));
-      }
-#pragma unroll
-    for (int k = 0; k < kRPT; ++k) {
-      const uint32_t f = fm[k] >> Smem::kFilterShift, bit = 1u << (f & 31u);
-      if (((live >> k) & 1u) && (old[k] & bit)) atomicOr(&S.dup[f >> 5], bit);
-    }
-    if (on && psi_local)
-      for (uint32_t q = threadIdx.x; q < npsi; q += THREADS) {
-        const uint32_t f = tile_mix(S.psik[buf][q]) >> Smem::kFilterShift;
-        const uint32_t bit = 1u << (f & 31u);
-        if (atomicOr(&S.seen[f >> 5], bit) & bit) atomicOr(&S.dup[f >> 5], bit);
-      }
-    __syncthreads();  // filters complete
-    if (on && psi_local) {
-      // psi markers: claim a slot, or flag the slot a record already holds
-      // (a marker whose filter bit is unmarked meets no record: left out)
-      for (uint32_t q = threadIdx.x; q < npsi; q += THREADS) {
-        const uint64_t key = S.psik[buf][q];
-        const uint32_t mix = tile_mix(key), f = mix >> Smem::kFilterShift;
-        if (!((S.dup[f >> 5] >> (f & 31u)) & 1u)) {
-          S.psi_slot[q] = kEndList;
-          continue;
-        }
-        uint32_t h = mix & (uint32_t)(kTab - 1);
-        uint16_t claimed = kEndList;
-        int probe = 0;
-        for (; probe < kTab; ++probe) {
-          uint32_t cur = S.slot[h];
-          if (cur == kEmptySlot) {
-            cur = atomicCAS(&S.slot[h], kEmptySlot, kPsiBit | q);
-            if (cur == kEmptySlot) {
-              claimed = (uint16_t)h;
-              break;
-            }
-          }
-          if (slot_key(S, buf, cur, packed, d.alpha) == key) break;
-          h = (h + 1) & (kTab - 1);
-        }
-        if (probe == kTab) atomicOr(C.err, kErrTile);  // cannot happen at load < 3/4
-        else atomicOr(&S.psibit[buf][h >> 5], 1u << (h & 31));
-        S.psi_slot[q] = claimed;
-      }
-    }
-    if (on) {
-      // singletons are scored and appended at once; every other record is
-      // linked into its target's list (warps append the slots they claim to
-      // the target list with one shared atomic per round)
-#pragma unroll
-      for (int k = 0; k < kRPT; ++k) {
-        const int base = k * THREADS;
-        if (base + warp_base >= nrec) break;
-        const int e = base + (int)threadIdx.x;
-        int claimed = -1;
-        bool single = false, pass1 = false;
-        uint64_t key = 0;
-        double v1 = 0.0;
-        const uint32_t mix = fm[k];
-        if ((live >> k) & 1u) {
-          key = rec_key(S, buf, (uint32_t)e, packed, d.alpha);
-          const uint32_t f = mix >> Smem::kFilterShift;
-          single = !((S.dup[f >> 5] >> (f & 31u)) & 1u);
-          if (single) {
-            ++my_unique;
-            if (!psi_local && psi_contains(C.psi_ht, C.psi_mask, key, C.err)) {
-              ++my_excl;
-            } else {
-              const StageRec r = S.rec[buf][e];
-              v1 = r.v;
-              pass1 = true;
-              if (C.tau > 0.0) {
-                bool okn;
-                const float nf = abs_as_float(r.v, &okn);
-                const float df = fabsf(r.den);
-                if (okn && df != 0.0f) pass1 = nf >= C.tau_f * df * 0.99999f;
-              }
-            }
-          }
-        }
-        {  // the singletons that pass the threshold
-          const unsigned bal = __ballot_sync(0xffffffffu, pass1);
-          if (bal) {
-            unsigned long long b0 = 0;
-            if (lane == 0) b0 = atomicAdd(C.cand_count, (unsigned long long)__popc(bal));
-            b0 = __shfl_sync(0xffffffffu, b0, 0);
-            if (pass1) {
-              const unsigned long long slotc = b0 + __popc(bal & ((1u << lane) - 1u));
-              if (slotc < C.cand_cap) {
-                C.cand_key[slotc] = key;
-                C.cand_score[slotc] = v1;  // the exact score is formed after the launch
-              }
-            }
-          }
-        }
-        if (((live >> k) & 1u) && !single) {
-          uint32_t h = mix & (uint32_t)(kTab - 1);
-          int probe = 0;
-          for (; probe < kTab; ++probe) {
-            uint32_t cur = S.slot[h];
-            if (cur == kEmptySlot) {
-              cur = atomicCAS(&S.slot[h], kEmptySlot, (uint32_t)e);
-              if (cur == kEmptySlot) {
-                S.next[e] = kEndList;
-                claimed = (int)h;
-                break;
-              }
-            }
-            if (slot_key(S, buf, cur, packed, d.alpha) == key) {
-              const uint32_t old = atomicExch(&S.slot[h], (uint32_t)e);
-              if (old & kPsiBit) {  // the first record of a psi marker's target
-                S.next[e] = kEndList;
-                claimed = (int)h;
-              } else {
-                S.next[e] = (uint16_t)old;
-              }
-              break;
-            }
-            h = (h + 1) & (kTab - 1);
-          }
-          if (probe == kTab) atomicOr(C.err, kErrTile);  // cannot happen at load < 3/4
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, claimed >= 0);
-        if (bal) {
-          uint32_t b0 = 0;
-          if (lane == 0) b0 = atomicAdd(&S.ntargets[buf], (uint32_t)__popc(bal));
-          b0 = __shfl_sync(0xffffffffu, b0, 0);
-          if (claimed >= 0) S.targets[b0 + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)claimed;
-        }
-      }
-    }
-    __syncthreads();  // lists complete
-    if (threadIdx.x == 0) S.ntargets[buf ^ 1] = 0;  // read by no one until the next barrier
-    // the filters are read by no one until the next tile's filter phase
-    for (int i = threadIdx.x; i < Smem::kFilterWords; i += THREADS) S.seen[i] = S.dup[i] = 0u;
-    if (on) {
-      // markers that no record joined are emptied by their inserting thread
-      if (psi_local)
-        for (uint32_t q = threadIdx.x; q < npsi; q += THREADS) {
-          const uint32_t h = S.psi_slot[q];
-          if (h != kEndList) {
-            const uint32_t v = S.slot[h];
-            if (v != kEmptySlot && (v & kPsiBit)) S.slot[h] = kEmptySlot;
-          }
-        }
-      // one target per thread: numerator, exclusion, threshold; the slot is
-      // emptied by its owner for the next tile
-      const int ntg = (int)S.ntargets[buf];
-      const float tau_f = C.tau > 0.0 ? C.tau_f : 0.0f;
-#pragma unroll 1
-      for (int base = 0; base + warp_base < ntg; base += THREADS) {
-        const int idx = base + (int)threadIdx.x;
-        bool live = false, deferred = false, reach = true;
-        double num = 0.0;
-        float den = 0.0f;
-        uint64_t key = 0;
-        unsigned long long fix = ~0ull;  // the list's k_long_sums entry, if its sum is left there
-        if (idx < ntg) {
-          const uint32_t h = S.targets[idx];
-          const uint32_t e = S.slot[h];
-          S.slot[h] = kEmptySlot;
-          key = rec_key(S, buf, e, packed, d.alpha);
-          ++my_unique;
-          const bool in_psi = psi_local ? ((S.psibit[buf][h >> 5] >> (h & 31)) & 1u) != 0u
-                                        : psi_contains(C.psi_ht, C.psi_mask, key, C.err);
-          if (in_psi) {
-            ++my_excl;
-          } else {
-            live = true;
-            den = S.rec[buf][e].den;
-            num = list_numerator(S, buf, e, tau_f, kHotWarp ? CAP / 32 : CAP, &reach, &deferred,
-                                 &fix, C);
-          }
-        }
-        // hot targets: each summed by the whole warp
-        if (kHotWarp)
-        for (unsigned m = __ballot_sync(0xffffffffu, deferred); m; m &= m - 1) {
-          const int src = __ffs(m) - 1;
-          bool r2 = true;
-          const double n2 = warp_numerator(S, buf, nrec, packed, d.alpha, C.screened != 0,
-                                           __shfl_sync(0xffffffffu, key, src), tau_f,
-                                           __shfl_sync(0xffffffffu, den, src), &r2, C.err);
-          if (lane == src) {
-            num = n2;
-            reach = r2;
-          }
-        }
-        bool pass = false;
-        if (live) {
-          pass = reach;
-          if (reach && C.tau > 0.0 && fix == ~0ull) {  // a deferred sum is appended untested
-            bool okn;
-            const float nf = abs_as_float(num, &okn);
-            const float df = fabsf(den);
-            if (okn && df != 0.0f) pass = nf >= C.tau_f * df * 0.99999f;  // else the exact test decides
-          }
-        }
-        const double sc = num;  // the exact score is formed after the launch (k_exact_scores)
-        const unsigned bal = __ballot_sync(0xffffffffu, pass);
-        if (bal) {
-          unsigned long long b0 = 0;
-          if (lane == 0) b0 = atomicAdd(C.cand_count, (unsigned long long)__popc(bal));
-          b0 = __shfl_sync(0xffffffffu, b0, 0);
-          if (pass) {
-            const unsigned long long slotc = b0 + __popc(bal & ((1u << lane) - 1u));
-            if (slotc < C.cand_cap) {
-              C.cand_key[slotc] = key;
-              C.cand_score[slotc] = sc;
-              if (fix != ~0ull) C.fix[fix].x = slotc;
-            } else if (fix != ~0ull) {
-              C.fix[fix].y = ~0ull;
-            }
-          }
-        }
-      }
-    }
-    d = dn;
-    dn = dnn;
-    on = on_n;
-  }
-  cp_async_wait_all();
-  for (int dl = 16; dl; dl >>= 1) {
-    my_unique += __shfl_xor_sync(0xffffffffu, my_unique, dl);
-    my_excl += __shfl_xor_sync(0xffffffffu, my_excl, dl);
-  }
-  if (lane == 0) {
-    if (my_unique) atomicAdd(C.n_unique, my_unique);
-    if (my_excl) atomicAdd(C.n_excluded, my_excl);
-  }
+  if (ovf) atomicOr(err, kErrAccum);
 }
 
 // ---------------------------------------------- oversized hash buckets ---
@@ -2506,25 +2381,28 @@ static CellArgs cell_args(const FusedCore &F, const Stage &st,
   return CA;
 }
 
-// Buffers of the exact sums that the tile kernels leave to k_long_sums, in a
-// scratch arena that outlives the launch and the fix-up that follows it,
-// sized from the launch's tiles (about seven lists of five or more records a
-// tile at (24e,30o), nine records long; with no threshold, as in ASCI-PT2,
-// every such list is deferred).  A list that finds no room is summed in the
-// tile kernel as before.
-static int enable_long_sums(CellArgs &CA, size_t ntiles, Arena &la) {
-  const unsigned long long kFixCap =
-      std::max<unsigned long long>(1ull << 20, (unsigned long long)ntiles * 8);
-  const unsigned long long kLvCap = kFixCap * 12;
+// Buffers of the targets that the tile kernels leave to k_long_sums, in a
+// scratch arena that outlives the launch and the fix-up that follows it.  With
+// a threshold few targets of several records reach it (at (24e,30o) six a
+// tile of kCap records, with 25 values), and the buffers hold 16 and 80 per
+// kCap records of capacity.  `full` gives room for every record (no threshold,
+// as in ASCI-PT2 and the first batch, where every such target is summed); a
+// launch whose buffers were too small sets kErrValues and is run again so.
+static int enable_long_sums(CellArgs &CA, size_t tiles, bool full, Arena &la) {
+  const unsigned long long t = tiles, all_fix = t * (kCap / 2), all_lv = t * kCap;
+  const unsigned long long fix_cap =
+      full ? all_fix : std::max(t * 16, std::min(all_fix, 1ull << 16));
+  const unsigned long long lv_cap = std::min<unsigned long long>(
+      full ? all_lv : std::max(t * 80, std::min(all_lv, 1ull << 18)), 0xffffffffull);
   unsigned long long *cnt;
-  ASCI_TRY(la.alloc(&CA.lv, (size_t)kLvCap));
-  ASCI_TRY(la.alloc(&CA.fix, (size_t)kFixCap));
+  ASCI_TRY(la.alloc(&CA.lv, (size_t)lv_cap));
+  ASCI_TRY(la.alloc(&CA.fix, (size_t)fix_cap));
   ASCI_TRY(la.alloc(&cnt, 2));
   ASCI_TRY_CUDA(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), la.stream()));
   CA.lv_count = cnt;
   CA.nfix = cnt + 1;
-  CA.lv_cap = kLvCap;
-  CA.fix_cap = kFixCap;
+  CA.lv_cap = lv_cap;
+  CA.fix_cap = fix_cap;
   return ASCI_OK;
 }
 
@@ -2535,6 +2413,12 @@ static int run_long_sums(const CellArgs &CA, int sms, cudaStream_t s) {
   return ASCI_OK;
 }
 
+// Tiles per launch when every record has room in the buffers of k_long_sums
+// (16 KB a tile): a quarter of the batch, between 128 MB and 2 GB of buffers.
+size_t full_tiles(size_t ntiles) {
+  return std::min<size_t>(std::max<size_t>(ntiles / 4, 8192), 131072);
+}
+
 // Reduce tiles [tile_begin, tile_end) of a staged batch on chip and append the
 // targets with |S| >= tau to the candidate buffer (at most kCap per tile).
 int fused_cells(const FusedCore &F, const void *tiles, const uint64_t *psi_list,
@@ -2542,7 +2426,7 @@ int fused_cells(const FusedCore &F, const void *tiles, const uint64_t *psi_list,
                 uint64_t *cand_key, double *cand_score,
                 unsigned long long *cand_count, unsigned long long cand_cap,
                 unsigned long long *n_unique, unsigned long long *n_excluded, unsigned *err,
-                Arena &arena) {
+                bool full, Arena &arena) {
   if (tile_end <= tile_begin) return ASCI_OK;
   cudaStream_t s = arena.stream();
   CellArgs CA = cell_args(F, st, tau, cand_key, cand_score, cand_count, cand_cap, n_unique,
@@ -2551,14 +2435,14 @@ int fused_cells(const FusedCore &F, const void *tiles, const uint64_t *psi_list,
   CA.psi_list = psi_list;
   CA.tile0 = tile_begin;
   CA.ntiles = tile_end;
-  const size_t cell_smem = sizeof(TileSmem);
+  const size_t cell_smem = sizeof(CellSmem<kCap>);
   // once (thread-safe static initialisation): attribute and occupancy
   static const int per_sm = [cell_smem]() {
     int p = 0;
-    if (cudaFuncSetAttribute(k_cells<kCap, kCellThreads, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(k_cells<kCap, kCellThreads, kCellCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)cell_smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &p, k_cells<kCap, kCellThreads, true>, kCellThreads, cell_smem) !=
+                &p, k_cells<kCap, kCellThreads, kCellCtas>, kCellThreads, cell_smem) !=
             cudaSuccess)
       return 0;
     return p < 1 ? 1 : p;
@@ -2574,8 +2458,8 @@ int fused_cells(const FusedCore &F, const void *tiles, const uint64_t *psi_list,
   const unsigned grid = (unsigned)std::min<size_t>((size_t)sms * per, tile_end - tile_begin);
   ASCI_TRACE("cells: launch grid=%u smem=%zu per_sm=%d", grid, cell_smem, per_sm);
   Arena la(s);
-  ASCI_TRY(enable_long_sums(CA, tile_end - tile_begin, la));
-  k_cells<kCap, kCellThreads, true><<<grid, kCellThreads, cell_smem, s>>>(CA);
+  ASCI_TRY(enable_long_sums(CA, tile_end - tile_begin, full, la));
+  k_cells<kCap, kCellThreads, kCellCtas><<<grid, kCellThreads, cell_smem, s>>>(CA);
   ASCI_CHECK_LAUNCH();
   ASCI_TRY(run_long_sums(CA, sms, s));
   return ASCI_OK;
@@ -2602,16 +2486,15 @@ int tile_info(const void *tiles, const std::vector<uint32_t> &list, const Spill 
 }
 
 // Launch the tile kernel of one size over tiles [t0, t1) of CA.tiles.
-template <int CAP, int THREADS>
+template <int CAP, int THREADS, int CTAS>
 static int launch_big_cells(CellArgs CA, uint32_t t0, uint32_t t1, int sms, cudaStream_t s) {
   if (t1 <= t0) return ASCI_OK;
-  using Smem = CellSmem<CAP, false>;
-  const size_t smem = sizeof(Smem);
+  const size_t smem = sizeof(CellSmem<CAP>);
   static const int per_sm = [smem]() {
     int p = 0;
-    if (cudaFuncSetAttribute(k_cells<CAP, THREADS, false>,
+    if (cudaFuncSetAttribute(k_cells<CAP, THREADS, CTAS>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k_cells<CAP, THREADS, false>, THREADS,
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k_cells<CAP, THREADS, CTAS>, THREADS,
                                                       smem) != cudaSuccess)
       return 0;
     return p < 1 ? 1 : p;
@@ -2623,7 +2506,7 @@ static int launch_big_cells(CellArgs CA, uint32_t t0, uint32_t t1, int sms, cuda
   CA.tile0 = t0;
   CA.ntiles = t1;
   const unsigned grid = (unsigned)std::min<size_t>((size_t)sms * per_sm, t1 - t0);
-  k_cells<CAP, THREADS, false><<<grid, THREADS, smem, s>>>(CA);
+  k_cells<CAP, THREADS, CTAS><<<grid, THREADS, smem, s>>>(CA);
   ASCI_CHECK_LAUNCH();
   return ASCI_OK;
 }
@@ -2638,7 +2521,7 @@ int fused_big_cells(const FusedCore &F, const void *tiles, const uint64_t *psi_l
                     const Stage &st, const Spill &spill, double tau, uint64_t *cand_key,
                     double *cand_score, unsigned long long *cand_count,
                     unsigned long long cand_cap, unsigned long long *n_unique,
-                    unsigned long long *n_excluded, unsigned *err, uint64_t *nrec_out,
+                    unsigned long long *n_excluded, unsigned *err, bool full, uint64_t *nrec_out,
                     Arena &arena) {
   cudaStream_t s = arena.stream();
   *nrec_out = 0;
@@ -2694,9 +2577,9 @@ int fused_big_cells(const FusedCore &F, const void *tiles, const uint64_t *psi_l
   int dev = 0, sms = 152;
   ASCI_TRY_CUDA(cudaGetDevice(&dev));
   ASCI_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  ASCI_TRY(enable_long_sums(CA, nt * 4, ta));
-  ASCI_TRY((launch_big_cells<kMidCap, kMidThreads>(CA, 0, (uint32_t)nmid, sms, s)));
-  ASCI_TRY((launch_big_cells<kBigCap, kBigThreads>(CA, (uint32_t)nmid, (uint32_t)nt, sms, s)));
+  ASCI_TRY(enable_long_sums(CA, nt * (kBigCap / kCap), full, ta));
+  ASCI_TRY((launch_big_cells<kMidCap, kMidThreads, 4>(CA, 0, (uint32_t)nmid, sms, s)));
+  ASCI_TRY((launch_big_cells<kBigCap, kBigThreads, 2>(CA, (uint32_t)nmid, (uint32_t)nt, sms, s)));
   ASCI_TRY(run_long_sums(CA, sms, s));
   ASCI_TRY_CUDA(cudaStreamSynchronize(s));  // the host vectors above are read by copies
   return ASCI_OK;

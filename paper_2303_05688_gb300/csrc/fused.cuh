@@ -47,6 +47,10 @@ struct Spill {
   uint32_t n;
 };
 
+// Bit of the device error word: the values of the targets to be summed found
+// no room (the launch is run again with room for all of them).
+constexpr unsigned kErrValues = 32u;
+
 // Everything the batch kernels read that stays fixed during one search.
 struct FusedCore {
   DevInts I;

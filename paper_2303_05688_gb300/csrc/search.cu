@@ -62,7 +62,7 @@ int fused_big_cells(const FusedCore &F, const void *tiles, const uint64_t *psi_l
                     const Spill &spill, double tau, uint64_t *cand_key, double *cand_score,
                     unsigned long long *cand_count, unsigned long long cand_cap,
                     unsigned long long *n_unique, unsigned long long *n_excluded, unsigned *err,
-                    uint64_t *nrec_out, Arena &arena);
+                    bool full, uint64_t *nrec_out, Arena &arena);
 int fused_big_tiles(const FusedCore &F, const uint32_t *info, size_t nt, const Stage &st,
                     const Spill &spill, double tau,
                     uint64_t *cand_key, double *cand_score, unsigned long long *cand_count,
@@ -74,7 +74,8 @@ int fused_cells(const FusedCore &F, const void *tiles, const uint64_t *psi_list,
                 uint64_t *cand_key, double *cand_score,
                 unsigned long long *cand_count, unsigned long long cand_cap,
                 unsigned long long *n_unique, unsigned long long *n_excluded, unsigned *err,
-                Arena &arena);
+                bool full, Arena &arena);
+size_t full_tiles(size_t ntiles);
 size_t tile_capacity();
 size_t big_tile_capacity();
 int exact_scores(const FusedCore &F, const uint64_t *key, double *score, size_t n,
@@ -911,6 +912,37 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
     ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
     return ASCI_OK;
   };
+  // The counters before a tile launch: when its values found no room (rare: a
+  // low threshold over crowded targets), they are put back and the launch, and
+  // those after it, run with room for every record, fewer tiles at a time.
+  unsigned long long hcount[3] = {0, 0, 0};
+  bool values_full = false;
+  auto read_counts = [&](bool full, const char *what, bool *again) -> int {
+    unsigned long long c[3];
+    unsigned he = 0;
+    *again = false;
+    ASCI_TRY_CUDA(cudaMemcpyAsync(c, dcount, sizeof(c), cudaMemcpyDefault, stream));
+    ASCI_TRY_CUDA(cudaMemcpyAsync(&he, derr2, sizeof(he), cudaMemcpyDefault, stream));
+    ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
+    if (he == kErrValues && !full) {
+      ASCI_TRACE("%s: values found no room; again with room for all", what);
+      values_full = *again = true;
+      hcount[0] = pool_n;
+      ASCI_TRY_CUDA(cudaMemsetAsync(derr2, 0, sizeof(unsigned), stream));
+      ASCI_TRY_CUDA(cudaMemcpyAsync(dcount, hcount, sizeof(hcount), cudaMemcpyDefault, stream));
+      ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
+      return ASCI_OK;
+    }
+    if (he) {
+      char msg[96];
+      snprintf(msg, sizeof(msg), "%s check failed (flags 0x%x)", what, he);
+      record_error(msg, __FILE__, __LINE__);
+      return ASCI_ECUDA;
+    }
+    if (c[0] > pool_cap) return ASCI_ECUDA;  // cannot happen: room bounds the appends
+    for (int i = 0; i < 3; ++i) hcount[i] = c[i];
+    return ASCI_OK;
+  };
   for (const Batch &b : batches) {
     Arena ba(stream);  // scratch of this batch, released when the batch ends
     uint32_t gg[2];
@@ -949,27 +981,19 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
         room = (pool_cap - pool_n) / tile_capacity();
         if (room == 0) return ASCI_ENOMEM;
       }
-      const size_t t1 = std::min(ntiles, t + room);
+      const bool full = tau <= 0.0 || values_full;
+      const size_t t1 = std::min(ntiles, t + (full ? std::min(room, full_tiles(ntiles)) : room));
       ASCI_TRACE("cells: tiles [%zu,%zu) tau=%.6g pool=%zu", t, t1, tau, pool_n);
       ktm.start();
       ASCI_TRY(fused_cells(F, tiles, psi_list, (uint32_t)t, (uint32_t)t1, stg, tau,
                            pool_k[pcur], pool_s[pcur], dcount, pool_cap, dcount + 1, dcount + 2,
-                           derr2, ba));
+                           derr2, full, ba));
       ktm.stop(&tl[3]);
       ++tile_launches;
-      unsigned long long c = 0;
-      unsigned he = 0;
-      ASCI_TRY_CUDA(cudaMemcpyAsync(&c, dcount, sizeof(c), cudaMemcpyDefault, stream));
-      ASCI_TRY_CUDA(cudaMemcpyAsync(&he, derr2, sizeof(he), cudaMemcpyDefault, stream));
-      ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
-      if (he) {
-        char msg[96];
-        snprintf(msg, sizeof(msg), "constraint-tile kernel check failed (flags 0x%x)", he);
-        record_error(msg, __FILE__, __LINE__);
-        return ASCI_ECUDA;
-      }
-      if (c > pool_cap) return ASCI_ECUDA;  // cannot happen: room bounds the appends
-      ASCI_TRY(consume(c));
+      bool again = false;
+      ASCI_TRY(read_counts(full, "constraint-tile kernel", &again));
+      if (again) continue;
+      ASCI_TRY(consume(hcount[0]));
       t = t1;
       if (pool_n > N && (pool_cap - pool_n) < pool_cap / 2) {
         tm.stop(&tl[5]);
@@ -1011,33 +1035,26 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
           }
           uint64_t room = pool_cap - pool_n, total = 0;
           size_t j = i;
-          while (j < cnt && total + recs(j) <= room) total += recs(j++);
+          const bool full = tau <= 0.0 || values_full;
+          const size_t most = pass == 0 && full ? i + full_tiles(0) / 4 : cnt;
+          while (j < cnt && j < most && total + recs(j) <= room) total += recs(j++);
           uint64_t nrec = 0;
           ktm.start();
           if (pass == 0)
             ASCI_TRY(fused_big_cells(F, tiles, psi_list, big_list.data() + i, inf.data() + 5 * i,
                                      j - i, stg, spill, tau, pool_k[pcur], pool_s[pcur], dcount,
-                                     pool_cap, dcount + 1, dcount + 2, derr2, &nrec, ba));
+                                     pool_cap, dcount + 1, dcount + 2, derr2, full, &nrec, ba));
           else
             ASCI_TRY(fused_big_tiles(F, inf.data() + 5 * i, j - i, stg, spill, tau, pool_k[pcur],
                                      pool_s[pcur], dcount, pool_cap, dcount + 1, dcount + 2,
                                      derr2, &nrec, ba));
           ktm.stop(&tl[4]);
+          bool again = false;
+          ASCI_TRY(read_counts(full || pass == 1, "oversized-tile reduction", &again));
+          if (again) continue;
           oversized_records += nrec;
           if (pass == 0) big_records += nrec;
-          unsigned long long c = 0;
-          unsigned he = 0;
-          ASCI_TRY_CUDA(cudaMemcpyAsync(&c, dcount, sizeof(c), cudaMemcpyDefault, stream));
-          ASCI_TRY_CUDA(cudaMemcpyAsync(&he, derr2, sizeof(he), cudaMemcpyDefault, stream));
-          ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
-          if (he) {
-            char msg[96];
-            snprintf(msg, sizeof(msg), "oversized-tile reduction check failed (flags 0x%x)", he);
-            record_error(msg, __FILE__, __LINE__);
-            return ASCI_ECUDA;
-          }
-          if (c > pool_cap) return ASCI_ECUDA;
-          ASCI_TRY(consume(c));
+          ASCI_TRY(consume(hcount[0]));
           ASCI_TRACE("oversized tiles (%s): [%zu,%zu) %llu records, pool=%zu",
                      pass == 0 ? "on chip" : "global", i, j, (unsigned long long)nrec, pool_n);
           i = j;
