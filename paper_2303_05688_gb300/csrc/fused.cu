@@ -119,6 +119,55 @@ __global__ void k_fx_single_tables(const double *h1, const double *eri, int n, i
   }
 }
 
+// Same-spin terms within the orbitals of m (with h_pp) and between m and r.
+__device__ int64_t chunk_within(const int64_t *hh, const int64_t *jk, int n, uint32_t m) {
+  int64_t v = 0;
+  for (; m; m &= m - 1) {
+    const int p = __ffs(m) - 1;
+    v += hh[p];
+    for (uint32_t r = m & (m - 1); r; r &= r - 1) v += jk[p * n + __ffs(r) - 1];
+  }
+  return v;
+}
+__device__ int64_t chunk_between(const int64_t *t, int n, uint32_t m, uint32_t r0) {
+  int64_t v = 0;
+  for (; m; m &= m - 1)
+    for (uint32_t r = r0; r; r &= r - 1) v += t[(__ffs(m) - 1) * n + __ffs(r) - 1];
+  return v;
+}
+
+// One table per blockIdx.y: the chunk pairs of xs, then the nc x nc tables of xo.
+__global__ void k_fx_chunks(const int64_t *hh, const int64_t *jk, const int64_t *jj, int n, int nc,
+                            int cb, int64_t *xs, int64_t *xo) {
+  const int npair = nc * (nc - 1) / 2;
+  const uint32_t mask = (1u << cb) - 1u, full = n >= 32 ? 0xffffffffu : ((1u << n) - 1u);
+  const int t = (int)blockIdx.y;
+  int k = 0, l = 1;
+  if (t < npair) {
+    for (int i = 0; i < t; ++i)
+      if (++l == nc) l = ++k + 1;
+  } else {
+    k = (t - npair) / nc;
+    l = (t - npair) % nc;
+  }
+  int64_t *out = t < npair ? xs + ((size_t)t << (2 * cb)) : xo + ((size_t)(t - npair) << (2 * cb));
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < 1u << (2 * cb);
+       i += gridDim.x * blockDim.x) {
+    // bits at or above n (in the last chunk) belong to no orbital
+    const uint32_t x = ((i >> cb) << (k * cb)) & full;
+    const uint32_t y = (uint32_t)((uint64_t)(i & mask) << (l * cb)) & full;
+    int64_t v;
+    if (t >= npair) {
+      v = chunk_between(jj, n, x, y);
+    } else {
+      v = chunk_between(jk, n, x, y);
+      if (k == 0) v += chunk_within(hh, jk, n, y);
+      if (k == 0 && l == 1) v += chunk_within(hh, jk, n, x);
+    }
+    out[i] = v;
+  }
+}
+
 }  // namespace
 
 // x * 2^-s rounded to the nearest double (ties to even), by integer
@@ -1980,6 +2029,19 @@ int build_fx(const double *h1, const double *eri, int n, int na, int nb, double 
   X.hh = hh;
   X.jk = jk;
   X.jj = jj;
+  // chunk tables of the diagonal: at most 8 bits a chunk, at least two chunks
+  X.nc = std::max(2, (n + 7) / 8);
+  X.cb = (n + X.nc - 1) / X.nc;
+  const int npair = X.nc * (X.nc - 1) / 2;
+  const size_t tab = (size_t)1 << (2 * X.cb);
+  int64_t *xs, *xo;
+  ASCI_TRY(arena.alloc(&xs, npair * tab));
+  ASCI_TRY(arena.alloc(&xo, X.nc * X.nc * tab));
+  k_fx_chunks<<<dim3((unsigned)((tab + 255) / 256), npair + X.nc * X.nc), 256, 0, s>>>(
+      hh, jk, jj, n, X.nc, X.cb, xs, xo);
+  ASCI_CHECK_LAUNCH();
+  X.xs = xs;
+  X.xo = xo;
   *out = X;
   *E0_x = llrint(ldexp(E0, sc));
   return ASCI_OK;
@@ -2662,13 +2724,13 @@ namespace {
 // at most three limbs; bits below the grid are truncated).  Integer addition
 // is exact and associative, so the sum does not depend on the order of the
 // terms, on the batches or on the tiles: the result is a function of the set
-// of targets.  Per-thread limb sums are reduced over the warp and the block,
-// then added to the counters with one atomic per limb and block; a launch
-// holds fewer than 2^31 terms, so no counter overflows.
+// of targets.  Per-thread limb sums in shared memory are reduced over the
+// block, then added to the counters with one atomic per limb and block; a
+// launch holds fewer than 2^31 terms, so no counter overflows.
 constexpr int kPt2Limbs = 8;
 constexpr int kPt2Grid = 216;  // the grid is 2^-216
 
-__device__ __forceinline__ void pt2_add(double t, long long *acc, unsigned *bad) {
+__device__ __forceinline__ void pt2_add(double t, long long (*acc)[256], unsigned *bad) {
   if (t == 0.0) return;
   if (!(fabs(t) < 0x1p40)) {  // also catches NaN and infinities
     *bad = 1u;
@@ -2687,120 +2749,86 @@ __device__ __forceinline__ void pt2_add(double t, long long *acc, unsigned *bad)
   const unsigned long long lo = m << o;
   const unsigned long long hi = o ? (m >> (64 - o)) : 0ull;
   const long long sg = t < 0.0 ? -1 : 1;
-  const long long l0 = sg * (long long)(lo & 0xffffffffull), l1 = sg * (long long)(lo >> 32),
-                  l2 = sg * (long long)(hi & 0xffffffffull);
-  // selects, not indexing, so that acc stays in registers
-#pragma unroll
-  for (int k = 0; k < kPt2Limbs; ++k)
-    acc[k] += k == k0 ? l0 : (k == k0 + 1 ? l1 : (k == k0 + 2 ? l2 : 0ll));
+  // |t| < 2^40: k0 + 2 is at most the last limb, or hi is zero
+  acc[k0][threadIdx.x] += sg * (long long)(lo & 0xffffffffull);
+  if (k0 + 1 < kPt2Limbs) acc[k0 + 1][threadIdx.x] += sg * (long long)(lo >> 32);
+  if (k0 + 2 < kPt2Limbs) acc[k0 + 2][threadIdx.x] += sg * (long long)hi;
 }
 
-// The exact fixed-point H_ii of the 32 targets of a warp (lanes with live
-// false take no part), equal bit for bit to fx_diag.  Targets of one tile
-// mostly share their alpha string, so the alpha part is formed once per
-// distinct alpha string of the warp (at most four; any others take fx_diag):
-// D_a = sum_{p in A} h_pp + sum_{p<r in A} jk_pr by the lanes p of A, and
-// J_A[q] = sum_{p in A} jj_pq by lane q; each lane then adds its beta part
-// sum_{q in B} (h_qq + J_A[q]) + sum_{q<r in B} jk_qr.
-__device__ __forceinline__ int64_t warp_diag(const FxInts &X, uint32_t A, uint32_t B,
-                                             bool live) {
-  const int n = X.n;
-  const uint32_t lane = threadIdx.x & 31u;
-  int64_t diag = 0;
-  uint32_t pending = __ballot_sync(0xffffffffu, live);
-  const int nbmax = (int)__reduce_max_sync(0xffffffffu, live ? (unsigned)__popc(B) : 0u);
-  for (int round = 0; pending && round < 4; ++round) {
-    const uint32_t AL = __shfl_sync(0xffffffffu, A, __ffs(pending) - 1);
-    int64_t part = 0, ja = 0;
-    if ((int)lane < n) {
-      if ((AL >> lane) & 1u) {
-        part = X.hh[lane];
-        for (uint32_t r = AL & ~((2u << lane) - 1u); r; r &= r - 1)
-          part += X.jk[lane * n + __ffs(r) - 1];
-      }
-      for (uint32_t p = AL; p; p &= p - 1) ja += X.jj[(__ffs(p) - 1) * n + lane];
-    }
-    for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    const bool mine = live && A == AL && ((pending >> lane) & 1u);
-    const uint32_t group = __ballot_sync(0xffffffffu, mine);
-    // each lane reads J_A[q] from lane q for the occupied beta orbitals q of
-    // its own B (every round is taken by the whole warp)
-    int64_t cross = 0;
-    uint32_t mB = B;
-    for (int it = 0; it < nbmax; ++it) {
-      const bool has = mB != 0u;
-      const int q = has ? __ffs(mB) - 1 : 0;
-      mB &= mB - 1u;
-      const int64_t t = __shfl_sync(0xffffffffu, ja, q);
-      if (mine && has) cross += t;
-    }
-    if (mine) {
-      int64_t s = X.ecore_x + part + cross;
-      for (uint32_t m = B; m; m &= m - 1) {
-        const int q = __ffs(m) - 1;
-        s += X.hh[q];
-        for (uint32_t r = m & (m - 1); r; r &= r - 1) s += X.jk[q * n + __ffs(r) - 1];
-      }
-      diag = s;
-    }
-    pending &= ~group;
+// The exact fixed-point H_ii of a target from the chunk tables of FxInts
+// (equal bit for bit to fx_diag: integer sums): 28 loads at 25 to 32 orbitals,
+// 15 at 17 to 24 and 6 below, against some 300 terms at (24e,30o).  The
+// tables (12 MB at 30 orbitals, built in a few microseconds) stay in L2, and
+// the rows that the targets of one alpha string share in L1.  Before, the
+// terms were added one by one, the alpha part once per alpha string of a warp:
+// ASCI-PT2 of 4000 determinants at (24e,30o) took 47.0 ms against 21.0, a
+// (24e,30o) search 223.4 against 214.8.
+template <int NC>
+__device__ __forceinline__ int64_t table_diag(const FxInts &X, uint32_t A, uint32_t B) {
+  const int cb = X.cb;
+  const uint32_t mask = (1u << cb) - 1u;
+  uint32_t a[NC], b[NC];
+#pragma unroll
+  for (int k = 0; k < NC; ++k) {
+    a[k] = (A >> (k * cb)) & mask;
+    b[k] = (B >> (k * cb)) & mask;
   }
-  if (live && ((pending >> lane) & 1u)) diag = fx_diag(X, A, B);
-  return diag;
+  int64_t s = X.ecore_x;
+  uint32_t t = 0;
+#pragma unroll
+  for (int k = 0; k < NC; ++k)
+#pragma unroll
+    for (int l = k + 1; l < NC; ++l, t += 1u << (2 * cb))
+      s += __ldg(X.xs + (t | (a[k] << cb) | a[l])) + __ldg(X.xs + (t | (b[k] << cb) | b[l]));
+  t = 0;
+#pragma unroll
+  for (int k = 0; k < NC; ++k)
+#pragma unroll
+    for (int l = 0; l < NC; ++l, t += 1u << (2 * cb)) s += __ldg(X.xo + (t | (a[k] << cb) | b[l]));
+  return s;
 }
 
 // Exact scores of appended candidates, which hold their numerator:
-// S = num / (E0 - H_ii), with H_ii summed in fixed point (exact; warp_diag
-// shares the alpha part among the warp's candidates, which come from a few
-// tiles and mostly share their alpha string) and E0 - H_ii rounded once to a
-// double.
+// S = num / (E0 - H_ii), with H_ii summed in fixed point (exact) and E0 - H_ii
+// rounded once to a double.
+template <int NC>
 __global__ void __launch_bounds__(256) k_exact_scores(const uint64_t *key, double *score, size_t n,
                                                       FxInts X, int64_t E0_x, double inv_scale) {
-  // warp-uniform loop: warp_diag needs every lane
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
-  for (size_t base = (size_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < n;
-       base += stride) {
-    const size_t i = base + (threadIdx.x & 31u);
-    const bool live = i < n;
-    const uint64_t k = live ? key[i] : 0ull;
-    const int64_t dg = warp_diag(X, key_alpha(k), (uint32_t)(k >> 32), live);
-    if (live) score[i] = score[i] / (__ll2double_rn(E0_x - dg) * inv_scale);
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (size_t)gridDim.x * blockDim.x) {
+    const uint64_t k = key[i];
+    const int64_t dg = table_diag<NC>(X, key_alpha(k), (uint32_t)(k >> 32));
+    score[i] = score[i] / (__ll2double_rn(E0_x - dg) * inv_scale);
   }
 }
 
+template <int NC>
 __global__ void __launch_bounds__(256) k_pt2_terms(const uint64_t *key, const double *num,
                                                    size_t n, FxInts X, int64_t E0_x,
                                                    double inv_scale, long long *limbs,
                                                    unsigned *err) {
-  __shared__ long long red[8][kPt2Limbs];
-  long long acc[kPt2Limbs];
-  for (int k = 0; k < kPt2Limbs; ++k) acc[k] = 0;
+  // limb sums of each thread, thread-contiguous so that any limbs are free of
+  // bank conflicts
+  __shared__ long long acc[kPt2Limbs][256];
+  for (int k = 0; k < kPt2Limbs; ++k) acc[k][threadIdx.x] = 0;
   unsigned bad = 0;
-  // warp-uniform loop: warp_diag needs every lane
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
-  for (size_t base = (size_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < n;
-       base += stride) {
-    const size_t i = base + (threadIdx.x & 31u);
-    const bool live = i < n;
-    const uint64_t k = live ? key[i] : 0ull;
-    const int64_t dg = warp_diag(X, key_alpha(k), (uint32_t)(k >> 32), live);
-    if (!live) continue;
-    const double den = __ll2double_rn(E0_x - dg) * inv_scale;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (size_t)gridDim.x * blockDim.x) {
+    const uint64_t k = key[i];
     const double v = num[i];
+    const int64_t dg = table_diag<NC>(X, key_alpha(k), (uint32_t)(k >> 32));
+    const double den = __ll2double_rn(E0_x - dg) * inv_scale;
     const double r = (fabs(den) >= 1e-30 && fabs(den) <= 1e30) ? recip_fast(den) : 1.0 / den;
     pt2_add(v * v * r, acc, &bad);
   }
   if (bad) atomicOr(err, kErrAccum);
-  for (int k = 0; k < kPt2Limbs; ++k)
-    for (int o = 16; o; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
-  if ((threadIdx.x & 31) == 0)
-    for (int k = 0; k < kPt2Limbs; ++k) red[threadIdx.x >> 5][k] = acc[k];
   __syncthreads();
-  if (threadIdx.x < kPt2Limbs) {
-    long long t = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w][threadIdx.x];
-    if (t) atomicAdd((unsigned long long *)&limbs[threadIdx.x], (unsigned long long)t);
-  }
+  const int k = threadIdx.x >> 5;  // a warp per limb
+  long long t = 0;
+  for (int j = threadIdx.x & 31; j < 256; j += 32) t += acc[k][j];
+  for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if ((threadIdx.x & 31) == 0 && t)
+    atomicAdd((unsigned long long *)&limbs[k], (unsigned long long)t);
 }
 
 // The counters as one double: the limbs in a fixed order, low to high.
@@ -2816,8 +2844,8 @@ __global__ void k_pt2_value(const long long *limbs, double *out) {
 int pt2_terms(const FusedCore &F, const uint64_t *key, const double *num, size_t n,
               long long *limbs, unsigned *err, cudaStream_t s) {
   if (!n) return ASCI_OK;
-  k_pt2_terms<<<grid_for(n, 152 * 8), 256, 0, s>>>(key, num, n, F.X, F.E0_x,
-                                                   ldexp(1.0, -F.X.s), limbs, err);
+  auto *k = F.X.nc == 2 ? k_pt2_terms<2> : (F.X.nc == 3 ? k_pt2_terms<3> : k_pt2_terms<4>);
+  k<<<grid_for(n, 152 * 8), 256, 0, s>>>(key, num, n, F.X, F.E0_x, ldexp(1.0, -F.X.s), limbs, err);
   ASCI_CHECK_LAUNCH();
   return ASCI_OK;
 }
@@ -2831,8 +2859,9 @@ int pt2_value(const long long *limbs, double *out, cudaStream_t s) {
 int exact_scores(const FusedCore &F, const uint64_t *key, double *score, size_t n,
                  cudaStream_t s) {
   if (!n) return ASCI_OK;
-  k_exact_scores<<<grid_for(n, 152 * 32), 256, 0, s>>>(key, score, n, F.X, F.E0_x,
-                                                      ldexp(1.0, -F.X.s));
+  auto *k = F.X.nc == 2 ? k_exact_scores<2>
+                        : (F.X.nc == 3 ? k_exact_scores<3> : k_exact_scores<4>);
+  k<<<grid_for(n, 152 * 32), 256, 0, s>>>(key, score, n, F.X, F.E0_x, ldexp(1.0, -F.X.s));
   ASCI_CHECK_LAUNCH();
   return ASCI_OK;
 }

@@ -18,6 +18,13 @@ struct FxInts {
   // h1x = h_ia, ssx[(i*n+a)*n+k] = (ia|kk) - (ik|ka), sox[(i*n+a)*n+k] = (ia|kk)
   int s1;
   const int64_t *h1x, *ssx, *sox;
+  // the diagonal by lookups: a string is cut into nc chunks of cb bits, and
+  // xs (one table of 2^cb x 2^cb per pair of chunks k < l, in the order 01, 02,
+  // ..., 12, ...) holds the same-spin terms between the chunks, the terms within
+  // a chunk and its h_pp folded into the first pair that has it; xo (nc x nc
+  // tables) the opposite-spin terms between an alpha and a beta chunk
+  int nc, cb;
+  const int64_t *xs, *xo;
 };
 
 // One staged pair (16 bytes, written with one vector store): the value
