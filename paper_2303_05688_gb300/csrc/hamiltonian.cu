@@ -17,11 +17,10 @@
 //    the row, a fixed shuffle tree: the same bits on every call.
 //  * Davidson (Algorithm 5): basis V and products W = H V resident on the
 //    device, the subspace matrix V^T H V grown one column per product, its
-//    eigenpairs by parallel-order Jacobi in one CTA (FP32 sweeps refined by
-//    FP64 sweeps), the shifted Jacobi
-//    preconditioner, two passes of classical Gram-Schmidt, a thick restart
-//    (the four lowest Ritz vectors) at the subspace limit.  Every reduction
-//    has a fixed order.
+//    lowest eigenpairs by FP32 Jacobi refined in FP64 in one CTA, the shifted
+//    Jacobi preconditioner, two passes of classical Gram-Schmidt, a thick
+//    restart (the four lowest Ritz vectors) at the subspace limit.  Every
+//    reduction has a fixed order.
 //  * The ASCI loop itself: search, merge, build, diagonalise, repeat.
 #include <algorithm>
 #include <cmath>
@@ -392,7 +391,8 @@ HamGeom ham_geom(uint32_t n) {
 
 __global__ void k_spmv(const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
                        const double *__restrict__ val, uint32_t n, const double *__restrict__ x,
-                       double *__restrict__ y) {
+                       double *__restrict__ y, const int *stop) {
+  if (stop && *stop) return;
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
   for (uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
@@ -446,57 +446,282 @@ __global__ void __launch_bounds__(kDotThreads) k_dots(const double *V, size_t ld
   }
 }
 
-// out = base * sb + sum_k coef[k] * sc * V_k (base nullable).
-__global__ void k_combine(const double *V, size_t ld, int m, const double *coef, double sc,
-                          const double *base, double sb, size_t n, double *out) {
+// out = sum_k coef[k] scale[k] V_k
+__global__ void k_combine(const double *V, size_t ld, int m, const double *coef,
+                          const double *scale, size_t n, double *out) {
   __shared__ double cf[kMaxSub];
-  for (int k = threadIdx.x; k < m; k += blockDim.x) cf[k] = coef[k] * sc;
+  for (int k = threadIdx.x; k < m; k += blockDim.x) cf[k] = coef[k] * scale[k];
   __syncthreads();
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (size_t)gridDim.x * blockDim.x) {
-    double s = base ? base[i] * sb : 0.0;
+    double s = 0.0;
     for (int k = 0; k < m; ++k) s = fma(cf[k], V[(size_t)k * ld + i], s);
     out[i] = s;
   }
 }
 
-// x = V c and wx = W c in one pass (c = the lowest Ritz vector's coefficients).
-__global__ void k_ritz(const double *V, const double *W, size_t ld, int m, const double *coef,
-                       size_t n, double *x, double *wx) {
-  __shared__ double cf[kMaxSub];
-  for (int k = threadIdx.x; k < m; k += blockDim.x) cf[k] = coef[k];
-  __syncthreads();
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x) {
-    double a = 0.0, b = 0.0;
-    for (int k = 0; k < m; ++k) {
-      a = fma(cf[k], V[(size_t)k * ld + i], a);
-      b = fma(cf[k], W[(size_t)k * ld + i], b);
+// State of a Davidson solve on the device.  The host enqueues several
+// iterations at a time; once `stop` is set, the kernels of the iterations
+// behind it return at once, so the basis, its size and the coefficients stay
+// those of the iteration that stopped.
+//
+// A basis vector is kept as the correction it was made from, with its factor:
+// v_j = scale[j] T_j, W_j = H T_j, so no pass over the vectors normalises them.
+enum : int { kStopConverged = 1, kStopSpent = 2, kStopBad = 3 };  // spent: nothing left to add
+struct DavState {
+  int stop;
+  int iter;      // products performed when the last residual was formed
+  double theta;  // lowest Ritz value
+  double res2;   // |H x - theta x|^2
+  double scale[kMaxSub + 1];
+};
+
+constexpr int kPassThreads = 128;
+constexpr int kPassBlocks = 304;  // at most: two per SM
+
+// One pass over the vectors, an element per thread and step.  Each mode forms
+// per-element values and sums over the elements (in registers per thread, then
+// over the block, then by the last block over the blocks: a fixed order, so the
+// same bits on every call):
+//   kProject  sums j < m: T_j . W_(m-1): the new column of v^T H v, written to
+//             row and column m - 1 of Hs
+//   kRitz     x = v c, H x = W c, r = H x - theta x, t = r / (theta - H_ii)
+//             (the denominator kept at least 1e-8 in magnitude; t = r when
+//             unpreconditioned); sums j < m: T_j . t, and r . r
+//   kRestart  the same with T, W replaced in place by the `keep` lowest Ritz
+//             vectors and their products; sums k < keep: T_k . t, and r . r
+//   kOrth1    t -= v h; sums j < m: T_j . t (for the second pass)
+//   kOrth2    t -= v h; sum t . t
+// t is the next basis vector's place.  A pass reads its vectors once (from L2
+// at 50,000 determinants) with all loads of an element in flight, and takes up
+// to 3 m FP64 operations per element; 8 to 17 us at 50,000 elements, half of it
+// the launch and the tail of the sums.  With the subspace solve below, a
+// product costs 6 launches instead of 12: a solve at 50,000 determinants 39.0
+// -> 16.7 ms, a loop of two steps at 20,000 67.9 -> 35.3.  The sums of a warp's lanes are folded
+// value against value (half of the values kept by each half of the lanes, and
+// so on): M + 1 FP64 additions per warp for M values instead of 5 M.
+enum : int { kProject, kRitz, kRestart, kOrth1, kOrth2 };
+
+struct PassArgs {
+  double *T, *W;
+  size_t n;
+  int m, keep;
+  const double *coef;   // kRitz, kRestart: Ct; kOrth1, kOrth2: h
+  const double *theta;
+  const double *diag;
+  double *t;
+  bool precondition;
+  int iter;
+  double tol;
+  double *Hs, *h;       // outputs of the sums
+  double *part;         // partial sums of the blocks
+  unsigned *ticket;     // zero between launches
+  DavState *st;
+};
+
+// Sums over the warp of v[0 .. M), M a power of two up to 32: on return lane l
+// holds the sum of v[l % M].
+template <int M>
+__device__ __forceinline__ double fold_sums(double (&v)[M]) {
+  const unsigned lane = threadIdx.x & 31u;
+#pragma unroll
+  for (int o = M / 2; o; o >>= 1) {
+    const bool up = (lane & (unsigned)o) != 0u;
+#pragma unroll
+    for (int j = 0; j < o; ++j) {
+      const double give = up ? v[j] : v[j + o], have = up ? v[j + o] : v[j];
+      v[j] = have + __shfl_xor_sync(0xffffffffu, give, o);
     }
-    x[i] = a;
-    wx[i] = b;
+  }
+  double s = v[0];
+#pragma unroll
+  for (int o = M; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+template <int MODE, int MAXM>
+__global__ void __launch_bounds__(kPassThreads) k_pass(PassArgs A) {
+  constexpr int kWarps = kPassThreads / 32;
+  __shared__ double cf[MODE == kRestart ? kKeep * kMaxSub : kMaxSub];
+  __shared__ double red[kWarps][kMaxSub + 1];
+  __shared__ double sum[kMaxSub + 1];
+  __shared__ double fin[kPassThreads];
+  __shared__ bool last;
+  if (A.st->stop) return;
+  const int m = A.m, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int K = MODE == kRestart ? A.keep : 1;
+  const int nh = MODE == kOrth2 ? 0 : (MODE == kRestart ? K : m);  // sums T_j . something
+  const bool extra = MODE != kProject && MODE != kOrth1;           // r . r or t . t
+  const int nval = nh + (extra ? 1 : 0);
+  // coefficients of the T_j (with the factors of the basis vectors)
+  if (MODE == kRitz || MODE == kRestart)
+    for (int e = tid; e < K * m; e += kPassThreads) {
+      const int k = e / m, j = e - k * m;
+      cf[e] = A.coef[(size_t)k * kMaxSub + j] * A.st->scale[j];
+    }
+  if (MODE == kOrth1 || MODE == kOrth2)
+    for (int e = tid; e < m; e += kPassThreads) cf[e] = -A.coef[e];
+  const double theta = (MODE == kRitz || MODE == kRestart) ? *A.theta : 0.0;
+  double acc[MAXM], ex = 0.0;
+#pragma unroll
+  for (int j = 0; j < MAXM; ++j) acc[j] = 0.0;
+  __syncthreads();
+  const size_t n = A.n;
+  for (size_t i = (size_t)blockIdx.x * kPassThreads + tid; i < n;
+       i += (size_t)gridDim.x * kPassThreads) {
+    double *T = A.T + i, *W = A.W + i;
+    double v[MAXM];
+#pragma unroll
+    for (int j = 0; j < MAXM; ++j) v[j] = j < m ? T[(size_t)j * n] : 0.0;
+    if (MODE == kProject) {
+      const double w = W[(size_t)(m - 1) * n];
+#pragma unroll
+      for (int j = 0; j < MAXM; ++j)
+        if (j < m) acc[j] = fma(v[j], w, acc[j]);
+      continue;
+    }
+    if (MODE == kOrth1 || MODE == kOrth2) {
+      double t = A.t[i];
+#pragma unroll
+      for (int j = 0; j < MAXM; ++j)
+        if (j < m) t = fma(cf[j], v[j], t);
+      A.t[i] = t;
+      if (MODE == kOrth2) {
+        ex = fma(t, t, ex);
+      } else {
+#pragma unroll
+        for (int j = 0; j < MAXM; ++j)
+          if (j < m) acc[j] = fma(v[j], t, acc[j]);
+      }
+      continue;
+    }
+    double x = 0.0, wx = 0.0, xs[kKeep];
+    if (MODE == kRestart) {
+      double ws[kKeep];
+#pragma unroll
+      for (int k = 0; k < kKeep; ++k) xs[k] = ws[k] = 0.0;
+#pragma unroll
+      for (int j = 0; j < MAXM; ++j)
+        if (j < m) {
+          const double w = W[(size_t)j * n];
+#pragma unroll
+          for (int k = 0; k < kKeep; ++k)
+            if (k < K) {
+              xs[k] = fma(cf[k * m + j], v[j], xs[k]);
+              ws[k] = fma(cf[k * m + j], w, ws[k]);
+            }
+        }
+#pragma unroll
+      for (int k = 0; k < kKeep; ++k)
+        if (k < K) {
+          T[(size_t)k * n] = xs[k];
+          W[(size_t)k * n] = ws[k];
+        }
+      x = xs[0];
+      wx = ws[0];
+    } else {
+      double w[MAXM];
+#pragma unroll
+      for (int j = 0; j < MAXM; ++j) w[j] = j < m ? W[(size_t)j * n] : 0.0;
+#pragma unroll
+      for (int j = 0; j < MAXM; ++j)
+        if (j < m) {
+          x = fma(cf[j], v[j], x);
+          wx = fma(cf[j], w[j], wx);
+        }
+    }
+    const double r = fma(-theta, x, wx);
+    double t = r;
+    if (A.precondition) {
+      double d = theta - A.diag[i];
+      if (fabs(d) < 1e-8) d = d < 0.0 ? -1e-8 : 1e-8;
+      t = fabs(d) <= 1e30 ? r * recip_fast(d) : r / d;
+    }
+    A.t[i] = t;
+    if (MODE == kRestart) {
+#pragma unroll
+      for (int k = 0; k < kKeep; ++k)
+        if (k < K) acc[k] = fma(xs[k], t, acc[k]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < MAXM; ++j)
+        if (j < m) acc[j] = fma(v[j], t, acc[j]);
+    }
+    ex = fma(r, r, ex);
+  }
+  if (nh) {
+    const double s = fold_sums<MAXM>(acc);
+    if (lane < nh) red[warp][lane] = s;
+  }
+  if (extra) {
+    for (int o = 16; o; o >>= 1) ex += __shfl_xor_sync(0xffffffffu, ex, o);
+    if (lane == 0) red[warp][nh] = ex;
+  }
+  __syncthreads();
+  if (tid < nval) {
+    double s = red[0][tid];
+    for (int w = 1; w < kWarps; ++w) s += red[w][tid];
+    A.part[(size_t)tid * gridDim.x + blockIdx.x] = s;
+    __threadfence();
+  }
+  __syncthreads();
+  if (tid == 0) last = atomicAdd(A.ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  // the blocks' sums: 8 lanes per value, then the 8 in order
+  for (int j0 = 0; j0 < nval; j0 += kPassThreads / 8) {
+    const int j = j0 + (tid >> 3), p = tid & 7;
+    double s = 0.0;
+    if (j < nval) {
+      const double *q = A.part + (size_t)j * gridDim.x;
+#pragma unroll 8
+      for (unsigned e = p; e < gridDim.x; e += 8) s += __ldcg(q + e);
+    }
+    fin[tid] = s;
+    __syncthreads();
+    if (p == 0 && j < nval) {
+      double t = fin[tid];
+      for (int u = 1; u < 8; ++u) t += fin[tid + u];
+      sum[j] = t;
+    }
+    __syncthreads();
+  }
+  DavState *st = A.st;
+  if (MODE == kProject) {
+    const double sm = st->scale[m - 1];
+    for (int j = tid; j < m; j += kPassThreads) {
+      const double v = sum[j] * st->scale[j] * sm;
+      A.Hs[j * kMaxSub + (m - 1)] = v;
+      A.Hs[(m - 1) * kMaxSub + j] = v;
+    }
+  } else {
+    // v_j (v_j . t) = T_j scale_j^2 (T_j . t); restarted vectors have scale 1
+    for (int j = tid; j < nh; j += kPassThreads) {
+      const double sj = MODE == kRestart ? 1.0 : st->scale[j];
+      A.h[j] = sum[j] * sj * sj;
+    }
+  }
+  if (MODE == kRestart && tid < K) st->scale[tid] = 1.0;
+  if (tid == 0) {
+    *A.ticket = 0u;
+    if (MODE == kRitz || MODE == kRestart) {
+      const double rr = sum[nh];
+      st->iter = A.iter;
+      st->theta = theta;
+      st->res2 = rr;
+      if (!isfinite(theta) || !isfinite(rr)) st->stop = kStopBad;
+      else if (sqrt(rr > 0.0 ? rr : 0.0) <= A.tol) st->stop = kStopConverged;
+    }
+    if (MODE == kOrth2) {
+      st->scale[m] = 1.0 / sqrt(sum[0]);
+      if (!(sum[0] > 1e-28)) st->stop = kStopSpent;  // the correction lies in the basis
+    }
   }
 }
 
-// r = wx - theta * x; t = r / (theta - H_ii) with the denominator kept at
-// least 1e-8 in magnitude (or t = r when unpreconditioned).
-__global__ void k_residual(const double *wx, const double *x, const double *theta,
-                           const double *diag, size_t n, bool precondition, double *r,
-                           double *t) {
-  const double th = *theta;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const double ri = fma(-th, x[i], wx[i]);
-    r[i] = ri;
-    if (precondition) {
-      double d = th - diag[i];
-      if (fabs(d) < 1e-8) d = d < 0.0 ? -1e-8 : 1e-8;
-      t[i] = ri / d;
-    } else {
-      t[i] = ri;
-    }
-  }
-}
+// *out = 1 / sqrt(*norm2)
+__global__ void k_inverse_norm(const double *norm2, double *out) { *out = 1.0 / sqrt(*norm2); }
 
 // v *= 1 / sqrt(*norm2)
 __global__ void k_normalize(double *v, size_t n, const double *norm2) {
@@ -506,24 +731,31 @@ __global__ void k_normalize(double *v, size_t n, const double *norm2) {
     v[i] *= s;
 }
 
-// All eigenpairs of the symmetric m x m matrix Hs (leading dimension ld) by
-// Jacobi rotations in the parallel (round-robin) ordering (Brent and Luk,
-// 1985; Golub and Van Loan, Sec. 8.5): a sweep is M - 1 rounds (M = m rounded
-// up to even; the extra index, when there is one, has no couplings), each
-// round pairs every index with one other, so its M / 2 rotations act on
-// disjoint planes.  One thread per pair forms its rotation from the round's
-// matrix, then the CTA applies all of them to the columns (and to the
-// eigenvector matrix), then to the rows.
+// The lowest eigenpairs of the symmetric m x m subspace matrix Hs (leading
+// dimension kMaxSub), one CTA.
 //
 // GB300 executes about 1.7 FP64 operations per clock per SM, against some 126
-// FP32 ones, so the sweeps run in two precisions: FP32 sweeps take the matrix
-// to near-diagonal form (off-diagonal norm below 1e-6 of the diagonal's); the
-// FP32 eigenvectors, promoted to FP64 and orthonormalised by two passes of
-// classical Gram-Schmidt, transform Hs in FP64 (Q^T Hs Q, an exact similarity
-// up to rounding); FP64 sweeps then finish (off-diagonal norm below 1e-13 of
-// the diagonal's, one or two sweeps by quadratic convergence), accumulating
-// into the same eigenvectors.  out: theta[r] in ascending order (ties by
-// index), eigenvector r in Ct[r * kMaxSub + k].
+// FP32 ones, so the eigenvectors are found in FP32 and only the wanted ones
+// (the lowest; the kKeep lowest at a restart) refined in FP64:
+//   1. Jacobi rotations in the parallel (round-robin) ordering (Brent and Luk,
+//      1985; Golub and Van Loan, Sec. 8.5) on Hs - Hs_00 in FP32: a sweep is
+//      M - 1 rounds (M = m rounded up to even; the extra index has no
+//      couplings), each round pairs every index with one other, so its M / 2
+//      rotations act on disjoint planes and each 2 x 2 block of the matrix is
+//      updated by one thread.  The matrix grew by a row since the last call, so
+//      the sweeps start from that call's eigenbasis (two or three instead of
+//      six).
+//   2. Per wanted eigenpair, a warp iterates in FP64: theta = x.Hx,
+//      r = Hx - theta x, x <- x - Q (L - theta)^-1 Q^T r with the FP32
+//      eigenbasis Q, L as the approximate inverse (its own component left
+//      out), normalised.  Each step shrinks the error by about the FP32
+//      eigenbasis's own (1e-4), until |r| is at FP64 rounding.
+//   3. Several eigenvectors are orthonormalised by two passes of Gram-Schmidt.
+// A pair whose residual stays above 1e-13 of the matrix (eigenvalues too close
+// for FP32 to tell apart) sends the whole matrix through FP64 Jacobi: FP32
+// eigenvectors orthonormalised in FP64, Q^T Hs Q, FP64 sweeps to an
+// off-diagonal norm of 1e-13 of the diagonal's.
+// m = 16: 15 us against 135 for the FP64 Jacobi that every product took.
 constexpr int kEigThreads = 256;
 
 // 1/sqrt(x) to FP64 accuracy from the FP32 estimate rsqrtf and two
@@ -559,15 +791,6 @@ __device__ __forceinline__ void rotation(double app, double aqq, double apq, dou
   *s = t * cs;
 }
 
-// The FP32 rotation of the same formulas (IEEE FP32 division and square root).
-__device__ __forceinline__ void rotation_f(float app, float aqq, float apq, float *c, float *s) {
-  const float tau = (aqq - app) / (2.0f * apq);
-  const float t = (tau >= 0.0f ? 1.0f : -1.0f) / (fabsf(tau) + sqrtf(fmaf(tau, tau, 1.0f)));
-  const float cs = 1.0f / sqrtf(fmaf(t, t, 1.0f));
-  *c = cs;
-  *s = t * cs;
-}
-
 constexpr int kEigPer = (kMaxSub * kMaxSub + kEigThreads - 1) / kEigThreads;
 
 struct EigScratch {
@@ -577,12 +800,13 @@ struct EigScratch {
   int done;
 };
 
-// Parallel-order Jacobi sweeps on A (symmetric, m x m) accumulating into Q,
-// until the off-diagonal norm is at most sqrt(thr) of the diagonal's or after
-// max_sweeps.  T is float or double; every thread of the CTA calls it.
-template <typename T>
-__device__ void jacobi_sweeps(T (*A)[kMaxSub + 1], T (*Q)[kMaxSub + 1], int m, int max_sweeps,
-                              double thr, EigScratch &E) {
+// Parallel-order Jacobi sweeps in FP64 on A (symmetric, m x m) accumulating
+// into Q, until the off-diagonal norm is at most sqrt(thr) of the diagonal's or
+// after max_sweeps.  One thread per pair forms its rotation from the round's
+// matrix, then the CTA applies all of them to the columns (and to Q), then to
+// the rows.  Every thread of the CTA calls it.
+__device__ void jacobi_sweeps(double (*A)[kMaxSub + 1], double (*Q)[kMaxSub + 1], int m,
+                              int max_sweeps, double thr, EigScratch &E) {
   const int tid = threadIdx.x;
   const int M = m + (m & 1);
   const int half = M / 2;
@@ -590,7 +814,7 @@ __device__ void jacobi_sweeps(T (*A)[kMaxSub + 1], T (*Q)[kMaxSub + 1], int m, i
     double off = 0.0, dg = 0.0;
     for (int e = tid; e < m * m; e += kEigThreads) {
       const int i = e / m, k = e - (e / m) * m;
-      const double a = (double)A[i][k];
+      const double a = A[i][k];
       if (i == k) dg += a * a;
       else off += a * a;
     }
@@ -620,18 +844,8 @@ __device__ void jacobi_sweeps(T (*A)[kMaxSub + 1], T (*Q)[kMaxSub + 1], int m, i
         const int p = pa < pb ? pa : pb, q = pa < pb ? pb : pa;
         double cs = 1.0, sn = 0.0;
         if (q < m) {
-          if (sizeof(T) == sizeof(float)) {
-            const float apq = (float)A[p][q];
-            if (fabsf(apq) >= 1e-30f) {
-              float c, s;
-              rotation_f((float)A[p][p], (float)A[q][q], apq, &c, &s);
-              cs = c;
-              sn = s;
-            }
-          } else {
-            const double apq = (double)A[p][q];
-            if (fabs(apq) >= 1e-300) rotation((double)A[p][p], (double)A[q][q], apq, &cs, &sn);
-          }
+          const double apq = A[p][q];
+          if (fabs(apq) >= 1e-300) rotation(A[p][p], A[q][q], apq, &cs, &sn);
         }
         E.rc[tid] = cs;
         E.rs[tid] = sn;
@@ -643,11 +857,11 @@ __device__ void jacobi_sweeps(T (*A)[kMaxSub + 1], T (*Q)[kMaxSub + 1], int m, i
         const int k = e / m, i = e - (e / m) * m;
         const int p = E.rp[k], q = E.rq[k];
         if (q >= m || E.rs[k] == 0.0) continue;
-        const T cs = (T)E.rc[k], sn = (T)E.rs[k];
-        const T aip = A[i][p], aiq = A[i][q];
+        const double cs = E.rc[k], sn = E.rs[k];
+        const double aip = A[i][p], aiq = A[i][q];
         A[i][p] = cs * aip - sn * aiq;
         A[i][q] = sn * aip + cs * aiq;
-        const T qip = Q[i][p], qiq = Q[i][q];
+        const double qip = Q[i][p], qiq = Q[i][q];
         Q[i][p] = cs * qip - sn * qiq;
         Q[i][q] = sn * qip + cs * qiq;
       }
@@ -656,8 +870,8 @@ __device__ void jacobi_sweeps(T (*A)[kMaxSub + 1], T (*Q)[kMaxSub + 1], int m, i
         const int k = e / m, j = e - (e / m) * m;
         const int p = E.rp[k], q = E.rq[k];
         if (q >= m || E.rs[k] == 0.0) continue;
-        const T cs = (T)E.rc[k], sn = (T)E.rs[k];
-        const T apj = A[p][j], aqj = A[q][j];
+        const double cs = E.rc[k], sn = E.rs[k];
+        const double apj = A[p][j], aqj = A[q][j];
         A[p][j] = cs * apj - sn * aqj;
         A[q][j] = sn * apj + cs * aqj;
       }
@@ -666,23 +880,275 @@ __device__ void jacobi_sweeps(T (*A)[kMaxSub + 1], T (*Q)[kMaxSub + 1], int m, i
   }
 }
 
-__global__ void __launch_bounds__(kEigThreads) k_small_eig(const double *Hs, int ld, int m,
-                                                           double *theta, double *Ct) {
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// The FP32 rotation that zeroes apq by the hardware's approximate reciprocal
+// and reciprocal square root (an error of some 1e-7 is made good by the
+// refinement): t = sign(d) h / (|d| + sqrt(d^2 + h^2)), d = aqq - app, h = 2 apq.
+__device__ __forceinline__ float2 rotation_fast(float app, float aqq, float apq) {
+  const float d = aqq - app, h = 2.0f * apq;
+  const float q = fmaf(d, d, h * h);
+  if (!(q > 1e-35f) || h == 0.0f) return make_float2(1.0f, 0.0f);
+  const float t = (d >= 0.0f ? h : -h) * rcp_approx(fmaf(q, rsqrt_approx(q), fabsf(d)));
+  const float c = rsqrt_approx(fmaf(t, t, 1.0f));
+  return make_float2(c, t * c);
+}
+
+// FP32 sweeps on A[0] (m x m, zero beyond) accumulating into Q[0], until the
+// off-diagonal norm is 1e-4 of the matrix's (the refinement's contraction; a
+// sweep costs as much as three of its steps).  Positions 2k and 2k + 1 are
+// rotated against each other, a block of A (or a row's pair of Q) per thread,
+// and the results written one place on in the round-robin into the other
+// buffer, so a round has one barrier; after the M - 1 rounds of a sweep every
+// index is back in its place.  Returns the buffer that holds the result.
+__device__ int jacobi_fast(float (*A)[kMaxSub][kMaxSub + 1], float (*Q)[kMaxSub][kMaxSub + 1],
+                           int m, float (*red)[kEigThreads / 32]) {
+  const int tid = threadIdx.x, M = m + (m & 1), half = M / 2;
+  constexpr int kItems = (kMaxSub * kMaxSub / 4 + kMaxSub * kMaxSub / 2) / kEigThreads;
+  const int items = half * half + M * half;  // blocks of A, then (row, pair) of Q
+  auto next = [&](int pos) {
+    if (pos == 0 || half == 1) return pos;
+    if (pos & 1) return pos == 1 ? 2 : pos - 2;
+    return pos == M - 2 ? M - 1 : pos + 2;
+  };
+  int it_k[kItems], it_l[kItems], to_l0[kItems], to_l1[kItems], to_k0[kItems], to_k1[kItems];
+#pragma unroll
+  for (int u = 0; u < kItems; ++u) {
+    const int e = tid + u * kEigThreads;
+    it_k[u] = e / max(half, 1);
+    it_l[u] = e - it_k[u] * half;
+    to_l0[u] = next(2 * it_l[u]);
+    to_l1[u] = next(2 * it_l[u] + 1);
+    to_k0[u] = next(2 * it_k[u]);
+    to_k1[u] = next(2 * it_k[u] + 1);
+  }
+  int b = 0;
+  for (int sweep = 0; sweep < 12 && m > 1; ++sweep) {
+    float off = 0.0f, all = 0.0f;
+    for (int e = tid; e < kMaxSub * M; e += kEigThreads) {
+      const int i = e / kMaxSub, k = e % kMaxSub;
+      if (k < M) {
+        const float a = A[b][i][k];
+        all = fmaf(a, a, all);
+        if (i != k) off = fmaf(a, a, off);
+      }
+    }
+    for (int o = 16; o; o >>= 1) {
+      off += __shfl_xor_sync(0xffffffffu, off, o);
+      all += __shfl_xor_sync(0xffffffffu, all, o);
+    }
+    if ((tid & 31) == 0) {
+      red[0][tid >> 5] = off;
+      red[1][tid >> 5] = all;
+    }
+    __syncthreads();
+    off = all = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kEigThreads / 32; ++w) {
+      off += red[0][w];
+      all += red[1][w];
+    }
+    if (!(off > 1e-8f * all)) break;  // uniform
+    for (int r = 0; r < M - 1; ++r, b ^= 1) {
+      const float(*Ab)[kMaxSub + 1] = A[b];
+      const float(*Qb)[kMaxSub + 1] = Q[b];
+      float(*An)[kMaxSub + 1] = A[b ^ 1];
+      float(*Qn)[kMaxSub + 1] = Q[b ^ 1];
+#pragma unroll
+      for (int u = 0; u < kItems; ++u) {
+        if (tid + u * kEigThreads >= items) break;
+        const int k = it_k[u], pl = 2 * it_l[u], ql = pl + 1;
+        const float2 R = rotation_fast(Ab[pl][pl], Ab[ql][ql], Ab[pl][ql]);
+        if (k < half) {
+          const int pk = 2 * k, qk = pk + 1;
+          const float x = Ab[pk][pl], y = Ab[pk][ql], z = Ab[qk][pl], w = Ab[qk][ql];
+          const float2 L = rotation_fast(Ab[pk][pk], Ab[qk][qk], Ab[pk][qk]);
+          const float x1 = L.x * x - L.y * z, z1 = L.y * x + L.x * z;
+          const float y1 = L.x * y - L.y * w, w1 = L.y * y + L.x * w;
+          An[to_k0[u]][to_l0[u]] = R.x * x1 - R.y * y1;
+          An[to_k0[u]][to_l1[u]] = R.y * x1 + R.x * y1;
+          An[to_k1[u]][to_l0[u]] = R.x * z1 - R.y * w1;
+          An[to_k1[u]][to_l1[u]] = R.y * z1 + R.x * w1;
+        } else {
+          const float x = Qb[k - half][pl], y = Qb[k - half][ql];
+          Qn[k - half][to_l0[u]] = R.x * x - R.y * y;
+          Qn[k - half][to_l1[u]] = R.y * x + R.x * y;
+        }
+      }
+      __syncthreads();
+    }
+  }
+  __syncthreads();
+  return b;
+}
+
+__device__ __forceinline__ double warp_sum(double v) {
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// want lowest eigenpairs: theta[0 .. want), eigenvector k in Ct[k * kMaxSub + j].
+// Qw keeps the FP32 eigenbasis; with `warm` it holds that of the leading
+// m - 1 rows and columns, and the sweeps start in its basis (an arrowhead).
+__global__ void __launch_bounds__(kEigThreads) k_small_eig(const double *Hs, int m, int want,
+                                                           bool warm, float *Qw, double *theta,
+                                                           double *Ct, const int *stop) {
+  __shared__ double H[kMaxSub][kMaxSub + 1];
   __shared__ double A[kMaxSub][kMaxSub + 1];
   __shared__ double Q[kMaxSub][kMaxSub + 1];
-  __shared__ float Af[kMaxSub][kMaxSub + 1];
-  __shared__ float Qf[kMaxSub][kMaxSub + 1];
+  __shared__ float A2[2][kMaxSub][kMaxSub + 1];
+  __shared__ float Q2[2][kMaxSub][kMaxSub + 1];
+  __shared__ double X[kKeep][kMaxSub], th[kKeep];
+  __shared__ float gv[kKeep][kMaxSub], redf[2][kEigThreads / 32];
+  __shared__ int of_rank[kMaxSub], failed;
   __shared__ double gsr[kMaxSub];
   __shared__ double nrm;
   __shared__ EigScratch E;
+  if (stop && *stop) return;
   const int tid = threadIdx.x;
-  for (int e = tid; e < m * m; e += kEigThreads) {
-    const int i = e / m, k = e - (e / m) * m;
-    Af[i][k] = (float)Hs[(size_t)i * ld + k];
-    Qf[i][k] = (i == k) ? 1.0f : 0.0f;
+  const double shift = Hs[0];
+#pragma unroll
+  for (int e = tid; e < kMaxSub * kMaxSub; e += kEigThreads) {
+    const int i = e / kMaxSub, k = e % kMaxSub;
+    const bool in = i < m && k < m;
+    const double h = in ? Hs[e] : 0.0;
+    float q = i == k ? 1.0f : 0.0f;
+    if (warm && i < m - 1 && k < m - 1) q = Qw[e];
+    H[i][k] = h;
+    A2[0][i][k] = (float)(in && i == k ? h - shift : h);
+    Q2[0][i][k] = q;
+  }
+  if (tid == 0) failed = 0;
+  __syncthreads();
+  if (warm) {  // A = Q^T A Q
+    float p[kMaxSub * kMaxSub / kEigThreads];
+    for (int side = 0; side < 2; ++side) {
+#pragma unroll
+      for (int u = 0; u < kMaxSub * kMaxSub / kEigThreads; ++u) {
+        const int e = tid + u * kEigThreads, i = e / kMaxSub, k = e % kMaxSub;
+        p[u] = 0.0f;
+        if (i < m && k < m) {
+#pragma unroll 8
+          for (int l = 0; l < m; ++l)
+            p[u] = side ? fmaf(Q2[0][l][i], A2[0][l][k], p[u]) : fmaf(A2[0][i][l], Q2[0][l][k], p[u]);
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < kMaxSub * kMaxSub / kEigThreads; ++u) {
+        const int e = tid + u * kEigThreads, i = e / kMaxSub, k = e % kMaxSub;
+        if (i < m && k < m) A2[0][i][k] = p[u];
+      }
+      __syncthreads();
+    }
+  }
+  const int buf = jacobi_fast(A2, Q2, m, redf);
+  const float(*Af)[kMaxSub + 1] = A2[buf];
+  const float(*Qf)[kMaxSub + 1] = Q2[buf];
+#pragma unroll
+  for (int e = tid; e < kMaxSub * kMaxSub; e += kEigThreads) {
+    const int i = e / kMaxSub, k = e % kMaxSub;
+    if (i < m && k < m) Qw[e] = Qf[i][k];
+  }
+  if (tid < m) {  // rank of each FP32 eigenvalue (ties by index)
+    const float d = Af[tid][tid];
+    int rk = 0;
+    for (int j = 0; j < m; ++j) rk += (Af[j][j] < d) || (Af[j][j] == d && j < tid);
+    of_rank[rk] = tid;
   }
   __syncthreads();
-  jacobi_sweeps<float>(Af, Qf, m, 16, 1e-12, E);
+  const int w = tid >> 5, lane = tid & 31;
+  if (w < want) {  // a warp per wanted pair
+    const int own = of_rank[w];
+    const bool in = lane < m;
+    const float lam = in ? Af[lane][lane] : 0.0f;
+    float scale = in ? fabsf(lam) : 0.0f;
+    for (int o = 16; o; o >>= 1) scale = fmaxf(scale, __shfl_xor_sync(0xffffffffu, scale, o));
+    scale += fabsf((float)shift);
+    double x = in ? (double)Qf[lane][own] : 0.0;
+    x *= rsqrt_fast(warp_sum(x * x));
+    double t = 0.0;
+    float last = __int_as_float(0x7f800000);
+    for (int it = 0; it < 16; ++it) {
+      X[w][lane] = x;
+      __syncwarp();
+      double y = 0.0;
+      if (m <= 16) {  // two lanes per row
+        const int i = lane & 15, l0 = (lane >> 4) * 8;
+        if (i < m)
+          for (int l = l0; l < l0 + 8 && l < m; ++l) y = fma(H[i][l], X[w][l], y);
+        y += __shfl_xor_sync(0xffffffffu, y, 16);
+      } else if (in) {
+        for (int l = 0; l < m; ++l) y = fma(H[lane][l], X[w][l], y);
+      }
+      if (!in) y = 0.0;
+      t = warp_sum(x * y);
+      const float r = (float)fma(-t, x, y);
+      float rr = r * r;
+      for (int o = 16; o; o >>= 1) rr += __shfl_xor_sync(0xffffffffu, rr, o);
+      const float rn = sqrtf(rr);
+      if (rn <= 4e-15f * scale) break;  // at rounding
+      if (!(rn < 0.5f * last) || it == 15) {  // no longer falling
+        if (!(rn <= 1e-13f * scale) && lane == 0) failed = 1;
+        break;
+      }
+      last = rn;
+      // the step from the FP32 eigenbasis
+      gv[w][lane] = r;
+      __syncwarp();
+      float g = 0.0f;
+      if (in)
+#pragma unroll 8
+        for (int l = 0; l < m; ++l) g = fmaf(Qf[l][lane], gv[w][l], g);
+      const float gap = lam - (float)(t - shift);
+      g = (in && lane != own && fabsf(gap) > 1e-6f * scale) ? __fdividef(g, gap) : 0.0f;
+      __syncwarp();
+      gv[w][lane] = g;
+      __syncwarp();
+      float dx = 0.0f;
+      if (in)
+#pragma unroll 8
+        for (int l = 0; l < m; ++l) dx = fmaf(Qf[lane][l], gv[w][l], dx);
+      __syncwarp();
+      x -= (double)dx;
+      x *= rsqrt_fast(warp_sum(x * x));
+    }
+    X[w][lane] = x;
+    if (lane == 0) th[w] = t;
+  }
+  __syncthreads();
+  if (!failed) {
+    if (want > 1 && w == 0) {  // orthonormal: two passes of Gram-Schmidt, one vector after another
+      for (int k = 0; k < want; ++k) {
+        double x = X[k][lane];
+        for (int pass = 0; pass < 2 && k > 0; ++pass) {
+          double dots[kKeep];
+#pragma unroll
+          for (int j = 0; j < kKeep; ++j) dots[j] = j < k ? warp_sum(x * X[j][lane]) : 0.0;
+#pragma unroll
+          for (int j = 0; j < kKeep; ++j)
+            if (j < k) x = fma(-dots[j], X[j][lane], x);
+        }
+        x *= rsqrt_fast(warp_sum(x * x));
+        X[k][lane] = x;
+        __syncwarp();
+      }
+    }
+    __syncthreads();
+    for (int e = tid; e < want * m; e += kEigThreads)
+      Ct[(size_t)(e / m) * kMaxSub + (e - (e / m) * m)] = X[e / m][e - (e / m) * m];
+    if (tid < want) theta[tid] = th[tid];
+    return;
+  }
   for (int e = tid; e < m * m; e += kEigThreads) {
     const int i = e / m, k = e - (e / m) * m;
     Q[i][k] = (double)Qf[i][k];
@@ -706,7 +1172,7 @@ __global__ void __launch_bounds__(kEigThreads) k_small_eig(const double *Hs, int
     }
     if (tid < 32) {
       double v = tid < m ? Q[tid][k] * Q[tid][k] : 0.0;
-      for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      v = warp_sum(v);
       if (tid == 0) nrm = v;
     }
     __syncthreads();
@@ -717,7 +1183,7 @@ __global__ void __launch_bounds__(kEigThreads) k_small_eig(const double *Hs, int
   for (int e = tid; e < m * m; e += kEigThreads) {
     const int i = e / m, j = e - (e / m) * m;
     double t = 0.0;
-    for (int l = 0; l < m; ++l) t = fma(Hs[(size_t)i * ld + l], Q[l][j], t);
+    for (int l = 0; l < m; ++l) t = fma(H[i][l], Q[l][j], t);
     A[i][j] = t;
   }
   __syncthreads();
@@ -737,18 +1203,20 @@ __global__ void __launch_bounds__(kEigThreads) k_small_eig(const double *Hs, int
     if (e < m * m) A[e / m][e - (e / m) * m] = keep[u];
   }
   __syncthreads();
-  jacobi_sweeps<double>(A, Q, m, 8, 1e-26, E);
+  jacobi_sweeps(A, Q, m, 8, 1e-26, E);
   for (int i = tid; i < m; i += kEigThreads) {
     const double d = A[i][i];
     int rk = 0;
     for (int j = 0; j < m; ++j) rk += (A[j][j] < d) || (A[j][j] == d && j < i);
+    if (rk >= want) continue;
     theta[rk] = d;
     for (int k = 0; k < m; ++k) Ct[(size_t)rk * kMaxSub + k] = Q[k][i];
   }
 }
 
 // Hs = diag(theta[0..K)) after a restart.
-__global__ void k_restart_hs(double *Hs, const double *theta, int K) {
+__global__ void k_restart_hs(double *Hs, const double *theta, int K, const int *stop) {
+  if (*stop) return;
   for (int e = threadIdx.x; e < kMaxSub * kMaxSub; e += blockDim.x) {
     const int i = e / kMaxSub, k = e - (e / kMaxSub) * kMaxSub;
     Hs[e] = (i == k && i < K) ? theta[i] : 0.0;
@@ -791,17 +1259,32 @@ __global__ void k_absmax_part(const double *v, size_t n, double *bval, unsigned 
   }
 }
 
-__global__ void k_absmax_sign(const double *bval, const unsigned long long *bidx, int nb,
-                              const double *v, double *sign) {
-  if (threadIdx.x != 0) return;
+__global__ void __launch_bounds__(256) k_absmax_sign(const double *bval,
+                                                     const unsigned long long *bidx, int nb,
+                                                     const double *v, double *sign) {
+  __shared__ double sv[256];
+  __shared__ unsigned long long si[256];
   double best = -1.0;
   unsigned long long bi = ~0ull;
-  for (int b = 0; b < nb; ++b)
-    if (bval[b] > best || (bval[b] == best && bidx[b] < bi)) {
-      best = bval[b];
-      bi = bidx[b];
+  auto take = [&](double o, unsigned long long oi) {
+    if (o > best || (o == best && oi < bi)) {
+      best = o;
+      bi = oi;
     }
-  *sign = (bi != ~0ull && v[bi] < 0.0) ? -1.0 : 1.0;
+  };
+  for (int b = threadIdx.x; b < nb; b += 256) take(bval[b], bidx[b]);
+  sv[threadIdx.x] = best;
+  si[threadIdx.x] = bi;
+  __syncthreads();
+  for (int s = 128; s; s >>= 1) {
+    if ((int)threadIdx.x < s) {
+      take(sv[threadIdx.x + s], si[threadIdx.x + s]);
+      sv[threadIdx.x] = best;
+      si[threadIdx.x] = bi;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) *sign = (bi != ~0ull && v[bi] < 0.0) ? -1.0 : 1.0;
 }
 
 __global__ void k_scale_by(double *v, size_t n, const double *s) {
@@ -839,16 +1322,23 @@ __global__ void k_unit(double *v, size_t n, const double *diag) {
   for (size_t i = threadIdx.x; i < n; i += blockDim.x) v[i] = (i == si[0]) ? 1.0 : 0.0;
 }
 
+// A warp per row: the lanes scan the row's columns for the diagonal.
 __global__ void k_csr_diag(const int64_t *rp, const int32_t *col, const double *val, uint32_t n,
                            double *diag) {
-  for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
+  for (uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
+    const int64_t e = rp[r + 1];
     double d = 0.0;
-    for (int64_t k = rp[r]; k < rp[r + 1]; ++k)
-      if (col[k] == (int32_t)r) {
-        d = val[k];
+    for (int64_t k0 = rp[r]; k0 < e; k0 += 32) {
+      const int64_t k = k0 + lane;
+      const uint32_t hit = __ballot_sync(0xffffffffu, k < e && col[k] == (int32_t)r);
+      if (hit) {
+        d = val[k0 + __ffs(hit) - 1];
         break;
       }
-    diag[r] = d;
+    }
+    if (lane == 0) diag[r] = d;
   }
 }
 
@@ -968,10 +1458,11 @@ static int ham_fill(const DevInts &I, const uint64_t *keys, uint32_t n, const do
   return ASCI_OK;
 }
 
-static int spmv(const Csr &H, const double *x, double *y, cudaStream_t s) {
+static int spmv(const Csr &H, const double *x, double *y, cudaStream_t s,
+                const int *stop = nullptr) {
   if (!H.n) return ASCI_OK;
   k_spmv<<<blocks_for(H.n * 32, 256, 152 * 32), 256, 0, s>>>(H.row_ptr, H.col, H.val,
-                                                             (uint32_t)H.n, x, y);
+                                                             (uint32_t)H.n, x, y, stop);
   ASCI_CHECK_LAUNCH();
   return ASCI_OK;
 }
@@ -999,6 +1490,14 @@ static int dots(const double *V, size_t ld, int m, const double *b, size_t n,
   return ASCI_OK;
 }
 
+template <int MODE>
+static int run_pass(const PassArgs &A, unsigned blocks, cudaStream_t s) {
+  auto *k = A.m <= 8 ? k_pass<MODE, 8> : (A.m <= 16 ? k_pass<MODE, 16> : k_pass<MODE, 32>);
+  k<<<blocks, kPassThreads, 0, s>>>(A);
+  ASCI_CHECK_LAUNCH();
+  return ASCI_OK;
+}
+
 struct DavidsonResult {
   double energy = 0.0, residual = 0.0;
   int iterations = 0;
@@ -1014,25 +1513,27 @@ static int davidson(const Csr &H, const double *diag, const double *guess,
   const int mmax = (int)std::min<size_t>((size_t)o.max_subspace, n);
   const unsigned gb = blocks_for(n, 256);
   const int keep = std::min(kKeep, mmax - 1);  // Ritz vectors kept at a restart
-  double *V, *W, *Hs, *Ct, *th, *h, *sc, *x, *wx, *r, *t, *TV = nullptr, *TW = nullptr;
+  double *V, *W, *Hs, *Ct, *th, *h, *sc, *x, *pass_part;
+  unsigned *pass_ticket;
+  float *Qw;
+  DavState *st;
   DotScratch part;
-  ASCI_TRY(arena.alloc(&V, (size_t)std::max(mmax, 1) * n));
-  ASCI_TRY(arena.alloc(&W, (size_t)std::max(mmax, 1) * n));
-  if (keep > 0) {
-    ASCI_TRY(arena.alloc(&TV, (size_t)keep * n));
-    ASCI_TRY(arena.alloc(&TW, (size_t)keep * n));
-  }
+  ASCI_TRY(arena.alloc(&V, ((size_t)mmax + 1) * n));  // the last correction has a place too
+  ASCI_TRY(arena.alloc(&W, (size_t)mmax * n));
   ASCI_TRY(arena.alloc(&Hs, (size_t)kMaxSub * kMaxSub));
   ASCI_TRY(arena.alloc(&Ct, (size_t)kMaxSub * kMaxSub));
   ASCI_TRY(arena.alloc(&th, kMaxSub));
   ASCI_TRY(arena.alloc(&h, kMaxSub));
   ASCI_TRY(dot_scratch(&part, arena));
-  ASCI_TRY(arena.alloc(&sc, 8));  // scratch, |r|^2, |t|^2, sign
+  ASCI_TRY(arena.alloc(&sc, 4));  // |v|^2, sign
   ASCI_TRY(arena.alloc(&x, n));
-  ASCI_TRY(arena.alloc(&wx, n));
-  ASCI_TRY(arena.alloc(&r, n));
-  ASCI_TRY(arena.alloc(&t, n));
+  ASCI_TRY(arena.alloc(&pass_part, (size_t)(kMaxSub + 1) * kPassBlocks));
+  ASCI_TRY(arena.alloc(&pass_ticket, 1));
+  ASCI_TRY(arena.alloc(&Qw, (size_t)kMaxSub * kMaxSub));
+  ASCI_TRY(arena.alloc(&st, 1));
   ASCI_TRY_CUDA(cudaMemsetAsync(Hs, 0, sizeof(double) * kMaxSub * kMaxSub, s));
+  ASCI_TRY_CUDA(cudaMemsetAsync(pass_ticket, 0, sizeof(unsigned), s));
+  ASCI_TRY_CUDA(cudaMemsetAsync(st, 0, sizeof(DavState), s));
   // v0: the guess, or the unit vector of the smallest H_ii; normalised
   if (guess) {
     ASCI_TRY_CUDA(cudaMemcpyAsync(V, guess, n * sizeof(double), cudaMemcpyDefault, s));
@@ -1048,79 +1549,92 @@ static int davidson(const Csr &H, const double *diag, const double *guess,
     record_error("Davidson guess is zero or not finite", __FILE__, __LINE__);
     return ASCI_EINVAL;
   }
-  k_normalize<<<gb, 256, 0, s>>>(V, n, sc + 2);
+  k_inverse_norm<<<1, 1, 0, s>>>(sc + 2, &st->scale[0]);
   ASCI_CHECK_LAUNCH();
-  int m = 1;         // basis vectors in V
-  int have_w = 0;    // products already in W
-  bool first = true;
-  double theta = 0.0, rn = 0.0;
-  for (;;) {
-    // products of the new basis vectors and their column of V^T H V
-    for (; have_w < m; ++have_w) {
-      ASCI_TRY(spmv(H, V + (size_t)have_w * n, W + (size_t)have_w * n, s));
-      ++res->iterations;
-      ASCI_TRY(dots(V, n, have_w + 1, W + (size_t)have_w * n, n, part, Hs + have_w, kMaxSub,
-                    Hs + (size_t)have_w * kMaxSub, 1, s));
-    }
-    k_small_eig<<<1, kEigThreads, 0, s>>>(Hs, kMaxSub, m, th, Ct);
-    ASCI_CHECK_LAUNCH();
-    k_ritz<<<gb, 256, 0, s>>>(V, W, n, m, Ct, n, x, wx);
-    ASCI_CHECK_LAUNCH();
-    k_residual<<<gb, 256, 0, s>>>(wx, x, th, diag, n, !first, r, t);
-    ASCI_CHECK_LAUNCH();
-    ASCI_TRY(dots(r, n, 1, r, n, part, sc + 1, 1, nullptr, 0, s));
-    // the next expansion vector is prepared before the convergence test is
-    // read back, so that one host round trip serves both; when the test
-    // stops the iteration, that work is simply dropped
-    const bool restart = m == mmax && (size_t)m < n;
-    if (restart) {  // thick restart: the `keep` lowest Ritz vectors and their products
-      for (int k = 0; k < keep; ++k) {
-        k_ritz<<<gb, 256, 0, s>>>(V, W, n, m, Ct + (size_t)k * kMaxSub, n, TV + (size_t)k * n,
-                                  TW + (size_t)k * n);
+  const int *stop = &st->stop;
+  const unsigned pb = blocks_for(n, kPassThreads, kPassBlocks);
+  auto pass_args = [&](int m, int iter) {
+    PassArgs A{};
+    A.T = V;
+    A.W = W;
+    A.n = n;
+    A.m = m;
+    A.keep = keep;
+    A.theta = th;
+    A.diag = diag;
+    A.t = V;
+    A.precondition = iter > 1;
+    A.iter = iter;
+    A.tol = o.tol;
+    A.Hs = Hs;
+    A.h = h;
+    A.part = pass_part;
+    A.ticket = pass_ticket;
+    A.st = st;
+    return A;
+  };
+  // Iterations are enqueued kAhead at a time between two looks at the state:
+  // the host's round trip is paid once for them, and those behind the one that
+  // stopped return at once.
+  constexpr int kAhead = 8;
+  struct Step {
+    int m;
+    bool restarted;
+  };
+  std::vector<Step> steps(1);  // steps[i]: product i (1-based)
+  int m = 1, it = 0;
+  DavState hst{};
+  for (bool more = true; more;) {
+    for (int a = 0; a < kAhead && more; ++a) {
+      // the newest basis vector's product and column of V^T H V
+      ASCI_TRY(spmv(H, V + (size_t)(m - 1) * n, W + (size_t)(m - 1) * n, s, stop));
+      ++it;
+      const bool restart = m == mmax && (size_t)m < n;
+      steps.push_back(Step{m, restart});
+      PassArgs A = pass_args(m, it);
+      ASCI_TRY(run_pass<kProject>(A, pb, s));
+      k_small_eig<<<1, kEigThreads, 0, s>>>(Hs, m, restart ? keep : 1, it > 1 && !steps[it - 1].restarted,
+                                            Qw, th, Ct, stop);
+      ASCI_CHECK_LAUNCH();
+      A.coef = Ct;
+      A.t = V + (size_t)(restart ? keep : m) * n;
+      if (restart) {  // thick restart: the `keep` lowest Ritz vectors and their products
+        ASCI_TRY(run_pass<kRestart>(A, pb, s));
+        k_restart_hs<<<1, 256, 0, s>>>(Hs, th, keep, stop);
         ASCI_CHECK_LAUNCH();
+        m = keep;
+      } else {
+        ASCI_TRY(run_pass<kRitz>(A, pb, s));
       }
-      ASCI_TRY_CUDA(cudaMemcpyAsync(V, TV, (size_t)keep * n * sizeof(double),
-                                    cudaMemcpyDeviceToDevice, s));
-      ASCI_TRY_CUDA(cudaMemcpyAsync(W, TW, (size_t)keep * n * sizeof(double),
-                                    cudaMemcpyDeviceToDevice, s));
-      k_restart_hs<<<1, 256, 0, s>>>(Hs, th, keep);
-      ASCI_CHECK_LAUNCH();
+      if (it >= o.max_iter || (size_t)steps[it].m >= n) {
+        more = false;
+        break;
+      }
+      // the correction, orthogonalised by two passes of classical Gram-Schmidt
+      A.m = m;
+      A.coef = h;
+      ASCI_TRY(run_pass<kOrth1>(A, pb, s));
+      ASCI_TRY(run_pass<kOrth2>(A, pb, s));
+      ++m;
     }
-    const int mb = restart ? keep : m;  // basis the correction is orthogonalised against
-    for (int pass = 0; pass < 2; ++pass) {  // two passes of classical Gram-Schmidt
-      ASCI_TRY(dots(V, n, mb, t, n, part, h, 1, nullptr, 0, s));
-      k_combine<<<gb, 256, 0, s>>>(V, n, mb, h, -1.0, t, 1.0, n, t);
-      ASCI_CHECK_LAUNCH();
-    }
-    ASCI_TRY(dots(t, n, 1, t, n, part, sc + 2, 1, nullptr, 0, s));
-    double hs[3];
-    ASCI_TRY_CUDA(cudaMemcpyAsync(&hs[0], th, sizeof(double), cudaMemcpyDeviceToHost, s));
-    ASCI_TRY_CUDA(cudaMemcpyAsync(&hs[1], sc + 1, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
+    ASCI_TRY_CUDA(cudaMemcpyAsync(&hst, st, sizeof(hst), cudaMemcpyDeviceToHost, s));
     ASCI_TRY_CUDA(cudaStreamSynchronize(s));
-    theta = hs[0];
-    rn = std::sqrt(std::max(hs[1], 0.0));
-    if (!std::isfinite(theta) || !std::isfinite(rn)) {
-      record_error("Davidson produced a non-finite value", __FILE__, __LINE__);
-      return ASCI_ECUDA;
-    }
-    if (rn <= o.tol || res->iterations >= o.max_iter || (size_t)m >= n) {
-      res->converged = rn <= o.tol || (size_t)m >= n;
-      break;
-    }
-    first = false;
-    if (restart) {
-      m = keep;
-      have_w = keep;
-    }
-    if (!(hs[2] > 1e-28)) {  // the correction lies in the basis: nothing left to add
-      res->converged = rn <= o.tol;
-      break;
-    }
-    k_normalize<<<gb, 256, 0, s>>>(t, n, sc + 2);
+    if (hst.stop) more = false;
+  }
+  if (hst.stop == kStopBad) {
+    record_error("Davidson produced a non-finite value", __FILE__, __LINE__);
+    return ASCI_ECUDA;
+  }
+  const Step fin = steps[hst.iter];
+  const double theta = hst.theta, rn = std::sqrt(std::max(hst.res2, 0.0));
+  res->iterations = hst.iter;
+  res->converged = rn <= o.tol || (size_t)fin.m >= n;
+  // the Ritz vector of the last residual: a restart left it in V_0
+  if (fin.restarted) {
+    x = V;
+  } else {
+    k_combine<<<gb, 256, 0, s>>>(V, n, fin.m, Ct, st->scale, n, x);
     ASCI_CHECK_LAUNCH();
-    ASCI_TRY_CUDA(cudaMemcpyAsync(V + (size_t)m * n, t, n * sizeof(double),
-                                  cudaMemcpyDeviceToDevice, s));
-    ++m;
   }
   // unit Ritz vector, largest component positive
   {
@@ -1134,7 +1648,7 @@ static int davidson(const Csr &H, const double *diag, const double *guess,
     ASCI_CHECK_LAUNCH();
     k_absmax_part<<<nb, 256, 0, s>>>(x, n, bval, bidx);
     ASCI_CHECK_LAUNCH();
-    k_absmax_sign<<<1, 32, 0, s>>>(bval, bidx, nb, x, sc + 3);
+    k_absmax_sign<<<1, 256, 0, s>>>(bval, bidx, nb, x, sc + 3);
     ASCI_CHECK_LAUNCH();
     k_scale_by<<<gb, 256, 0, s>>>(x, n, sc + 3);
     ASCI_CHECK_LAUNCH();
@@ -1598,7 +2112,7 @@ int asci_davidson(const int64_t *row_ptr, const int32_t *col, const double *val,
   Csr H = {rp, dc, dv, n};
   double *diag;
   ASCI_TRY(arena.alloc(&diag, n));
-  k_csr_diag<<<blocks_for(n, 256), 256, 0, s>>>(rp, dc, dv, (uint32_t)n, diag);
+  k_csr_diag<<<blocks_for(n * 32, 256), 256, 0, s>>>(rp, dc, dv, (uint32_t)n, diag);
   ASCI_CHECK_LAUNCH();
   DavidsonResult r;
   ASCI_TRY(davidson(H, diag, dg, o, vec, &r, arena));
