@@ -380,10 +380,16 @@ int sort_accumulate(uint64_t **keys, uint64_t **keys_alt, double **vals, double 
 // H_ii of packed keys.
 int diagonal_packed(const DevInts &I, const uint64_t *keys, size_t n, double *out, Arena &arena);
 
-// Top-N by |score| with key tie-break; compacts into out arrays (may not alias
-// the inputs).  Returns the count on the host.
+// Top-N by |score| with key tie-break (distinct keys); compacts into out arrays
+// (may not alias the inputs) in input order.  *host_out_n = min(n, N), without
+// waiting for the device; with host_min, waits and returns a lower bound of the
+// selected |scores| that every entry left out is at or below.
 int select_topn_packed(const uint64_t *keys, const double *scores, size_t n, size_t N,
-                       uint64_t *out_keys, double *out_scores, size_t *host_out_n, Arena &arena);
+                       uint64_t *out_keys, double *out_scores, size_t *host_out_n, Arena &arena,
+                       double *host_min = nullptr);
+
+// Smallest |score| among n candidates (host result).
+int abs_min(const double *s, size_t n, double *host_min, Arena &arena);
 
 // Histogram of byte `digit` of the rank word (~bits(|S|), key) over entries
 // matching pre on the bits of msk ({hi, lo}); hist is host memory.

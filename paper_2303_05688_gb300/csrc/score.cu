@@ -1,10 +1,20 @@
 // Sort-and-accumulate (Sec. 2.2), the diagonal H_ii and the score of Eq. 1,
 // exclusion of psi, and the top-N selection that replaces a full sort.
+#include <algorithm>
+#include <cstring>
+
 #include "asci_internal.cuh"
 
 namespace asci {
 
 namespace {
+
+struct SelState {
+  uint64_t pre[2];      // fixed bits of R_N: {hi, lo}
+  uint64_t thr[2];      // entries with R <= thr are selected, once done
+  uint64_t remaining;   // rank of R_N among the entries that match the prefix
+  unsigned done, ticket;
+};
 
 // ------------------------- segmented accumulate ----------------------------
 
@@ -104,6 +114,128 @@ __global__ void k_select_hist(const uint64_t *keys, const double *scores, size_t
   if (h[threadIdx.x]) atomicAdd(&hist[threadIdx.x], (unsigned long long)h[threadIdx.x]);
 }
 
+// Top-N selection on the device: the same digit choice with digits of 11 bits
+// (six per word, the last of 9), made by the last block of each round, so that
+// the rounds follow one another without the host.  A round whose selection is
+// settled returns at once; the host enqueues all of them.  (With 8-bit digits
+// and the choice on the host, a selection waited for a copy per digit: up to 16
+// round trips, 0.4 ms.)
+constexpr int kSelBits = 11, kSelBins = 1 << kSelBits, kSelRounds = 12;
+__host__ __device__ inline int sel_shift(int round) {
+  const int d = round % 6;
+  return d == 5 ? 0 : 64 - kSelBits * (d + 1);
+}
+
+__global__ void __launch_bounds__(256) k_select_round(const uint64_t *keys, const double *scores,
+                                                      size_t n, int round, SelState *st,
+                                                      uint32_t *hist) {
+  __shared__ uint32_t h[kSelBins];
+  __shared__ uint32_t part[256];
+  __shared__ bool last;
+  if (st->done) return;
+  for (int i = threadIdx.x; i < kSelBins; i += 256) h[i] = 0;
+  const uint64_t p_hi = st->pre[0], p_lo = st->pre[1];
+  const int word = round / 6, sh = sel_shift(round);
+  // the bits fixed so far: every higher digit of the word (and the high word)
+  const int top = round % 6 == 0 ? 64 : sel_shift(round - 1);
+  const uint64_t mask = top == 64 ? 0ull : ~0ull << top;
+  const uint32_t bins = round % 6 == 5 ? 1u << 9 : (uint32_t)kSelBins;
+  __syncthreads();
+  // warp-uniform loop: equal digits of a warp are counted with one atomic
+  // (the leading digits are the exponents, nearly all alike)
+  const uint32_t lane = threadIdx.x & 31u;
+  for (size_t i0 = (size_t)blockIdx.x * 256 + (threadIdx.x & ~31u); i0 < n;
+       i0 += (size_t)gridDim.x * 256) {
+    const size_t i = i0 + lane;
+    uint32_t d = kSelBins;
+    if (i < n) {
+      const uint64_t hi = ~((uint64_t)__double_as_longlong(fabs(scores[i])));
+      bool in;
+      uint64_t w = hi;
+      if (word == 0) {
+        in = (hi & mask) == p_hi;
+      } else {
+        in = hi == p_hi;
+        if (in) {
+          w = keys[i];
+          in = (w & mask) == p_lo;
+        }
+      }
+      if (in) d = (uint32_t)(w >> sh) & (bins - 1u);
+    }
+    if (!__any_sync(0xffffffffu, d < (uint32_t)kSelBins)) continue;
+    const uint32_t peers = __match_any_sync(0xffffffffu, d);
+    if (d < (uint32_t)kSelBins && (int)lane == __ffs(peers) - 1) atomicAdd(&h[d], __popc(peers));
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < kSelBins; i += 256)
+    if (h[i]) atomicAdd(&hist[i], h[i]);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&st->ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  // thread t: bins [8 t, 8 t + 8); the bin that holds the remaining-th entry
+  constexpr int kPer = kSelBins / 256;
+  uint32_t c[kPer], own = 0;
+  for (int k = 0; k < kPer; ++k) {
+    c[k] = __ldcg(&hist[threadIdx.x * kPer + k]);
+    hist[threadIdx.x * kPer + k] = 0;
+    own += c[k];
+  }
+  part[threadIdx.x] = own;
+  __syncthreads();
+  for (int o = 1; o < 256; o <<= 1) {
+    const uint32_t y = (int)threadIdx.x >= o ? part[threadIdx.x - o] : 0u;
+    __syncthreads();
+    part[threadIdx.x] += y;
+    __syncthreads();
+  }
+  const uint64_t remaining = st->remaining;
+  uint64_t below = part[threadIdx.x] - own;
+  __syncthreads();
+  if (threadIdx.x == 0) st->ticket = 0u;
+  if (below < remaining && below + own >= remaining) {
+    int k = 0;
+    for (; k < kPer - 1 && below + c[k] < remaining; ++k) below += c[k];
+    const uint64_t digit = (uint64_t)(threadIdx.x * kPer + k);
+    const uint64_t pre = st->pre[word] | (digit << sh);
+    st->pre[word] = pre;
+    st->remaining = remaining - below;
+    // the whole bin is selected: every lower bit of the threshold is set
+    const bool whole = c[k] == remaining - below;
+    if (whole || round == kSelRounds - 1) {
+      const uint64_t low = whole ? ~(~0ull << sh) : 0ull;
+      st->thr[0] = word == 0 ? pre | low : st->pre[0];
+      st->thr[1] = word == 0 ? ~0ull : pre | low;
+      st->done = 1;
+    }
+  }
+}
+
+__global__ void k_select_marks(const uint64_t *keys, const double *scores, size_t n,
+                               const SelState *st, uint32_t *flag) {
+  const uint64_t t_hi = st->thr[0], t_lo = st->thr[1];
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (size_t)gridDim.x * blockDim.x) {
+    const uint64_t hi = ~((uint64_t)__double_as_longlong(fabs(scores[i])));
+    flag[i] = (hi < t_hi || (hi == t_hi && keys[i] <= t_lo)) ? 1u : 0u;
+  }
+}
+
+// Marked entries of both arrays, at most m of them.
+__global__ void k_select_compact(const uint64_t *keys, const double *scores, const uint32_t *flag,
+                                 const uint32_t *pos, size_t n, size_t m, uint64_t *out_keys,
+                                 double *out_scores) {
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (size_t)gridDim.x * blockDim.x)
+    if (flag[i] && pos[i] < m) {
+      out_keys[pos[i]] = keys[i];
+      out_scores[pos[i]] = scores[i];
+    }
+}
+
 __global__ void k_select_flags(const uint64_t *keys, const double *scores, size_t n,
                                uint64_t t_hi, uint64_t t_lo, uint32_t *flag) {
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -184,61 +316,46 @@ int diagonal_packed(const DevInts &I, const uint64_t *keys, size_t n, double *ou
 
 int select_topn_packed(const uint64_t *keys, const double *scores, size_t n, size_t N,
                        uint64_t *out_keys, double *out_scores, size_t *host_out_n,
-                       Arena &arena) {
+                       Arena &arena, double *host_min) {
   *host_out_n = 0;
   if (!n || !N) return ASCI_OK;
   cudaStream_t s = arena.stream();
-  uint32_t *flag, *pos;
+  const size_t m = std::min(n, N);
+  *host_out_n = m;
+  if (N >= n) {  // everything is selected
+    ASCI_TRY_CUDA(cudaMemcpyAsync(out_keys, keys, n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
+    ASCI_TRY_CUDA(cudaMemcpyAsync(out_scores, scores, n * sizeof(double), cudaMemcpyDeviceToDevice,
+                                  s));
+    if (host_min) ASCI_TRY(abs_min(scores, n, host_min, arena));
+    return ASCI_OK;
+  }
+  uint32_t *flag, *pos, *hist;
+  SelState *st;
   ASCI_TRY(arena.alloc(&flag, n));
   ASCI_TRY(arena.alloc(&pos, n));
-  uint64_t t_hi = ~0ull, t_lo = ~0ull;  // select everything when N >= n
-  if (N < n) {
-    unsigned long long *dhist;
-    ASCI_TRY(arena.alloc(&dhist, 256));
-    uint64_t pre_hi = 0, pre_lo = 0, m_hi = 0, m_lo = 0;
-    uint64_t remaining = N;
-    for (int digit = 15; digit >= 0; --digit) {
-      ASCI_TRY_CUDA(cudaMemsetAsync(dhist, 0, 256 * sizeof(unsigned long long), s));
-      k_select_hist<<<grid_for(n), 256, 0, s>>>(keys, scores, n, digit, pre_hi, pre_lo, m_hi,
-                                                m_lo, dhist);
-      ASCI_CHECK_LAUNCH();
-      unsigned long long h[256];
-      ASCI_TRY_CUDA(cudaMemcpyAsync(h, dhist, sizeof(h), cudaMemcpyDeviceToHost, s));
-      ASCI_TRY_CUDA(cudaStreamSynchronize(s));
-      uint64_t cum = 0;
-      int d = 0;
-      for (; d < 256; ++d) {
-        if (cum + h[d] >= remaining) break;
-        cum += h[d];
-      }
-      if (d == 256) return ASCI_ECUDA;  // inconsistent histogram
-      remaining -= cum;
-      uint64_t dv = (uint64_t)d;
-      if (digit >= 8) {
-        pre_hi |= dv << ((digit - 8) * 8);
-        m_hi |= 0xffull << ((digit - 8) * 8);
-      } else {
-        pre_lo |= dv << (digit * 8);
-        m_lo |= 0xffull << (digit * 8);
-      }
-      if (h[d] == remaining) {
-        // the whole bucket is selected: threshold = prefix with all lower bits set
-        t_hi = pre_hi | ~m_hi;
-        t_lo = pre_lo | ~m_lo;
-        break;
-      }
-      t_hi = pre_hi;
-      t_lo = pre_lo;
-    }
+  ASCI_TRY(arena.alloc(&hist, (size_t)kSelBins));
+  ASCI_TRY(arena.alloc(&st, 1));
+  SelState init{};
+  init.remaining = N;
+  ASCI_TRY_CUDA(cudaMemsetAsync(hist, 0, kSelBins * sizeof(uint32_t), s));
+  ASCI_TRY_CUDA(cudaMemcpyAsync(st, &init, sizeof(init), cudaMemcpyHostToDevice, s));
+  for (int round = 0; round < kSelRounds; ++round) {
+    k_select_round<<<grid_for(n, 152 * 4), 256, 0, s>>>(keys, scores, n, round, st, hist);
+    ASCI_CHECK_LAUNCH();
   }
-  k_select_flags<<<grid_for(n), 256, 0, s>>>(keys, scores, n, t_hi, t_lo, flag);
+  k_select_marks<<<grid_for(n), 256, 0, s>>>(keys, scores, n, st, flag);
   ASCI_CHECK_LAUNCH();
   ASCI_TRY(scan_exclusive_u32(flag, pos, n, arena));
-  size_t m = 0;
-  ASCI_TRY(kept_count(flag, pos, n, &m, arena));
-  ASCI_TRY(compact_u64(keys, flag, pos, n, out_keys, arena));
-  ASCI_TRY(compact_f64(scores, flag, pos, n, out_scores, arena));
-  *host_out_n = m;
+  k_select_compact<<<grid_for(n), 256, 0, s>>>(keys, scores, flag, pos, n, m, out_keys, out_scores);
+  ASCI_CHECK_LAUNCH();
+  if (host_min) {
+    // the selected entry of largest R has the smallest |S|: thr bounds it from
+    // below (its free low bits are set)
+    ASCI_TRY_CUDA(cudaMemcpyAsync(&init, st, sizeof(init), cudaMemcpyDeviceToHost, s));
+    ASCI_TRY_CUDA(cudaStreamSynchronize(s));
+    const uint64_t bits = ~init.thr[0];
+    memcpy(host_min, &bits, sizeof(bits));
+  }
   return ASCI_OK;
 }
 

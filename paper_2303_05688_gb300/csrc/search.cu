@@ -80,7 +80,6 @@ size_t tile_capacity();
 size_t big_tile_capacity();
 int exact_scores(const FusedCore &F, const uint64_t *key, double *score, size_t n,
                  cudaStream_t s);
-int abs_min(const double *s, size_t n, double *host_min, Arena &arena);
 int pt2_terms(const FusedCore &F, const uint64_t *key, const double *num, size_t n,
               long long *limbs, unsigned *err, cudaStream_t s);
 int pt2_value(const long long *limbs, double *out, cudaStream_t s);
@@ -902,11 +901,12 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   // the final cutoff, so nothing that can still be selected is ever dropped).
   auto prune = [&](Arena &pa) -> int {
     size_t m2 = 0;
+    double least = 0.0;
     ASCI_TRY(select_topn_packed(pool_k[pcur], pool_s[pcur], pool_n, N, pool_k[pcur ^ 1],
-                                pool_s[pcur ^ 1], &m2, pa));
+                                pool_s[pcur ^ 1], &m2, pa, &least));
     pcur ^= 1;
     pool_n = m2;
-    if (m2 >= N && N > 0) ASCI_TRY(abs_min(pool_s[pcur], pool_n, &tau, pa));
+    if (m2 >= N && N > 0) tau = least;
     unsigned long long c = pool_n;
     ASCI_TRY_CUDA(cudaMemcpyAsync(dcount, &c, sizeof(c), cudaMemcpyDefault, stream));
     ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
