@@ -206,6 +206,12 @@ __host__ __device__ inline uint64_t pack_key(uint32_t a, uint32_t b) {
 __host__ __device__ inline uint32_t key_alpha(uint64_t k) { return (uint32_t)k; }
 __host__ __device__ inline uint32_t key_beta(uint64_t k) { return (uint32_t)(k >> 32); }
 
+// The bits of packed keys that determinants of n orbitals use.
+__host__ __device__ inline uint64_t key_bits(int n) {
+  const uint64_t w = n >= 32 ? 0xffffffffull : (1ull << n) - 1ull;
+  return (w << 32) | w;
+}
+
 // Sign of the single p -> q on string s: (-1)^popc(s & bits strictly between).
 __device__ __forceinline__ int single_parity(uint32_t s, int p, int q) {
   int lo = p < q ? p : q, hi = p < q ? q : p;
@@ -355,13 +361,16 @@ int scan_item_heads(const uint64_t *items, uint64_t T, uint32_t *excl, Arena &ar
 // each pair are swapped as passes proceed).  n < 2^32.
 int radix_sort_u64(uint64_t **keys, uint64_t **keys_alt, size_t n, int begin_bit, int end_bit,
                    Arena &arena);
+// With *varying the caller names the bits that may vary among the keys (a digit
+// with none of them is skipped; others would be left unsorted); without it they
+// are found first, which waits for the device when n > 4096.
 int radix_sort_u64_u32(uint64_t **keys, uint64_t **keys_alt, uint32_t **vals, uint32_t **vals_alt,
-                       size_t n, int begin_bit, int end_bit, Arena &arena);
+                       size_t n, int begin_bit, int end_bit, Arena &arena,
+                       const uint64_t *varying = nullptr);
 int radix_sort_u64_f64(uint64_t **keys, uint64_t **keys_alt, double **vals, double **vals_alt,
-                       size_t n, int begin_bit, int end_bit, Arena &arena);
-// The same keys-only sort when the caller knows which bits vary among the
-// keys (a digit with no varying bit is skipped; varying bits outside the mask
-// would be left unsorted).
+                       size_t n, int begin_bit, int end_bit, Arena &arena,
+                       const uint64_t *varying = nullptr);
+// The same for keys alone.
 int radix_sort_u64_varying(uint64_t **keys, uint64_t **keys_alt, size_t n, int begin_bit,
                            int end_bit, uint64_t varying, Arena &arena);
 

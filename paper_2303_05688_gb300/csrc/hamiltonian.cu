@@ -1686,7 +1686,7 @@ static int det_keys(const asci_det *dets, size_t n, int norb, uint64_t *keys, in
   k_det_keys<<<blocks_for(n, 256), 256, 0, s>>>(dets, n, norb, *na, *nb, keys, err);
   ASCI_CHECK_LAUNCH();
   ASCI_TRY_CUDA(cudaMemcpyAsync(sk, keys, n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
-  ASCI_TRY(radix_sort_u64(&sk, &sk_alt, n, 0, 64, arena));
+  ASCI_TRY(radix_sort_u64_varying(&sk, &sk_alt, n, 0, 64, key_bits(norb), arena));
   k_adjacent_equal<<<blocks_for(n, 256), 256, 0, s>>>(sk, n, err);
   ASCI_CHECK_LAUNCH();
   unsigned herr = 0;
@@ -1787,7 +1787,8 @@ static int loop_impl(const asci_det *dets_in, const double *coeffs_in, size_t nd
   ASCI_TRY(arena.alloc(&c, nd));
   ASCI_TRY(arena.alloc(&c_alt, nd));
   ASCI_TRY_CUDA(cudaMemcpyAsync(c, coeffs, nd * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  ASCI_TRY(radix_sort_u64_f64(&keys, &keys_alt, &c, &c_alt, nd, 0, 64, arena));
+  const uint64_t used = key_bits(norb);
+  ASCI_TRY(radix_sort_u64_f64(&keys, &keys_alt, &c, &c_alt, nd, 0, 64, arena, &used));
   double *sc;
   DotScratch part;
   ASCI_TRY(dot_scratch(&part, arena));
@@ -1877,7 +1878,7 @@ static int loop_impl(const asci_det *dets_in, const double *coeffs_in, size_t nd
     ASCI_TRY(sa.alloc(&sel_v_alt, keep));
     size_t nsel = 0;
     ASCI_TRY(select_topn_packed(uk, uv, tot, o.ntdets, sel_k, sel_v, &nsel, sa));
-    ASCI_TRY(radix_sort_u64_f64(&sel_k, &sel_k_alt, &sel_v, &sel_v_alt, nsel, 0, 64, sa));
+    ASCI_TRY(radix_sort_u64_f64(&sel_k, &sel_k_alt, &sel_v, &sel_v_alt, nsel, 0, 64, sa, &used));
     // determinants that entered (selected keys absent from psi_k)
     unsigned long long entered = 0;
     {
@@ -1993,7 +1994,8 @@ int asci_hamiltonian(const asci_det *dets, size_t n, const asci_ints *ints, int6
   // key order, and whether the caller's order already is key order
   k_iota<<<blocks_for(n, 256), 256, 0, s>>>(perm, (uint32_t)n);
   ASCI_CHECK_LAUNCH();
-  ASCI_TRY(radix_sort_u64_u32(&keys, &keys_alt, &perm, &perm_alt, n, 0, 64, arena));
+  const uint64_t used = key_bits(ints->norb);
+  ASCI_TRY(radix_sort_u64_u32(&keys, &keys_alt, &perm, &perm_alt, n, 0, 64, arena, &used));
   unsigned *flag, hflag = 0;
   ASCI_TRY(arena.alloc(&flag, 1));
   ASCI_TRY_CUDA(cudaMemsetAsync(flag, 0, sizeof(unsigned), s));

@@ -32,8 +32,7 @@
 namespace asci {
 
 int make_items(const ExcCounts &X, int n, const uint32_t *grp_alpha, uint32_t ngroups,
-               uint32_t o_begin, uint32_t nops, int opbits, uint64_t *items,
-               uint64_t *varying, Arena &arena);
+               uint32_t o_begin, uint32_t nops, int opbits, uint64_t *items, Arena &arena);
 int compact_u64(const uint64_t *in, const uint32_t *keep, const uint32_t *pos, size_t n,
                 uint64_t *out, Arena &arena);
 int compact_f64(const double *in, const uint32_t *keep, const uint32_t *pos, size_t n, double *out,
@@ -129,7 +128,7 @@ enum : uint32_t {
 };
 
 __global__ void k_prepare_psi(const asci_det *dets, const double *c, size_t nd, int norb, int na,
-                              int nb, uint64_t *keys, uint32_t *idx, unsigned *err) {
+                              int nb, uint64_t *keys, uint64_t *keys2, unsigned *err) {
   const uint64_t hi = ~((1ull << norb) - 1ull);  // norb <= 32
   unsigned e = 0;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nd;
@@ -138,8 +137,9 @@ __global__ void k_prepare_psi(const asci_det *dets, const double *c, size_t nd, 
     if ((d.alpha & hi) || (d.beta & hi)) e |= kBadRange;
     if (na >= 0 && (__popcll(d.alpha) != na || __popcll(d.beta) != nb)) e |= kBadCount;
     if (!isfinite(c[i])) e |= kBadValue;
-    keys[i] = pack_key((uint32_t)d.alpha, (uint32_t)d.beta);
-    idx[i] = (uint32_t)i;
+    const uint64_t k = pack_key((uint32_t)d.alpha, (uint32_t)d.beta);
+    keys[i] = k;
+    if (keys2) keys2[i] = k;
   }
   if (e) atomicOr(err, e);
 }
@@ -160,32 +160,11 @@ __global__ void k_check_dups(const uint64_t *sorted, size_t n, unsigned *err) {
   if (e) atomicOr(err, e);
 }
 
-// key for the core order: ~bits(|c|) ascending = |c| descending
-__global__ void k_abs_keys(const uint32_t *idx, const double *c, size_t n, uint64_t *out) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x)
-    out[i] = ~(uint64_t)__double_as_longlong(fabs(c[idx[i]]));
-}
-
-// gather the core: alpha as the sort key (low word), payload = core position
-__global__ void k_gather_core(const uint32_t *core_idx, const uint64_t *psi_keys_by_input,
-                              const double *c, size_t m, uint64_t *alpha_keys, uint32_t *pos,
-                              uint64_t *core_keys, double *core_c) {
+// core determinants as sort keys with the alpha string in the high word
+__global__ void k_core_alpha(const uint64_t *core_keys, size_t m, uint64_t *out) {
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < m;
-       j += (size_t)gridDim.x * blockDim.x) {
-    uint32_t i = core_idx[j];
-    uint64_t k = psi_keys_by_input[i];
-    core_keys[j] = k;
-    core_c[j] = c[i];
-    alpha_keys[j] = (uint64_t)key_alpha(k);
-    pos[j] = (uint32_t)j;
-  }
-}
-
-__global__ void k_low_words(const uint64_t *in, size_t n, uint32_t *out) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x)
-    out[i] = (uint32_t)in[i];
+       j += (size_t)gridDim.x * blockDim.x)
+    out[j] = (core_keys[j] << 32) | (core_keys[j] >> 32);
 }
 
 __global__ void k_input_keys(const asci_det *dets, size_t nd, uint64_t *keys) {
@@ -206,25 +185,23 @@ __global__ void k_input_keys_checked(const asci_det *dets, size_t nd, uint64_t *
   }
 }
 
-// core sorted by alpha: group heads, per-det beta and coefficient in that order
-__global__ void k_group_heads(const uint64_t *alpha_sorted, const uint32_t *pos,
-                              const uint64_t *core_keys, const double *core_c, size_t m,
-                              uint32_t *head, uint32_t *beta_sorted, double *c_sorted) {
+// core sorted by alpha: group heads, both strings of each determinant
+__global__ void k_group_heads(const uint64_t *sorted, size_t m, uint32_t *head, uint32_t *alpha,
+                              uint32_t *beta) {
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < m;
        j += (size_t)gridDim.x * blockDim.x) {
-    head[j] = (j == 0 || alpha_sorted[j] != alpha_sorted[j - 1]) ? 1u : 0u;
-    uint32_t p = pos[j];
-    beta_sorted[j] = key_beta(core_keys[p]);
-    c_sorted[j] = core_c[p];
+    head[j] = (j == 0 || (sorted[j] >> 32) != (sorted[j - 1] >> 32)) ? 1u : 0u;
+    alpha[j] = (uint32_t)(sorted[j] >> 32);
+    beta[j] = (uint32_t)sorted[j];
   }
 }
 
-__global__ void k_group_table(const uint32_t *head, const uint32_t *gid, const uint64_t *alpha_sorted,
+__global__ void k_group_table(const uint32_t *head, const uint32_t *gid, const uint32_t *alpha,
                               size_t m, uint32_t *grp_alpha, uint32_t *grp_start) {
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < m;
        j += (size_t)gridDim.x * blockDim.x)
     if (head[j]) {
-      grp_alpha[gid[j]] = (uint32_t)alpha_sorted[j];
+      grp_alpha[gid[j]] = alpha[j];
       grp_start[gid[j]] = (uint32_t)j;
     }
 }
@@ -602,25 +579,62 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   unsigned *derr;
   ASCI_TRY(arena.alloc(&derr, 1));
   ASCI_TRY_CUDA(cudaMemsetAsync(derr, 0, sizeof(unsigned), stream));
-  uint64_t *pkeys, *pkeys_alt, *absk, *absk_alt;
-  uint32_t *pidx, *pidx_alt;
+  uint64_t *pkeys, *pkeys_alt, *in_keys;
   ASCI_TRY(arena.alloc(&pkeys, nd));
   ASCI_TRY(arena.alloc(&pkeys_alt, nd));
-  ASCI_TRY(arena.alloc(&pidx, nd));
-  ASCI_TRY(arena.alloc(&pidx_alt, nd));
-  k_prepare_psi<<<grid_for(nd), 256, 0, stream>>>(dets, coeffs, nd, n, na, nb, pkeys, pidx, derr);
+  ASCI_TRY(arena.alloc(&in_keys, nd));
+  k_prepare_psi<<<grid_for(nd), 256, 0, stream>>>(dets, coeffs, nd, n, na, nb, in_keys, pkeys, derr);
   ASCI_CHECK_LAUNCH();
   k_check_finite<<<grid_for((size_t)n * n * n * n), 256, 0, stream>>>(eri, (size_t)n * n * n * n,
                                                                        derr);
   ASCI_CHECK_LAUNCH();
   k_check_finite<<<grid_for((size_t)n * n), 256, 0, stream>>>(h1, (size_t)n * n, derr);
   ASCI_CHECK_LAUNCH();
-  // psi keys sorted (exclusion table) with input positions
-  ASCI_TRY(radix_sort_u64_u32(&pkeys, &pkeys_alt, &pidx, &pidx_alt, nd, 0, 64, arena));
+  // psi keys sorted (exclusion table)
+  const uint64_t used = key_bits(n), used_alpha = used & 0xffffffff00000000ull;
+  ASCI_TRY(radix_sort_u64_varying(&pkeys, &pkeys_alt, nd, 0, 64, used, arena));
   k_check_dups<<<grid_for(nd), 256, 0, stream>>>(pkeys, nd, derr);
   ASCI_CHECK_LAUNCH();
+  const uint64_t *psi_sorted = pkeys;
+  // the core: the m determinants of largest |c|, ties by key.  Their order does
+  // not matter (they are grouped by alpha string next), so they are selected,
+  // not sorted: eight digit passes over psi took 0.3 of the 1.0 ms of the
+  // preparation at 1e6 determinants.
+  const size_t m = std::min(C, nd);
+  const uint64_t *core_keys = in_keys;
+  double *core_c_sorted, *core_c_alt;
+  uint64_t *alpha_k, *alpha_k_alt;
+  ASCI_TRY(arena.alloc(&core_c_sorted, m));
+  ASCI_TRY(arena.alloc(&core_c_alt, m));
+  ASCI_TRY(arena.alloc(&alpha_k, m));
+  ASCI_TRY(arena.alloc(&alpha_k_alt, m));
+  if (m < nd) {
+    uint64_t *sel;
+    size_t got = 0;
+    ASCI_TRY(arena.alloc(&sel, m));
+    ASCI_TRY(select_topn_packed(in_keys, coeffs, nd, m, sel, core_c_sorted, &got, arena));
+    core_keys = sel;
+  } else {
+    ASCI_TRY_CUDA(cudaMemcpyAsync(core_c_sorted, coeffs, m * sizeof(double),
+                                  cudaMemcpyDeviceToDevice, stream));
+  }
+  k_core_alpha<<<grid_for(m), 256, 0, stream>>>(core_keys, m, alpha_k);
+  ASCI_CHECK_LAUNCH();
+  ASCI_TRY(radix_sort_u64_f64(&alpha_k, &alpha_k_alt, &core_c_sorted, &core_c_alt, m, 32, 64, arena,
+                              &used_alpha));
+  uint32_t *ghead, *gid, *core_alpha, *core_beta;
+  ASCI_TRY(arena.alloc(&ghead, m));
+  ASCI_TRY(arena.alloc(&gid, m));
+  ASCI_TRY(arena.alloc(&core_alpha, m));
+  ASCI_TRY(arena.alloc(&core_beta, m));
+  k_group_heads<<<grid_for(m), 256, 0, stream>>>(alpha_k, m, ghead, core_alpha, core_beta);
+  ASCI_CHECK_LAUNCH();
+  ASCI_TRY(scan_exclusive_u32(ghead, gid, m, arena));
   unsigned herr = 0;
+  uint32_t lastg[2];
   ASCI_TRY_CUDA(cudaMemcpyAsync(&herr, derr, sizeof(herr), cudaMemcpyDefault, stream));
+  ASCI_TRY_CUDA(cudaMemcpyAsync(&lastg[0], gid + m - 1, 4, cudaMemcpyDefault, stream));
+  ASCI_TRY_CUDA(cudaMemcpyAsync(&lastg[1], ghead + m - 1, 4, cudaMemcpyDefault, stream));
   ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
   if (herr) {
     record_error(herr & kDuplicate   ? "duplicate determinants in psi"
@@ -630,49 +644,12 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
                  __FILE__, __LINE__);
     return ASCI_EINVAL;
   }
-  const uint64_t *psi_sorted = pkeys;
-  // the psi key buffer stays live; reuse the alternates for the core order
-  ASCI_TRY(arena.alloc(&absk, nd));
-  ASCI_TRY(arena.alloc(&absk_alt, nd));
-  k_abs_keys<<<grid_for(nd), 256, 0, stream>>>(pidx, coeffs, nd, absk);
-  ASCI_CHECK_LAUNCH();
-  ASCI_TRY(radix_sort_u64_u32(&absk, &absk_alt, &pidx, &pidx_alt, nd, 0, 64, arena));
-  const size_t m = std::min(C, nd);
-  // keys of psi by input position (for gathering the core)
-  uint64_t *in_keys;
-  ASCI_TRY(arena.alloc(&in_keys, nd));
-  k_input_keys<<<grid_for(nd), 256, 0, stream>>>(dets, nd, in_keys);
-  ASCI_CHECK_LAUNCH();
-  uint64_t *core_keys, *alpha_k, *alpha_k_alt;
-  double *core_c;
-  uint32_t *cpos, *cpos_alt;
-  ASCI_TRY(arena.alloc(&core_keys, m));
-  ASCI_TRY(arena.alloc(&core_c, m));
-  ASCI_TRY(arena.alloc(&alpha_k, m));
-  ASCI_TRY(arena.alloc(&alpha_k_alt, m));
-  ASCI_TRY(arena.alloc(&cpos, m));
-  ASCI_TRY(arena.alloc(&cpos_alt, m));
-  k_gather_core<<<grid_for(m), 256, 0, stream>>>(pidx, in_keys, coeffs, m, alpha_k, cpos, core_keys,
-                                                 core_c);
-  ASCI_CHECK_LAUNCH();
-  ASCI_TRY(radix_sort_u64_u32(&alpha_k, &alpha_k_alt, &cpos, &cpos_alt, m, 0, 32, arena));
-  uint32_t *ghead, *gid, *core_beta;
-  double *core_c_sorted;
-  ASCI_TRY(arena.alloc(&ghead, m));
-  ASCI_TRY(arena.alloc(&gid, m));
-  ASCI_TRY(arena.alloc(&core_beta, m));
-  ASCI_TRY(arena.alloc(&core_c_sorted, m));
-  k_group_heads<<<grid_for(m), 256, 0, stream>>>(alpha_k, cpos, core_keys, core_c, m, ghead,
-                                                 core_beta, core_c_sorted);
-  ASCI_CHECK_LAUNCH();
-  ASCI_TRY(scan_exclusive_u32(ghead, gid, m, arena));
-  size_t ngroups = 0;
-  ASCI_TRY(kept_count(ghead, gid, m, &ngroups, arena));
+  const size_t ngroups = (size_t)lastg[0] + lastg[1];
   uint32_t *grp_alpha, *grp_start, *grp_count;
   ASCI_TRY(arena.alloc(&grp_alpha, ngroups));
   ASCI_TRY(arena.alloc(&grp_start, ngroups));
   ASCI_TRY(arena.alloc(&grp_count, ngroups));
-  k_group_table<<<grid_for(m), 256, 0, stream>>>(ghead, gid, alpha_k, m, grp_alpha, grp_start);
+  k_group_table<<<grid_for(m), 256, 0, stream>>>(ghead, gid, core_alpha, m, grp_alpha, grp_start);
   ASCI_CHECK_LAUNCH();
   k_group_count<<<grid_for(ngroups), 256, 0, stream>>>(grp_start, (uint32_t)ngroups, (uint32_t)m,
                                                        grp_count);
@@ -717,10 +694,8 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   if (T > 0) {
     ASCI_TRY(arena.alloc(&items, T));
     ASCI_TRY(arena.alloc(&items_alt, T));
-    uint64_t varying = 0;  // bits in which the target strings differ
-    ASCI_TRY(make_items(X, n, grp_alpha, (uint32_t)ngroups, o_begin, nops, opbits, items, &varying,
-                        arena));
-    ASCI_TRY(radix_sort_u64_varying(&items, &items_alt, T, 32, 32 + n, varying, arena));
+    ASCI_TRY(make_items(X, n, grp_alpha, (uint32_t)ngroups, o_begin, nops, opbits, items, arena));
+    ASCI_TRY(radix_sort_u64_varying(&items, &items_alt, T, 32, 32 + n, used_alpha, arena));
     ASCI_TRY(arena.alloc(&Wexcl, T + 1));
     ASCI_TRY(scan_item_weights(items, T, opbits, grp_count, X, Wexcl, arena));
     ASCI_TRY_CUDA(cudaMemcpyAsync(&P, Wexcl + T, 8, cudaMemcpyDefault, stream));
@@ -828,15 +803,11 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   ASCI_TRY(build_fx(h1, eri, n, na, nb, ints->ecore, E0, arena, &F.X, &F.E0_x));
   if (st) st->diag_grid_bits = (uint64_t)F.X.s;
   {
-    uint32_t *core_alpha32;
     int64_t *Dx, *Fa, *Fb;
-    ASCI_TRY(arena.alloc(&core_alpha32, m));
     ASCI_TRY(arena.alloc(&Dx, m));
     ASCI_TRY(arena.alloc(&Fa, m * n));
     ASCI_TRY(arena.alloc(&Fb, m * n));
-    k_low_words<<<grid_for(m), 256, 0, stream>>>(alpha_k, m, core_alpha32);
-    ASCI_CHECK_LAUNCH();
-    ASCI_TRY(core_fock(F.X, core_alpha32, core_beta, m, Dx, Fa, Fb, arena));
+    ASCI_TRY(core_fock(F.X, core_alpha, core_beta, m, Dx, Fa, Fb, arena));
     F.Dx = Dx;
     F.Fa = Fa;
     F.Fb = Fb;
@@ -1127,7 +1098,7 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
       double *s2;
       ASCI_TRY(arena.alloc(&k2, nsel));
       ASCI_TRY(arena.alloc(&s2, nsel));
-      ASCI_TRY(radix_sort_u64_f64(&sel_k, &k2, &sel_s, &s2, nsel, 0, 64, arena));
+      ASCI_TRY(radix_sort_u64_f64(&sel_k, &k2, &sel_s, &s2, nsel, 0, 64, arena, &used));
     }
     asci_det *dout = out_dets;
     double *sout = out_scores;
@@ -1313,15 +1284,13 @@ int asci_excitations(const asci_ints *ints, const asci_det *core, const double *
   {
     unsigned *derr;
     uint64_t *tk;
-    uint32_t *ti;
     double *tc;
     ASCI_TRY(arena.alloc(&derr, 1));
     ASCI_TRY(arena.alloc(&tk, ncore));
-    ASCI_TRY(arena.alloc(&ti, ncore));
     ASCI_TRY(arena.alloc(&tc, ncore));
     ASCI_TRY_CUDA(cudaMemsetAsync(derr, 0, sizeof(unsigned), s));
     ASCI_TRY_CUDA(cudaMemsetAsync(tc, 0, ncore * sizeof(double), s));
-    k_prepare_psi<<<grid_for(ncore), 256, 0, s>>>(dcore, tc, ncore, n, na, nb, tk, ti, derr);
+    k_prepare_psi<<<grid_for(ncore), 256, 0, s>>>(dcore, tc, ncore, n, na, nb, tk, nullptr, derr);
     ASCI_CHECK_LAUNCH();
     unsigned herr = 0;
     ASCI_TRY_CUDA(cudaMemcpyAsync(&herr, derr, sizeof(herr), cudaMemcpyDefault, s));
@@ -1367,15 +1336,13 @@ int asci_diagonal(const asci_ints *ints, const asci_det *dets, size_t n, double 
     // no bits at or above norb (they would index past the integral tables)
     unsigned *derr;
     uint64_t *tk;
-    uint32_t *ti;
     double *tc;
     ASCI_TRY(arena.alloc(&derr, 1));
     ASCI_TRY(arena.alloc(&tk, n));
-    ASCI_TRY(arena.alloc(&ti, n));
     ASCI_TRY(arena.alloc(&tc, n));
     ASCI_TRY_CUDA(cudaMemsetAsync(derr, 0, sizeof(unsigned), s));
     ASCI_TRY_CUDA(cudaMemsetAsync(tc, 0, n * sizeof(double), s));
-    k_prepare_psi<<<grid_for(n), 256, 0, s>>>(dd, tc, n, ints->norb, -1, -1, tk, ti, derr);
+    k_prepare_psi<<<grid_for(n), 256, 0, s>>>(dd, tc, n, ints->norb, -1, -1, tk, nullptr, derr);
     ASCI_CHECK_LAUNCH();
     unsigned herr = 0;
     ASCI_TRY_CUDA(cudaMemcpyAsync(&herr, derr, sizeof(herr), cudaMemcpyDefault, s));

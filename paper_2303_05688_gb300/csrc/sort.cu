@@ -272,12 +272,124 @@ __global__ void __launch_bounds__(kSortThreads, 4)
   }
 }
 
+// The whole sort of at most one tile (4096 keys) in one CTA: 16 warps of 256
+// consecutive elements each, the digits that vary one after another in shared
+// memory (the ranks as in the scatter above, so just as stable).  A sort of a
+// small list through the tile kernels takes four or more launches a digit and a
+// host round trip for the varying bits: 2000 (key, index) pairs 95 us in 8
+// digits, against 20 here.
+constexpr int kSmallThreads = 512;
+constexpr int kSmallItems = kSortTile / kSmallThreads;
+constexpr int kSmallWarps = kSmallThreads / 32;
+
+template <typename V, bool kHasVals>
+constexpr size_t small_smem() {
+  return (size_t)kSortTile * (sizeof(uint64_t) + (kHasVals ? sizeof(V) : 0)) +
+         (size_t)(kSmallWarps + 1) * kRadix * sizeof(uint32_t);
+}
+
+template <typename V, bool kHasVals>
+__global__ void __launch_bounds__(kSmallThreads) k_sort_small(uint64_t *keys, V *vals, uint32_t n,
+                                                              int begin_bit, int end_bit) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ uint32_t differ[2];
+  uint64_t *sk = reinterpret_cast<uint64_t *>(sm);
+  V *sv = reinterpret_cast<V *>(sk + kSortTile);
+  uint32_t *wb = reinterpret_cast<uint32_t *>(sm + (size_t)kSortTile * (sizeof(uint64_t) +
+                                                                        (kHasVals ? sizeof(V) : 0)));
+  uint32_t *dstart = wb + kSmallWarps * kRadix;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t base = (uint32_t)warp * (32 * kSmallItems) + lane;
+  if (threadIdx.x < 2) differ[threadIdx.x] = 0;
+  const uint64_t k0 = keys[0];
+  uint64_t k[kSmallItems], acc = 0;
+  V v[kSmallItems];
+#pragma unroll
+  for (int r = 0; r < kSmallItems; ++r) {
+    const uint32_t i = base + 32 * r;
+    k[r] = i < n ? keys[i] : 0ull;
+    if (kHasVals) v[r] = i < n ? vals[i] : V(0);
+    if (i < n) acc |= k[r] ^ k0;
+  }
+  __syncthreads();
+  const uint32_t a0 = __reduce_or_sync(0xffffffffu, (uint32_t)acc);
+  const uint32_t a1 = __reduce_or_sync(0xffffffffu, (uint32_t)(acc >> 32));
+  if (lane == 0) {
+    if (a0) atomicOr(&differ[0], a0);
+    if (a1) atomicOr(&differ[1], a1);
+  }
+  __syncthreads();
+  const uint64_t mask = ((uint64_t)differ[1] << 32) | differ[0];
+  const uint32_t lt = (1u << lane) - 1u;
+  for (int shift = begin_bit; shift < end_bit; shift += 8) {
+    const uint64_t dm = end_bit - shift < 8 ? (1ull << (end_bit - shift)) - 1ull : 0xffull;
+    if (!((mask >> shift) & dm)) continue;  // uniform
+    for (int i = threadIdx.x; i < kSmallWarps * kRadix; i += kSmallThreads) wb[i] = 0;
+    __syncthreads();
+    uint32_t rank[kSmallItems];  // among the warp's keys of the same digit
+#pragma unroll
+    for (int r = 0; r < kSmallItems; ++r) {
+      const bool ok = base + 32 * r < n;
+      const uint32_t d = ok ? (uint32_t)((k[r] >> shift) & 0xffu) : (uint32_t)kRadix;
+      const uint32_t peers = __match_any_sync(0xffffffffu, d);
+      uint32_t before = 0;
+      if (ok) before = wb[warp * kRadix + d];
+      __syncwarp();
+      if (ok && lane == __ffs(peers) - 1) wb[warp * kRadix + d] = before + __popc(peers);
+      __syncwarp();
+      rank[r] = before + __popc(peers & lt);
+    }
+    __syncthreads();
+    uint32_t cnt = 0;
+    if (threadIdx.x < kRadix)
+      for (int w = 0; w < kSmallWarps; ++w) {
+        const uint32_t c = wb[w * kRadix + threadIdx.x];
+        wb[w * kRadix + threadIdx.x] = cnt;
+        cnt += c;
+      }
+    const uint32_t first = block_exclusive_scan<uint32_t>(cnt, nullptr);
+    if (threadIdx.x < kRadix) dstart[threadIdx.x] = first;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSmallItems; ++r)
+      if (base + 32 * r < n) {
+        const uint32_t d = (uint32_t)((k[r] >> shift) & 0xffu);
+        const uint32_t pos = dstart[d] + wb[warp * kRadix + d] + rank[r];
+        sk[pos] = k[r];
+        if (kHasVals) sv[pos] = v[r];
+      }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSmallItems; ++r)
+      if (base + 32 * r < n) {
+        k[r] = sk[base + 32 * r];
+        if (kHasVals) v[r] = sv[base + 32 * r];
+      }
+  }
+#pragma unroll
+  for (int r = 0; r < kSmallItems; ++r)
+    if (base + 32 * r < n) {
+      keys[base + 32 * r] = k[r];
+      if (kHasVals) vals[base + 32 * r] = v[r];
+    }
+}
+
 template <typename V, bool kHasVals>
 int radix_sort_impl(uint64_t **keys, uint64_t **keys_alt, V **vals, V **vals_alt, size_t n,
                     int begin_bit, int end_bit, Arena &arena, const uint64_t *known_mask = nullptr) {
   if (n <= 1 || begin_bit >= end_bit) return ASCI_OK;
   if (n >= (1ull << 32)) return ASCI_EINVAL;
   cudaStream_t s = arena.stream();
+  if (n <= (size_t)kSortTile) {
+    static const cudaError_t small_attr = cudaFuncSetAttribute(
+        k_sort_small<V, kHasVals>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        (int)small_smem<V, kHasVals>());
+    ASCI_TRY_CUDA(small_attr);
+    k_sort_small<V, kHasVals><<<1, kSmallThreads, small_smem<V, kHasVals>(), s>>>(
+        *keys, kHasVals ? *vals : nullptr, (uint32_t)n, begin_bit, end_bit);
+    ASCI_CHECK_LAUNCH();
+    return ASCI_OK;
+  }
   uint32_t ntiles = (uint32_t)((n + kSortTile - 1) / kSortTile);
   uint32_t *hist = nullptr;
   ASCI_TRY(arena.alloc(&hist, (size_t)kRadix * ntiles));
@@ -370,14 +482,16 @@ int radix_sort_u64_varying(uint64_t **keys, uint64_t **keys_alt, size_t n, int b
                                           arena, &varying);
 }
 int radix_sort_u64_u32(uint64_t **keys, uint64_t **keys_alt, uint32_t **vals, uint32_t **vals_alt,
-                       size_t n, int begin_bit, int end_bit, Arena &arena) {
+                       size_t n, int begin_bit, int end_bit, Arena &arena,
+                       const uint64_t *varying) {
   return radix_sort_impl<uint32_t, true>(keys, keys_alt, vals, vals_alt, n, begin_bit, end_bit,
-                                         arena);
+                                         arena, varying);
 }
 int radix_sort_u64_f64(uint64_t **keys, uint64_t **keys_alt, double **vals, double **vals_alt,
-                       size_t n, int begin_bit, int end_bit, Arena &arena) {
+                       size_t n, int begin_bit, int end_bit, Arena &arena,
+                       const uint64_t *varying) {
   return radix_sort_impl<double, true>(keys, keys_alt, vals, vals_alt, n, begin_bit, end_bit,
-                                       arena);
+                                       arena, varying);
 }
 
 }  // namespace asci
