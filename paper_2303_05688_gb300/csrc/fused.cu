@@ -38,33 +38,39 @@ namespace asci {
 
 namespace {
 
-__global__ void k_fx_bound(const double *h1, const double *eri, int n, double *out3) {
-  // out3[0] = max |h_pp|, out3[1] = max_{p!=q} |J-K|, out3[2] = max_{p,q} |J|
-  double a = 0, b = 0, c = 0;
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-    int p = t / n, q = t % n;
-    double J = eri[(((size_t)p * n + p) * n + q) * n + q];
-    double K = eri[(((size_t)p * n + q) * n + q) * n + p];
-    if (p == q) a = fmax(a, fabs(h1[p * n + p]));
-    if (p != q) b = fmax(b, fabs(J - K));
-    c = fmax(c, fabs(J));
-  }
-  __shared__ double sh[3][256];
-  sh[0][threadIdx.x] = a;
-  sh[1][threadIdx.x] = b;
-  sh[2][threadIdx.x] = c;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s0 = 0, s1 = 0, s2 = 0;
-    for (int i = 0; i < blockDim.x; ++i) {
-      s0 = fmax(s0, sh[0][i]);
-      s1 = fmax(s1, sh[1][i]);
-      s2 = fmax(s2, sh[2][i]);
+// out[0] = max |h_pp|, out[1] = max_{p!=q} |J-K|, out[2] = max_{p,q} |J|, and
+// out[3] = the largest single-excitation bound over (i, a): |h_ia| + sum_k
+// (|(ia|kk) - (ik|ka)| + |(ia|kk)|), as bit patterns (ordered like the values,
+// which are not negative).  A warp per pair (p, q); out is zero before.  (One CTA
+// whose first thread compared all 256 partial maxima took 45 and 20 us.)
+__global__ void __launch_bounds__(256) k_fx_bounds(const double *h1, const double *eri, int n,
+                                                   unsigned long long *out) {
+  const int lane = threadIdx.x & 31, t = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  double m[4] = {0, 0, 0, 0};
+  if (t < n * n) {
+    const int p = t / n, q = t - p * n;
+    const double J = eri[(((size_t)p * n + p) * n + q) * n + q];
+    const double K = eri[(((size_t)p * n + q) * n + q) * n + p];
+    if (p == q) m[0] = fabs(h1[t]);
+    if (p != q) m[1] = fabs(J - K);
+    m[2] = fabs(J);
+    double b = 0.0;
+    if (lane < n) {
+      const double ijkk = eri[(((size_t)p * n + q) * n + lane) * n + lane];
+      const double ikkj = eri[(((size_t)p * n + lane) * n + lane) * n + q];
+      b = fabs(ijkk - ikkj) + fabs(ijkk);
     }
-    out3[0] = s0;
-    out3[1] = s1;
-    out3[2] = s2;
+    for (int o = 16; o; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+    m[3] = fabs(h1[t]) + b;
   }
+  __shared__ unsigned long long best[4];
+  if (threadIdx.x < 4) best[threadIdx.x] = 0;
+  __syncthreads();
+  if (lane == 0)
+    for (int k = 0; k < 4; ++k)
+      atomicMax(&best[k], (unsigned long long)__double_as_longlong(m[k]));
+  __syncthreads();
+  if (threadIdx.x < 4 && best[threadIdx.x]) atomicMax(&out[threadIdx.x], best[threadIdx.x]);
 }
 
 __global__ void k_fx_tables(const double *h1, const double *eri, int n, int s, int64_t *hh,
@@ -77,30 +83,6 @@ __global__ void k_fx_tables(const double *h1, const double *eri, int n, int s, i
     jk[t] = (p == q) ? 0 : __double2ll_rn((J - K) * sc);
     jj[t] = __double2ll_rn(J * sc);
     if (p == q) hh[p] = __double2ll_rn(h1[p * n + p] * sc);
-  }
-}
-
-// Largest single-excitation magnitude bound over (i, a):
-// |h_ia| + sum_k |(ia|kk) - (ik|ka)| + sum_k |(ia|kk)|.
-__global__ void k_fx_single_bound(const double *h1, const double *eri, int n, double *out) {
-  double m = 0;
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-    const int i = t / n, a = t % n;
-    double b = fabs(h1[t]);
-    for (int k = 0; k < n; ++k) {
-      const double iakk = eri[(((size_t)i * n + a) * n + k) * n + k];
-      const double ikka = eri[(((size_t)i * n + k) * n + k) * n + a];
-      b += fabs(iakk - ikka) + fabs(iakk);
-    }
-    m = fmax(m, b);
-  }
-  __shared__ double sh[256];
-  sh[threadIdx.x] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double r = 0;
-    for (int i = 0; i < blockDim.x; ++i) r = fmax(r, sh[i]);
-    *out = r;
   }
 }
 
@@ -219,28 +201,31 @@ namespace {
 // diagonals.  Fb is determinant-major (Fb[j n + p]: a warp's lanes read one
 // determinant's row); Fa is orbital-major (Fa[p m + j]: the lanes of an
 // alpha-double step read one orbital of consecutive determinants).
+// A thread per (orbital, determinant), determinants fastest; the thread of
+// orbital n forms H_jj.
 __global__ void k_core_fock(FxInts X, const uint32_t *core_alpha, const uint32_t *core_beta,
                             size_t m, int64_t *Dx, int64_t *Fa, int64_t *Fb) {
-  const int n = X.n;
+  const int n = X.n, p = (int)blockIdx.y;
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < m;
        j += (size_t)gridDim.x * blockDim.x) {
     const uint32_t A = core_alpha[j], B = core_beta[j];
-    Dx[j] = fx_diag(X, A, B);
-    for (int p = 0; p < n; ++p) {
-      int64_t fa = X.hh[p], fb = X.hh[p];
-      for (uint32_t r = A; r; r &= r - 1) {
-        int q = __ffs(r) - 1;
-        fa += X.jk[p * n + q];
-        fb += X.jj[p * n + q];
-      }
-      for (uint32_t r = B; r; r &= r - 1) {
-        int q = __ffs(r) - 1;
-        fb += X.jk[p * n + q];
-        fa += X.jj[p * n + q];
-      }
-      Fa[(size_t)p * m + j] = fa;
-      Fb[j * n + p] = fb;
+    if (p == n) {
+      Dx[j] = fx_diag(X, A, B);
+      continue;
     }
+    int64_t fa = X.hh[p], fb = X.hh[p];
+    for (uint32_t r = A; r; r &= r - 1) {
+      const int q = __ffs(r) - 1;
+      fa += X.jk[p * n + q];
+      fb += X.jj[p * n + q];
+    }
+    for (uint32_t r = B; r; r &= r - 1) {
+      const int q = __ffs(r) - 1;
+      fb += X.jk[p * n + q];
+      fa += X.jj[p * n + q];
+    }
+    Fa[(size_t)p * m + j] = fa;
+    Fb[j * n + p] = fb;
   }
 }
 
@@ -1620,43 +1605,43 @@ __global__ void __launch_bounds__(THREADS, CTAS) k_cells(CellArgs C) {
 // (the correctly rounded exact sum), three or four by the ordered FP64 sum,
 // more by the 128-bit fixed-point accumulator anchored to the largest
 // exponent.  Each depends only on the multiset of values, so not on the order
-// in which they were copied.  One thread per list of at most kWalk values; a
-// longer one is summed by the whole warp (integer additions: the same bits).
-constexpr unsigned long long kWalk = 32;
+// in which they were copied.  Lists of two to four values take one thread, those
+// of up to 64 eight lanes, longer ones the warp (integer additions: the same
+// bits); a thread that walked lists of up to 32 values alone, load after load,
+// made the launch wait 50 us for the longest ones.
+constexpr unsigned kLaneList = 64;
 
-__device__ __forceinline__ double list_sum(const double *x, unsigned len, unsigned *ovf) {
-  if (len == 2) return x[0] + x[1];
-  if (len == 3) return sum4_ordered(0.0, x[0], x[1], x[2]);
-  if (len == 4) return sum4_ordered(x[0], x[1], x[2], x[3]);
+// The rule for five or more values, by the LANES lanes of a group (a power of
+// two); every lane of the warp takes part, len = 0 for an idle group.  The
+// first HELD values of each lane stay in registers, loaded together.
+template <unsigned LANES>
+__device__ __forceinline__ double group_list_sum(const double *x, unsigned len, unsigned *ovf) {
+  constexpr unsigned kHeld = kLaneList / 8;
+  const unsigned lane = threadIdx.x & (LANES - 1u);
+  double v[kHeld];
+#pragma unroll
+  for (unsigned k = 0; k < kHeld; ++k) v[k] = lane + k * LANES < len ? x[lane + k * LANES] : 0.0;
   int emax = 1;
-  for (unsigned j = 0; j < len; ++j) {
-    const int ex = fx_exponent(x[j]);
-    emax = ex > emax ? ex : emax;
-  }
+#pragma unroll
+  for (unsigned k = 0; k < kHeld; ++k) emax = max(emax, fx_exponent(v[k]));
+  for (unsigned j = lane + kHeld * LANES; j < len; j += LANES) emax = max(emax, fx_exponent(x[j]));
+#pragma unroll
+  for (unsigned o = LANES / 2; o; o >>= 1)
+    emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
   const int frac = fx128_frac_for(emax);
   Fx128 acc = {0, 0};
-  for (unsigned j = 0; j < len; ++j) {
+#pragma unroll
+  for (unsigned k = 0; k < kHeld; ++k)
+    if (lane + k * LANES < len) {
+      Fx128 t = fx128_from_double(v[k], frac, ovf);
+      fx128_add(acc, t);
+    }
+  for (unsigned j = lane + kHeld * LANES; j < len; j += LANES) {
     Fx128 t = fx128_from_double(x[j], frac, ovf);
     fx128_add(acc, t);
   }
-  return fx128_to_double(acc, frac);
-}
-
-__device__ __forceinline__ double warp_list_sum(const double *x, unsigned len, unsigned *ovf) {
-  const unsigned lane = threadIdx.x & 31u;
-  int emax = 1;
-  for (unsigned j = lane; j < len; j += 32) {
-    const int ex = fx_exponent(x[j]);
-    emax = ex > emax ? ex : emax;
-  }
-  emax = (int)__reduce_max_sync(0xffffffffu, (unsigned)emax);
-  const int frac = fx128_frac_for(emax);
-  Fx128 acc = {0, 0};
-  for (unsigned j = lane; j < len; j += 32) {
-    Fx128 t = fx128_from_double(x[j], frac, ovf);
-    fx128_add(acc, t);
-  }
-  for (int o = 16; o; o >>= 1) {
+#pragma unroll
+  for (unsigned o = LANES / 2; o; o >>= 1) {
     Fx128 t;
     t.lo = __shfl_xor_sync(0xffffffffu, acc.lo, o);
     t.hi = __shfl_xor_sync(0xffffffffu, acc.hi, o);
@@ -1670,21 +1655,35 @@ __global__ void __launch_bounds__(256) k_long_sums(const ulonglong2 *fix,
                                                    unsigned long long fix_cap, const double *lv,
                                                    double *cand_score, unsigned *err) {
   const unsigned long long n = *nfix < fix_cap ? *nfix : fix_cap;
+  const unsigned lane = threadIdx.x & 31u;
   unsigned ovf = 0;
-  // warp-uniform loop: long lists are summed by the whole warp
+  // warp-uniform loop: the longer lists are shared by the warp's lanes
   for (unsigned long long base = (unsigned long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
        base < n; base += (unsigned long long)gridDim.x * blockDim.x) {
-    const unsigned long long i = base + (threadIdx.x & 31u);
     ulonglong2 f = make_ulonglong2(0, ~0ull);
-    if (i < n) f = fix[i];
+    if (base + lane < n) f = fix[base + lane];
     const bool used = f.y != ~0ull;
-    const unsigned long long len = f.y & 0xffffull;
-    if (used && len <= kWalk) cand_score[f.x] = list_sum(lv + (f.y >> 16), (unsigned)len, &ovf);
-    for (unsigned m = __ballot_sync(0xffffffffu, used && len > kWalk); m; m &= m - 1) {
+    const unsigned len = (unsigned)(f.y & 0xffffull);
+    const double *x = lv + (f.y >> 16);
+    if (used && len == 2) cand_score[f.x] = x[0] + x[1];
+    if (used && len == 3) cand_score[f.x] = sum4_ordered(0.0, x[0], x[1], x[2]);
+    if (used && len == 4) cand_score[f.x] = sum4_ordered(x[0], x[1], x[2], x[3]);
+    for (unsigned m = __ballot_sync(0xffffffffu, used && len > 4u && len <= kLaneList); m;) {
+      // the next four lists, one per group of eight lanes
+      int src = -1;
+      for (unsigned g = 0; g < 4 && m; ++g, m &= m - 1)
+        if (g == lane >> 3) src = __ffs(m) - 1;
+      const unsigned long long y = __shfl_sync(0xffffffffu, f.y, src < 0 ? 0 : src);
+      const unsigned long long at = __shfl_sync(0xffffffffu, f.x, src < 0 ? 0 : src);
+      const double s = group_list_sum<8>(lv + (src < 0 ? 0ull : y >> 16),
+                                         src < 0 ? 0u : (unsigned)(y & 0xffffull), &ovf);
+      if (src >= 0 && (lane & 7u) == 0u) cand_score[at] = s;
+    }
+    for (unsigned m = __ballot_sync(0xffffffffu, used && len > kLaneList); m; m &= m - 1) {
       const int src = __ffs(m) - 1;
       const unsigned long long y = __shfl_sync(0xffffffffu, f.y, src);
-      const double s = warp_list_sum(lv + (y >> 16), (unsigned)(y & 0xffffull), &ovf);
-      if ((int)(threadIdx.x & 31u) == src) cand_score[f.x] = s;
+      const double s = group_list_sum<32>(lv + (y >> 16), (unsigned)(y & 0xffffull), &ovf);
+      if ((int)lane == src) cand_score[f.x] = s;
     }
   }
   if (ovf) atomicOr(err, kErrAccum);
@@ -1706,8 +1705,13 @@ __global__ void k_tile_gather(const TileDesc *tiles, const uint32_t *list, uint3
       const uint32_t mid = (lo + hi) >> 1;
       if ((uint32_t)(spill_keys[mid] >> 32) < t) lo = mid + 1; else hi = mid;
     }
+    // its end by another search (a hot tile spills thousands of records)
     uint32_t e = lo;
-    while (e < nspill && (uint32_t)(spill_keys[e] >> 32) == t) ++e;
+    hi = nspill;
+    while (e < hi) {
+      const uint32_t mid = (e + hi) >> 1;
+      if ((uint32_t)(spill_keys[mid] >> 32) <= t) e = mid + 1; else hi = mid;
+    }
     info[5 * i] = d.start;
     info[5 * i + 1] = d.npairs < (uint32_t)kCap ? d.npairs : (uint32_t)kCap;
     info[5 * i + 2] = d.alpha;
@@ -1989,12 +1993,13 @@ int kept_count(const uint32_t *keep, const uint32_t *pos, size_t n, size_t *host
 int build_fx(const double *h1, const double *eri, int n, int na, int nb, double ecore, double E0,
              Arena &arena, FxInts *out, int64_t *E0_x) {
   cudaStream_t s = arena.stream();
-  double *d3;
-  ASCI_TRY(arena.alloc(&d3, 3));
-  k_fx_bound<<<1, 256, 0, s>>>(h1, eri, n, d3);
+  unsigned long long *dmax;
+  double h3[4];
+  ASCI_TRY(arena.alloc(&dmax, 4));
+  ASCI_TRY_CUDA(cudaMemsetAsync(dmax, 0, 4 * sizeof(unsigned long long), s));
+  k_fx_bounds<<<(unsigned)((n * n * 32 + 255) / 256), 256, 0, s>>>(h1, eri, n, dmax);
   ASCI_CHECK_LAUNCH();
-  double h3[3];
-  ASCI_TRY_CUDA(cudaMemcpyAsync(h3, d3, sizeof(h3), cudaMemcpyDefault, s));
+  ASCI_TRY_CUDA(cudaMemcpyAsync(h3, dmax, sizeof(h3), cudaMemcpyDefault, s));
   ASCI_TRY_CUDA(cudaStreamSynchronize(s));
   // B bounds |E0|, every diagonal element and every Fock-like diagonal value:
   // (na+nb) one-body terms, C(na,2)+C(nb,2) same-spin and na*nb opposite-spin
@@ -2019,13 +2024,7 @@ int build_fx(const double *h1, const double *eri, int n, int na, int nb, double 
   ASCI_CHECK_LAUNCH();
   // single excitations: a sum of at most n + 1 table values stays below the
   // bound Bs, and s1 = 61 - log2(Bs) keeps it inside 64 bits
-  double *d1;
-  ASCI_TRY(arena.alloc(&d1, 1));
-  k_fx_single_bound<<<1, 256, 0, s>>>(h1, eri, n, d1);
-  ASCI_CHECK_LAUNCH();
-  double bs = 0;
-  ASCI_TRY_CUDA(cudaMemcpyAsync(&bs, d1, sizeof(bs), cudaMemcpyDefault, s));
-  ASCI_TRY_CUDA(cudaStreamSynchronize(s));
+  const double bs = h3[3];
   int e1 = 0;
   frexp(bs + 1e-300, &e1);
   int s1 = 61 - e1;
@@ -2070,7 +2069,8 @@ int build_fx(const double *h1, const double *eri, int n, int na, int nb, double 
 int core_fock(const FxInts &X, const uint32_t *core_alpha, const uint32_t *core_beta, size_t m,
               int64_t *Dx, int64_t *Fa, int64_t *Fb, Arena &arena) {
   if (!m) return ASCI_OK;
-  k_core_fock<<<grid_for(m), 256, 0, arena.stream()>>>(X, core_alpha, core_beta, m, Dx, Fa, Fb);
+  k_core_fock<<<dim3(grid_for(m, 152 * 4), X.n + 1), 256, 0, arena.stream()>>>(X, core_alpha, core_beta,
+                                                                              m, Dx, Fa, Fb);
   ASCI_CHECK_LAUNCH();
   return ASCI_OK;
 }
@@ -2463,17 +2463,20 @@ static CellArgs cell_args(const FusedCore &F, const Stage &st,
 
 // Buffers of the targets that the tile kernels leave to k_long_sums, in a
 // scratch arena that outlives the launch and the fix-up that follows it.  With
-// a threshold few targets of several records reach it (at (24e,30o) six a
-// tile of kCap records, with 25 values), and the buffers hold 16 and 80 per
-// kCap records of capacity.  `full` gives room for every record (no threshold,
-// as in ASCI-PT2 and the first batch, where every such target is summed); a
-// launch whose buffers were too small sets kErrValues and is run again so.
+// a threshold few targets of several records can reach it, most where targets
+// collect many records (at most 6 a tile with 75 values at (24e,30o), C = 1e5;
+// 25 with 300 at (16e,16o), C = 1e4): the buffers hold 48 and 512 per kCap
+// records of capacity, 4.9 KB against the 16 KB of the records.  (16 and 80
+// made those two searches run their first launches twice: 209 ms against 199,
+// 6.3 against 5.6.)  `full` gives room for every record (no threshold, as in
+// ASCI-PT2 and the first batch, where every such target is summed); a launch
+// whose buffers were too small sets kErrValues and is run again so.
 static int enable_long_sums(CellArgs &CA, size_t tiles, bool full, Arena &la) {
   const unsigned long long t = tiles, all_fix = t * (kCap / 2), all_lv = t * kCap;
   const unsigned long long fix_cap =
-      full ? all_fix : std::max(t * 16, std::min(all_fix, 1ull << 16));
+      full ? all_fix : std::max(t * 48, std::min(all_fix, 1ull << 16));
   const unsigned long long lv_cap = std::min<unsigned long long>(
-      full ? all_lv : std::max(t * 80, std::min(all_lv, 1ull << 18)), 0xffffffffull);
+      full ? all_lv : std::max(t * 512, std::min(all_lv, 1ull << 18)), 0xffffffffull);
   unsigned long long *cnt;
   ASCI_TRY(la.alloc(&CA.lv, (size_t)lv_cap));
   ASCI_TRY(la.alloc(&CA.fix, (size_t)fix_cap));
@@ -2487,7 +2490,7 @@ static int enable_long_sums(CellArgs &CA, size_t tiles, bool full, Arena &la) {
 }
 
 static int run_long_sums(const CellArgs &CA, int sms, cudaStream_t s) {
-  k_long_sums<<<(unsigned)sms * 4, 256, 0, s>>>(CA.fix, CA.nfix, CA.fix_cap, CA.lv, CA.cand_score,
+  k_long_sums<<<(unsigned)sms * 8, 256, 0, s>>>(CA.fix, CA.nfix, CA.fix_cap, CA.lv, CA.cand_score,
                                                  CA.err);
   ASCI_CHECK_LAUNCH();
   return ASCI_OK;

@@ -119,7 +119,7 @@ __global__ void k_select_hist(const uint64_t *keys, const double *scores, size_t
 // the rounds follow one another without the host.  A round whose selection is
 // settled returns at once; the host enqueues all of them.  (With 8-bit digits
 // and the choice on the host, a selection waited for a copy per digit: up to 16
-// round trips, 0.4 ms.)
+// round trips, 0.4 ms.)  Lists of at most 16384 entries take one CTA instead.
 constexpr int kSelBits = 11, kSelBins = 1 << kSelBits, kSelRounds = 12;
 __host__ __device__ inline int sel_shift(int round) {
   const int d = round % 6;
@@ -211,6 +211,107 @@ __global__ void __launch_bounds__(256) k_select_round(const uint64_t *keys, cons
       st->thr[1] = word == 0 ? ~0ull : pre | low;
       st->done = 1;
     }
+  }
+}
+
+// The whole selection of at most kSmallSelect entries by one CTA: the same
+// digits, as many as it takes, then the selected entries in input order.
+constexpr size_t kSmallSelect = 16384;
+
+__global__ void __launch_bounds__(1024) k_select_small(const uint64_t *keys, const double *scores,
+                                                       uint32_t n, uint32_t N, uint64_t *out_keys,
+                                                       double *out_scores, SelState *st) {
+  __shared__ uint32_t h[kSelBins];
+  __shared__ uint32_t warp_sum[32];
+  __shared__ uint64_t pre[2], thr[2];
+  __shared__ uint32_t remaining, done;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  if (tid == 0) {
+    pre[0] = pre[1] = 0;
+    remaining = N;
+    done = 0;
+  }
+  // exclusive prefix of v over the CTA
+  auto scan = [&](uint32_t v) {
+    uint32_t x = v;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if ((int)lane >= o) x += y;
+    }
+    if (lane == 31) warp_sum[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+      uint32_t w = warp_sum[lane];
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
+        if ((int)lane >= o) w += y;
+      }
+      warp_sum[lane] = w;
+    }
+    __syncthreads();
+    const uint32_t before = warp ? warp_sum[warp - 1] : 0u;
+    return before + x - v;
+  };
+  for (int round = 0; round < kSelRounds; ++round) {
+    for (uint32_t i = tid; i < kSelBins; i += 1024) h[i] = 0;
+    __syncthreads();
+    if (done) break;
+    const int word = round / 6, sh = sel_shift(round);
+    const int top = round % 6 == 0 ? 64 : sel_shift(round - 1);
+    const uint64_t mask = top == 64 ? 0ull : ~0ull << top, p_hi = pre[0], p_lo = pre[1];
+    const uint32_t bins = round % 6 == 5 ? 1u << 9 : (uint32_t)kSelBins;
+    for (uint32_t i0 = tid & ~31u; i0 < n; i0 += 1024) {
+      const uint32_t i = i0 + lane;
+      uint32_t d = kSelBins;
+      if (i < n) {
+        const uint64_t hi = ~((uint64_t)__double_as_longlong(fabs(scores[i])));
+        const uint64_t w = word == 0 ? hi : keys[i];
+        if (word == 0 ? (hi & mask) == p_hi : (hi == p_hi && (w & mask) == p_lo))
+          d = (uint32_t)(w >> sh) & (bins - 1u);
+      }
+      const uint32_t peers = __match_any_sync(0xffffffffu, d);
+      if (d < (uint32_t)kSelBins && (int)lane == __ffs(peers) - 1) atomicAdd(&h[d], __popc(peers));
+    }
+    __syncthreads();
+    const uint32_t c0 = h[2 * tid], c1 = h[2 * tid + 1], want = remaining;
+    const uint32_t below = scan(c0 + c1);
+    if (below < want && below + c0 + c1 >= want) {
+      const bool second = below + c0 < want;
+      const uint32_t under = below + (second ? c0 : 0u);
+      const uint64_t p = pre[word] | ((uint64_t)(2 * tid + (second ? 1u : 0u)) << sh);
+      const bool whole = (second ? c1 : c0) == want - under;
+      pre[word] = p;
+      remaining = want - under;
+      if (whole || round == kSelRounds - 1) {
+        const uint64_t low = whole ? ~(~0ull << sh) : 0ull;
+        thr[0] = word == 0 ? p | low : pre[0];
+        thr[1] = word == 0 ? ~0ull : p | low;
+        done = 1;
+      }
+    }
+    __syncthreads();
+  }
+  __syncthreads();
+  const uint64_t t_hi = thr[0], t_lo = thr[1];
+  uint32_t at = 0;
+  for (uint32_t i0 = 0; i0 < n; i0 += 1024) {
+    const uint32_t i = i0 + tid;
+    bool in = false;
+    if (i < n) {
+      const uint64_t hi = ~((uint64_t)__double_as_longlong(fabs(scores[i])));
+      in = hi < t_hi || (hi == t_hi && keys[i] <= t_lo);
+    }
+    const uint32_t pos = at + scan(in ? 1u : 0u);
+    if (in && pos < N) {
+      out_keys[pos] = keys[i];
+      out_scores[pos] = scores[i];
+    }
+    at += warp_sum[31];
+    __syncthreads();
+  }
+  if (tid == 0) {
+    st->thr[0] = t_hi;
+    st->thr[1] = t_lo;
   }
 }
 
@@ -329,25 +430,31 @@ int select_topn_packed(const uint64_t *keys, const double *scores, size_t n, siz
     if (host_min) ASCI_TRY(abs_min(scores, n, host_min, arena));
     return ASCI_OK;
   }
-  uint32_t *flag, *pos, *hist;
-  SelState *st;
-  ASCI_TRY(arena.alloc(&flag, n));
-  ASCI_TRY(arena.alloc(&pos, n));
-  ASCI_TRY(arena.alloc(&hist, (size_t)kSelBins));
+  SelState *st, init{};
   ASCI_TRY(arena.alloc(&st, 1));
-  SelState init{};
-  init.remaining = N;
-  ASCI_TRY_CUDA(cudaMemsetAsync(hist, 0, kSelBins * sizeof(uint32_t), s));
-  ASCI_TRY_CUDA(cudaMemcpyAsync(st, &init, sizeof(init), cudaMemcpyHostToDevice, s));
-  for (int round = 0; round < kSelRounds; ++round) {
-    k_select_round<<<grid_for(n, 152 * 4), 256, 0, s>>>(keys, scores, n, round, st, hist);
+  if (n <= kSmallSelect) {
+    k_select_small<<<1, 1024, 0, s>>>(keys, scores, (uint32_t)n, (uint32_t)N, out_keys, out_scores,
+                                      st);
+    ASCI_CHECK_LAUNCH();
+  } else {
+    uint32_t *flag, *pos, *hist;
+    ASCI_TRY(arena.alloc(&flag, n));
+    ASCI_TRY(arena.alloc(&pos, n));
+    ASCI_TRY(arena.alloc(&hist, (size_t)kSelBins));
+    init.remaining = N;
+    ASCI_TRY_CUDA(cudaMemsetAsync(hist, 0, kSelBins * sizeof(uint32_t), s));
+    ASCI_TRY_CUDA(cudaMemcpyAsync(st, &init, sizeof(init), cudaMemcpyHostToDevice, s));
+    for (int round = 0; round < kSelRounds; ++round) {
+      k_select_round<<<grid_for(n, 152 * 4), 256, 0, s>>>(keys, scores, n, round, st, hist);
+      ASCI_CHECK_LAUNCH();
+    }
+    k_select_marks<<<grid_for(n), 256, 0, s>>>(keys, scores, n, st, flag);
+    ASCI_CHECK_LAUNCH();
+    ASCI_TRY(scan_exclusive_u32(flag, pos, n, arena));
+    k_select_compact<<<grid_for(n), 256, 0, s>>>(keys, scores, flag, pos, n, m, out_keys,
+                                                 out_scores);
     ASCI_CHECK_LAUNCH();
   }
-  k_select_marks<<<grid_for(n), 256, 0, s>>>(keys, scores, n, st, flag);
-  ASCI_CHECK_LAUNCH();
-  ASCI_TRY(scan_exclusive_u32(flag, pos, n, arena));
-  k_select_compact<<<grid_for(n), 256, 0, s>>>(keys, scores, flag, pos, n, m, out_keys, out_scores);
-  ASCI_CHECK_LAUNCH();
   if (host_min) {
     // the selected entry of largest R has the smallest |S|: thr bounds it from
     // below (its free low bits are set)
