@@ -60,7 +60,9 @@ void count_launch();
   } while (0)
 
 // Stream-ordered scratch arena: every allocation is released when the arena
-// goes out of scope (cudaFreeAsync on the same stream).
+// goes out of scope (cudaFreeAsync on the same stream).  Small allocations are
+// carved from chunks: a pool allocation and its release cost 2 us, and some 20
+// where several threads allocate at once, and a search makes a hundred.
 class Arena {
  public:
   explicit Arena(cudaStream_t s) : stream_(s) {
@@ -95,29 +97,52 @@ class Arena {
       *p = nullptr;
       return ASCI_ENOMEM;
     }
-    cudaError_t e = pool_ ? cudaMallocFromPoolAsync(&q, bytes, pool_, stream_)
-                          : cudaMallocAsync(&q, bytes, stream_);
+    if (bytes <= kChunk / 4) {
+      const size_t need = (bytes + 255) & ~(size_t)255;
+      if (need > chunk_left_ && pool_alloc(&q, kChunk) == cudaSuccess) {
+        chunk_ = static_cast<char *>(q);
+        chunk_left_ = kChunk;
+      }
+      if (need <= chunk_left_) {
+        *p = reinterpret_cast<T *>(chunk_);
+        chunk_ += need;
+        chunk_left_ -= need;
+        return ASCI_OK;
+      }
+    }
+    const cudaError_t e = pool_alloc(&q, bytes);
     if (e != cudaSuccess) {
-      cudaGetLastError();
       record_error(cudaGetErrorString(e), __FILE__, __LINE__);
       *p = nullptr;
       return ASCI_ENOMEM;
     }
-    ptrs_.push_back(q);
     *p = static_cast<T *>(q);
     return ASCI_OK;
   }
   void release() {
     for (void *q : ptrs_) cudaFreeAsync(q, stream_);
     ptrs_.clear();
+    chunk_left_ = 0;
     bump_off_ = 0;
   }
   cudaStream_t stream() const { return stream_; }
 
  private:
+  static constexpr size_t kChunk = 2u << 20;
+  // One allocation of the pool, released with the arena.
+  cudaError_t pool_alloc(void **q, size_t bytes) {
+    const cudaError_t e = pool_ ? cudaMallocFromPoolAsync(q, bytes, pool_, stream_)
+                                : cudaMallocAsync(q, bytes, stream_);
+    if (e == cudaSuccess) ptrs_.push_back(*q);
+    else cudaGetLastError();
+    return e;
+  }
+
   cudaStream_t stream_;
   cudaMemPool_t pool_ = nullptr;
   std::vector<void *> ptrs_;
+  char *chunk_ = nullptr;
+  size_t chunk_left_ = 0;
   char *bump_base_ = nullptr;
   size_t bump_cap_ = 0, bump_off_ = 0;
 };
@@ -167,30 +192,55 @@ int finish_out(T *user, const T *dev, size_t count, cudaStream_t s) {
 }
 
 // Device time between start() and stop() on one stream, added to *acc in
-// milliseconds (stop() waits for the stream to reach the end event).
+// milliseconds once read() has waited for the stream to reach the last event
+// (stop() itself does not wait).
 struct StageTimer {
   cudaStream_t s;
-  cudaEvent_t ev[2];
-  bool ok = false;
-  explicit StageTimer(cudaStream_t st) : s(st) {
-    ok = cudaEventCreate(&ev[0]) == cudaSuccess && cudaEventCreate(&ev[1]) == cudaSuccess;
-  }
-  ~StageTimer() {
-    if (ok) {
-      cudaEventDestroy(ev[0]);
-      cudaEventDestroy(ev[1]);
-    }
-  }
+  struct Span {
+    cudaEvent_t ev[2];
+    double *acc;
+  };
+  std::vector<Span> spans;
+  bool open = false;
+  explicit StageTimer(cudaStream_t st) : s(st) {}
+  StageTimer(const StageTimer &) = delete;
+  StageTimer &operator=(const StageTimer &) = delete;
+  ~StageTimer() { drop(); }
   void start() {
-    if (ok) cudaEventRecord(ev[0], s);
+    Span sp{};
+    if (open || cudaEventCreate(&sp.ev[0]) != cudaSuccess) return;
+    if (cudaEventCreate(&sp.ev[1]) != cudaSuccess) {
+      cudaEventDestroy(sp.ev[0]);
+      return;
+    }
+    cudaEventRecord(sp.ev[0], s);
+    spans.push_back(sp);
+    open = true;
   }
   void stop(double *acc) {
-    if (!ok) return;
-    cudaEventRecord(ev[1], s);
-    cudaEventSynchronize(ev[1]);
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, ev[0], ev[1]);
-    *acc += ms;
+    if (!open) return;
+    spans.back().acc = acc;
+    cudaEventRecord(spans.back().ev[1], s);
+    open = false;
+  }
+  void read() {
+    for (Span &sp : spans) {
+      float ms = 0.f;
+      if (sp.acc && cudaEventSynchronize(sp.ev[1]) == cudaSuccess &&
+          cudaEventElapsedTime(&ms, sp.ev[0], sp.ev[1]) == cudaSuccess)
+        *sp.acc += ms;
+    }
+    drop();
+  }
+
+ private:
+  void drop() {
+    for (Span &sp : spans) {
+      cudaEventDestroy(sp.ev[0]);
+      cudaEventDestroy(sp.ev[1]);
+    }
+    spans.clear();
+    open = false;
   }
 };
 

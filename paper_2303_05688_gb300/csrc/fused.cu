@@ -999,7 +999,7 @@ __global__ void __launch_bounds__(kAdThreads) k_emit_ad(EmitArgs A) {
 // alpha-double flag.
 __global__ void k_batch_counts(const uint64_t *items, uint64_t t0, uint64_t nt, int opbits,
                                uint32_t sa, uint32_t npieces, const uint32_t *grp_count,
-                               uint32_t *rcnt, uint32_t *adf) {
+                               uint32_t *rcnt, uint32_t *adf, uint32_t *adw) {
   const uint32_t omask = (1u << opbits) - 1u;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nt;
        i += (uint64_t)gridDim.x * blockDim.x) {
@@ -1007,13 +1007,36 @@ __global__ void k_batch_counts(const uint64_t *items, uint64_t t0, uint64_t nt, 
     const uint32_t k = lo >> opbits, o = lo & omask;
     rcnt[i] = o == 0 ? grp_count[k] * npieces : (o <= sa ? grp_count[k] : 0u);
     adf[i] = o > sa ? 1u : 0u;
+    adw[i] = o > sa ? grp_count[k] : 0u;
   }
+}
+
+// Totals of the batch plan's scans, for one copy to the host: staging slots,
+// bucket cells, tiles, runs, alpha-double items and their pairs.
+struct PlanTotals {
+  uint64_t slots, cells, tiles, runs, ad, ad_pairs;
+};
+__global__ void k_plan_totals(uint32_t ng, const uint64_t *soff, const uint64_t *slots,
+                              const uint32_t *cellbase, const uint32_t *nb,
+                              const uint32_t *tile_base, const uint32_t *ntile, uint64_t nt,
+                              const uint32_t *roff, const uint32_t *rcnt, const uint32_t *adpos,
+                              const uint32_t *adf, const uint32_t *adsum, const uint32_t *adw,
+                              PlanTotals *out) {
+  const uint32_t g = ng - 1;
+  const uint64_t i = nt - 1;
+  out->slots = soff[g] + slots[g];
+  out->cells = (uint64_t)cellbase[g] + nb[g];
+  out->tiles = (uint64_t)tile_base[g] + ntile[g];
+  out->runs = (uint64_t)roff[i] + rcnt[i];
+  out->ad = (uint64_t)adpos[i] + adf[i];
+  out->ad_pairs = (uint64_t)adsum[i] + adw[i];
 }
 
 __global__ void k_batch_lists(const uint64_t *items, uint64_t t0, uint64_t nt, int opbits,
                               uint32_t sa, const uint32_t *grp_count, const uint32_t *rcnt,
-                              const uint32_t *roff, const uint32_t *adpos, uint64_t *runs,
-                              uint32_t *adl, uint32_t *adw, const uint32_t *grp_alpha, int n,
+                              const uint32_t *roff, const uint32_t *adpos, const uint32_t *adsum,
+                              uint64_t *runs, uint32_t *adl, uint32_t *ad_off,
+                              const uint32_t *grp_alpha, int n,
                               FastDiv dv_va, uint32_t *opinfo) {
   const uint32_t omask = (1u << opbits) - 1u;
   const uint32_t full = n >= 32 ? 0xffffffffu : ((1u << n) - 1u);
@@ -1042,7 +1065,7 @@ __global__ void k_batch_lists(const uint64_t *items, uint64_t t0, uint64_t nt, i
         opinfo[i] = oi;
       } else {
         adl[adpos[i]] = (uint32_t)i;
-        adw[adpos[i]] = grp_count[k];
+        ad_off[adpos[i]] = adsum[i];
       }
     }
     for (uint32_t have = __ballot_sync(0xffffffffu, cnt != 0); have; have &= have - 1) {
@@ -1990,17 +2013,17 @@ inline unsigned grid_for(size_t n, unsigned cap = 152 * 16) {
 int kept_count(const uint32_t *keep, const uint32_t *pos, size_t n, size_t *host_count,
                Arena &arena);
 
-int build_fx(const double *h1, const double *eri, int n, int na, int nb, double ecore, double E0,
-             Arena &arena, FxInts *out, int64_t *E0_x) {
-  cudaStream_t s = arena.stream();
-  unsigned long long *dmax;
-  double h3[4];
-  ASCI_TRY(arena.alloc(&dmax, 4));
-  ASCI_TRY_CUDA(cudaMemsetAsync(dmax, 0, 4 * sizeof(unsigned long long), s));
-  k_fx_bounds<<<(unsigned)((n * n * 32 + 255) / 256), 256, 0, s>>>(h1, eri, n, dmax);
+// The four maxima that size the fixed-point grids (k_fx_bounds), to `out`
+// (zeroed by the caller).
+int fx_bounds(const double *h1, const double *eri, int n, unsigned long long *out, cudaStream_t s) {
+  k_fx_bounds<<<(unsigned)((n * n * 32 + 255) / 256), 256, 0, s>>>(h1, eri, n, out);
   ASCI_CHECK_LAUNCH();
-  ASCI_TRY_CUDA(cudaMemcpyAsync(h3, dmax, sizeof(h3), cudaMemcpyDefault, s));
-  ASCI_TRY_CUDA(cudaStreamSynchronize(s));
+  return ASCI_OK;
+}
+
+int build_fx(const double *h1, const double *eri, int n, int na, int nb, double ecore, double E0,
+             const double h3[4], Arena &arena, FxInts *out, int64_t *E0_x) {
+  cudaStream_t s = arena.stream();
   // B bounds |E0|, every diagonal element and every Fock-like diagonal value:
   // (na+nb) one-body terms, C(na,2)+C(nb,2) same-spin and na*nb opposite-spin
   // pair terms.  With s = 58 - log2(B) a sum of up to 32 such values cannot
@@ -2075,43 +2098,48 @@ int core_fock(const FxInts &X, const uint32_t *core_alpha, const uint32_t *core_
   return ASCI_OK;
 }
 
+namespace {
+__global__ void k_item_totals(const uint32_t *item_group, const uint64_t *Wexcl, uint64_t T,
+                              uint64_t *out) {
+  out[0] = item_group[T];
+  out[1] = Wexcl[T];
+}
+}  // namespace
+
 // Groups (distinct target alpha strings) of the sorted item list.  item_group
 // has T + 1 entries; the group tables have G + 1 rows (row G: T and P).
+// *P receives the total weight, read with the group count.
 int item_groups(const uint64_t *items, const uint64_t *Wexcl, uint64_t T, uint32_t *item_group,
-                uint32_t **g_alpha, uint64_t **g_P0, uint64_t **g_item0, size_t *G,
+                uint32_t **g_alpha, uint64_t **g_P0, uint64_t **g_item0, size_t *G, uint64_t *P,
                 Arena &arena) {
   cudaStream_t s = arena.stream();
   ASCI_TRY(scan_item_heads(items, T, item_group, arena));
-  uint32_t ng = 0;
-  ASCI_TRY_CUDA(cudaMemcpyAsync(&ng, item_group + T, 4, cudaMemcpyDefault, s));
+  uint64_t *d_tot, tot[2] = {0, 0};
+  ASCI_TRY(arena.alloc(&d_tot, 2));
+  k_item_totals<<<1, 1, 0, s>>>(item_group, Wexcl, T, d_tot);
+  ASCI_CHECK_LAUNCH();
+  ASCI_TRY_CUDA(cudaMemcpyAsync(tot, d_tot, sizeof(tot), cudaMemcpyDeviceToHost, s));
   ASCI_TRY_CUDA(cudaStreamSynchronize(s));
-  ASCI_TRY(arena.alloc(g_alpha, (size_t)ng + 1));
-  ASCI_TRY(arena.alloc(g_P0, (size_t)ng + 1));
-  ASCI_TRY(arena.alloc(g_item0, (size_t)ng + 1));
+  const size_t ng = (size_t)tot[0];
+  ASCI_TRY(arena.alloc(g_alpha, ng + 1));
+  ASCI_TRY(arena.alloc(g_P0, ng + 1));
+  ASCI_TRY(arena.alloc(g_item0, ng + 1));
   k_group_tab<<<grid_for(T), 256, 0, s>>>(items, item_group, Wexcl, T, *g_alpha, *g_P0, *g_item0);
   ASCI_CHECK_LAUNCH();
   *G = ng;
+  *P = tot[1];
   return ASCI_OK;
 }
 
 int psi_hash_build(const uint64_t *psi_keys, size_t nd, uint64_t **ht, uint64_t *mask,
-                   Arena &arena) {
+                   unsigned *err, Arena &arena) {
   uint64_t size = 1024;
   while (size < 4 * (uint64_t)nd) size <<= 1;
   ASCI_TRY(arena.alloc(ht, size));
   cudaStream_t s = arena.stream();
   ASCI_TRY_CUDA(cudaMemsetAsync(*ht, 0xff, size * sizeof(uint64_t), s));
-  unsigned *err, herr = 0;
-  ASCI_TRY(arena.alloc(&err, 1));
-  ASCI_TRY_CUDA(cudaMemsetAsync(err, 0, sizeof(unsigned), s));
   k_psi_insert<<<grid_for(nd), 256, 0, s>>>(psi_keys, nd, *ht, size - 1, err);
   ASCI_CHECK_LAUNCH();
-  ASCI_TRY_CUDA(cudaMemcpyAsync(&herr, err, sizeof(herr), cudaMemcpyDeviceToHost, s));
-  ASCI_TRY_CUDA(cudaStreamSynchronize(s));
-  if (herr) {
-    record_error("psi hash table full", __FILE__, __LINE__);
-    return ASCI_ECUDA;
-  }
   *mask = size - 1;
   return ASCI_OK;
 }
@@ -2175,70 +2203,67 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   ASCI_CHECK_LAUNCH();
   ASCI_TRACE("stage: classified %u groups", ng);
   ASCI_TRY(scan_exclusive_u64(slots, soff, ng, arena));
-  {
-    uint64_t last[2];
-    ASCI_TRY_CUDA(cudaMemcpyAsync(&last[0], soff + ng - 1, 8, cudaMemcpyDefault, s));
-    ASCI_TRY_CUDA(cudaMemcpyAsync(&last[1], slots + ng - 1, 8, cudaMemcpyDefault, s));
-    ASCI_TRY_CUDA(cudaStreamSynchronize(s));
-    if (last[0] + last[1] > st.cap) {
-      record_error("staging buffer too small for the batch's hash buckets (lower max_batch_pairs)",
-                   __FILE__, __LINE__);
-      return ASCI_ENOMEM;
-    }
-  }
   ASCI_TRY(scan_exclusive_u64(small_pairs, Ws, ng, arena));
   ASCI_TRY(scan_exclusive_u32(nb, cellbase, ng, arena));
-  size_t ncells = 0, ntiles = 0;
-  ASCI_TRY(kept_count(nb, cellbase, ng, &ncells, arena));
   k_tile_count<<<grid_for(ng), 256, 0, s>>>(ng, kind, nb, Ws, ntile);
   ASCI_CHECK_LAUNCH();
   ASCI_TRY(scan_exclusive_u32(ntile, tile_base, ng, arena));
-  ASCI_TRY(kept_count(ntile, tile_base, ng, &ntiles, arena));
+
+  // work lists of the batch: determinant runs and alpha-double items
+  const uint64_t nt = t1 - t0;
+  if (nt >= (1ull << 32)) return ASCI_EINVAL;
+  uint32_t *rcnt, *roff, *adf, *adpos, *adw, *adsum;
+  ASCI_TRY(arena.alloc(&rcnt, nt));
+  ASCI_TRY(arena.alloc(&roff, nt));
+  ASCI_TRY(arena.alloc(&adf, nt));
+  ASCI_TRY(arena.alloc(&adpos, nt));
+  ASCI_TRY(arena.alloc(&adw, nt));
+  ASCI_TRY(arena.alloc(&adsum, nt));
+  const uint32_t npieces =
+      (uint32_t)std::max<uint64_t>(1, ((uint64_t)F.E.sb + F.E.dbb + kPiecePairs - 1) / kPiecePairs);
+  k_batch_counts<<<grid_for(nt), 256, 0, s>>>(F.items, t0, nt, F.opbits, F.E.sa, npieces,
+                                              F.grp_count, rcnt, adf, adw);
+  ASCI_CHECK_LAUNCH();
+  ASCI_TRY(scan_exclusive_u32(rcnt, roff, nt, arena));
+  ASCI_TRY(scan_exclusive_u32(adf, adpos, nt, arena));
+  ASCI_TRY(scan_exclusive_u32(adw, adsum, nt, arena));
+  // every total the host needs, in one copy (one round trip for the plan)
+  PlanTotals *d_tot, tot{};
+  ASCI_TRY(arena.alloc(&d_tot, 1));
+  k_plan_totals<<<1, 1, 0, s>>>(ng, soff, slots, cellbase, nb, tile_base, ntile, nt, roff, rcnt,
+                                adpos, adf, adsum, adw, d_tot);
+  ASCI_CHECK_LAUNCH();
+  ASCI_TRY_CUDA(cudaMemcpyAsync(&tot, d_tot, sizeof(tot), cudaMemcpyDeviceToHost, s));
+  ASCI_TRY_CUDA(cudaStreamSynchronize(s));
+  if (tot.slots > st.cap) {
+    record_error("staging buffer too small for the batch's hash buckets (lower max_batch_pairs)",
+                 __FILE__, __LINE__);
+    return ASCI_ENOMEM;
+  }
+  const size_t ncells = tot.cells, ntiles = tot.tiles, nruns = tot.runs, nad = tot.ad,
+               ad_total = tot.ad_pairs;
   ASCI_TRACE("stage: cells=%zu tiles=%zu", ncells, ntiles);
   if (ncells > P1 - P0 || ntiles > P1 - P0) {
     record_error("inconsistent tile plan", __FILE__, __LINE__);
     return ASCI_ECUDA;
   }
-
-  // work lists of the batch: determinant runs and alpha-double items
-  const uint64_t nt = t1 - t0;
-  if (nt >= (1ull << 32)) return ASCI_EINVAL;
-  uint32_t *rcnt, *roff, *adf, *adpos;
-  ASCI_TRY(arena.alloc(&rcnt, nt));
-  ASCI_TRY(arena.alloc(&roff, nt));
-  ASCI_TRY(arena.alloc(&adf, nt));
-  ASCI_TRY(arena.alloc(&adpos, nt));
-  const uint32_t npieces =
-      (uint32_t)std::max<uint64_t>(1, ((uint64_t)F.E.sb + F.E.dbb + kPiecePairs - 1) / kPiecePairs);
-  k_batch_counts<<<grid_for(nt), 256, 0, s>>>(F.items, t0, nt, F.opbits, F.E.sa, npieces,
-                                              F.grp_count, rcnt, adf);
-  ASCI_CHECK_LAUNCH();
-  ASCI_TRY(scan_exclusive_u32(rcnt, roff, nt, arena));
-  ASCI_TRY(scan_exclusive_u32(adf, adpos, nt, arena));
-  size_t nruns = 0, nad = 0;
-  ASCI_TRY(kept_count(rcnt, roff, nt, &nruns, arena));
-  ASCI_TRY(kept_count(adf, adpos, nt, &nad, arena));
+  if (ad_total > P1 - P0) {
+    record_error("alpha-double pairs exceed the batch", __FILE__, __LINE__);
+    return ASCI_ECUDA;
+  }
   uint64_t *runs;
-  uint32_t *adl, *adw, *ad_off, *opinfo;
+  uint32_t *adl, *ad_off, *opinfo;
   ASCI_TRY(arena.alloc(&opinfo, nt));
   ASCI_TRY(arena.alloc(&runs, nruns + 1));
   ASCI_TRY(arena.alloc(&adl, nad + 1));
-  ASCI_TRY(arena.alloc(&adw, nad + 1));
   ASCI_TRY(arena.alloc(&ad_off, nad + 1));
   k_batch_lists<<<grid_for(nt), 256, 0, s>>>(F.items, t0, nt, F.opbits, F.E.sa, F.grp_count, rcnt,
-                                             roff, adpos, runs, adl, adw, F.grp_alpha, F.X.n,
-                                             FastDiv(F.E.va ? F.E.va : 1), opinfo);
+                                             roff, adpos, adsum, runs, adl, ad_off, F.grp_alpha,
+                                             F.X.n, FastDiv(F.E.va ? F.E.va : 1), opinfo);
   ASCI_CHECK_LAUNCH();
-  size_t ad_total = 0;
   uint32_t ad_tiles = 0;
   uint32_t *ad_tile_item = nullptr;
   if (nad) {
-    ASCI_TRY(scan_exclusive_u32(adw, ad_off, nad, arena));
-    ASCI_TRY(kept_count(adw, ad_off, nad, &ad_total, arena));
-    if (ad_total > P1 - P0) {
-      record_error("alpha-double pairs exceed the batch", __FILE__, __LINE__);
-      return ASCI_ECUDA;
-    }
     ad_tiles = (uint32_t)((ad_total + kAdTile - 1) / kAdTile);
     ASCI_TRY(arena.alloc(&ad_tile_item, (size_t)ad_tiles + 1));
     k_ad_tile_items<<<grid_for((size_t)ad_tiles + 1), 256, 0, s>>>(

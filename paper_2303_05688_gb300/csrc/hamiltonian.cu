@@ -1903,6 +1903,7 @@ static int loop_impl(const asci_det *dets_in, const double *coeffs_in, size_t nd
     double *nc = buf_c[which];
     ASCI_TRY(davidson(H, diag, sel_v, o.davidson, nc, &dr, sa));
     tm.stop(&t_dav);
+    tm.read();
     if (!dr.converged) {
       record_error("Davidson did not converge within max_iter", __FILE__, __LINE__);
       return ASCI_ETIMEOUT;

@@ -40,15 +40,16 @@ int compact_f64(const double *in, const uint32_t *keep, const uint32_t *pos, siz
 int kept_count(const uint32_t *keep, const uint32_t *pos, size_t n, size_t *host_count,
                Arena &arena);
 
+int fx_bounds(const double *h1, const double *eri, int n, unsigned long long *out, cudaStream_t s);
 int build_fx(const double *h1, const double *eri, int n, int na, int nb, double ecore, double E0,
-             Arena &arena, FxInts *out, int64_t *E0_x);
+             const double h3[4], Arena &arena, FxInts *out, int64_t *E0_x);
 int core_fock(const FxInts &X, const uint32_t *core_alpha, const uint32_t *core_beta, size_t m,
               int64_t *Dx, int64_t *Fa, int64_t *Fb, Arena &arena);
 int item_groups(const uint64_t *items, const uint64_t *Wexcl, uint64_t T, uint32_t *item_group,
-                uint32_t **g_alpha, uint64_t **g_P0, uint64_t **g_item0, size_t *G,
+                uint32_t **g_alpha, uint64_t **g_P0, uint64_t **g_item0, size_t *G, uint64_t *P,
                 Arena &arena);
 int psi_hash_build(const uint64_t *psi_keys, size_t nd, uint64_t **ht, uint64_t *mask,
-                   Arena &arena);
+                   unsigned *err, Arena &arena);
 int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint64_t P1,
                 uint32_t gb0, uint32_t gb1, const Stage &st, double eps,
                 unsigned long long *survivors, unsigned *err,
@@ -127,10 +128,15 @@ enum : uint32_t {
   kDuplicate = 8u,    // repeated determinant
 };
 
+// na = -2: the electron counts are those of the first determinant; -1: unchecked.
 __global__ void k_prepare_psi(const asci_det *dets, const double *c, size_t nd, int norb, int na,
                               int nb, uint64_t *keys, uint64_t *keys2, unsigned *err) {
   const uint64_t hi = ~((1ull << norb) - 1ull);  // norb <= 32
   unsigned e = 0;
+  if (na == -2) {
+    na = __popcll(dets[0].alpha);
+    nb = __popcll(dets[0].beta);
+  }
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nd;
        i += (size_t)gridDim.x * blockDim.x) {
     asci_det d = dets[i];
@@ -241,6 +247,19 @@ __global__ void k_class_list(const uint32_t *head, const uint32_t *pos, uint64_t
     }
 }
 
+// What the host needs from the preparation, in one copy.
+struct PrepTotals {
+  double bounds[4];  // k_fx_bounds, written in place
+  asci_det d0;
+  uint64_t groups;
+  unsigned err;
+};
+__global__ void k_prep_totals(const asci_det *dets, const uint32_t *gid, const uint32_t *head,
+                              size_t m, PrepTotals *out) {
+  out->d0 = dets[0];
+  out->groups = (uint64_t)gid[m - 1] + head[m - 1];
+}
+
 __global__ void k_unpack(const uint64_t *keys, size_t n, asci_det *out) {
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (size_t)gridDim.x * blockDim.x) {
@@ -321,7 +340,12 @@ int shard_items(uint64_t **items, uint64_t **items_alt, const uint64_t *Wexcl, u
   uint64_t *g_P0, *g_item0;
   size_t G = 0;
   ASCI_TRY(sa.alloc(&item_group, T + 1));
-  ASCI_TRY(item_groups(*items, Wexcl, T, item_group, &g_alpha, &g_P0, &g_item0, &G, sa));
+  uint64_t total = 0;
+  ASCI_TRY(item_groups(*items, Wexcl, T, item_group, &g_alpha, &g_P0, &g_item0, &G, &total, sa));
+  if (total != P) {
+    record_error("pair count does not match the closed form", __FILE__, __LINE__);
+    return ASCI_ECUDA;
+  }
   const uint64_t heavy = std::max<uint64_t>(1, P / (64ull * (uint64_t)W));
   const uint32_t heavy_cap = (uint32_t)std::min<uint64_t>(G, 64ull * W + 1);
   int32_t *shard;
@@ -394,7 +418,8 @@ int bits_for(uint32_t v) {
 }
 
 struct Batch {
-  uint64_t t0, t1, P0, P1;
+  uint64_t t0, t1, P0, P1;  // items and pairs
+  uint64_t g0, g1;          // target groups
 };
 
 // Cut items [0, T) into batches of at most bmax pairs at class boundaries
@@ -466,15 +491,16 @@ class Planner {
     cur_open_ = false;
   }
 
-  void add(uint64_t cs, uint64_t ce, uint64_t ws, uint64_t we) {
+  void add(uint64_t cs, uint64_t ce, uint64_t ws, uint64_t we, uint64_t gs, uint64_t ge) {
     const uint64_t cap = batches_.empty() ? first_cap_ : bmax_;
     if (cur_open_ && (we - cur_.P0) > cap) flush();
     if (!cur_open_) {
-      cur_ = Batch{cs, ce, ws, we};
+      cur_ = Batch{cs, ce, ws, we, gs, ge};
       cur_open_ = true;
     } else {
       cur_.t1 = ce;
       cur_.P1 = we;
+      cur_.g1 = ge;
     }
   }
 
@@ -492,7 +518,7 @@ class Planner {
         flush();
         ASCI_TRY(visit(g0, g1, i1, w1, L + 1));
       } else {
-        add(i0, i1, w0, w1);
+        add(i0, i1, w0, w1, g0, g1);
       }
     }
     return ASCI_OK;
@@ -558,6 +584,11 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   double tl[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // per-stage device milliseconds
   uint64_t tile_launches = 0, staged_records = 0, oversized_records = 0, big_records = 0;
   StageTimer tm(stream), total_tm(stream), ktm(stream);
+  auto read_timers = [&]() {
+    tm.read();
+    ktm.read();
+    total_tm.read();
+  };
   total_tm.start();
   tm.start();
   const int n = ints->norb;
@@ -569,21 +600,16 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   ASCI_TRY(to_device(ints->eri, (size_t)n * n * n * n, &eri, arena));
 
   ASCI_TRACE("search: ndets=%zu norb=%d C=%zu N=%zu eps=%g", nd, n, C, N, o.eps_search);
-  // electron counts from the first determinant
-  asci_det d0;
-  ASCI_TRY_CUDA(cudaMemcpyAsync(&d0, dets, sizeof(d0), cudaMemcpyDefault, stream));
-  ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
-  const int na = __builtin_popcountll(d0.alpha), nb = __builtin_popcountll(d0.beta);
-  if (na > n || nb > n) return ASCI_EINVAL;
-
-  unsigned *derr;
-  ASCI_TRY(arena.alloc(&derr, 1));
-  ASCI_TRY_CUDA(cudaMemsetAsync(derr, 0, sizeof(unsigned), stream));
+  PrepTotals *prep, hp{};
+  ASCI_TRY(arena.alloc(&prep, 1));
+  ASCI_TRY_CUDA(cudaMemsetAsync(prep, 0, sizeof(PrepTotals), stream));
+  unsigned *derr = &prep->err;
+  ASCI_TRY(fx_bounds(h1, eri, n, reinterpret_cast<unsigned long long *>(prep->bounds), stream));
   uint64_t *pkeys, *pkeys_alt, *in_keys;
   ASCI_TRY(arena.alloc(&pkeys, nd));
   ASCI_TRY(arena.alloc(&pkeys_alt, nd));
   ASCI_TRY(arena.alloc(&in_keys, nd));
-  k_prepare_psi<<<grid_for(nd), 256, 0, stream>>>(dets, coeffs, nd, n, na, nb, in_keys, pkeys, derr);
+  k_prepare_psi<<<grid_for(nd), 256, 0, stream>>>(dets, coeffs, nd, n, -2, -2, in_keys, pkeys, derr);
   ASCI_CHECK_LAUNCH();
   k_check_finite<<<grid_for((size_t)n * n * n * n), 256, 0, stream>>>(eri, (size_t)n * n * n * n,
                                                                        derr);
@@ -630,12 +656,14 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   k_group_heads<<<grid_for(m), 256, 0, stream>>>(alpha_k, m, ghead, core_alpha, core_beta);
   ASCI_CHECK_LAUNCH();
   ASCI_TRY(scan_exclusive_u32(ghead, gid, m, arena));
-  unsigned herr = 0;
-  uint32_t lastg[2];
-  ASCI_TRY_CUDA(cudaMemcpyAsync(&herr, derr, sizeof(herr), cudaMemcpyDefault, stream));
-  ASCI_TRY_CUDA(cudaMemcpyAsync(&lastg[0], gid + m - 1, 4, cudaMemcpyDefault, stream));
-  ASCI_TRY_CUDA(cudaMemcpyAsync(&lastg[1], ghead + m - 1, 4, cudaMemcpyDefault, stream));
+  k_prep_totals<<<1, 1, 0, stream>>>(dets, gid, ghead, m, prep);
+  ASCI_CHECK_LAUNCH();
+  ASCI_TRY_CUDA(cudaMemcpyAsync(&hp, prep, sizeof(hp), cudaMemcpyDeviceToHost, stream));
   ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
+  // electron counts from the first determinant
+  const unsigned herr = hp.err;
+  const int na = __builtin_popcountll(hp.d0.alpha), nb = __builtin_popcountll(hp.d0.beta);
+  if (na > n || nb > n) return ASCI_EINVAL;
   if (herr) {
     record_error(herr & kDuplicate   ? "duplicate determinants in psi"
                  : herr & kBadCount  ? "determinants with different electron counts"
@@ -644,7 +672,7 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
                  __FILE__, __LINE__);
     return ASCI_EINVAL;
   }
-  const size_t ngroups = (size_t)lastg[0] + lastg[1];
+  const size_t ngroups = (size_t)hp.groups;
   uint32_t *grp_alpha, *grp_start, *grp_count;
   ASCI_TRY(arena.alloc(&grp_alpha, ngroups));
   ASCI_TRY(arena.alloc(&grp_start, ngroups));
@@ -698,12 +726,7 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
     ASCI_TRY(radix_sort_u64_varying(&items, &items_alt, T, 32, 32 + n, used_alpha, arena));
     ASCI_TRY(arena.alloc(&Wexcl, T + 1));
     ASCI_TRY(scan_item_weights(items, T, opbits, grp_count, X, Wexcl, arena));
-    ASCI_TRY_CUDA(cudaMemcpyAsync(&P, Wexcl + T, 8, cudaMemcpyDefault, stream));
-    ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
-    if (P != (uint64_t)m * X.total) {
-      record_error("pair count does not match the closed form", __FILE__, __LINE__);
-      return ASCI_ECUDA;
-    }
+    P = (uint64_t)m * X.total;  // compared with the scan's total below
     if (W > 1) {  // this shard's classes only
       uint64_t T1 = 0;
       ASCI_TRY(shard_items(&items, &items_alt, Wexcl, T, P, o.shard_index, W, &T1, arena));
@@ -711,11 +734,7 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
                  (unsigned long long)T1, (unsigned long long)T);
       T = T1;
       P = 0;
-      if (T) {
-        ASCI_TRY(scan_item_weights(items, T, opbits, grp_count, X, Wexcl, arena));
-        ASCI_TRY_CUDA(cudaMemcpyAsync(&P, Wexcl + T, 8, cudaMemcpyDefault, stream));
-        ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
-      }
+      if (T) ASCI_TRY(scan_item_weights(items, T, opbits, grp_count, X, Wexcl, arena));
     }
   }
   // the distinct target alpha strings (groups) of the items
@@ -725,7 +744,13 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   size_t G = 0;
   if (T > 0) {
     ASCI_TRY(arena.alloc(&item_group, T + 1));
-    ASCI_TRY(item_groups(items, Wexcl, T, item_group, &g_alpha, &g_P0, &g_item0, &G, arena));
+    uint64_t total = 0;
+    ASCI_TRY(item_groups(items, Wexcl, T, item_group, &g_alpha, &g_P0, &g_item0, &G, &total, arena));
+    if (W > 1) P = total;
+    if (P != total) {
+      record_error("pair count does not match the closed form", __FILE__, __LINE__);
+      return ASCI_ECUDA;
+    }
   }
   if (cq) {  // the classes of one level, in constraint order, and their pairs
     cq->n = 0;
@@ -744,7 +769,9 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   }
   if (T > 0 && P > 0) {
     uint64_t bmax = o.max_batch_pairs;
-    if (bmax == 0) {
+    if (bmax == 0 && P <= (1ull << 20)) {
+      bmax = 1ull << 20;  // the least that free memory would allow
+    } else if (bmax == 0) {
       size_t fr = 0, tot = 0;
       ASCI_TRY_CUDA(cudaMemGetInfo(&fr, &tot));
       bmax = (uint64_t)(fr / 2) / 40;  // staging: 1.5 slots of 20 bytes per pair
@@ -755,8 +782,13 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
     const int L0 = std::min(3, lmax);
     // a small first batch fixes the selection threshold early
     const uint64_t first_cap = std::min<uint64_t>(bmax, std::max<uint64_t>(1ull << 22, P / 64));
-    Planner planner(g_alpha, g_item0, g_P0, G, bmax, first_cap, lmax, arena);
-    ASCI_TRY(planner.run(T, P, L0, &batches, &max_level));
+    if (P <= first_cap) {  // one batch, whatever its classes
+      batches.push_back(Batch{0, T, 0, P, 0, G});
+      max_level = L0;
+    } else {
+      Planner planner(g_alpha, g_item0, g_P0, G, bmax, first_cap, lmax, arena);
+      ASCI_TRY(planner.run(T, P, L0, &batches, &max_level));
+    }
   }
   uint64_t bcap = 0;
   for (auto &b : batches) bcap = std::max(bcap, b.P1 - b.P0);
@@ -791,7 +823,12 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   F.core_c = core_c_sorted;
   uint64_t *psi_ht = nullptr;
   uint64_t psi_mask = 0;
-  ASCI_TRY(psi_hash_build(psi_sorted, nd, &psi_ht, &psi_mask, arena));
+  // [0] candidates, [1] unique, [2] excluded, [3] survivors, [4] error bits: one copy reads them
+  unsigned long long *dcount = nullptr;
+  ASCI_TRY(arena.alloc(&dcount, 5));
+  ASCI_TRY_CUDA(cudaMemsetAsync(dcount, 0, 5 * sizeof(unsigned long long), stream));
+  unsigned *derr2 = reinterpret_cast<unsigned *>(dcount + 4);
+  ASCI_TRY(psi_hash_build(psi_sorted, nd, &psi_ht, &psi_mask, derr2, arena));
   F.psi_ht = psi_ht;
   F.psi_keys = psi_sorted;
   F.npsi = nd;
@@ -800,7 +837,7 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   F.prec = o.precision == ASCI_FP32_INT_COMP_ACC ? 2 : (o.precision == ASCI_FP32_INT_FP64_ACC ? 1 : 0);
   F.screened = o.eps_search > 0.0 ? 1 : 0;
   F.ctas_per_sm = o.ctas_per_sm;
-  ASCI_TRY(build_fx(h1, eri, n, na, nb, ints->ecore, E0, arena, &F.X, &F.E0_x));
+  ASCI_TRY(build_fx(h1, eri, n, na, nb, ints->ecore, E0, hp.bounds, arena, &F.X, &F.E0_x));
   if (st) st->diag_grid_bits = (uint64_t)F.X.s;
   {
     int64_t *Dx, *Fa, *Fb;
@@ -830,8 +867,6 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   Stage stg = {nullptr, nullptr, scap};
   uint64_t *pool_k[2] = {nullptr, nullptr};
   double *pool_s[2] = {nullptr, nullptr};
-  unsigned long long *dcount = nullptr;  // [0] candidates, [1] unique, [2] excluded, [3] survivors
-  unsigned *derr2 = nullptr;
   if (bcap) {
     ASCI_TRY(arena.alloc(&stg.rec, scap));
     ASCI_TRY(arena.alloc(&stg.alpha, scap));
@@ -839,10 +874,6 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
       ASCI_TRY(arena.alloc(&pool_k[i], pool_cap));
       ASCI_TRY(arena.alloc(&pool_s[i], pool_cap));
     }
-    ASCI_TRY(arena.alloc(&dcount, 4));
-    ASCI_TRY(arena.alloc(&derr2, 1));
-    ASCI_TRY_CUDA(cudaMemsetAsync(dcount, 0, 4 * sizeof(unsigned long long), stream));
-    ASCI_TRY_CUDA(cudaMemsetAsync(derr2, 0, sizeof(unsigned), stream));
   }
   size_t pool_n = 0;
   int pcur = 0;
@@ -860,7 +891,6 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
                          pt2_limbs, derr2, stream));
       const unsigned long long keep = pool_n;
       ASCI_TRY_CUDA(cudaMemcpyAsync(dcount, &keep, sizeof(keep), cudaMemcpyHostToDevice, stream));
-      ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
       return ASCI_OK;
     }
     ASCI_TRY(exact_scores(F, pool_k[pcur] + pool_n, pool_s[pcur] + pool_n, (size_t)c - pool_n,
@@ -878,30 +908,28 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
     pcur ^= 1;
     pool_n = m2;
     if (m2 >= N && N > 0) tau = least;
-    unsigned long long c = pool_n;
-    ASCI_TRY_CUDA(cudaMemcpyAsync(dcount, &c, sizeof(c), cudaMemcpyDefault, stream));
-    ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
+    const unsigned long long c = pool_n;
+    ASCI_TRY_CUDA(cudaMemcpyAsync(dcount, &c, sizeof(c), cudaMemcpyHostToDevice, stream));
     return ASCI_OK;
   };
   // The counters before a tile launch: when its values found no room (rare: a
   // low threshold over crowded targets), they are put back and the launch, and
   // those after it, run with room for every record, fewer tiles at a time.
-  unsigned long long hcount[3] = {0, 0, 0};
+  unsigned long long hcount[4] = {0, 0, 0, 0};
   bool values_full = false;
   auto read_counts = [&](bool full, const char *what, bool *again) -> int {
-    unsigned long long c[3];
-    unsigned he = 0;
+    unsigned long long c[5];
     *again = false;
-    ASCI_TRY_CUDA(cudaMemcpyAsync(c, dcount, sizeof(c), cudaMemcpyDefault, stream));
-    ASCI_TRY_CUDA(cudaMemcpyAsync(&he, derr2, sizeof(he), cudaMemcpyDefault, stream));
+    ASCI_TRY_CUDA(cudaMemcpyAsync(c, dcount, sizeof(c), cudaMemcpyDeviceToHost, stream));
     ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
+    const unsigned he = (unsigned)c[4];
     if (he == kErrValues && !full) {
       ASCI_TRACE("%s: values found no room; again with room for all", what);
       values_full = *again = true;
       hcount[0] = pool_n;
       ASCI_TRY_CUDA(cudaMemsetAsync(derr2, 0, sizeof(unsigned), stream));
-      ASCI_TRY_CUDA(cudaMemcpyAsync(dcount, hcount, sizeof(hcount), cudaMemcpyDefault, stream));
-      ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
+      ASCI_TRY_CUDA(cudaMemcpyAsync(dcount, hcount, 3 * sizeof(hcount[0]), cudaMemcpyHostToDevice,
+                                    stream));
       return ASCI_OK;
     }
     if (he) {
@@ -911,15 +939,12 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
       return ASCI_ECUDA;
     }
     if (c[0] > pool_cap) return ASCI_ECUDA;  // cannot happen: room bounds the appends
-    for (int i = 0; i < 3; ++i) hcount[i] = c[i];
+    for (int i = 0; i < 4; ++i) hcount[i] = c[i];
     return ASCI_OK;
   };
   for (const Batch &b : batches) {
     Arena ba(stream);  // scratch of this batch, released when the batch ends
-    uint32_t gg[2];
-    ASCI_TRY_CUDA(cudaMemcpyAsync(&gg[0], item_group + b.t0, 4, cudaMemcpyDefault, stream));
-    ASCI_TRY_CUDA(cudaMemcpyAsync(&gg[1], item_group + b.t1 - 1, 4, cudaMemcpyDefault, stream));
-    ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
+    const uint32_t gg[2] = {(uint32_t)b.g0, (uint32_t)b.g1 - 1u};
     tm.start();
     void *tiles = nullptr;
     size_t ntiles = 0;
@@ -1033,7 +1058,7 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
       }
     }
     tm.stop(&tl[5]);
-    if (pool_n > N) {  // tighten tau before the next batch
+    if (pool_n > N && &b != &batches.back()) {  // tighten tau before the next batch
       tm.start();
       ASCI_TRY(prune(ba));
       tm.stop(&tl[6]);
@@ -1041,12 +1066,9 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   }
   uint64_t unique = 0, excluded = 0, surviving = P;
   if (bcap) {
-    unsigned long long hc[4];
-    ASCI_TRY_CUDA(cudaMemcpyAsync(hc, dcount, sizeof(hc), cudaMemcpyDefault, stream));
-    ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
-    unique = hc[1];
-    excluded = hc[2];
-    if (o.eps_search > 0.0) surviving = hc[3];
+    unique = hcount[1];
+    excluded = hcount[2];
+    if (o.eps_search > 0.0) surviving = hcount[3];
   }
   if (pt2_out) {
     double v = 0.0;
@@ -1073,6 +1095,7 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
       st->selected = 0;
     }
     total_tm.stop(&tl[7]);
+    read_timers();
     if (st) {
       memcpy(st->t_stage, tl, sizeof(tl));
       st->tile_launches = tile_launches;
@@ -1130,6 +1153,7 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   (void)g_item0;
   (void)G;
   total_tm.stop(&tl[7]);
+  read_timers();
   if (st) {
     memcpy(st->t_stage, tl, sizeof(tl));
     st->tile_launches = tile_launches;
