@@ -197,20 +197,42 @@ __device__ __forceinline__ int64_t fx_diag(const FxInts &X, uint32_t A, uint32_t
 
 namespace {
 
+// The staged denominator only serves screens (|v| against tau |E0 - H_ii|), so
+// without the eps screen, which tests it exactly, it is summed in 32-bit fixed
+// point: multiples of 2^29 units of the 64-bit grid (|E0 - H_ii| < 2^59 of
+// those), each term rounded to nearest, and stored as a lower bound of the
+// magnitude: a sum of at most 15 such terms is within 8 units.  Half the
+// registers, shuffles, table bytes and additions of 64 bits.
+constexpr int kDenShift = 29;
+constexpr int32_t kDenSlack = 8;
+template <bool EPS>
+struct DenType {
+  using T = uint32_t;  // two's complement; sums may wrap on the way
+};
+template <>
+struct DenType<true> {
+  using T = int64_t;
+};
+template <typename T>
+__host__ __device__ __forceinline__ T den_round(int64_t x) {
+  return sizeof(T) == 8 ? (T)x : (T)((x + (1ll << (kDenShift - 1))) >> kDenShift);
+}
+
 // Parent data of each core det (alpha-sorted order): H_jj and both Fock-like
 // diagonals.  Fb is determinant-major (Fb[j n + p]: a warp's lanes read one
 // determinant's row); Fa is orbital-major (Fa[p m + j]: the lanes of an
 // alpha-double step read one orbital of consecutive determinants).
 // A thread per (orbital, determinant), determinants fastest; the thread of
-// orbital n forms H_jj.
+// orbital n forms H_jj.  D is the emission's diagonal type (den_round).
+template <typename D>
 __global__ void k_core_fock(FxInts X, const uint32_t *core_alpha, const uint32_t *core_beta,
-                            size_t m, int64_t *Dx, int64_t *Fa, int64_t *Fb) {
+                            size_t m, D *Dx, D *Fa, D *Fb) {
   const int n = X.n, p = (int)blockIdx.y;
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < m;
        j += (size_t)gridDim.x * blockDim.x) {
     const uint32_t A = core_alpha[j], B = core_beta[j];
     if (p == n) {
-      Dx[j] = fx_diag(X, A, B);
+      Dx[j] = den_round<D>(fx_diag(X, A, B));
       continue;
     }
     int64_t fa = X.hh[p], fb = X.hh[p];
@@ -224,8 +246,15 @@ __global__ void k_core_fock(FxInts X, const uint32_t *core_alpha, const uint32_t
       fb += X.jk[p * n + q];
       fa += X.jj[p * n + q];
     }
-    Fa[(size_t)p * m + j] = fa;
-    Fb[j * n + p] = fb;
+    Fa[(size_t)p * m + j] = den_round<D>(fa);
+    Fb[j * n + p] = den_round<D>(fb);
+  }
+}
+
+__global__ void k_den_tables(FxInts X, uint32_t *jk, uint32_t *jj) {
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < X.n * X.n; t += gridDim.x * blockDim.x) {
+    jk[t] = den_round<uint32_t>(X.jk[t]);
+    jj[t] = den_round<uint32_t>(X.jj[t]);
   }
 }
 
@@ -482,7 +511,7 @@ struct EmitArgs {
   DevInts I;
   FxInts X;
   ExcCounts E;
-  FastDiv dv_va, dv_vb, dv_pa_p, dv_pb_p;
+  FastDiv dv_vb, dv_pb_p, dv_pieces;
   uint32_t npd0, npd1;        // pairs per determinant for o = 0 and for an alpha single
   uint32_t npieces;           // pieces of kPiecePairs pairs a determinant's o = 0 run is cut into
   const uint64_t *items, *Wexcl;
@@ -491,7 +520,9 @@ struct EmitArgs {
   int opbits;
   const uint32_t *grp_alpha, *grp_start, *grp_count, *core_beta;
   const double *core_c;
-  const int64_t *Dx, *Fa, *Fb;
+  // H_jj and the Fock-like diagonals of the core, and jk and jj, in the type of
+  // the emission's diagonal (DenType): 64 bits with the eps screen, else 32
+  const void *Dx, *Fa, *Fb, *jk, *jj;
   uint32_t gb0;
   const uint32_t *kind, *nb, *cellbase;
   const uint64_t *soff;       // first staging slot of each class of the batch
@@ -508,7 +539,6 @@ struct EmitArgs {
   const uint32_t *adl;        // alpha-double items (item - t0)
   const uint32_t *ad_off;     // first flat pair of each (exclusive prefix)
   uint32_t nad, ad_total;
-  const uint32_t *opinfo;     // per batch item: alpha single i | a << 5 | parity << 10
   const uint32_t *ad_tile_item;  // first alpha-double item of each CTA step
   uint32_t ad_tiles;
   Stage st;
@@ -516,34 +546,31 @@ struct EmitArgs {
   float eps_f;                // eps as a float (the screen's float pre-test)
   int64_t E0_x;
   double inv_scale;
+  int32_t E0_32;
+  float scale32;              // a unit of the 32-bit diagonal
   unsigned long long *survivors;
   uint32_t ncore;
   unsigned *err;
 };
 
-__device__ __forceinline__ void dec_single(uint32_t s, uint32_t virt, uint32_t idx,
-                                           const FastDiv &dv, int *i, int *a) {
-  uint32_t q = dv.div(idx);
-  *i = nth_set_bit(s, (int)q);
-  *a = nth_set_bit(virt, (int)(idx - q * dv.d));
+// An excitation from the two strings: its holes and particles are the bits in
+// which they differ.  Parities: with n(x) the occupied orbitals of s below x, a
+// single i -> a crosses n(a) + n(i) + [a > i] (mod 2) of them, and a double i <
+// j -> a < b, taken as i -> a then j -> b, n(a) + n(b) + n(i) + n(j) + 1 plus the
+// particles between i and j.
+__device__ __forceinline__ uint32_t below(int x) { return (1u << x) - 1u; }
+
+__device__ __forceinline__ uint32_t single_orbitals(uint32_t s, uint32_t t, int *i, int *a) {
+  *i = __ffs(s & ~t) - 1;
+  *a = __ffs(t & ~s) - 1;
+  return (uint32_t)__popc(s & (below(*i) ^ below(*a))) + (*a > *i ? 1u : 0u);
 }
 
-__device__ __forceinline__ void dec_double(uint32_t s, uint32_t virt, uint32_t idx,
-                                           const FastDiv &dv, int *i, int *j, int *a, int *b) {
-  uint32_t q = dv.div(idx);
-  int h1, h2, p1, p2;
-  unrank_pair(q, &h1, &h2);
-  unrank_pair(idx - q * dv.d, &p1, &p2);
-  *i = nth_set_bit(s, h1);
-  *j = nth_set_bit(s, h2);
-  *a = nth_set_bit(virt, p1);
-  *b = nth_set_bit(virt, p2);
-}
-
-__device__ __forceinline__ int par_double(uint32_t s, int i, int j, int a, int b) {
-  int p1 = single_parity(s, i, a);
-  uint32_t s1 = s ^ (1u << i) ^ (1u << a);
-  return p1 ^ single_parity(s1, j, b);
+// Parity (bit 0) of the double from the holes i < j and the particle mask pm.
+__device__ __forceinline__ uint32_t double_sign(uint32_t s, int i, int j, int a, int b) {
+  const uint32_t m = below(i) ^ below(j) ^ below(a) ^ below(b);
+  const uint32_t between = below(j) & ~((2u << i) - 1u);
+  return (uint32_t)__popc(s & m) + (uint32_t)__popc(((1u << a) | (1u << b)) & between) + 1u;
 }
 
 // Single excitation i -> a of the string s (the other spin's string o) in
@@ -558,10 +585,6 @@ __device__ __forceinline__ int64_t fx_single(const FxInts &X, uint32_t s, uint32
   for (uint32_t m = s; m; m &= m - 1) v += ss[__ffs(m) - 1];
   for (uint32_t m = o; m; m &= m - 1) v += so[__ffs(m) - 1];
   return v;
-}
-
-__device__ __forceinline__ int64_t shfl64(int64_t x, int src) {
-  return (int64_t)__shfl_sync(0xffffffffu, (long long)x, src);
 }
 
 // A float widened to a double exactly, by operations on the bits (a widening
@@ -615,11 +638,13 @@ __device__ __forceinline__ float abs_as_float(double x, bool *ok) {
   return __uint_as_float(((uint32_t)e << 23) | (uint32_t)((b >> 29) & 0x7fffffu));
 }
 
+// den = E0 - H_ii in the emission's diagonal type.
 template <bool EPS>
 __device__ __forceinline__ void write_record(const EmitArgs &A, uint32_t pos, bool spill,
                                              uint32_t cell, uint32_t talpha, uint32_t tb,
-                                             bool packed, double v, int64_t haa, bool *kept) {
-  const float df = scaled_as_float(A.E0_x - haa, A.X.s);
+                                             bool packed, double v,
+                                             typename DenType<EPS>::T den, bool *kept) {
+  float df;
   if (EPS) {
     // Alg. 2's screen |v / (E0 - H_ii)| > eps, without a division.  A float
     // test settles every pair that is not within 4e-6 relative of the
@@ -627,6 +652,7 @@ __device__ __forceinline__ void write_record(const EmitArgs &A, uint32_t pos, bo
     // below their values, eps_f within 2^-24 of eps, the product within
     // 2^-24); the rest take the FP64 test, so every decision is the FP64
     // test's.  (FP64 instructions are scarce on this GPU.)
+    df = scaled_as_float((int64_t)den, A.X.s);
     bool okv;
     const float vf = abs_as_float(v, &okv);
     const float t = A.eps_f * fabsf(df);
@@ -636,11 +662,14 @@ __device__ __forceinline__ void write_record(const EmitArgs &A, uint32_t pos, bo
     } else if (okv && t > 1e-37f && t < 1e37f && vf < t * 0.999996f) {
       keep = false;
     } else {
-      const double den = __ll2double_rn(A.E0_x - haa) * A.inv_scale;
-      keep = fabs(v) > A.eps * fabs(den);
+      const double d = __ll2double_rn((int64_t)den) * A.inv_scale;
+      keep = fabs(v) > A.eps * fabs(d);
     }
     if (!keep) v = drop_marker();
     *kept = keep;
+  } else {
+    const int32_t a = abs((int32_t)den) - kDenSlack;  // |den| < 2^30
+    df = (float)(a > 0 ? a : 0) * A.scale32;
   }
   const uint64_t vb = (uint64_t)__double_as_longlong(v);
   const uint4 r = make_uint4((uint32_t)vb, (uint32_t)(vb >> 32), tb, __float_as_uint(df));
@@ -657,6 +686,20 @@ __device__ __forceinline__ void write_record(const EmitArgs &A, uint32_t pos, bo
   }
 }
 
+// Next free slot of the lane's bucket cell (lanes with `big`): the slot number
+// within the cell.  Lanes of one cell share an atomic when the class has few
+// buckets; with many, two lanes seldom meet and each takes its own.
+__device__ __forceinline__ uint32_t claim_slot(uint32_t *fill, uint32_t cell, bool big, bool few) {
+  if (!few) return big ? atomicAdd(&fill[cell], 1u) : 0u;
+  const int lane = threadIdx.x & 31;
+  const uint32_t peers = __match_any_sync(0xffffffffu, big ? cell : 0xffffffffu);
+  const int leader = __ffs(peers) - 1;
+  uint32_t base = 0;
+  if (big && lane == leader) base = atomicAdd(&fill[cell], (uint32_t)__popc(peers));
+  base = __shfl_sync(0xffffffffu, base, leader);
+  return base + __popc(peers & ((1u << lane) - 1u));
+}
+
 // The pairs an emission thread kept under the eps screen, added to the
 // search's counter once per warp when the kernel ends (one counter for the
 // whole grid: an atomic per chunk would serialise on it).
@@ -665,31 +708,63 @@ __device__ __forceinline__ void add_survivors(const EmitArgs &A, unsigned long l
   if ((threadIdx.x & 31) == 0 && kept) atomicAdd(A.survivors, kept);
 }
 
+// What a warp needs of one run, set up by one lane for each run of a claim (so
+// that the chain of loads, run -> item -> group -> determinant, is walked once
+// for all of them) and read back by the warp in a few wide loads.
+struct __align__(16) RunInfo {
+  uint32_t B, talpha, Ak, off0;       // off0: in-place slot of the run's first pair
+  uint32_t cls0, cell0, nbk, jdx;     // bucket b's slots start at cls0 + b kCap
+  uint32_t ebeg, eend, orb, flags;    // orb: i | a << 8 of the alpha single
+  double c;
+  int64_t base;                       // E0 - H_jj, less the alpha single's change
+};
+enum : uint32_t { kRunZero = 1u, kRunBig = 2u, kRunPacked = 4u, kRunFew = 8u, kRunOdd = 16u };
+constexpr uint32_t kFewBuckets = 32;
+
 // EPS compiles Alg. 2's screen in (eps > 0); PREC selects the pair-value
 // precision (pair_value).
+//
+// Bound: instruction issue and the latency of the bucket atomics.  Seven pairs
+// in ten combine an alpha single with a beta single; such a pair takes its
+// ranks from a table, its orbitals and their diagonal terms from the
+// determinant's lists in shared memory (one 8-byte load each), and its sign
+// from the ranks: the occupied orbitals below the h-th occupied one are h, those
+// below the p-th virtual orbital x are x - p.
 template <bool EPS, int PREC>
 __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
-  extern __shared__ int64_t s_fx[];  // emit mode: jk[n*n], jj[n*n]
+  using D = typename DenType<EPS>::T;
+  struct __align__(8) Orb {
+    D z;          // diagonal term of removing or adding the orbital
+    int32_t x;    // the orbital
+  };
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint16_t s_pair[kPairTab];
+  __shared__ uint16_t s_sp[256];  // beta single f: hole rank | particle rank << 8
+  __shared__ RunInfo s_run[kRunThreads / 32][kRunClaim];
+  __shared__ Orb s_occ[kRunThreads / 32][32], s_vir[kRunThreads / 32][32];
   const int n = A.I.n;
-  int64_t *s_jk = s_fx, *s_jj = s_fx + n * n;
+  D *s_jk = reinterpret_cast<D *>(smem_raw), *s_jj = s_jk + n * n;
   for (int t = threadIdx.x; t < n * n; t += kRunThreads) {
-    s_jk[t] = A.X.jk[t];
-    s_jj[t] = A.X.jj[t];
+    s_jk[t] = static_cast<const D *>(A.jk)[t];
+    s_jj[t] = static_cast<const D *>(A.jj)[t];
   }
   for (int r = threadIdx.x; r < kPairTab; r += kRunThreads) {
     int x, y;
     unrank_pair((uint32_t)r, &x, &y);
     s_pair[r] = (uint16_t)(x | (y << 8));
   }
-  __syncthreads();
-  const uint32_t full = n >= 32 ? 0xffffffffu : ((1u << n) - 1u);
-  const uint32_t omask = (1u << A.opbits) - 1u;
-  const int lane = threadIdx.x & 31;
   const uint32_t sb = A.E.sb, vb = A.E.vb;
+  for (uint32_t f = threadIdx.x; f < sb; f += kRunThreads) {
+    const uint32_t h = A.dv_vb.div(f);
+    s_sp[f] = (uint16_t)(h | ((f - h * vb) << 8));
+  }
+  __syncthreads();
+  const uint32_t omask = (1u << A.opbits) - 1u;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  Orb *occ = s_occ[warp], *vir = s_vir[warp];
   unsigned long long my_kept = 0;  // pairs kept by the eps screen (EPS)
   // runs are claimed kRunClaim at a time from a shared counter (their lengths
-  // differ by a factor of about fifty); the next claim is issued before the
+  // differ by a factor of about five); the next claim is issued before the
   // claimed runs are emitted
   unsigned long long claim = 0;
   if (lane == 0) claim = atomicAdd(A.run_next, (unsigned long long)kRunClaim);
@@ -697,207 +772,236 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
 #pragma unroll 1
   for (; r0 < A.nruns; r0 = (uint64_t)__shfl_sync(0xffffffffu, claim, 0)) {
     if (lane == 0) claim = atomicAdd(A.run_next, (unsigned long long)kRunClaim);
-    const uint64_t r1 = r0 + kRunClaim < A.nruns ? r0 + kRunClaim : A.nruns;
-#pragma unroll 1
-  for (uint64_t r = r0; r < r1; ++r) {
-    const uint64_t run = A.runs[r];
-    const uint64_t t = A.t0 + (run >> 32);
-    const uint64_t it = A.items[t];
-    const uint32_t k = (uint32_t)it >> A.opbits, o = (uint32_t)it & omask;
-    // determinant m of the group; for o = 0, piece number m % npieces of its run
-    const uint32_t mr = (uint32_t)run;
-    const uint32_t m = o == 0 ? mr / A.npieces : mr;
-    const uint32_t ebeg = o == 0 ? (mr - m * A.npieces) * kPiecePairs : 0u;
-    const uint32_t gi = A.item_group[t] - A.gb0;
-    const uint32_t kd = A.kind[gi];
-    const bool big = kd == kTileBucket, packed = kd == kTilePacked;
-    const uint32_t jdx = A.grp_start[k] + m;
-    if (jdx >= A.ncore) {
-      if (lane == 0) atomicOr(A.err, kErrCore);
-      continue;
-    }
-    const uint32_t talpha = (uint32_t)(it >> 32);
-    const uint32_t Ak = A.grp_alpha[k], B = A.core_beta[jdx];
-    const uint32_t npd = o == 0 ? A.npd0 : A.npd1;
-    const uint32_t eend = npd < ebeg + kPiecePairs ? npd : ebeg + kPiecePairs;
-    const uint64_t p0 = A.Wexcl[t] + (uint64_t)m * npd;
-    // in-place staging slot of the run's first pair (classes that fit a tile)
-    const uint32_t off0 = (uint32_t)(A.soff[gi] + (p0 - A.g_P0[A.gb0 + gi]));
-    const uint32_t cell0 = big ? A.cellbase[gi] : 0u, nbk = big ? A.nb[gi] : 1u;
-    const uint32_t cls0 = (uint32_t)A.soff[gi];  // bucket b's slots start at cls0 + b kCap
-    // lane L: the L-th occupied and the L-th virtual beta orbital of B
-    const int occL = lane < (int)A.E.nb ? nth_set_bit(B, lane) : 0;
-    const int virL = lane < (int)vb ? nth_set_bit(~B & full, lane) : 0;
-    // emit mode: coefficient, alpha part of the diagonal change, and per lane
-    // the diagonal terms of removing occL / adding virL (Fock-like diagonal of
-    // B, plus the alpha-beta Coulomb change when o is an alpha single)
-    double c = 0.0;
-    int64_t base_x = 0, Vo = 0, Vv = 0;
-    int ia = 0, aa = 0;
-    uint32_t pa = 0;
-    double h0 = 0.0;  // the alpha single alone
-    const double *erow = A.I.eri;
-    const float *erow32 = A.I.eri32;
-    float cf = 0.0f;
-    {
-      c = A.core_c[jdx];
-      cf = (float)c;
-      base_x = A.Dx[jdx];
-      const int64_t *Fb = A.Fb + (size_t)jdx * n;
-      Vo = Fb[occL];
-      Vv = Fb[virL];
+    const int nr = (int)(A.nruns - r0 < (uint64_t)kRunClaim ? A.nruns - r0 : (uint64_t)kRunClaim);
+    __syncwarp();  // the previous claim's runs have been read
+    if (lane < nr) {
+      const uint64_t run = A.runs[r0 + lane];
+      const uint64_t t = A.t0 + (run >> 32);
+      const uint64_t it = A.items[t];
+      const uint32_t k = (uint32_t)it >> A.opbits, o = (uint32_t)it & omask;
+      // determinant m of the group; for o = 0, piece number mr % npieces of its run
+      const uint32_t mr = (uint32_t)run;
+      const uint32_t m = o == 0 ? A.dv_pieces.div(mr) : mr;
+      const uint32_t gi = A.item_group[t] - A.gb0, kd = A.kind[gi];
+      const uint32_t npd = o == 0 ? A.npd0 : A.npd1;
+      RunInfo R;
+      R.jdx = A.grp_start[k] + m;
+      R.flags = (o == 0 ? kRunZero : 0u) | (kd == kTileBucket ? kRunBig : 0u) |
+                (kd == kTilePacked ? kRunPacked : 0u);
+      R.ebeg = o == 0 ? (mr - m * A.npieces) * kPiecePairs : 0u;
+      R.eend = npd < R.ebeg + kPiecePairs ? npd : R.ebeg + kPiecePairs;
+      R.cls0 = (uint32_t)A.soff[gi];
+      R.off0 = (uint32_t)(A.soff[gi] + (A.Wexcl[t] + (uint64_t)m * npd - A.g_P0[A.gb0 + gi]));
+      R.cell0 = kd == kTileBucket ? A.cellbase[gi] : 0u;
+      R.nbk = kd == kTileBucket ? A.nb[gi] : 1u;
+      if (R.nbk < kFewBuckets) R.flags |= kRunFew;
+      R.talpha = (uint32_t)(it >> 32);
+      R.Ak = A.grp_alpha[k];
+      R.orb = 0;
+      if (R.jdx >= A.ncore) {
+        atomicOr(A.err, kErrCore);
+        R.eend = R.ebeg;
+        R.jdx = 0;
+      }
+      R.B = A.core_beta[R.jdx];
+      R.c = A.core_c[R.jdx];
+      const D *Fa = static_cast<const D *>(A.Fa) + R.jdx;
+      D base = (sizeof(D) == 8 ? (D)A.E0_x : (D)A.E0_32) - static_cast<const D *>(A.Dx)[R.jdx];
       if (o != 0) {
-        const uint32_t oi = A.opinfo[t - A.t0];
-        ia = (int)(oi & 31u);
-        aa = (int)((oi >> 5) & 31u);
-        pa = (oi >> 10) & 1u;
-        // its matrix element, summed across the warp: lane L adds the terms of
-        // the L-th occupied alpha and beta orbitals
-        const int occA = lane < (int)A.E.na ? nth_set_bit(Ak, lane) : 0;
+        int i, a;
+        const uint32_t odd = single_orbitals(R.Ak, R.talpha, &i, &a);
+        R.orb = (uint32_t)i | ((uint32_t)a << 8);
+        if (odd & 1u) R.flags |= kRunOdd;
+        base -= Fa[(size_t)a * A.ncore] - Fa[(size_t)i * A.ncore] - s_jk[a * n + i];
+      }
+      R.base = (int64_t)base;
+      s_run[warp][lane] = R;
+    }
+#pragma unroll 1
+    for (int r = 0; r < nr; ++r) {
+      __syncwarp();  // the runs are set up; the previous run's lists have been read
+      const RunInfo &R = s_run[warp][r];
+      const uint32_t B = R.B, talpha = R.talpha, flags = R.flags, ebeg = R.ebeg, eend = R.eend;
+      const uint32_t cls0 = R.cls0, off0 = R.off0, cell0 = R.cell0, nbk = R.nbk;
+      const bool zero = (flags & kRunZero) != 0u, big = (flags & kRunBig) != 0u;
+      const bool packed = (flags & kRunPacked) != 0u, few = (flags & kRunFew) != 0u;
+      const uint32_t pa = (flags & kRunOdd) ? 1u : 0u;
+      const double c = R.c;
+      const float cf = (float)c;
+      const D base = (D)R.base;
+      const int ia = (int)(R.orb & 0xffu), aa = (int)(R.orb >> 8);
+      // the determinant's occupied and virtual beta orbitals by rank, with the
+      // Fock-like diagonal (and, for an alpha single, its Coulomb change)
+      if (lane < n) {
+        Orb q;
+        q.x = lane;
+        q.z = static_cast<const D *>(A.Fb)[(size_t)R.jdx * n + lane];
+        if (!zero) q.z += s_jj[aa * n + lane] - s_jj[ia * n + lane];
+        const uint32_t nb = (uint32_t)__popc(B & below(lane));
+        if ((B >> lane) & 1u) occ[nb] = q;
+        else vir[lane - nb] = q;
+      }
+      double h0 = 0.0;  // the alpha single alone
+      const double *erow = A.I.eri;
+      const float *erow32 = A.I.eri32;
+      if (!zero) {
+        // its matrix element, summed across the warp: lane p adds the terms of
+        // orbital p where alpha and beta occupy it
         const size_t row = ((size_t)ia * n + aa) * n;
-        int64_t part = (lane < (int)A.E.na ? A.X.ssx[row + occA] : 0) +
-                       (lane < (int)A.E.nb ? A.X.sox[row + occL] : 0);
+        int64_t part = 0;
+        if (lane < n) {
+          if ((R.Ak >> lane) & 1u) part = A.X.ssx[row + lane];
+          if ((B >> lane) & 1u) part += A.X.sox[row + lane];
+        }
 #pragma unroll
         for (int d = 16; d; d >>= 1) part += (int64_t)__shfl_xor_sync(0xffffffffu, (long long)part, d);
         h0 = flip_sign(fx64_to_double(part + A.X.h1x[ia * n + aa], A.X.s1), pa);
-        base_x += A.Fa[(size_t)aa * A.ncore + jdx] - A.Fa[(size_t)ia * A.ncore + jdx] -
-                  s_jk[aa * n + ia];
-        Vo += s_jj[aa * n + occL] - s_jj[ia * n + occL];
-        Vv += s_jj[aa * n + virL] - s_jj[ia * n + virL];
         erow = A.I.eri + ((size_t)ia * n + aa) * n * n;
         if (PREC != 0) erow32 = A.I.eri32 + ((size_t)ia * n + aa) * n * n;
       }
-    }
-    // one chunk of 32 pairs: the beta operation as positions in the occupied /
-    // virtual lists (op 0: none, the alpha single alone; 1: beta single;
-    // 2: beta double), its orbitals and the target beta string
-    struct Chunk {
-      uint32_t h1, h2, p1, p2;
-      int op, bi, bj, ba, bb;
-      uint32_t tb, pos, cell;
-      bool valid, wr, spill;
-      double g;  // the gathered integral (beta double; alpha x beta single), issued ahead
-    };
-    auto decode = [&](uint32_t e0, Chunk &q) {
-      const uint32_t e = e0 + lane;
-      q.valid = e < eend;
-      q.op = 0;
-      q.h1 = q.h2 = q.p1 = q.p2 = 0;
-      if (q.valid) {
-        if (o == 0 && e >= sb) {
-          q.op = 2;
-          const uint32_t f = e - sb, qq = A.dv_pb_p.div(f);
-          const uint32_t hp = s_pair[qq], pp = s_pair[f - qq * A.dv_pb_p.d];
-          q.h1 = hp & 0xffu;
-          q.h2 = hp >> 8;
-          q.p1 = pp & 0xffu;
-          q.p2 = pp >> 8;
-        } else if (o == 0 || e > 0) {
-          q.op = 1;
-          const uint32_t f = o == 0 ? e : e - 1, qq = A.dv_vb.div(f);
-          q.h1 = qq;
-          q.p1 = f - qq * vb;
-        }
-      }
-      q.bi = __shfl_sync(0xffffffffu, occL, (int)q.h1);
-      q.bj = __shfl_sync(0xffffffffu, occL, (int)q.h2);
-      q.ba = __shfl_sync(0xffffffffu, virL, (int)q.p1);
-      q.bb = __shfl_sync(0xffffffffu, virL, (int)q.p2);
-      q.tb = B;
-      if (q.op == 1) q.tb ^= (1u << q.bi) | (1u << q.ba);
-      if (q.op == 2) q.tb ^= (1u << q.bi) | (1u << q.bj) | (1u << q.ba) | (1u << q.bb);
-      const uint32_t bkt = big ? bucket_of(q.tb, nbk) : 0u;
-      q.cell = cell0 + bkt;
-      q.pos = 0;
-      q.spill = false;
-      q.wr = q.valid;
-      if (big) {  // warp-uniform: the next free slot of the lane's bucket cell
-        const uint32_t peers = __match_any_sync(0xffffffffu, q.valid ? q.cell : 0xffffffffu);
-        const int leader = __ffs(peers) - 1;
-        uint32_t base = 0;
-        if (q.valid && lane == leader) base = atomicAdd(&A.fill[q.cell], (uint32_t)__popc(peers));
-        base = __shfl_sync(0xffffffffu, base, leader);
-        const uint32_t slot = base + __popc(peers & ((1u << lane) - 1u));
-        if (slot < (uint32_t)kCap) {
+      const D Bz = base;
+      __syncwarp();
+      // one chunk of 32 pairs: target, place, denominator and matrix element
+      struct Chunk {
+        uint32_t tb, pos, sign;
+        D den;
+        bool valid, spill;
+        double g;   // the gathered integral, requested a chunk ahead
+        float gf;   // the same from the FP32 tables
+      };
+      auto place = [&](Chunk &q, uint32_t e) {
+        q.spill = false;
+        if (big) {  // warp-uniform: the next free slot of the lane's bucket cell
+          const uint32_t bkt = bucket_of(q.tb, nbk);
+          const uint32_t slot = claim_slot(A.fill, cell0 + bkt, q.valid, few);
           q.pos = cls0 + bkt * (uint32_t)kCap + slot;
-        } else if (q.valid) {  // the cell is full: the spill list
-          q.spill = true;
-          q.pos = atomicAdd(A.n_spill, 1u);
+          if (q.valid && slot >= (uint32_t)kCap) {  // the cell is full: the spill list
+            q.spill = true;
+            q.pos = atomicAdd(A.n_spill, 1u);
+          }
+        } else {
+          q.pos = off0 + e;
+        }
+      };
+      auto emit = [&](const Chunk &q, double h, bool is_double) {
+        // is_double: h holds the value; else the gathered integral is it
+        double v;
+        if (PREC == 2) {
+          const float hf = is_double ? (float)h : __uint_as_float(__float_as_uint(q.gf) ^ (q.sign << 31));
+          v = widen(hf * cf);
+        } else {
+          const double hh = is_double ? h : flip_sign(PREC == 1 ? widen(q.gf) : q.g, q.sign);
+          v = hh * c;
+        }
+        bool kept = false;
+        if (q.valid)
+          write_record<EPS>(A, q.pos, q.spill, cell0 + (big ? bucket_of(q.tb, nbk) : 0u), talpha, q.tb,
+                            packed, v, q.den, &kept);
+        if (EPS) my_kept += kept ? 1u : 0u;
+      };
+      if (!zero) {
+        auto decode = [&](uint32_t e0, Chunk &q) {
+          const uint32_t e = e0 + lane;
+          q.valid = e < eend;
+          q.tb = B;
+          q.den = Bz;
+          q.sign = 0;
+          q.g = 0.0;
+          q.gf = 0.0f;
+          if (q.valid && e > 0) {
+            const uint32_t sp = s_sp[e - 1], h = sp & 0xffu, p = sp >> 8;
+            const Orb i = occ[h], a = vir[p];
+            q.tb = B ^ (1u << i.x) ^ (1u << a.x);
+            q.den = Bz - (a.z - i.z - s_jk[a.x * n + i.x]);
+            q.sign = (pa + h + (uint32_t)a.x - p + (a.x > i.x ? 1u : 0u)) & 1u;
+            const int ix = i.x * n + a.x;
+            if (PREC != 0) q.gf = erow32[ix];
+            else q.g = erow[ix];
+          }
+          place(q, e);
+        };
+        // software-pipelined: the next chunk's slots (an atomic for big
+        // classes) and integrals are requested before this chunk is written
+        Chunk cur, nxt;
+        decode(0, cur);
+#pragma unroll 1
+        for (uint32_t e0 = 0; e0 < eend; e0 += 32) {
+          if (e0 + 32 < eend) decode(e0 + 32, nxt);  // warp-uniform
+          emit(cur, h0, e0 + lane == 0);
+          cur = nxt;
         }
       } else {
-        q.pos = off0 + e;
-      }
-      // the chunk's integral gather, issued now and used one chunk later
-      q.g = 0.0;
-      if (q.op == 2) {
-        const size_t ix = (((size_t)q.bj * n + q.bb) * n + q.bi) * n + q.ba;
-        q.g = PREC != 0 ? widen(A.I.asymT32[ix]) : A.I.asymT[ix];
-      } else if (q.op == 1 && o != 0) {
-        q.g = PREC != 0 ? widen(erow32[q.bi * n + q.ba]) : erow[q.bi * n + q.ba];
-      }
-    };
-    // software-pipelined: the next chunk's staging slots (an atomic for big
-    // classes) and integrals are requested before this chunk's matrix
-    // elements are formed
-    Chunk cur, nxt;
-    decode(ebeg, cur);
+        auto decode = [&](uint32_t e0, Chunk &q) {
+          const uint32_t e = e0 + lane;
+          q.valid = e < eend;
+          q.tb = B;
+          q.den = Bz;
+          q.sign = 0;
+          q.g = 0.0;
+          q.gf = 0.0f;
+          if (q.valid && e >= sb) {
+            const uint32_t f = e - sb, qq = A.dv_pb_p.div(f);
+            const uint32_t hp = s_pair[qq], pp = s_pair[f - qq * A.dv_pb_p.d];
+            const uint32_t h1 = hp & 0xffu, h2 = hp >> 8, p1 = pp & 0xffu, p2 = pp >> 8;
+            const Orb i = occ[h1], j = occ[h2], a = vir[p1], b = vir[p2];
+            const uint32_t pm = (1u << a.x) | (1u << b.x);
+            q.tb = B ^ ((1u << i.x) | (1u << j.x)) ^ pm;
+            q.den = Bz - (a.z + b.z - i.z - j.z + s_jk[i.x * n + j.x] + s_jk[a.x * n + b.x] -
+                          s_jk[a.x * n + i.x] - s_jk[a.x * n + j.x] - s_jk[b.x * n + i.x] -
+                          s_jk[b.x * n + j.x]);
+            const uint32_t between = below(j.x) & ~((2u << i.x) - 1u);
+            q.sign = (h1 + h2 + (uint32_t)a.x - p1 + (uint32_t)b.x - p2 + 1u +
+                      (uint32_t)__popc(pm & between)) & 1u;
+            const size_t ix = (((size_t)j.x * n + b.x) * n + i.x) * n + a.x;
+            if (PREC != 0) q.gf = A.I.asymT32[ix];
+            else q.g = A.I.asymT[ix];
+          } else if (q.valid) {  // beta single
+            const uint32_t sp = s_sp[e], h = sp & 0xffu, p = sp >> 8;
+            const Orb i = occ[h], a = vir[p];
+            q.tb = B ^ (1u << i.x) ^ (1u << a.x);
+            q.den = Bz - (a.z - i.z - s_jk[a.x * n + i.x]);
+            q.sign = (h + (uint32_t)a.x - p + (a.x > i.x ? 1u : 0u)) & 1u;
+            q.g = flip_sign(fx64_to_double(fx_single(A.X, B, R.Ak, i.x, a.x), A.X.s1), q.sign);
+          }
+          place(q, e);
+        };
+        Chunk cur, nxt;
+        decode(ebeg, cur);
 #pragma unroll 1
-    for (uint32_t e0 = ebeg; e0 < eend; e0 += 32) {
-      if (e0 + 32 < eend) decode(e0 + 32, nxt);  // warp-uniform
-      double h = 0.0;
-      int64_t dh = 0;
-      {
-        const int64_t vo1 = shfl64(Vo, (int)cur.h1), vv1 = shfl64(Vv, (int)cur.p1);
-        int64_t vo2 = 0, vv2 = 0;
-        if (o == 0) {  // warp-uniform
-          vo2 = shfl64(Vo, (int)cur.h2);
-          vv2 = shfl64(Vv, (int)cur.p2);
-        }
-        const int bi = cur.bi, bj = cur.bj, ba = cur.ba, bb = cur.bb;
-        if (cur.op == 0) {
-          h = h0;
-        } else if (cur.op == 1) {
-          if (o == 0)
-            h = flip_sign(fx64_to_double(fx_single(A.X, B, Ak, bi, ba), A.X.s1),
-                          (uint32_t)single_parity(B, bi, ba));
-          else
-            h = flip_sign(cur.g, pa ^ (uint32_t)single_parity(B, bi, ba));
-          dh = vv1 - vo1 - s_jk[ba * n + bi];
-        } else {
-          h = flip_sign(cur.g, (uint32_t)par_double(B, bi, bj, ba, bb));
-          dh = vv1 + vv2 - vo1 - vo2 + s_jk[bi * n + bj] + s_jk[ba * n + bb] - s_jk[ba * n + bi] -
-               s_jk[ba * n + bj] - s_jk[bb * n + bi] - s_jk[bb * n + bj];
+        for (uint32_t e0 = ebeg; e0 < eend; e0 += 32) {
+          if (e0 + 32 < eend) decode(e0 + 32, nxt);
+          emit(cur, cur.g, e0 + lane < sb);
+          cur = nxt;
         }
       }
-      bool kept = false;
-      if (cur.wr)
-        write_record<EPS>(A, cur.pos, cur.spill, cur.cell, talpha, cur.tb, packed,
-                          pair_value<PREC>(h, c, cf), base_x + dh, &kept);
-      if (EPS) my_kept += kept ? 1u : 0u;
-      cur = nxt;
     }
-  }
   }
   if (EPS) add_survivors(A, my_kept);
 }
 
 // Alpha-double pairs, flat: CTA step s covers flat pairs [s * kAdTile, ...).
+// An item's orbitals are the bits in which its target differs from its group's
+// alpha string (unranking the operation's number took some 300 instructions an
+// item, of 2.2 pairs at (24e,30o)).
 template <bool EPS, int PREC>
 __global__ void __launch_bounds__(kAdThreads) k_emit_ad(EmitArgs A) {
+  using D = typename DenType<EPS>::T;
   __shared__ uint32_t sF[kAdTile + 1];    // first flat pair of each item in the step
   __shared__ uint32_t sPos[kAdTile + 1];  // in-place staging slot of the item's first pair
   __shared__ uint32_t sG[kAdTile + 1];    // first core determinant of the item's group
-  __shared__ uint32_t sOrb[kAdTile + 1];  // i | a << 5 | j << 10 | b << 15
+  __shared__ uint32_t sOrb[kAdTile + 1];  // i | a << 5 | j << 10 | b << 15 | kind << 20
   __shared__ uint32_t sTA[kAdTile + 1];   // target alpha string
-  __shared__ uint32_t sCls[kAdTile + 1];  // class (relative to the batch)
+  __shared__ uint32_t sNb[kAdTile + 1];   // buckets and first cell of the item's class
+  __shared__ uint32_t sCell[kAdTile + 1];
   __shared__ uint32_t sBase[kAdTile + 1]; // first staging slot of the class
   __shared__ double sH[kAdTile + 1];      // signed matrix element
-  __shared__ int64_t sD[kAdTile + 1];     // determinant-independent diagonal change
+  __shared__ D sD[kAdTile + 1];           // determinant-independent diagonal change
   __shared__ uint16_t sItem[kAdTile];     // item of each pair of the step
   const int n = A.I.n;
-  const uint32_t full = n >= 32 ? 0xffffffffu : ((1u << n) - 1u);
   const uint32_t omask = (1u << A.opbits) - 1u;
   const int lane = threadIdx.x & 31;
+  const D *jk = static_cast<const D *>(A.jk), *Dx = static_cast<const D *>(A.Dx);
+  const D E0 = sizeof(D) == 8 ? (D)A.E0_x : (D)A.E0_32;
   unsigned long long my_kept = 0;  // pairs kept by the eps screen (EPS)
 #pragma unroll 1
   for (uint32_t step = blockIdx.x; step < A.ad_tiles; step += gridDim.x) {
@@ -910,26 +1014,26 @@ __global__ void __launch_bounds__(kAdThreads) k_emit_ad(EmitArgs A) {
     for (int i = threadIdx.x; i < nspan; i += kAdThreads) {
       const uint64_t t = A.t0 + A.adl[ja + i];
       const uint64_t it = A.items[t];
-      const uint32_t k = (uint32_t)it >> A.opbits, o = (uint32_t)it & omask;
+      const uint32_t k = (uint32_t)it >> A.opbits;
       const uint32_t gi = A.item_group[t] - A.gb0;
+      const uint32_t kd = A.kind[gi], Ak = A.grp_alpha[k], At = (uint32_t)(it >> 32);
+      const uint64_t so = A.soff[gi];
       sF[i] = A.ad_off[ja + i];
-      sPos[i] = (uint32_t)(A.soff[gi] + (A.Wexcl[t] - A.g_P0[A.gb0 + gi]));
-      sBase[i] = (uint32_t)A.soff[gi];
+      sPos[i] = (uint32_t)(so + (A.Wexcl[t] - A.g_P0[A.gb0 + gi]));
+      sBase[i] = (uint32_t)so;
       sG[i] = A.grp_start[k];
-      sTA[i] = (uint32_t)(it >> 32);
-      sCls[i] = gi;
-      {
-        const uint32_t Ak = A.grp_alpha[k];
-        int ia, ja2, aa, ba;
-        dec_double(Ak, ~Ak & full, o - 1 - A.E.sa, A.dv_pa_p, &ia, &ja2, &aa, &ba);
-        sOrb[i] = (uint32_t)ia | ((uint32_t)aa << 5) | ((uint32_t)ja2 << 10) | ((uint32_t)ba << 15);
-        const size_t ix = (((size_t)ia * n + aa) * n + ja2) * n + ba;
-        sH[i] = flip_sign(PREC != 0 ? widen(A.I.asym32[ix]) : A.I.asym[ix],
-                          (uint32_t)par_double(Ak, ia, ja2, aa, ba));
-        const int64_t *jk = A.X.jk;
-        sD[i] = jk[ia * n + ja2] + jk[aa * n + ba] - jk[aa * n + ia] - jk[aa * n + ja2] -
-                jk[ba * n + ia] - jk[ba * n + ja2];
-      }
+      sTA[i] = At;
+      sNb[i] = kd == kTileBucket ? A.nb[gi] : 0u;
+      sCell[i] = kd == kTileBucket ? A.cellbase[gi] : 0u;
+      const uint32_t hm = Ak & ~At, pm = At & ~Ak;
+      const int ia = __ffs(hm) - 1, ja2 = 31 - __clz(hm), aa = __ffs(pm) - 1, ba = 31 - __clz(pm);
+      sOrb[i] = (uint32_t)ia | ((uint32_t)aa << 5) | ((uint32_t)ja2 << 10) | ((uint32_t)ba << 15) |
+                (kd << 20);
+      const size_t ix = (((size_t)ia * n + aa) * n + ja2) * n + ba;
+      sH[i] = flip_sign(PREC != 0 ? widen(A.I.asym32[ix]) : A.I.asym[ix],
+                        double_sign(Ak, ia, ja2, aa, ba));
+      sD[i] = jk[ia * n + ja2] + jk[aa * n + ba] - jk[aa * n + ia] - jk[aa * n + ja2] -
+              jk[ba * n + ia] - jk[ba * n + ja2];
     }
     __syncthreads();
     // pair -> item map of the step: each item marks its pairs
@@ -947,9 +1051,8 @@ __global__ void __launch_bounds__(kAdThreads) k_emit_ad(EmitArgs A) {
       const int lo = valid ? (int)sItem[f - fb] : 0;
       const uint32_t q = valid ? f - sF[lo] : 0u;
       uint32_t jdx = sG[lo] + q;
-      const uint32_t gi = sCls[lo];
-      const bool bigl = valid && A.kind[gi] == kTileBucket;
-      const bool big = __any_sync(0xffffffffu, bigl);
+      const uint32_t ob = sOrb[lo], kd = ob >> 20;
+      const bool bigl = valid && kd == kTileBucket;
       if (valid && jdx >= A.ncore) {
         atomicOr(A.err, kErrCore);
         jdx = 0;
@@ -958,17 +1061,12 @@ __global__ void __launch_bounds__(kAdThreads) k_emit_ad(EmitArgs A) {
       // lanes of one warp may straddle classes of both kinds: position per lane
       uint32_t pos = sPos[lo] + q, cell = 0;
       bool spill = false;
-      uint32_t bkt = 0;
-      if (big) {
-        bkt = bigl ? bucket_of(B, A.nb[gi]) : 0u;
-        cell = bigl ? A.cellbase[gi] + bkt : 0u;
-        const uint32_t peers = __match_any_sync(0xffffffffu, bigl ? cell : 0xffffffffu);
-        const int leader = __ffs(peers) - 1;
-        uint32_t base = 0;
-        if (bigl && lane == leader) base = atomicAdd(&A.fill[cell], (uint32_t)__popc(peers));
-        base = __shfl_sync(0xffffffffu, base, leader);
+      if (__any_sync(0xffffffffu, bigl)) {
+        const uint32_t bkt = bigl ? bucket_of(B, sNb[lo]) : 0u;
+        cell = sCell[lo] + bkt;
+        const bool few = __any_sync(0xffffffffu, bigl && sNb[lo] < kFewBuckets);
+        const uint32_t slot = claim_slot(A.fill, cell, bigl, few);
         if (bigl) {
-          const uint32_t slot = base + __popc(peers & ((1u << lane) - 1u));
           if (slot < (uint32_t)kCap) {
             pos = sBase[lo] + bkt * (uint32_t)kCap + slot;
           } else {
@@ -979,14 +1077,13 @@ __global__ void __launch_bounds__(kAdThreads) k_emit_ad(EmitArgs A) {
       }
       bool kept = false;
       if (valid) {
-        const uint32_t ob = sOrb[lo];
-        const int64_t *Fa = A.Fa + jdx;  // orbital p at Fa[p * ncore]
+        const D *Fa = static_cast<const D *>(A.Fa) + jdx;  // orbital p at Fa[p * ncore]
         const size_t m = A.ncore;
-        const int64_t dh = sD[lo] + Fa[((ob >> 5) & 31u) * m] + Fa[((ob >> 15) & 31u) * m] -
-                           Fa[(ob & 31u) * m] - Fa[((ob >> 10) & 31u) * m];
-        write_record<EPS>(A, pos, spill, cell, sTA[lo], B, A.kind[gi] == kTilePacked,
-                          pair_value<PREC>(sH[lo], A.core_c[jdx], (float)A.core_c[jdx]),
-                          A.Dx[jdx] + dh, &kept);
+        const D dh = sD[lo] + Fa[((ob >> 5) & 31u) * m] + Fa[((ob >> 15) & 31u) * m] -
+                     Fa[(ob & 31u) * m] - Fa[((ob >> 10) & 31u) * m];
+        const double c = A.core_c[jdx];
+        write_record<EPS>(A, pos, spill, cell, sTA[lo], B, kd == kTilePacked,
+                          pair_value<PREC>(sH[lo], c, (float)c), E0 - Dx[jdx] - dh, &kept);
       }
       if (EPS) my_kept += kept ? 1u : 0u;
     }
@@ -1033,13 +1130,10 @@ __global__ void k_plan_totals(uint32_t ng, const uint64_t *soff, const uint64_t 
 }
 
 __global__ void k_batch_lists(const uint64_t *items, uint64_t t0, uint64_t nt, int opbits,
-                              uint32_t sa, const uint32_t *grp_count, const uint32_t *rcnt,
-                              const uint32_t *roff, const uint32_t *adpos, const uint32_t *adsum,
-                              uint64_t *runs, uint32_t *adl, uint32_t *ad_off,
-                              const uint32_t *grp_alpha, int n,
-                              FastDiv dv_va, uint32_t *opinfo) {
+                              uint32_t sa, const uint32_t *rcnt, const uint32_t *roff,
+                              const uint32_t *adpos, const uint32_t *adsum,
+                              uint64_t *runs, uint32_t *adl, uint32_t *ad_off) {
   const uint32_t omask = (1u << opbits) - 1u;
-  const uint32_t full = n >= 32 ? 0xffffffffu : ((1u << n) - 1u);
   const int lane = (int)(threadIdx.x & 31u);
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   // warps take 32 items at a time (warp-uniform loop); the runs of the 32
@@ -1051,18 +1145,10 @@ __global__ void k_batch_lists(const uint64_t *items, uint64_t t0, uint64_t nt, i
     uint32_t cnt = 0, start = 0;
     if (i < nt) {
       const uint32_t lo = (uint32_t)items[t0 + i];
-      const uint32_t k = lo >> opbits, o = lo & omask;
+      const uint32_t o = lo & omask;
       if (o <= sa) {
         cnt = rcnt[i];
         start = roff[i];
-        uint32_t oi = 0;
-        if (o != 0) {
-          const uint32_t Ak = grp_alpha[k];
-          int ia, aa;
-          dec_single(Ak, ~Ak & full, o - 1, dv_va, &ia, &aa);
-          oi = (uint32_t)ia | ((uint32_t)aa << 5) | ((uint32_t)single_parity(Ak, ia, aa) << 10);
-        }
-        opinfo[i] = oi;
       } else {
         adl[adpos[i]] = (uint32_t)i;
         ad_off[adpos[i]] = adsum[i];
@@ -2089,12 +2175,42 @@ int build_fx(const double *h1, const double *eri, int n, int na, int nb, double 
   return ASCI_OK;
 }
 
+// H_jj, the Fock-like diagonals of the core and the pair tables in the type of
+// the emission's diagonal: 64 bits when the eps screen is on, else 32.
 int core_fock(const FxInts &X, const uint32_t *core_alpha, const uint32_t *core_beta, size_t m,
-              int64_t *Dx, int64_t *Fa, int64_t *Fb, Arena &arena) {
-  if (!m) return ASCI_OK;
-  k_core_fock<<<dim3(grid_for(m, 152 * 4), X.n + 1), 256, 0, arena.stream()>>>(X, core_alpha, core_beta,
-                                                                              m, Dx, Fa, Fb);
+              FusedCore *F, Arena &arena) {
+  const int n = X.n;
+  const dim3 grid(grid_for(m, 152 * 4), n + 1);
+  cudaStream_t s = arena.stream();
+  if (F->screened) {
+    int64_t *Dx, *Fa, *Fb;
+    ASCI_TRY(arena.alloc(&Dx, m));
+    ASCI_TRY(arena.alloc(&Fa, m * n));
+    ASCI_TRY(arena.alloc(&Fb, m * n));
+    k_core_fock<int64_t><<<grid, 256, 0, s>>>(X, core_alpha, core_beta, m, Dx, Fa, Fb);
+    ASCI_CHECK_LAUNCH();
+    F->Dx = Dx;
+    F->Fa = Fa;
+    F->Fb = Fb;
+    F->ejk = X.jk;
+    F->ejj = X.jj;
+    return ASCI_OK;
+  }
+  uint32_t *Dx, *Fa, *Fb, *jk, *jj;
+  ASCI_TRY(arena.alloc(&Dx, m));
+  ASCI_TRY(arena.alloc(&Fa, m * n));
+  ASCI_TRY(arena.alloc(&Fb, m * n));
+  ASCI_TRY(arena.alloc(&jk, (size_t)n * n));
+  ASCI_TRY(arena.alloc(&jj, (size_t)n * n));
+  k_core_fock<uint32_t><<<grid, 256, 0, s>>>(X, core_alpha, core_beta, m, Dx, Fa, Fb);
   ASCI_CHECK_LAUNCH();
+  k_den_tables<<<(n * n + 255) / 256, 256, 0, s>>>(X, jk, jj);
+  ASCI_CHECK_LAUNCH();
+  F->Dx = Dx;
+  F->Fa = Fa;
+  F->Fb = Fb;
+  F->ejk = jk;
+  F->ejj = jj;
   return ASCI_OK;
 }
 
@@ -2252,14 +2368,12 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
     return ASCI_ECUDA;
   }
   uint64_t *runs;
-  uint32_t *adl, *ad_off, *opinfo;
-  ASCI_TRY(arena.alloc(&opinfo, nt));
+  uint32_t *adl, *ad_off;
   ASCI_TRY(arena.alloc(&runs, nruns + 1));
   ASCI_TRY(arena.alloc(&adl, nad + 1));
   ASCI_TRY(arena.alloc(&ad_off, nad + 1));
-  k_batch_lists<<<grid_for(nt), 256, 0, s>>>(F.items, t0, nt, F.opbits, F.E.sa, F.grp_count, rcnt,
-                                             roff, adpos, adsum, runs, adl, ad_off, F.grp_alpha,
-                                             F.X.n, FastDiv(F.E.va ? F.E.va : 1), opinfo);
+  k_batch_lists<<<grid_for(nt), 256, 0, s>>>(F.items, t0, nt, F.opbits, F.E.sa, rcnt, roff, adpos,
+                                             adsum, runs, adl, ad_off);
   ASCI_CHECK_LAUNCH();
   uint32_t ad_tiles = 0;
   uint32_t *ad_tile_item = nullptr;
@@ -2323,10 +2437,9 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   A.I = F.I;
   A.X = F.X;
   A.E = F.E;
-  A.dv_va = FastDiv(F.E.va ? F.E.va : 1);
   A.dv_vb = FastDiv(F.E.vb ? F.E.vb : 1);
-  A.dv_pa_p = FastDiv(F.E.pa_p ? F.E.pa_p : 1);
   A.dv_pb_p = FastDiv(F.E.pb_p ? F.E.pb_p : 1);
+  A.dv_pieces = FastDiv(npieces);
   A.npd0 = (uint32_t)(F.E.sb + F.E.dbb);
   A.npd1 = 1u + F.E.sb;
   A.npieces = npieces;
@@ -2344,6 +2457,8 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   A.Dx = F.Dx;
   A.Fa = F.Fa;
   A.Fb = F.Fb;
+  A.jk = F.ejk;
+  A.jj = F.ejj;
   A.gb0 = gb0;
   A.kind = kind;
   A.nb = nb;
@@ -2359,7 +2474,6 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   A.runs = runs;
   A.nruns = nruns;
   A.adl = adl;
-  A.opinfo = opinfo;
   A.ad_off = ad_off;
   A.nad = (uint32_t)nad;
   A.ad_total = (uint32_t)ad_total;
@@ -2370,10 +2484,12 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   A.eps_f = (float)eps;
   A.E0_x = F.E0_x;
   A.inv_scale = ldexp(1.0, -F.X.s);
+  A.E0_32 = (int32_t)den_round<uint32_t>(F.E0_x);
+  A.scale32 = (float)ldexp(1.0, kDenShift - F.X.s);
   A.survivors = survivors;
   A.ncore = F.ncore;
   A.err = err;
-  const size_t emit_smem = 2 * (size_t)F.X.n * F.X.n * sizeof(int64_t);
+  const size_t emit_smem = 2 * (size_t)F.X.n * F.X.n * (F.screened ? sizeof(int64_t) : sizeof(uint32_t));
   unsigned long long *run_next;
   ASCI_TRY(arena.alloc(&run_next, 1));
   A.run_next = run_next;

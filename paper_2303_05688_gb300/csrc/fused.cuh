@@ -68,7 +68,7 @@ struct FusedCore {
   int opbits;
   const uint32_t *grp_alpha, *grp_start, *grp_count, *core_beta;
   const double *core_c;
-  const int64_t *Dx, *Fa, *Fb;
+  const void *Dx, *Fa, *Fb, *ejk, *ejj;  // the emission's diagonal tables (core_fock)
   const uint32_t *g_alpha;
   const uint64_t *g_P0;
   int64_t E0_x;

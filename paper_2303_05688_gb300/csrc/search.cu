@@ -44,7 +44,7 @@ int fx_bounds(const double *h1, const double *eri, int n, unsigned long long *ou
 int build_fx(const double *h1, const double *eri, int n, int na, int nb, double ecore, double E0,
              const double h3[4], Arena &arena, FxInts *out, int64_t *E0_x);
 int core_fock(const FxInts &X, const uint32_t *core_alpha, const uint32_t *core_beta, size_t m,
-              int64_t *Dx, int64_t *Fa, int64_t *Fb, Arena &arena);
+              FusedCore *F, Arena &arena);
 int item_groups(const uint64_t *items, const uint64_t *Wexcl, uint64_t T, uint32_t *item_group,
                 uint32_t **g_alpha, uint64_t **g_P0, uint64_t **g_item0, size_t *G, uint64_t *P,
                 Arena &arena);
@@ -839,16 +839,7 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   F.ctas_per_sm = o.ctas_per_sm;
   ASCI_TRY(build_fx(h1, eri, n, na, nb, ints->ecore, E0, hp.bounds, arena, &F.X, &F.E0_x));
   if (st) st->diag_grid_bits = (uint64_t)F.X.s;
-  {
-    int64_t *Dx, *Fa, *Fb;
-    ASCI_TRY(arena.alloc(&Dx, m));
-    ASCI_TRY(arena.alloc(&Fa, m * n));
-    ASCI_TRY(arena.alloc(&Fb, m * n));
-    ASCI_TRY(core_fock(F.X, core_alpha, core_beta, m, Dx, Fa, Fb, arena));
-    F.Dx = Dx;
-    F.Fa = Fa;
-    F.Fb = Fb;
-  }
+  ASCI_TRY(core_fock(F.X, core_alpha, core_beta, m, &F, arena));
   F.item_group = item_group;
   F.g_alpha = g_alpha;
   F.g_P0 = g_P0;
