@@ -197,42 +197,45 @@ __device__ __forceinline__ int64_t fx_diag(const FxInts &X, uint32_t A, uint32_t
 
 namespace {
 
-// The staged denominator only serves screens (|v| against tau |E0 - H_ii|), so
-// without the eps screen, which tests it exactly, it is summed in 32-bit fixed
-// point: multiples of 2^29 units of the 64-bit grid (|E0 - H_ii| < 2^59 of
-// those), each term rounded to nearest, and stored as a lower bound of the
-// magnitude: a sum of at most 15 such terms is within 8 units.  Half the
-// registers, shuffles, table bytes and additions of 64 bits.
+// The staged denominator E0 - H_ii serves screens only, so it is summed in
+// 32-bit fixed point: multiples of 2^29 units of the 64-bit grid (|E0 - H_ii| <
+// 2^59 of those), each term rounded to nearest; a sum of at most 15 such terms
+// is within 8 units of the exact value, and what is stored is a lower bound of
+// the magnitude.  A test that these 8 units could decide forms the exact value.
+// Half the registers, shuffles, table bytes and additions of 64 bits.  (Unsigned:
+// sums may wrap on the way.)
 constexpr int kDenShift = 29;
 constexpr int32_t kDenSlack = 8;
-template <bool EPS>
-struct DenType {
-  using T = uint32_t;  // two's complement; sums may wrap on the way
-};
-template <>
-struct DenType<true> {
-  using T = int64_t;
-};
-template <typename T>
-__host__ __device__ __forceinline__ T den_round(int64_t x) {
-  return sizeof(T) == 8 ? (T)x : (T)((x + (1ll << (kDenShift - 1))) >> kDenShift);
+__host__ __device__ __forceinline__ uint32_t den_round(int64_t x) {
+  return (uint32_t)((x + (1ll << (kDenShift - 1))) >> kDenShift);
 }
+
+// A core determinant as the emission reads it: one 16-byte load.
+struct __align__(16) CoreRec {
+  uint32_t beta;
+  uint32_t den;  // E0 - H_jj
+  double c;
+};
 
 // Parent data of each core det (alpha-sorted order): H_jj and both Fock-like
 // diagonals.  Fb is determinant-major (Fb[j n + p]: a warp's lanes read one
 // determinant's row); Fa is orbital-major (Fa[p m + j]: the lanes of an
 // alpha-double step read one orbital of consecutive determinants).
 // A thread per (orbital, determinant), determinants fastest; the thread of
-// orbital n forms H_jj.  D is the emission's diagonal type (den_round).
-template <typename D>
-__global__ void k_core_fock(FxInts X, const uint32_t *core_alpha, const uint32_t *core_beta,
-                            size_t m, D *Dx, D *Fa, D *Fb) {
+// orbital n forms H_jj and the determinant's record.
+__global__ void k_core_fock(FxInts X, int64_t E0_x, const uint32_t *core_alpha,
+                            const uint32_t *core_beta, const double *core_c, size_t m,
+                            CoreRec *rec, uint32_t *Fa, uint32_t *Fb) {
   const int n = X.n, p = (int)blockIdx.y;
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < m;
        j += (size_t)gridDim.x * blockDim.x) {
     const uint32_t A = core_alpha[j], B = core_beta[j];
     if (p == n) {
-      Dx[j] = den_round<D>(fx_diag(X, A, B));
+      CoreRec r;
+      r.beta = B;
+      r.den = den_round(E0_x - fx_diag(X, A, B));
+      r.c = core_c[j];
+      rec[j] = r;
       continue;
     }
     int64_t fa = X.hh[p], fb = X.hh[p];
@@ -246,15 +249,15 @@ __global__ void k_core_fock(FxInts X, const uint32_t *core_alpha, const uint32_t
       fb += X.jk[p * n + q];
       fa += X.jj[p * n + q];
     }
-    Fa[(size_t)p * m + j] = den_round<D>(fa);
-    Fb[j * n + p] = den_round<D>(fb);
+    Fa[(size_t)p * m + j] = den_round(fa);
+    Fb[j * n + p] = den_round(fb);
   }
 }
 
 __global__ void k_den_tables(FxInts X, uint32_t *jk, uint32_t *jj) {
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < X.n * X.n; t += gridDim.x * blockDim.x) {
-    jk[t] = den_round<uint32_t>(X.jk[t]);
-    jj[t] = den_round<uint32_t>(X.jj[t]);
+    jk[t] = den_round(X.jk[t]);
+    jj[t] = den_round(X.jj[t]);
   }
 }
 
@@ -518,11 +521,11 @@ struct EmitArgs {
   const uint32_t *item_group;
   uint64_t t0, P0;
   int opbits;
-  const uint32_t *grp_alpha, *grp_start, *grp_count, *core_beta;
-  const double *core_c;
-  // H_jj and the Fock-like diagonals of the core, and jk and jj, in the type of
-  // the emission's diagonal (DenType): 64 bits with the eps screen, else 32
-  const void *Dx, *Fa, *Fb, *jk, *jj;
+  const uint32_t *grp_alpha, *grp_start, *grp_count;
+  // the core's records, its Fock-like diagonals and jk, jj in units of the
+  // 32-bit denominator
+  const CoreRec *core;
+  const uint32_t *Fa, *Fb, *jk, *jj;
   uint32_t gb0;
   const uint32_t *kind, *nb, *cellbase;
   const uint64_t *soff;       // first staging slot of each class of the batch
@@ -542,12 +545,12 @@ struct EmitArgs {
   const uint32_t *ad_tile_item;  // first alpha-double item of each CTA step
   uint32_t ad_tiles;
   Stage st;
+  uint32_t st_cap;            // st.cap (below 2^32)
   double eps;                 // Alg. 2 screen; 0 keeps every pair
   float eps_f;                // eps as a float (the screen's float pre-test)
   int64_t E0_x;
   double inv_scale;
-  int32_t E0_32;
-  float scale32;              // a unit of the 32-bit diagonal
+  float scale32;              // a unit of the 32-bit denominator
   unsigned long long *survivors;
   uint32_t ncore;
   unsigned *err;
@@ -616,18 +619,6 @@ __device__ __forceinline__ double pair_value(double h, double c, float cf) {
   return h * c;
 }
 
-// z * 2^-s as a float built from the bits (truncated, relative error below
-// 2^-23); 0 when z is zero or the value lies outside the normal float range.
-__device__ __forceinline__ float scaled_as_float(int64_t z, int s) {
-  if (!z) return 0.0f;
-  const uint64_t u = z < 0 ? 0ull - (uint64_t)z : (uint64_t)z;
-  const int lz = __clzll((long long)u);
-  const int e = 63 - lz - s + 127;
-  if (e < 1 || e > 254) return 0.0f;
-  const uint32_t mant = (uint32_t)((u << lz) >> 40) & 0x7fffffu;
-  return __uint_as_float((z < 0 ? 0x80000000u : 0u) | ((uint32_t)e << 23) | mant);
-}
-
 // |x| as a float built from the bits, truncated (relative error below 2^-23);
 // *ok is false when |x| lies outside the normal float range.
 __device__ __forceinline__ float abs_as_float(double x, bool *ok) {
@@ -638,38 +629,34 @@ __device__ __forceinline__ float abs_as_float(double x, bool *ok) {
   return __uint_as_float(((uint32_t)e << 23) | (uint32_t)((b >> 29) & 0x7fffffu));
 }
 
-// den = E0 - H_ii in the emission's diagonal type.
 template <bool EPS>
 __device__ __forceinline__ void write_record(const EmitArgs &A, uint32_t pos, bool spill,
                                              uint32_t cell, uint32_t talpha, uint32_t tb,
-                                             bool packed, double v,
-                                             typename DenType<EPS>::T den, bool *kept) {
-  float df;
+                                             bool packed, double v, uint32_t den, bool *kept) {
+  const int32_t mag = abs((int32_t)den);  // |den| < 2^30
+  const float df = (float)max(mag - kDenSlack, 0) * A.scale32;
   if (EPS) {
     // Alg. 2's screen |v / (E0 - H_ii)| > eps, without a division.  A float
-    // test settles every pair that is not within 4e-6 relative of the
-    // threshold (|v| and |E0 - H_ii| truncated to floats lie within 2^-23
-    // below their values, eps_f within 2^-24 of eps, the product within
-    // 2^-24); the rest take the FP64 test, so every decision is the FP64
-    // test's.  (FP64 instructions are scarce on this GPU.)
-    df = scaled_as_float((int64_t)den, A.X.s);
+    // test settles every pair whose |v| is not within 4e-6 relative of eps
+    // times the bounds of |E0 - H_ii| (|v| truncated to a float lies within
+    // 2^-23 below its value, eps_f and the bounds within 2^-24 of theirs, the
+    // product within 2^-24); the rest take the FP64 test on the exact
+    // denominator, so every decision is that test's.  (FP64 instructions are
+    // scarce on this GPU.)
     bool okv;
     const float vf = abs_as_float(v, &okv);
-    const float t = A.eps_f * fabsf(df);
+    const float lo = A.eps_f * df, hi = A.eps_f * ((float)(mag + kDenSlack) * A.scale32);
     bool keep;
-    if (okv && t > 1e-37f && t < 1e37f && vf > t * 1.000004f) {
+    if (okv && hi > 1e-37f && hi < 1e37f && vf > hi * 1.000004f) {
       keep = true;
-    } else if (okv && t > 1e-37f && t < 1e37f && vf < t * 0.999996f) {
+    } else if (okv && lo > 1e-37f && lo < 1e37f && vf < lo * 0.999996f) {
       keep = false;
     } else {
-      const double d = __ll2double_rn((int64_t)den) * A.inv_scale;
+      const double d = __ll2double_rn(A.E0_x - fx_diag(A.X, talpha, tb)) * A.inv_scale;
       keep = fabs(v) > A.eps * fabs(d);
     }
     if (!keep) v = drop_marker();
     *kept = keep;
-  } else {
-    const int32_t a = abs((int32_t)den) - kDenSlack;  // |den| < 2^30
-    df = (float)(a > 0 ? a : 0) * A.scale32;
   }
   const uint64_t vb = (uint64_t)__double_as_longlong(v);
   const uint4 r = make_uint4((uint32_t)vb, (uint32_t)(vb >> 32), tb, __float_as_uint(df));
@@ -678,7 +665,7 @@ __device__ __forceinline__ void write_record(const EmitArgs &A, uint32_t pos, bo
       reinterpret_cast<uint4 *>(A.spill_rec)[pos] = r;
       A.spill_cell[pos] = cell;
     }
-  } else if (pos < A.st.cap) {
+  } else if (pos < A.st_cap) {
     reinterpret_cast<uint4 *>(A.st.rec)[pos] = r;
     if (packed) A.st.alpha[pos] = talpha;
   } else {
@@ -716,7 +703,7 @@ struct __align__(16) RunInfo {
   uint32_t cls0, cell0, nbk, jdx;     // bucket b's slots start at cls0 + b kCap
   uint32_t ebeg, eend, orb, flags;    // orb: i | a << 8 of the alpha single
   double c;
-  int64_t base;                       // E0 - H_jj, less the alpha single's change
+  uint32_t base, pad;                 // E0 - H_jj, less the alpha single's change
 };
 enum : uint32_t { kRunZero = 1u, kRunBig = 2u, kRunPacked = 4u, kRunFew = 8u, kRunOdd = 16u };
 constexpr uint32_t kFewBuckets = 32;
@@ -729,10 +716,14 @@ constexpr uint32_t kFewBuckets = 32;
 // ranks from a table, its orbitals and their diagonal terms from the
 // determinant's lists in shared memory (one 8-byte load each), and its sign
 // from the ranks: the occupied orbitals below the h-th occupied one are h, those
-// below the p-th virtual orbital x are x - p.
+// below the p-th virtual orbital x are x - p.  Two chunks are in flight, in turn
+// (a copy of one into the other costs 20 moves per pair), and a determinant's
+// beta string, coefficient and denominator arrive in one load: with the 32-bit
+// screen of write_record 3482 -> 3319 us for a (13e,19o) search with eps (64-bit
+// denominators spilled registers there), 181.9 -> 178.6 ms at (24e,30o).
 template <bool EPS, int PREC>
 __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
-  using D = typename DenType<EPS>::T;
+  using D = uint32_t;
   struct __align__(8) Orb {
     D z;          // diagonal term of removing or adding the orbital
     int32_t x;    // the orbital
@@ -743,10 +734,11 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
   __shared__ RunInfo s_run[kRunThreads / 32][kRunClaim];
   __shared__ Orb s_occ[kRunThreads / 32][32], s_vir[kRunThreads / 32][32];
   const int n = A.I.n;
+  // jk with the hole as the row (the lanes' particles are then on distinct banks)
   D *s_jk = reinterpret_cast<D *>(smem_raw), *s_jj = s_jk + n * n;
   for (int t = threadIdx.x; t < n * n; t += kRunThreads) {
-    s_jk[t] = static_cast<const D *>(A.jk)[t];
-    s_jj[t] = static_cast<const D *>(A.jj)[t];
+    s_jk[(t % n) * n + t / n] = A.jk[t];
+    s_jj[t] = A.jj[t];
   }
   for (int r = threadIdx.x; r < kPairTab; r += kRunThreads) {
     int x, y;
@@ -803,18 +795,19 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
         R.eend = R.ebeg;
         R.jdx = 0;
       }
-      R.B = A.core_beta[R.jdx];
-      R.c = A.core_c[R.jdx];
-      const D *Fa = static_cast<const D *>(A.Fa) + R.jdx;
-      D base = (sizeof(D) == 8 ? (D)A.E0_x : (D)A.E0_32) - static_cast<const D *>(A.Dx)[R.jdx];
+      const CoreRec cr = A.core[R.jdx];
+      R.B = cr.beta;
+      R.c = cr.c;
+      R.base = cr.den;
+      R.pad = 0;
       if (o != 0) {
         int i, a;
         const uint32_t odd = single_orbitals(R.Ak, R.talpha, &i, &a);
         R.orb = (uint32_t)i | ((uint32_t)a << 8);
         if (odd & 1u) R.flags |= kRunOdd;
-        base -= Fa[(size_t)a * A.ncore] - Fa[(size_t)i * A.ncore] - s_jk[a * n + i];
+        R.base -= A.Fa[(size_t)a * A.ncore + R.jdx] - A.Fa[(size_t)i * A.ncore + R.jdx] -
+                  s_jk[i * n + a];
       }
-      R.base = (int64_t)base;
       s_run[warp][lane] = R;
     }
 #pragma unroll 1
@@ -828,14 +821,14 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
       const uint32_t pa = (flags & kRunOdd) ? 1u : 0u;
       const double c = R.c;
       const float cf = (float)c;
-      const D base = (D)R.base;
+      const D Bz = R.base;
       const int ia = (int)(R.orb & 0xffu), aa = (int)(R.orb >> 8);
       // the determinant's occupied and virtual beta orbitals by rank, with the
       // Fock-like diagonal (and, for an alpha single, its Coulomb change)
       if (lane < n) {
         Orb q;
         q.x = lane;
-        q.z = static_cast<const D *>(A.Fb)[(size_t)R.jdx * n + lane];
+        q.z = A.Fb[(size_t)R.jdx * n + lane];
         if (!zero) q.z += s_jj[aa * n + lane] - s_jj[ia * n + lane];
         const uint32_t nb = (uint32_t)__popc(B & below(lane));
         if ((B >> lane) & 1u) occ[nb] = q;
@@ -859,7 +852,6 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
         erow = A.I.eri + ((size_t)ia * n + aa) * n * n;
         if (PREC != 0) erow32 = A.I.eri32 + ((size_t)ia * n + aa) * n * n;
       }
-      const D Bz = base;
       __syncwarp();
       // one chunk of 32 pairs: target, place, denominator and matrix element
       struct Chunk {
@@ -911,10 +903,10 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
           if (q.valid && e > 0) {
             const uint32_t sp = s_sp[e - 1], h = sp & 0xffu, p = sp >> 8;
             const Orb i = occ[h], a = vir[p];
-            q.tb = B ^ (1u << i.x) ^ (1u << a.x);
-            q.den = Bz - (a.z - i.z - s_jk[a.x * n + i.x]);
-            q.sign = (pa + h + (uint32_t)a.x - p + (a.x > i.x ? 1u : 0u)) & 1u;
             const int ix = i.x * n + a.x;
+            q.tb = B ^ (1u << i.x) ^ (1u << a.x);
+            q.den = Bz - (a.z - i.z - s_jk[ix]);
+            q.sign = (pa + h + (uint32_t)a.x - p + (a.x > i.x ? 1u : 0u)) & 1u;
             if (PREC != 0) q.gf = erow32[ix];
             else q.g = erow[ix];
           }
@@ -922,13 +914,15 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
         };
         // software-pipelined: the next chunk's slots (an atomic for big
         // classes) and integrals are requested before this chunk is written
-        Chunk cur, nxt;
-        decode(0, cur);
+        Chunk x, y;
+        decode(0, x);
 #pragma unroll 1
-        for (uint32_t e0 = 0; e0 < eend; e0 += 32) {
-          if (e0 + 32 < eend) decode(e0 + 32, nxt);  // warp-uniform
-          emit(cur, h0, e0 + lane == 0);
-          cur = nxt;
+        for (uint32_t e0 = 0; e0 < eend; e0 += 64) {  // warp-uniform
+          if (e0 + 32 < eend) decode(e0 + 32, y);
+          emit(x, h0, e0 + lane == 0);
+          if (e0 + 32 >= eend) break;
+          if (e0 + 64 < eend) decode(e0 + 64, x);
+          emit(y, h0, false);
         }
       } else {
         auto decode = [&](uint32_t e0, Chunk &q) {
@@ -946,9 +940,9 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
             const Orb i = occ[h1], j = occ[h2], a = vir[p1], b = vir[p2];
             const uint32_t pm = (1u << a.x) | (1u << b.x);
             q.tb = B ^ ((1u << i.x) | (1u << j.x)) ^ pm;
-            q.den = Bz - (a.z + b.z - i.z - j.z + s_jk[i.x * n + j.x] + s_jk[a.x * n + b.x] -
-                          s_jk[a.x * n + i.x] - s_jk[a.x * n + j.x] - s_jk[b.x * n + i.x] -
-                          s_jk[b.x * n + j.x]);
+            q.den = Bz - (a.z + b.z - i.z - j.z + s_jk[j.x * n + i.x] + s_jk[b.x * n + a.x] -
+                          s_jk[i.x * n + a.x] - s_jk[j.x * n + a.x] - s_jk[i.x * n + b.x] -
+                          s_jk[j.x * n + b.x]);
             const uint32_t between = below(j.x) & ~((2u << i.x) - 1u);
             q.sign = (h1 + h2 + (uint32_t)a.x - p1 + (uint32_t)b.x - p2 + 1u +
                       (uint32_t)__popc(pm & between)) & 1u;
@@ -959,7 +953,7 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
             const uint32_t sp = s_sp[e], h = sp & 0xffu, p = sp >> 8;
             const Orb i = occ[h], a = vir[p];
             q.tb = B ^ (1u << i.x) ^ (1u << a.x);
-            q.den = Bz - (a.z - i.z - s_jk[a.x * n + i.x]);
+            q.den = Bz - (a.z - i.z - s_jk[i.x * n + a.x]);
             q.sign = (h + (uint32_t)a.x - p + (a.x > i.x ? 1u : 0u)) & 1u;
             q.g = flip_sign(fx64_to_double(fx_single(A.X, B, R.Ak, i.x, a.x), A.X.s1), q.sign);
           }
@@ -985,7 +979,7 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
 // item, of 2.2 pairs at (24e,30o)).
 template <bool EPS, int PREC>
 __global__ void __launch_bounds__(kAdThreads) k_emit_ad(EmitArgs A) {
-  using D = typename DenType<EPS>::T;
+  using D = uint32_t;
   __shared__ uint32_t sF[kAdTile + 1];    // first flat pair of each item in the step
   __shared__ uint32_t sPos[kAdTile + 1];  // in-place staging slot of the item's first pair
   __shared__ uint32_t sG[kAdTile + 1];    // first core determinant of the item's group
@@ -1000,8 +994,7 @@ __global__ void __launch_bounds__(kAdThreads) k_emit_ad(EmitArgs A) {
   const int n = A.I.n;
   const uint32_t omask = (1u << A.opbits) - 1u;
   const int lane = threadIdx.x & 31;
-  const D *jk = static_cast<const D *>(A.jk), *Dx = static_cast<const D *>(A.Dx);
-  const D E0 = sizeof(D) == 8 ? (D)A.E0_x : (D)A.E0_32;
+  const D *jk = A.jk;
   unsigned long long my_kept = 0;  // pairs kept by the eps screen (EPS)
 #pragma unroll 1
   for (uint32_t step = blockIdx.x; step < A.ad_tiles; step += gridDim.x) {
@@ -1057,7 +1050,9 @@ __global__ void __launch_bounds__(kAdThreads) k_emit_ad(EmitArgs A) {
         atomicOr(A.err, kErrCore);
         jdx = 0;
       }
-      const uint32_t B = valid ? A.core_beta[jdx] : 0u;
+      CoreRec cr = {0u, 0u, 0.0};
+      if (valid) cr = A.core[jdx];
+      const uint32_t B = cr.beta;
       // lanes of one warp may straddle classes of both kinds: position per lane
       uint32_t pos = sPos[lo] + q, cell = 0;
       bool spill = false;
@@ -1077,13 +1072,12 @@ __global__ void __launch_bounds__(kAdThreads) k_emit_ad(EmitArgs A) {
       }
       bool kept = false;
       if (valid) {
-        const D *Fa = static_cast<const D *>(A.Fa) + jdx;  // orbital p at Fa[p * ncore]
+        const D *Fa = A.Fa + jdx;  // orbital p at Fa[p * ncore]
         const size_t m = A.ncore;
         const D dh = sD[lo] + Fa[((ob >> 5) & 31u) * m] + Fa[((ob >> 15) & 31u) * m] -
                      Fa[(ob & 31u) * m] - Fa[((ob >> 10) & 31u) * m];
-        const double c = A.core_c[jdx];
         write_record<EPS>(A, pos, spill, cell, sTA[lo], B, kd == kTilePacked,
-                          pair_value<PREC>(sH[lo], c, (float)c), E0 - Dx[jdx] - dh, &kept);
+                          pair_value<PREC>(sH[lo], cr.c, (float)cr.c), cr.den - dh, &kept);
       }
       if (EPS) my_kept += kept ? 1u : 0u;
     }
@@ -2175,38 +2169,25 @@ int build_fx(const double *h1, const double *eri, int n, int na, int nb, double 
   return ASCI_OK;
 }
 
-// H_jj, the Fock-like diagonals of the core and the pair tables in the type of
-// the emission's diagonal: 64 bits when the eps screen is on, else 32.
-int core_fock(const FxInts &X, const uint32_t *core_alpha, const uint32_t *core_beta, size_t m,
+// The core's records, its Fock-like diagonals and the pair tables in units of
+// the emission's denominator.
+int core_fock(const uint32_t *core_alpha, const uint32_t *core_beta, const double *core_c, size_t m,
               FusedCore *F, Arena &arena) {
-  const int n = X.n;
-  const dim3 grid(grid_for(m, 152 * 4), n + 1);
+  const int n = F->X.n;
   cudaStream_t s = arena.stream();
-  if (F->screened) {
-    int64_t *Dx, *Fa, *Fb;
-    ASCI_TRY(arena.alloc(&Dx, m));
-    ASCI_TRY(arena.alloc(&Fa, m * n));
-    ASCI_TRY(arena.alloc(&Fb, m * n));
-    k_core_fock<int64_t><<<grid, 256, 0, s>>>(X, core_alpha, core_beta, m, Dx, Fa, Fb);
-    ASCI_CHECK_LAUNCH();
-    F->Dx = Dx;
-    F->Fa = Fa;
-    F->Fb = Fb;
-    F->ejk = X.jk;
-    F->ejj = X.jj;
-    return ASCI_OK;
-  }
-  uint32_t *Dx, *Fa, *Fb, *jk, *jj;
-  ASCI_TRY(arena.alloc(&Dx, m));
+  CoreRec *rec;
+  uint32_t *Fa, *Fb, *jk, *jj;
+  ASCI_TRY(arena.alloc(&rec, m));
   ASCI_TRY(arena.alloc(&Fa, m * n));
   ASCI_TRY(arena.alloc(&Fb, m * n));
   ASCI_TRY(arena.alloc(&jk, (size_t)n * n));
   ASCI_TRY(arena.alloc(&jj, (size_t)n * n));
-  k_core_fock<uint32_t><<<grid, 256, 0, s>>>(X, core_alpha, core_beta, m, Dx, Fa, Fb);
+  k_core_fock<<<dim3(grid_for(m, 152 * 4), n + 1), 256, 0, s>>>(F->X, F->E0_x, core_alpha, core_beta,
+                                                               core_c, m, rec, Fa, Fb);
   ASCI_CHECK_LAUNCH();
-  k_den_tables<<<(n * n + 255) / 256, 256, 0, s>>>(X, jk, jj);
+  k_den_tables<<<(n * n + 255) / 256, 256, 0, s>>>(F->X, jk, jj);
   ASCI_CHECK_LAUNCH();
-  F->Dx = Dx;
+  F->core = rec;
   F->Fa = Fa;
   F->Fb = Fb;
   F->ejk = jk;
@@ -2452,9 +2433,7 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   A.grp_alpha = F.grp_alpha;
   A.grp_start = F.grp_start;
   A.grp_count = F.grp_count;
-  A.core_beta = F.core_beta;
-  A.core_c = F.core_c;
-  A.Dx = F.Dx;
+  A.core = static_cast<const CoreRec *>(F.core);
   A.Fa = F.Fa;
   A.Fb = F.Fb;
   A.jk = F.ejk;
@@ -2480,16 +2459,16 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   A.ad_tile_item = ad_tile_item;
   A.ad_tiles = ad_tiles;
   A.st = st;
+  A.st_cap = (uint32_t)std::min<uint64_t>(st.cap, 0xffffffffull);
   A.eps = eps;
   A.eps_f = (float)eps;
   A.E0_x = F.E0_x;
   A.inv_scale = ldexp(1.0, -F.X.s);
-  A.E0_32 = (int32_t)den_round<uint32_t>(F.E0_x);
   A.scale32 = (float)ldexp(1.0, kDenShift - F.X.s);
   A.survivors = survivors;
   A.ncore = F.ncore;
   A.err = err;
-  const size_t emit_smem = 2 * (size_t)F.X.n * F.X.n * (F.screened ? sizeof(int64_t) : sizeof(uint32_t));
+  const size_t emit_smem = 2 * (size_t)F.X.n * F.X.n * sizeof(uint32_t);
   unsigned long long *run_next;
   ASCI_TRY(arena.alloc(&run_next, 1));
   A.run_next = run_next;

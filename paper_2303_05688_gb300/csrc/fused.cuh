@@ -66,9 +66,9 @@ struct FusedCore {
   const uint64_t *items, *Wexcl;
   const uint32_t *item_group;
   int opbits;
-  const uint32_t *grp_alpha, *grp_start, *grp_count, *core_beta;
-  const double *core_c;
-  const void *Dx, *Fa, *Fb, *ejk, *ejj;  // the emission's diagonal tables (core_fock)
+  const uint32_t *grp_alpha, *grp_start, *grp_count;
+  const void *core;  // the core's records and diagonal tables of the emission (core_fock)
+  const uint32_t *Fa, *Fb, *ejk, *ejj;
   const uint32_t *g_alpha;
   const uint64_t *g_P0;
   int64_t E0_x;

@@ -43,7 +43,7 @@ int kept_count(const uint32_t *keep, const uint32_t *pos, size_t n, size_t *host
 int fx_bounds(const double *h1, const double *eri, int n, unsigned long long *out, cudaStream_t s);
 int build_fx(const double *h1, const double *eri, int n, int na, int nb, double ecore, double E0,
              const double h3[4], Arena &arena, FxInts *out, int64_t *E0_x);
-int core_fock(const FxInts &X, const uint32_t *core_alpha, const uint32_t *core_beta, size_t m,
+int core_fock(const uint32_t *core_alpha, const uint32_t *core_beta, const double *core_c, size_t m,
               FusedCore *F, Arena &arena);
 int item_groups(const uint64_t *items, const uint64_t *Wexcl, uint64_t T, uint32_t *item_group,
                 uint32_t **g_alpha, uint64_t **g_P0, uint64_t **g_item0, size_t *G, uint64_t *P,
@@ -819,8 +819,6 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   F.grp_alpha = grp_alpha;
   F.grp_start = grp_start;
   F.grp_count = grp_count;
-  F.core_beta = core_beta;
-  F.core_c = core_c_sorted;
   uint64_t *psi_ht = nullptr;
   uint64_t psi_mask = 0;
   // [0] candidates, [1] unique, [2] excluded, [3] survivors, [4] error bits: one copy reads them
@@ -839,7 +837,7 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   F.ctas_per_sm = o.ctas_per_sm;
   ASCI_TRY(build_fx(h1, eri, n, na, nb, ints->ecore, E0, hp.bounds, arena, &F.X, &F.E0_x));
   if (st) st->diag_grid_bits = (uint64_t)F.X.s;
-  ASCI_TRY(core_fock(F.X, core_alpha, core_beta, m, &F, arena));
+  ASCI_TRY(core_fock(core_alpha, core_beta, core_c_sorted, m, &F, arena));
   F.item_group = item_group;
   F.g_alpha = g_alpha;
   F.g_P0 = g_P0;
