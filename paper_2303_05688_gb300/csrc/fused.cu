@@ -501,11 +501,16 @@ __device__ __forceinline__ uint32_t bucket_of(uint32_t beta, uint32_t nb) {
 // fit a tile are staged in place and big classes go through bucket counters.
 
 constexpr int kRunThreads = 256;
-constexpr int kRunClaim = 4;   // runs a warp claims at a time
+constexpr int kRunClaim = 4;   // runs a warp claims at a time, at most
 // A determinant's o = 0 run (its beta singles and doubles, 10,314 pairs at
-// (24e,30o)) is emitted in pieces of at most this many pairs, so that the
-// last runs of a launch are short and its warps finish together.
-constexpr uint32_t kPiecePairs = 1024;
+// (24e,30o)) is emitted in pieces, so that the last runs of a launch are short
+// and its warps finish together: at most kPiecePairs pairs, fewer when the batch
+// would give each of the kEmitWarps warps that the GPU holds less than four.
+// (The small first batch of a search is nearly all o = 0 runs: 3.9 M pairs of
+// (16e,16o) in 261 us with pieces of 1024 pairs claimed four at a time, which left
+// half of the warps without work, and with the atomics waited for at once; 115 now.)
+constexpr uint32_t kPiecePairs = 1024, kMinPiece = 128;
+constexpr uint32_t kEmitWarps = 152 * 32;
 constexpr int kPairTab = 496;  // C(32, 2): unranked index pairs
 constexpr int kAdThreads = 256;
 constexpr int kAdTile = 512;   // alpha-double pairs per CTA step
@@ -516,7 +521,8 @@ struct EmitArgs {
   ExcCounts E;
   FastDiv dv_vb, dv_pb_p, dv_pieces;
   uint32_t npd0, npd1;        // pairs per determinant for o = 0 and for an alpha single
-  uint32_t npieces;           // pieces of kPiecePairs pairs a determinant's o = 0 run is cut into
+  uint32_t piece, run_claim;  // pairs of a piece; runs a warp claims at a time
+  uint32_t npieces;           // pieces of `piece` pairs a determinant's o = 0 run is cut into
   const uint64_t *items, *Wexcl;
   const uint32_t *item_group;
   uint64_t t0, P0;
@@ -673,18 +679,22 @@ __device__ __forceinline__ void write_record(const EmitArgs &A, uint32_t pos, bo
   }
 }
 
-// Next free slot of the lane's bucket cell (lanes with `big`): the slot number
-// within the cell.  Lanes of one cell share an atomic when the class has few
-// buckets; with many, two lanes seldom meet and each takes its own.
-__device__ __forceinline__ uint32_t claim_slot(uint32_t *fill, uint32_t cell, bool big, bool few) {
+// Next free slot of the lane's bucket cell (lanes with `big`), in two steps so
+// that the atomic's latency can pass while other pairs are worked on: claim_slot
+// issues the atomic, claimed_slot gives the slot number within the cell.  Lanes of
+// one cell share an atomic when the class has few buckets (peers: the lanes of
+// this lane's cell); with many, two lanes seldom meet and each takes its own.
+__device__ __forceinline__ uint32_t claim_slot(uint32_t *fill, uint32_t cell, bool big, bool few,
+                                               uint32_t *peers) {
   if (!few) return big ? atomicAdd(&fill[cell], 1u) : 0u;
-  const int lane = threadIdx.x & 31;
-  const uint32_t peers = __match_any_sync(0xffffffffu, big ? cell : 0xffffffffu);
-  const int leader = __ffs(peers) - 1;
-  uint32_t base = 0;
-  if (big && lane == leader) base = atomicAdd(&fill[cell], (uint32_t)__popc(peers));
-  base = __shfl_sync(0xffffffffu, base, leader);
-  return base + __popc(peers & ((1u << lane) - 1u));
+  *peers = __match_any_sync(0xffffffffu, big ? cell : 0xffffffffu);
+  if (!big || (int)(threadIdx.x & 31) != __ffs(*peers) - 1) return 0u;
+  return atomicAdd(&fill[cell], (uint32_t)__popc(*peers));
+}
+__device__ __forceinline__ uint32_t claimed_slot(uint32_t raw, bool few, uint32_t peers) {
+  if (!few) return raw;
+  return __shfl_sync(0xffffffffu, raw, __ffs(peers) - 1) +
+         __popc(peers & ((1u << (threadIdx.x & 31)) - 1u));
 }
 
 // The pairs an emission thread kept under the eps screen, added to the
@@ -759,12 +769,12 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
   // differ by a factor of about five); the next claim is issued before the
   // claimed runs are emitted
   unsigned long long claim = 0;
-  if (lane == 0) claim = atomicAdd(A.run_next, (unsigned long long)kRunClaim);
+  if (lane == 0) claim = atomicAdd(A.run_next, (unsigned long long)A.run_claim);
   uint64_t r0 = (uint64_t)__shfl_sync(0xffffffffu, claim, 0);
 #pragma unroll 1
   for (; r0 < A.nruns; r0 = (uint64_t)__shfl_sync(0xffffffffu, claim, 0)) {
-    if (lane == 0) claim = atomicAdd(A.run_next, (unsigned long long)kRunClaim);
-    const int nr = (int)(A.nruns - r0 < (uint64_t)kRunClaim ? A.nruns - r0 : (uint64_t)kRunClaim);
+    if (lane == 0) claim = atomicAdd(A.run_next, (unsigned long long)A.run_claim);
+    const int nr = (int)(A.nruns - r0 < (uint64_t)A.run_claim ? A.nruns - r0 : (uint64_t)A.run_claim);
     __syncwarp();  // the previous claim's runs have been read
     if (lane < nr) {
       const uint64_t run = A.runs[r0 + lane];
@@ -780,8 +790,8 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
       R.jdx = A.grp_start[k] + m;
       R.flags = (o == 0 ? kRunZero : 0u) | (kd == kTileBucket ? kRunBig : 0u) |
                 (kd == kTilePacked ? kRunPacked : 0u);
-      R.ebeg = o == 0 ? (mr - m * A.npieces) * kPiecePairs : 0u;
-      R.eend = npd < R.ebeg + kPiecePairs ? npd : R.ebeg + kPiecePairs;
+      R.ebeg = o == 0 ? (mr - m * A.npieces) * A.piece : 0u;
+      R.eend = o == 0 && R.ebeg + A.piece < npd ? R.ebeg + A.piece : npd;
       R.cls0 = (uint32_t)A.soff[gi];
       R.off0 = (uint32_t)(A.soff[gi] + (A.Wexcl[t] + (uint64_t)m * npd - A.g_P0[A.gb0 + gi]));
       R.cell0 = kd == kTileBucket ? A.cellbase[gi] : 0u;
@@ -855,25 +865,16 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
       __syncwarp();
       // one chunk of 32 pairs: target, place, denominator and matrix element
       struct Chunk {
-        uint32_t tb, pos, sign;
+        uint32_t tb, pos, sign, peers;
         D den;
-        bool valid, spill;
+        bool valid;
         double g;   // the gathered integral, requested a chunk ahead
         float gf;   // the same from the FP32 tables
       };
       auto place = [&](Chunk &q, uint32_t e) {
-        q.spill = false;
-        if (big) {  // warp-uniform: the next free slot of the lane's bucket cell
-          const uint32_t bkt = bucket_of(q.tb, nbk);
-          const uint32_t slot = claim_slot(A.fill, cell0 + bkt, q.valid, few);
-          q.pos = cls0 + bkt * (uint32_t)kCap + slot;
-          if (q.valid && slot >= (uint32_t)kCap) {  // the cell is full: the spill list
-            q.spill = true;
-            q.pos = atomicAdd(A.n_spill, 1u);
-          }
-        } else {
-          q.pos = off0 + e;
-        }
+        // big: the next free slot of the lane's bucket cell (warp-uniform)
+        q.pos = big ? claim_slot(A.fill, cell0 + bucket_of(q.tb, nbk), q.valid, few, &q.peers)
+                    : off0 + e;
       };
       auto emit = [&](const Chunk &q, double h, bool is_double) {
         // is_double: h holds the value; else the gathered integral is it
@@ -885,10 +886,18 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
           const double hh = is_double ? h : flip_sign(PREC == 1 ? widen(q.gf) : q.g, q.sign);
           v = hh * c;
         }
-        bool kept = false;
-        if (q.valid)
-          write_record<EPS>(A, q.pos, q.spill, cell0 + (big ? bucket_of(q.tb, nbk) : 0u), talpha, q.tb,
-                            packed, v, q.den, &kept);
+        uint32_t pos = q.pos, cell = cell0;
+        bool spill = false, kept = false;
+        if (big) {  // warp-uniform
+          const uint32_t slot = claimed_slot(q.pos, few, q.peers), bkt = bucket_of(q.tb, nbk);
+          cell += bkt;
+          pos = cls0 + bkt * (uint32_t)kCap + slot;
+          if (q.valid && slot >= (uint32_t)kCap) {  // the cell is full: the spill list
+            spill = true;
+            pos = atomicAdd(A.n_spill, 1u);
+          }
+        }
+        if (q.valid) write_record<EPS>(A, pos, spill, cell, talpha, q.tb, packed, v, q.den, &kept);
         if (EPS) my_kept += kept ? 1u : 0u;
       };
       if (!zero) {
@@ -959,13 +968,15 @@ __global__ void __launch_bounds__(kRunThreads, 4) k_emit_runs(EmitArgs A) {
           }
           place(q, e);
         };
-        Chunk cur, nxt;
-        decode(ebeg, cur);
+        Chunk x, y;
+        decode(ebeg, x);
 #pragma unroll 1
-        for (uint32_t e0 = ebeg; e0 < eend; e0 += 32) {
-          if (e0 + 32 < eend) decode(e0 + 32, nxt);
-          emit(cur, cur.g, e0 + lane < sb);
-          cur = nxt;
+        for (uint32_t e0 = ebeg; e0 < eend; e0 += 64) {
+          if (e0 + 32 < eend) decode(e0 + 32, y);
+          emit(x, x.g, e0 + lane < sb);
+          if (e0 + 32 >= eend) break;
+          if (e0 + 64 < eend) decode(e0 + 64, x);
+          emit(y, y.g, e0 + 32 + lane < sb);
         }
       }
     }
@@ -1060,7 +1071,9 @@ __global__ void __launch_bounds__(kAdThreads) k_emit_ad(EmitArgs A) {
         const uint32_t bkt = bigl ? bucket_of(B, sNb[lo]) : 0u;
         cell = sCell[lo] + bkt;
         const bool few = __any_sync(0xffffffffu, bigl && sNb[lo] < kFewBuckets);
-        const uint32_t slot = claim_slot(A.fill, cell, bigl, few);
+        uint32_t peers = 0;
+        const uint32_t raw = claim_slot(A.fill, cell, bigl, few, &peers);
+        const uint32_t slot = claimed_slot(raw, few, peers);
         if (bigl) {
           if (slot < (uint32_t)kCap) {
             pos = sBase[lo] + bkt * (uint32_t)kCap + slot;
@@ -2316,8 +2329,10 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   ASCI_TRY(arena.alloc(&adpos, nt));
   ASCI_TRY(arena.alloc(&adw, nt));
   ASCI_TRY(arena.alloc(&adsum, nt));
+  const uint32_t piece = (uint32_t)std::min<uint64_t>(
+      kPiecePairs, std::max<uint64_t>(kMinPiece, (P1 - P0) / (4ull * kEmitWarps) / 32 * 32));
   const uint32_t npieces =
-      (uint32_t)std::max<uint64_t>(1, ((uint64_t)F.E.sb + F.E.dbb + kPiecePairs - 1) / kPiecePairs);
+      (uint32_t)std::max<uint64_t>(1, ((uint64_t)F.E.sb + F.E.dbb + piece - 1) / piece);
   k_batch_counts<<<grid_for(nt), 256, 0, s>>>(F.items, t0, nt, F.opbits, F.E.sa, npieces,
                                               F.grp_count, rcnt, adf, adw);
   ASCI_CHECK_LAUNCH();
@@ -2424,6 +2439,8 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   A.npd0 = (uint32_t)(F.E.sb + F.E.dbb);
   A.npd1 = 1u + F.E.sb;
   A.npieces = npieces;
+  A.piece = piece;
+  A.run_claim = (uint32_t)std::min<uint64_t>(kRunClaim, std::max<uint64_t>(1, nruns / kEmitWarps));
   A.items = F.items;
   A.Wexcl = F.Wexcl;
   A.item_group = F.item_group;
