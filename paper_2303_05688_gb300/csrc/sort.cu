@@ -1,9 +1,9 @@
 // Device-wide primitives: exclusive scan and a stable LSD radix sort.
 //
 // The sort is the "sort" of the paper's sort-and-accumulate (Sec. 2.2); it is
-// written for this library: 8-bit digits, one histogram (upsweep) kernel, a
-// device-wide scan of the digit-major histogram, and a scatter (downsweep)
-// kernel that ranks each tile's keys stably with warp ballots.
+// written for this library: 8-bit digits, one kernel that counts every digit of
+// the keys, and one kernel per digit that ranks each tile's keys stably, learns
+// from the tiles before it where its runs begin, and moves the keys.
 #include "asci_internal.cuh"
 
 namespace asci {
@@ -169,54 +169,109 @@ constexpr int kSortItems = 16;  // per thread
 constexpr int kSortTile = kSortThreads * kSortItems;
 constexpr int kRadix = 256;
 
-__global__ void k_digit_hist(const uint64_t *keys, size_t n, int shift, uint32_t *hist,
-                             uint32_t ntiles) {
-  __shared__ uint32_t h[kRadix];
-  h[threadIdx.x] = 0;
+// The digits of a sort that vary, lowest first (at most eight).
+struct DigitShifts {
+  int count;
+  int shift[8];
+};
+
+// Counts of every digit in one pass over the keys (hist[digit][value]).
+__global__ void __launch_bounds__(512) k_digit_counts(const uint64_t *keys, size_t n,
+                                                      DigitShifts D, uint32_t *hist) {
+  extern __shared__ uint32_t h[];
+  for (int i = threadIdx.x; i < D.count * kRadix; i += blockDim.x) h[i] = 0;
   __syncthreads();
-  size_t base = (size_t)blockIdx.x * kSortTile;
-#pragma unroll 4
-  for (int i = 0; i < kSortItems; ++i) {
-    size_t idx = base + (size_t)i * kSortThreads + threadIdx.x;
-    if (idx < n) atomicAdd(&h[(keys[idx] >> shift) & 0xffu], 1u);
+  const size_t step = (size_t)gridDim.x * blockDim.x * 4;
+  for (size_t base = (size_t)blockIdx.x * blockDim.x * 4; base < n; base += step) {
+    uint64_t k[4] = {0, 0, 0, 0};
+    uint32_t ok = 0;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const size_t i = base + (size_t)r * blockDim.x + threadIdx.x;
+      if (i < n) {
+        k[r] = keys[i];
+        ok |= 1u << r;
+      }
+    }
+    for (int d = 0; d < D.count; ++d) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const uint32_t v = (uint32_t)(k[r] >> D.shift[d]) & 0xffu;
+        // kept together from one addition to the next: 57.7 M keys of four digits take
+        // 154 us, without this 445 (557 without the branch)
+        __syncwarp();
+        if ((ok >> r) & 1u) atomicAdd(&h[d * kRadix + v], 1u);
+      }
+    }
   }
   __syncthreads();
-  hist[(size_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
+  for (int i = threadIdx.x; i < D.count * kRadix; i += blockDim.x)
+    if (h[i]) atomicAdd(&hist[i], h[i]);
 }
 
+// A word of the tiles' digit counts: the value (a count or a prefix, both at most
+// n < 2^32) below a tag, 4 x (number of the pass) + state.  The words of one pass
+// are distinct from those of the passes before, so they are cleared once a sort.
+constexpr uint32_t kTileCount = 1u;   // the tile's own count of the digit
+constexpr uint32_t kTilePrefix = 2u;  // the count in this tile and all before it
+__device__ __forceinline__ uint64_t ld_relaxed(const uint64_t *p) {
+  uint64_t v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed(uint64_t *p, uint64_t v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+constexpr int kLook = 8;               // predecessors read at a time
+constexpr uint32_t kLookLimit = 1u << 18;  // polls before a tile counts for itself
+
 // Shared memory of the scatter: the tile's keys (and values) in digit order,
-// per-warp digit counters, and each digit's tile start and global offset.
+// per-warp digit counters, and each digit's offset from the tile to the output.
 template <typename V, bool kHasVals>
 constexpr size_t scatter_smem() {
   return (size_t)kSortTile * sizeof(uint64_t) + (kHasVals ? (size_t)kSortTile * sizeof(V) : 0) +
-         (size_t)(kSortWarps + 2) * kRadix * sizeof(uint32_t);
+         (size_t)(kSortWarps + 1) * kRadix * sizeof(uint32_t);
 }
 
-// Stable scatter of one tile.  Warp w owns elements [w*32*kSortItems, ...) of
-// the tile in rounds of 32 consecutive elements, so tile order is preserved.
-// The tile is first placed in shared memory in digit order; each digit's run
-// is then written to its global position with consecutive threads on
-// consecutive addresses.
+// Stable scatter by one digit, a tile per CTA.  Warp w owns elements
+// [w*32*kSortItems, ...) of the tile in rounds of 32 consecutive elements, so tile
+// order is preserved.  Tiles are numbered in the order in which CTAs start, so a
+// tile's predecessors are running or done; each publishes its digit counts before
+// it looks at theirs, so the wait below always ends.  Thread d adds up digit d of
+// the tiles before, kLook at a time, back to the nearest one that knows its prefix.
+// (Should a predecessor not answer within kLookLimit polls, the CTA counts the
+// keys before its tile itself.)  The tile is then placed in shared memory in digit
+// order and each digit's run is written with consecutive threads on consecutive
+// addresses.
+//
+// Bound: shared-memory wavefronts (78% of their rate) before memory: 16 bytes a
+// key and digit, at 2.8 TB/s.  Against a histogram kernel, its scan and a scatter
+// that ranked twice, a digit of 57.7 M keys 620 -> 330 us with its share of the
+// counts, of 1e5 keys 30 (five launches) -> 9.
 template <typename V, bool kHasVals>
 __global__ void __launch_bounds__(kSortThreads, 4)
     k_digit_scatter(const uint64_t *keys_in, const V *vals_in, uint64_t *keys_out, V *vals_out,
-                    size_t n, int shift, const uint32_t *offsets, uint32_t ntiles) {
+                    size_t n, int shift, uint32_t pass, const uint32_t *hist, uint64_t *words,
+                    uint32_t *ticket) {
   extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ uint32_t s_tile;
   uint64_t *sk = reinterpret_cast<uint64_t *>(sm);
   V *sv = reinterpret_cast<V *>(sk + kSortTile);
   uint32_t *wb = reinterpret_cast<uint32_t *>(sm + (size_t)kSortTile * sizeof(uint64_t) +
                                               (kHasVals ? (size_t)kSortTile * sizeof(V) : 0));
-  uint32_t *dstart = wb + kSortWarps * kRadix;  // digit start within the tile
-  uint32_t *dglob = dstart + kRadix;            // digit start in the output
+  uint32_t *dmove = wb + kSortWarps * kRadix;  // from a key's place in the tile to the output
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
   for (int i = threadIdx.x; i < kSortWarps * kRadix; i += kSortThreads) wb[i] = 0;
   __syncthreads();
-  const size_t base = (size_t)blockIdx.x * kSortTile;
+  const uint32_t tile = s_tile;
+  const size_t base = (size_t)tile * kSortTile;
   const size_t wbase = base + (size_t)warp * 32 * kSortItems;
-  // the tile's keys stay in registers (four CTAs of 256 threads per SM); a
-  // key's digit is recomputed where it is needed, out-of-range slots get the
-  // digit kRadix, which no counter holds
+  const uint32_t lt = (1u << lane) - 1u;
+  // the tile's keys and their ranks among the warp's keys of the same digit stay in
+  // registers; out-of-range slots get the digit kRadix, which no counter holds
   uint64_t k[kSortItems];
+  uint32_t rank2[kSortItems / 2];  // two 16-bit ranks a word
 #pragma unroll
   for (int r = 0; r < kSortItems; ++r) {
     const size_t idx = wbase + (size_t)r * 32 + lane;
@@ -227,36 +282,79 @@ __global__ void __launch_bounds__(kSortThreads, 4)
     const bool ok = wbase + (size_t)r * 32 + lane < n;
     const uint32_t d = ok ? (uint32_t)((k[r] >> shift) & 0xffu) : (uint32_t)kRadix;
     const uint32_t peers = __match_any_sync(0xffffffffu, d);
-    if (ok && lane == __ffs(peers) - 1) wb[warp * kRadix + d] += __popc(peers);
+    uint32_t before = 0;
+    if (ok) before = wb[warp * kRadix + d];
+    __syncwarp();
+    if (ok && lane == __ffs(peers) - 1) wb[warp * kRadix + d] = before + __popc(peers);
+    __syncwarp();
+    const uint32_t rk = before + __popc(peers & lt);
+    rank2[r >> 1] = (r & 1) ? rank2[r >> 1] | (rk << 16) : rk;
   }
   __syncthreads();
   {
-    // per digit: offsets of the warps within the digit's run, the run's start
-    // in the tile (scan over digits) and in the output
     const int dig = threadIdx.x;  // kSortThreads == kRadix
-    uint32_t cnt = 0;
+    uint32_t cnt = 0, first[kSortWarps];  // the warps' keys within the digit's run
+#pragma unroll
     for (int w = 0; w < kSortWarps; ++w) {
-      const uint32_t c = wb[w * kRadix + dig];
-      wb[w * kRadix + dig] = cnt;
-      cnt += c;
+      first[w] = cnt;
+      cnt += wb[w * kRadix + dig];
     }
-    dstart[dig] = block_exclusive_scan<uint32_t>(cnt, nullptr);
-    dglob[dig] = offsets[(size_t)dig * ntiles + blockIdx.x];
+    uint64_t *mine = words + (size_t)tile * kRadix + dig;
+    const uint64_t tag = (uint64_t)(4u * pass) << 32;
+    st_relaxed(mine, tag | ((uint64_t)(tile ? kTileCount : kTilePrefix) << 32) | cnt);
+    // starts of the digit in the tile and in the output: both sums stay below 2^32
+    const uint64_t st = block_exclusive_scan<uint64_t>(((uint64_t)cnt << 32) | hist[dig], nullptr);
+    const uint32_t dstart = (uint32_t)(st >> 32);
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) wb[w * kRadix + dig] = dstart + first[w];
+    uint32_t before = 0;  // the digit's keys in the tiles before
+    bool lost = false;
+    if (tile) {
+      uint32_t t = tile, polls = 0;  // tiles [t, tile) are in `before`
+      bool done = false;
+      while (!done) {
+        uint64_t w[kLook];
+#pragma unroll
+        for (int j = 0; j < kLook; ++j) {
+          const uint32_t b = (uint32_t)j + 1u <= t ? t - 1u - (uint32_t)j : 0u;
+          w[j] = ld_relaxed(words + (size_t)b * kRadix + dig);
+        }
+        bool open = true;
+#pragma unroll
+        for (int j = 0; j < kLook; ++j) {
+          const uint32_t hi = (uint32_t)(w[j] >> 32);
+          open = open && !done && hi >= 4u * pass + kTileCount;
+          if (open) {
+            before += (uint32_t)w[j];
+            --t;
+            done = hi == 4u * pass + kTilePrefix;
+          }
+        }
+        if (!done && ++polls > kLookLimit + tile) {
+          lost = true;
+          break;
+        }
+      }
+    }
+    if (__syncthreads_or(lost)) {
+      dmove[dig] = 0;
+      __syncthreads();
+      for (size_t i = threadIdx.x; i < base; i += kSortThreads)
+        atomicAdd(&dmove[(keys_in[i] >> shift) & 0xffu], 1u);
+      __syncthreads();
+      before = dmove[dig];
+      __syncthreads();
+    }
+    if (tile) st_relaxed(mine, tag | ((uint64_t)kTilePrefix << 32) | (before + cnt));
+    dmove[dig] = (uint32_t)st + before - dstart;
   }
   __syncthreads();
-  const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll
   for (int r = 0; r < kSortItems; ++r) {
     const size_t idx = wbase + (size_t)r * 32 + lane;
-    const bool ok = idx < n;
-    const uint32_t d = ok ? (uint32_t)((k[r] >> shift) & 0xffu) : (uint32_t)kRadix;
-    const uint32_t peers = __match_any_sync(0xffffffffu, d);
-    uint32_t pos = 0;
-    if (ok) pos = dstart[d] + wb[warp * kRadix + d] + __popc(peers & lt);
-    __syncwarp();
-    if (ok && lane == __ffs(peers) - 1) wb[warp * kRadix + d] += __popc(peers);
-    __syncwarp();
-    if (ok) {
+    if (idx < n) {
+      const uint32_t d = (uint32_t)((k[r] >> shift) & 0xffu);
+      const uint32_t pos = wb[warp * kRadix + d] + ((rank2[r >> 1] >> (16 * (r & 1))) & 0xffffu);
       sk[pos] = k[r];
       if (kHasVals) sv[pos] = vals_in[idx];
     }
@@ -266,7 +364,7 @@ __global__ void __launch_bounds__(kSortThreads, 4)
   for (uint32_t i = threadIdx.x; i < tn; i += kSortThreads) {
     const uint64_t key = sk[i];
     const uint32_t dg = (uint32_t)((key >> shift) & 0xffu);
-    const uint32_t gpos = dglob[dg] + (i - dstart[dg]);
+    const uint32_t gpos = dmove[dg] + i;
     keys_out[gpos] = key;
     if (kHasVals) vals_out[gpos] = sv[i];
   }
@@ -390,9 +488,7 @@ int radix_sort_impl(uint64_t **keys, uint64_t **keys_alt, V **vals, V **vals_alt
     ASCI_CHECK_LAUNCH();
     return ASCI_OK;
   }
-  uint32_t ntiles = (uint32_t)((n + kSortTile - 1) / kSortTile);
-  uint32_t *hist = nullptr;
-  ASCI_TRY(arena.alloc(&hist, (size_t)kRadix * ntiles));
+  const uint32_t ntiles = (uint32_t)((n + kSortTile - 1) / kSortTile);
   // once per instantiation (thread-safe static initialisation)
   static const cudaError_t attr = cudaFuncSetAttribute(
       k_digit_scatter<V, kHasVals>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -401,16 +497,28 @@ int radix_sort_impl(uint64_t **keys, uint64_t **keys_alt, V **vals, V **vals_alt
   uint64_t mask = 0;
   if (known_mask) mask = *known_mask;  // the caller knows which bits vary
   else ASCI_TRY(varying_bits_u64(*keys, n, &mask, arena));
+  DigitShifts D;
+  D.count = 0;
   for (int shift = begin_bit; shift < end_bit; shift += 8) {
     uint64_t dmask = (0xffull << shift);
     if (end_bit - shift < 8) dmask &= ((end_bit >= 64) ? ~0ull : ((1ull << end_bit) - 1));
-    if ((mask & dmask) == 0) continue;  // digit constant over the input
-    k_digit_hist<<<ntiles, kSortThreads, 0, s>>>(*keys, n, shift, hist, ntiles);
-    ASCI_CHECK_LAUNCH();
-    ASCI_TRY(scan_exclusive<uint32_t>(hist, hist, (size_t)kRadix * ntiles, arena));
+    if (mask & dmask) D.shift[D.count++] = shift;  // else constant over the input
+  }
+  if (D.count == 0) return ASCI_OK;
+  // the tiles' words, then the counts and the tickets of the passes
+  uint64_t *words;
+  const size_t nwords = (size_t)kRadix * ntiles, extra = (size_t)D.count * (kRadix + 1);
+  ASCI_TRY(arena.alloc(&words, nwords + (extra + 1) / 2));
+  ASCI_TRY_CUDA(cudaMemsetAsync(words, 0, (nwords + (extra + 1) / 2) * sizeof(uint64_t), s));
+  uint32_t *hist = reinterpret_cast<uint32_t *>(words + nwords);
+  uint32_t *ticket = hist + (size_t)D.count * kRadix;
+  k_digit_counts<<<(unsigned)std::min<size_t>(152 * 4, (n + 2047) / 2048), 512,
+                   (size_t)D.count * kRadix * sizeof(uint32_t), s>>>(*keys, n, D, hist);
+  ASCI_CHECK_LAUNCH();
+  for (int p = 0; p < D.count; ++p) {
     k_digit_scatter<V, kHasVals><<<ntiles, kSortThreads, scatter_smem<V, kHasVals>(), s>>>(
-        *keys, kHasVals ? *vals : nullptr, *keys_alt, kHasVals ? *vals_alt : nullptr, n, shift,
-        hist, ntiles);
+        *keys, kHasVals ? *vals : nullptr, *keys_alt, kHasVals ? *vals_alt : nullptr, n,
+        D.shift[p], (uint32_t)(p + 1), hist + (size_t)p * kRadix, words, ticket + p);
     ASCI_CHECK_LAUNCH();
     uint64_t *t = *keys;
     *keys = *keys_alt;
