@@ -4,10 +4,10 @@
 //  * H over a determinant list (Sec. 2.3, CSR): the paper's double loop over
 //    determinant pairs, pruned by the structure of the keys.  In key order
 //    (beta word high) each beta string's determinants are one group; a row
-//    visits only the groups whose beta string is within two excitations (a
-//    group graph built by a tiled double loop over the beta strings), tests
-//    the alpha distance against 4 - popc(beta_i ^ beta_j), and for groups a
-//    beta double away looks its own alpha string up by binary search.
+//    visits the groups whose beta string is within one excitation (a group
+//    graph built by a tiled double loop over the beta strings), where it tests
+//    the alpha distance against 4 - popc(beta_i ^ beta_j), and, merged with
+//    them, the determinants of its own alpha string a beta double away.
 //    Connected pairs get H_ij by the Slater-Condon rules, evaluated 32 at a
 //    time from a per-warp queue; nonzero elements are stored, each row's
 //    columns ascending.  A counting pass and a scan give the row pointers, the
@@ -126,12 +126,11 @@ __device__ double offdiag_element(const DevInts &I, uint32_t ai, uint32_t bi, ui
 // every beta string's determinants form one contiguous group.  Two
 // determinants are within two excitations iff
 //   popc(alpha_i ^ alpha_j) + popc(beta_i ^ beta_j) <= 4,
-// so a row only has to visit the groups whose beta string is within two
-// excitations of its own (the group graph, built once per list by a tiled
-// double loop over the G group strings), and inside such a group only the
-// alpha test remains, with the threshold 4 - popc(beta_i ^ beta_j) (for beta
-// strings a double apart, alpha_j must equal alpha_i: a binary search in the
-// alpha-sorted group).  A warp takes a row and walks its neighbour groups in
+// so a row has to visit the groups whose beta string is equal or a single
+// excitation away (the group graph, built once per list by a tiled double loop
+// over the G group strings), where only the alpha test remains, and the
+// determinants of its own alpha string whose beta string is a double away (from
+// the list in alpha order).  A warp takes a row and walks both, merged in
 // ascending order, 32 columns at a time; a ballot places the hits, so each
 // row's columns come out ascending.  A counting pass gives the row lengths, a scan the row
 // pointers, and the filling pass writes (never past a row's counted end).
@@ -158,7 +157,7 @@ __global__ void k_beta_groups(const uint64_t *keys, uint32_t n, const uint32_t *
 }
 
 // Group graph: count (kFill false) or list (kFill true) the groups g2 with
-// popc(beta_g1 ^ beta_g2) <= 4, for the groups g1 = [blockIdx.x * 256, +256)
+// popc(beta_g1 ^ beta_g2) <= 2, for the groups g1 = [blockIdx.x * 256, +256)
 // (one per thread) against the groups [blockIdx.y * chunk, +chunk) staged in
 // shared memory.
 template <bool kFill>
@@ -185,7 +184,7 @@ __global__ void __launch_bounds__(kRowThreads) k_beta_pairs(const uint32_t *gbet
     if (!live) continue;
 #pragma unroll 4
     for (uint32_t t = 0; t < m; ++t) {
-      if (__popc(b1 ^ sb[t]) > 4) continue;
+      if (__popc(b1 ^ sb[t]) > 2) continue;
       if (kFill) {
         if (pos < end) nbr[pos] = s + t;
         ++pos;
@@ -197,12 +196,50 @@ __global__ void __launch_bounds__(kRowThreads) k_beta_pairs(const uint32_t *gbet
   if (!kFill && live) cnt_off[slot] = cnt;
 }
 
+// Rows in alpha order: akey = alpha << 32 | row, to be sorted by alpha (stably,
+// so rows of one alpha string stay in ascending order).
+__global__ void k_alpha_keys(const uint64_t *keys, uint32_t n, uint64_t *akey) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    akey[i] = ((uint64_t)key_alpha(keys[i]) << 32) | i;
+}
+// mates[t] = (row, its beta string) in alpha order; span[row] = the row's
+// [first, end) there, the rows of its own alpha string.
+__global__ void k_alpha_mates(const uint64_t *keys, const uint64_t *akey, uint32_t n, uint2 *mates,
+                              uint2 *span) {
+  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+    const uint32_t r = (uint32_t)akey[t], a = (uint32_t)(akey[t] >> 32);
+    mates[t] = make_uint2(r, key_beta(keys[r]));
+    uint32_t lo = 0, hi = t;  // first position of alpha a
+    while (lo < hi) {
+      const uint32_t mid = lo + ((hi - lo) >> 1);
+      if ((uint32_t)(akey[mid] >> 32) < a) lo = mid + 1;
+      else hi = mid;
+    }
+    uint32_t lo2 = t, hi2 = n;  // first position past alpha a
+    while (lo2 < hi2) {
+      const uint32_t mid = lo2 + ((hi2 - lo2) >> 1);
+      if ((uint32_t)(akey[mid] >> 32) <= a) lo2 = mid + 1;
+      else hi2 = mid;
+    }
+    span[r] = make_uint2(lo, lo2);
+  }
+}
+
 // Row lengths (kFill false: rp[r] = count) or elements (kFill true: rp holds
 // the row pointers) of rows r = warp, warp + warps, ...  The diagonal is
 // always stored; off-diagonal elements when nonzero.  The columns that pass
 // the excitation test are queued in shared memory (in column order) and
 // evaluated 32 at a time, one per lane, so that the Slater-Condon work runs
 // on full warps rather than on the one or two lanes that hit in a step.
+//
+// Bound: latency of the gathers (integrals, columns' keys).  Looking the row's own
+// alpha string up in every group a beta double away (some 700 binary searches a
+// row at 16 orbitals) took 1.75 ms a counting pass over 1e5 random-walk
+// determinants; its mates, merged, take 1.34 (build 6.5 -> 5.2 ms).  Products of
+// whole string sets gain nothing, their rows having more mates than doubles: 320 x
+// 320 neighbouring strings 21.1 ms before and now, 300 x 300 random ones 2.2 and
+// 2.3, 8 x 12870 16.7 and 18.5 (20.4 with 48 registers instead of 32: the gathers
+// want warps).
 constexpr int kRowWarps = 8;
 
 template <bool kFill>
@@ -241,12 +278,17 @@ __device__ __forceinline__ void flush_queue(const DevInts &I, const uint64_t *ke
 }
 
 template <bool kFill>
-__global__ void __launch_bounds__(kRowWarps * 32) k_ham_rows(
+__global__ void __launch_bounds__(kRowWarps * 32, 8) k_ham_rows(
     DevInts I, const uint64_t *__restrict__ keys, uint32_t n, const uint32_t *__restrict__ of_row,
     const uint32_t *__restrict__ gstart, const uint32_t *__restrict__ gbeta,
     const int64_t *__restrict__ nbr_ptr, const uint32_t *__restrict__ nbr,
+    const uint2 *__restrict__ mates, const uint2 *__restrict__ span,
     const double *__restrict__ diag, int64_t *rp, int32_t *col, double *val) {
   __shared__ uint32_t queue[kRowWarps][64];
+  __shared__ uint2 place[kRowWarps][32];
+  __shared__ uint32_t found[kRowWarps][64];
+  uint2 *pl = place[threadIdx.x >> 5];
+  uint32_t *yq = found[threadIdx.x >> 5];
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t below = (1u << lane) - 1u;
   uint32_t *q = queue[threadIdx.x >> 5];
@@ -261,33 +303,77 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_ham_rows(
       end = rp[r + 1];
     }
     int qn = 0;  // queued columns (warp-uniform, < 64)
-    // 32 neighbour groups at a time: lane k holds group k's first column,
-    // length and alpha threshold; their columns are walked as one
-    // concatenated range, 32 columns per step, each lane finding its group
-    // by a binary search over the lanes' offsets
-    const int64_t e1 = nbr_ptr[g + 1];
-    for (int64_t e0 = nbr_ptr[g]; e0 < e1; e0 += 32) {
+    // two ascending lists, merged 32 entries at a time: the neighbour groups (x,
+    // first column and length) and the row's alpha mates a beta double away (y,
+    // one column each); lane k then holds entry k's first column, length and
+    // alpha threshold, and the columns are walked as one concatenated range, 32
+    // per step, each lane finding its entry by a binary search over the lanes'
+    // offsets
+    int64_t x0 = nbr_ptr[g];
+    const int64_t x1 = nbr_ptr[g + 1];
+    const uint2 ys = span[r];
+    constexpr uint32_t kNone = 0xffffffffu;  // n < 2^31
+    uint32_t y0 = ys.x;
+    int yn = 0;  // mates in hand (warp-uniform, < 64)
+    while (true) {
+      for (; yn < 32 && y0 < ys.y; y0 += 32) {
+        uint2 m = make_uint2(0u, bi);
+        if (ys.y - y0 > lane) m = mates[y0 + lane];
+        const bool hit = __popc(bi ^ m.y) == 4;
+        const uint32_t bal = __ballot_sync(0xffffffffu, hit);
+        if (!bal) continue;
+        if (hit) yq[yn + __popc(bal & below)] = m.x;
+        yn += __popc(bal);
+      }
+      __syncwarp();
+      if (x0 >= x1 && yn == 0) break;
+      // groups that start past the mates seen so far wait for the next mates
+      const uint32_t lim = y0 < ys.y ? mates[y0 - 1u].x : kNone;
+      const uint32_t yj = (int)lane < yn ? yq[lane] : kNone;
+      uint32_t xs = kNone, xl = 0, xt = 0;
+      if (x1 - x0 > (int64_t)lane) {
+        const uint32_t g2 = nbr[x0 + lane];
+        xs = gstart[g2];
+        xl = gstart[g2 + 1] - xs;
+        xt = 4u - (uint32_t)__popc(bi ^ gbeta[g2]);  // 4 or 2
+      }
+      uint32_t nx = 0, ny = 0;  // groups up to this lane's mate, mates before its group
+      for (int step = 16; step; step >>= 1) {
+        const uint32_t a = __shfl_sync(0xffffffffu, xs, nx + step - 1);
+        const uint32_t b = __shfl_sync(0xffffffffu, yj, ny + step - 1);
+        if (a <= yj) nx += step;
+        if (b < xs) ny += step;
+      }
+      const uint32_t xlast = __shfl_sync(0xffffffffu, xs, 31);
+      if (nx == 31 && xlast <= yj) nx = 32;
+      const uint32_t y32 = __shfl_sync(0xffffffffu, yj, 31);
+      if (ny == 31 && y32 < xs) ny = 32;
+      const uint32_t rx = lane + ny, ry = lane + nx;
+      const bool take_x = xs != kNone && xs <= lim && rx < 32u, take_y = yj != kNone && ry < 32u;
+      // the threshold's two bits (0, 2 or 4) above the column and the length
+      if (take_x) pl[rx] = make_uint2(xs | ((xt & 2u) << 30), xl | ((xt & 4u) << 29));
+      if (take_y) pl[ry] = make_uint2(yj, 1u);
+      const uint32_t tx = __ballot_sync(0xffffffffu, take_x), ty = __ballot_sync(0xffffffffu, take_y);
+      __syncwarp();
       uint32_t gs = 0, len = 0;
       int thr = -1;
-      if (e0 + lane < e1) {
-        const uint32_t g2 = nbr[e0 + lane];
-        gs = gstart[g2];
-        len = gstart[g2 + 1] - gs;
-        thr = 4 - __popc(bi ^ gbeta[g2]);
-        if (thr == 0) {
-          // beta strings a double apart: only alpha_j == alpha_i connects, and
-          // the group is sorted by alpha, so one binary search replaces the
-          // walk (the group becomes that one column, or nothing)
-          uint32_t lo = gs, hi = gs + len;
-          while (lo < hi) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (key_alpha(keys[mid]) < ai) lo = mid + 1;
-            else hi = mid;
-          }
-          const bool found = lo < gs + len && key_alpha(keys[lo]) == ai;
-          gs = lo;
-          len = found ? 1u : 0u;
-        }
+      if ((int)lane < __popc(tx) + __popc(ty)) {
+        const uint2 e = pl[lane];
+        gs = e.x & 0x7fffffffu;
+        len = e.y & 0x7fffffffu;
+        thr = (int)(((e.x >> 30) & 2u) | ((e.y >> 29) & 4u));
+      }
+      __syncwarp();
+      x0 += __popc(tx);
+      if (ty) {
+        const int k = __popc(ty);
+        const uint32_t a = (int)lane + k < yn ? yq[lane + k] : 0u;
+        const uint32_t b = (int)lane + 32 + k < yn ? yq[lane + 32 + k] : 0u;
+        __syncwarp();
+        yn -= k;
+        if ((int)lane < yn) yq[lane] = a;
+        if ((int)lane + 32 < yn) yq[lane + 32] = b;
+        __syncwarp();
       }
       uint32_t off = len;  // inclusive scan of the lengths
       for (int o = 1; o < 32; o <<= 1) {
@@ -1382,9 +1468,10 @@ struct BetaGraph {
   uint32_t G = 0;
   uint32_t *of_row = nullptr, *gstart = nullptr, *gbeta = nullptr, *nbr = nullptr;
   int64_t *nbr_ptr = nullptr;
+  uint2 *mates = nullptr, *span = nullptr;  // rows in alpha order
 };
 
-static int beta_graph(const uint64_t *keys, uint32_t n, BetaGraph *bg, Arena &arena) {
+static int beta_graph(const uint64_t *keys, uint32_t n, int norb, BetaGraph *bg, Arena &arena) {
   cudaStream_t s = arena.stream();
   uint32_t *head, *gid;
   ASCI_TRY(arena.alloc(&head, n));
@@ -1423,6 +1510,17 @@ static int beta_graph(const uint64_t *keys, uint32_t n, BetaGraph *bg, Arena &ar
   k_beta_pairs<true><<<dim3(g.gx, g.gy), kRowThreads, 0, s>>>(bg->gbeta, G, g.chunk, g.gy, off,
                                                                bg->nbr);
   ASCI_CHECK_LAUNCH();
+  uint64_t *akey, *akey_alt;
+  ASCI_TRY(arena.alloc(&akey, n));
+  ASCI_TRY(arena.alloc(&akey_alt, n));
+  ASCI_TRY(arena.alloc(&bg->mates, n));
+  ASCI_TRY(arena.alloc(&bg->span, n));
+  k_alpha_keys<<<blocks_for(n, 256), 256, 0, s>>>(keys, n, akey);
+  ASCI_CHECK_LAUNCH();
+  ASCI_TRY(radix_sort_u64_varying(&akey, &akey_alt, n, 32, 32 + norb,
+                                  ((1ull << norb) - 1ull) << 32, arena));
+  k_alpha_mates<<<blocks_for(n, 256), 256, 0, s>>>(keys, akey, n, bg->mates, bg->span);
+  ASCI_CHECK_LAUNCH();
   bg->G = G;
   return ASCI_OK;
 }
@@ -1437,7 +1535,7 @@ static int ham_count(const DevInts &I, const uint64_t *keys, uint32_t n, const d
   cudaStream_t s = arena.stream();
   ASCI_TRY_CUDA(cudaMemsetAsync(rp + n, 0, sizeof(int64_t), s));
   k_ham_rows<false><<<row_blocks(n), kRowWarps * 32, 0, s>>>(I, keys, n, bg.of_row, bg.gstart, bg.gbeta,
-                                                   bg.nbr_ptr, bg.nbr, diag, rp, nullptr,
+                                                   bg.nbr_ptr, bg.nbr, bg.mates, bg.span, diag, rp, nullptr,
                                                    nullptr);
   ASCI_CHECK_LAUNCH();
   ASCI_TRY(scan_exclusive_u64(reinterpret_cast<uint64_t *>(rp), reinterpret_cast<uint64_t *>(rp),
@@ -1452,7 +1550,7 @@ static int ham_count(const DevInts &I, const uint64_t *keys, uint32_t n, const d
 static int ham_fill(const DevInts &I, const uint64_t *keys, uint32_t n, const double *diag,
                     const BetaGraph &bg, int64_t *rp, int32_t *col, double *val, Arena &arena) {
   k_ham_rows<true><<<row_blocks(n), kRowWarps * 32, 0, arena.stream()>>>(I, keys, n, bg.of_row, bg.gstart,
-                                                              bg.gbeta, bg.nbr_ptr, bg.nbr, diag,
+                                                              bg.gbeta, bg.nbr_ptr, bg.nbr, bg.mates, bg.span, diag,
                                                               rp, col, val);
   ASCI_CHECK_LAUNCH();
   return ASCI_OK;
@@ -1734,7 +1832,7 @@ static int ham_build(const DevInts &I, const uint64_t *keys, size_t n, Arena &ar
   ASCI_TRY(arena.alloc(&rp, n + 1));
   ASCI_TRY(diagonal_packed(I, keys, n, diag, arena));
   BetaGraph bg;
-  ASCI_TRY(beta_graph(keys, (uint32_t)n, &bg, arena));
+  ASCI_TRY(beta_graph(keys, (uint32_t)n, I.n, &bg, arena));
   size_t nnz = 0;
   ASCI_TRY(ham_count(I, keys, (uint32_t)n, diag, bg, rp, &nnz, arena));
   int32_t *col;
@@ -2008,7 +2106,7 @@ int asci_hamiltonian(const asci_det *dets, size_t n, const asci_ints *ints, int6
   ASCI_TRY(arena.alloc(&diag, n));
   ASCI_TRY(diagonal_packed(I, keys, n, diag, arena));
   BetaGraph bg;
-  ASCI_TRY(beta_graph(keys, (uint32_t)n, &bg, arena));
+  ASCI_TRY(beta_graph(keys, (uint32_t)n, I.n, &bg, arena));
   const bool same_order = hflag == 0;
   int64_t *rp, *urp;
   ASCI_TRY(out_buffer(row_ptr, n + 1, &urp, arena));
