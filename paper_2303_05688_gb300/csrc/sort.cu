@@ -114,11 +114,11 @@ __device__ __forceinline__ uint64_t warp_sum(uint64_t v) {
 // same array: a tile writes only after it has published, so an input whose word
 // is still unknown after it was read was read unchanged).
 //
-// Bound: memory and the look back's latency: 57.7 M item weights 267 us (312 for
+// Bound: memory and the look back's latency: 57.7 M item weights 248 us (312 for
 // reduce, scan of the partial sums and scan, which read twice), 1e5 words 4 (9 in
 // three launches).
 template <typename T, typename In>
-__global__ void __launch_bounds__(kScanThreads, 4) k_scan(In in, T *out, size_t n, uint64_t *words) {
+__global__ void __launch_bounds__(kScanThreads, 5) k_scan(In in, T *out, size_t n, uint64_t *words) {
   __shared__ T tile[kScanTile + kScanTile / (128 / sizeof(T))];
   __shared__ uint32_t s_tile;
   __shared__ uint64_t s_before;
