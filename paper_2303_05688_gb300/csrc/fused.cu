@@ -4,8 +4,8 @@
 // Work is partitioned by target alpha string A' (the finest constraint class:
 // all occupied alpha orbitals fixed).  Items sorted by A' (see excite.cu) make
 // each class a contiguous range; a batch of classes is generated into a
-// staging buffer as records (beta', v = H_ij c_j, H_ii) and then reduced tile
-// by tile on chip:
+// staging buffer as records (beta', v = H_ij c_j, a lower bound of |E0 - H_ii|)
+// and then reduced tile by tile on chip:
 //   small classes (<= kCap/2 pairs)   packed, several per tile, in item order
 //   medium classes (<= kCap pairs)    one tile each, in item order
 //   big classes                       split into hash buckets of beta' (each a
@@ -13,15 +13,16 @@
 //                                     land in the same bucket
 // A tile groups its records by target in a shared-memory hash table, drops
 // targets in psi, and appends the targets whose |score| can reach the running
-// top-N threshold; their values are summed after the launch by a rule that
-// does not depend on the order of the contributions, so that it equals the
-// sort-and-accumulate result bit for bit, and scored in FP64.
+// top-N threshold.  A target's values are summed by a rule that does not depend
+// on the order of the contributions (long lists after the launch), so that the
+// sum equals the sort-and-accumulate result bit for bit, and scored in FP64.
 //
-// The diagonal H_ii is carried exactly in 64-bit fixed point: the integral
-// terms are rounded once to multiples of 2^-s, and each pair's H_ii is the
-// parent's H_jj plus the excitation's change, computed from the parent's
-// Fock-like diagonals F_s(p) = h_pp + sum_{q in s} (J-K)_pq + sum_{q in s'} J_pq.
-// Integer sums are exact, so every path to a target gives the same H_ii.
+// The diagonal H_ii is exact in 64-bit fixed point: the integral terms are
+// rounded once to multiples of 2^-s, and integer sums do not depend on their
+// order.  Where a score or a decision needs it, it is summed from chunk tables;
+// the bound that a record carries is the parent's H_jj plus the excitation's
+// change, from the parent's Fock-like diagonals F_s(p) = h_pp + sum_{q in s}
+// (J-K)_pq + sum_{q in s'} J_pq, in 32 bits.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
