@@ -1445,6 +1445,12 @@ __global__ void __launch_bounds__(THREADS, CTAS) k_cells(CellArgs C) {
   constexpr uint32_t kTabMask = (uint32_t)Smem::kTab - 1u;
   static_assert(CAP == kRPT * THREADS && THREADS >= kPsiCap, "records per thread");
   static_assert(kRPT == 8 && W::kThr < 256 && Smem::kTab <= 65536, "packed bounds and slots");
+  // a warp's candidates, lists and values in one word
+  constexpr int kListShift = 9, kValueShift = 18;
+  constexpr uint32_t kWarpMask = (1u << kListShift) - 1u;
+  static_assert(32 * kRPT <= (int)kWarpMask && kValueShift == 2 * kListShift &&
+                    (uint32_t)CAP <= (0xffffffffu >> kValueShift),
+                "a warp's counts must fit their fields");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Smem &S = *reinterpret_cast<Smem *>(smem_raw);
   const int lane = threadIdx.x & 31;
@@ -1603,7 +1609,7 @@ __global__ void __launch_bounds__(THREADS, CTAS) k_cells(CellArgs C) {
     __syncthreads();  // every slot word is complete
     // the claiming thread decides on its target and empties the slot, unless
     // the target's values are to be copied out
-    uint32_t pass = 0, multi = 0, own = 0;  // own: candidates, lists << 9, values << 17
+    uint32_t pass = 0, multi = 0, own = 0;  // own: candidates, lists, values (packed)
     my_unique += (uint32_t)__popc(claimed);
 #pragma unroll
     for (int k = 0; k < kRPT; ++k) {
@@ -1620,7 +1626,7 @@ __global__ void __launch_bounds__(THREADS, CTAS) k_cells(CellArgs C) {
         pass |= 1u << k;
         if (more) {
           multi |= 1u << k;
-          own += (1u << 9) + ((more + 1u) << 17);
+          own += (1u << kListShift) + ((more + 1u) << kValueShift);
           continue;
         }
       }
@@ -1632,7 +1638,8 @@ __global__ void __launch_bounds__(THREADS, CTAS) k_cells(CellArgs C) {
       S.slot[marker] = W::kEmpty;
     if (__any_sync(0xffffffffu, pass != 0u)) {
       // candidates, targets to be summed and their values: one scan over the
-      // warp (at most 256 candidates, 128 lists and CAP values)
+      // warp (at most a candidate and a list for each of its records, whose
+      // targets' other records may all be other warps', and CAP values)
       own += (uint32_t)__popc(pass);
       uint32_t sum = own;
 #pragma unroll
@@ -1641,14 +1648,14 @@ __global__ void __launch_bounds__(THREADS, CTAS) k_cells(CellArgs C) {
         if (lane >= o) sum += y;
       }
       const uint32_t all = __shfl_sync(0xffffffffu, sum, 31);
-      const uint32_t nf = (all >> 9) & 0xffu;
+      const uint32_t nf = (all >> kListShift) & kWarpMask;
       unsigned long long b0 = 0, f0 = 0, l0 = 0;
       uint32_t c0 = 0;
       if (lane == 0) {
-        b0 = atomicAdd(C.cand_count, (unsigned long long)(all & 0x1ffu));
+        b0 = atomicAdd(C.cand_count, (unsigned long long)(all & kWarpMask));
         if (nf) {
           f0 = atomicAdd(C.nfix, (unsigned long long)nf);
-          l0 = atomicAdd(C.lv_count, (unsigned long long)(all >> 17));
+          l0 = atomicAdd(C.lv_count, (unsigned long long)(all >> kValueShift));
           c0 = atomicAdd(&S.ncur, nf);
         }
       }
@@ -1659,10 +1666,10 @@ __global__ void __launch_bounds__(THREADS, CTAS) k_cells(CellArgs C) {
         c0 = __shfl_sync(0xffffffffu, c0, 0);
       }
       const uint32_t before = sum - own;
-      b0 += before & 0x1ffu;
-      f0 += (before >> 9) & 0xffu;
-      c0 += (before >> 9) & 0xffu;
-      l0 += before >> 17;
+      b0 += before & kWarpMask;
+      f0 += (before >> kListShift) & kWarpMask;
+      c0 += (before >> kListShift) & kWarpMask;
+      l0 += before >> kValueShift;
 #pragma unroll
       for (int k = 0; k < kRPT; ++k) {
         if (!((pass >> k) & 1u)) continue;
