@@ -126,6 +126,13 @@ __host__ __device__ inline int sel_shift(int round) {
   return d == 5 ? 0 : 64 - kSelBits * (d + 1);
 }
 
+// The state before the first round, for the n largest.
+__global__ void k_select_init(SelState *st, uint64_t n) {
+  SelState s{};
+  s.remaining = n;
+  *st = s;
+}
+
 __global__ void __launch_bounds__(256) k_select_round(const uint64_t *keys, const double *scores,
                                                       size_t n, int round, SelState *st,
                                                       uint32_t *hist) {
@@ -430,7 +437,7 @@ int select_topn_packed(const uint64_t *keys, const double *scores, size_t n, siz
     if (host_min) ASCI_TRY(abs_min(scores, n, host_min, arena));
     return ASCI_OK;
   }
-  SelState *st, init{};
+  SelState *st;
   ASCI_TRY(arena.alloc(&st, 1));
   if (n <= kSmallSelect) {
     k_select_small<<<1, 1024, 0, s>>>(keys, scores, (uint32_t)n, (uint32_t)N, out_keys, out_scores,
@@ -441,9 +448,9 @@ int select_topn_packed(const uint64_t *keys, const double *scores, size_t n, siz
     ASCI_TRY(arena.alloc(&flag, n));
     ASCI_TRY(arena.alloc(&pos, n));
     ASCI_TRY(arena.alloc(&hist, (size_t)kSelBins));
-    init.remaining = N;
     ASCI_TRY_CUDA(cudaMemsetAsync(hist, 0, kSelBins * sizeof(uint32_t), s));
-    ASCI_TRY_CUDA(cudaMemcpyAsync(st, &init, sizeof(init), cudaMemcpyHostToDevice, s));
+    k_select_init<<<1, 1, 0, s>>>(st, N);
+    ASCI_CHECK_LAUNCH();
     for (int round = 0; round < kSelRounds; ++round) {
       k_select_round<<<grid_for(n, 152 * 4), 256, 0, s>>>(keys, scores, n, round, st, hist);
       ASCI_CHECK_LAUNCH();
@@ -458,9 +465,10 @@ int select_topn_packed(const uint64_t *keys, const double *scores, size_t n, siz
   if (host_min) {
     // the selected entry of largest R has the smallest |S|: thr bounds it from
     // below (its free low bits are set)
-    ASCI_TRY_CUDA(cudaMemcpyAsync(&init, st, sizeof(init), cudaMemcpyDeviceToHost, s));
+    SelState done;
+    ASCI_TRY_CUDA(cudaMemcpyAsync(&done, st, sizeof(done), cudaMemcpyDeviceToHost, s));
     ASCI_TRY_CUDA(cudaStreamSynchronize(s));
-    const uint64_t bits = ~init.thr[0];
+    const uint64_t bits = ~done.thr[0];
     memcpy(host_min, &bits, sizeof(bits));
   }
   return ASCI_OK;

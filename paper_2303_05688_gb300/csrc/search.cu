@@ -260,6 +260,16 @@ __global__ void k_prep_totals(const asci_det *dets, const uint32_t *gid, const u
   out->groups = (uint64_t)gid[m - 1] + head[m - 1];
 }
 
+// Counters set on the stream by value: a copy from a host variable would need the
+// variable until the copy is done.
+__global__ void k_set_count(unsigned long long *count, unsigned long long v) { *count = v; }
+__global__ void k_set_counts(unsigned long long *count, ulonglong3 v, unsigned *err) {
+  count[0] = v.x;
+  count[1] = v.y;
+  count[2] = v.z;
+  *err = 0;
+}
+
 __global__ void k_unpack(const uint64_t *keys, size_t n, asci_det *out) {
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (size_t)gridDim.x * blockDim.x) {
@@ -878,8 +888,8 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
     if (pt2_out) {
       ASCI_TRY(pt2_terms(F, pool_k[pcur] + pool_n, pool_s[pcur] + pool_n, (size_t)c - pool_n,
                          pt2_limbs, derr2, stream));
-      const unsigned long long keep = pool_n;
-      ASCI_TRY_CUDA(cudaMemcpyAsync(dcount, &keep, sizeof(keep), cudaMemcpyHostToDevice, stream));
+      k_set_count<<<1, 1, 0, stream>>>(dcount, pool_n);
+      ASCI_CHECK_LAUNCH();
       return ASCI_OK;
     }
     ASCI_TRY(exact_scores(F, pool_k[pcur] + pool_n, pool_s[pcur] + pool_n, (size_t)c - pool_n,
@@ -897,8 +907,8 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
     pcur ^= 1;
     pool_n = m2;
     if (m2 >= N && N > 0) tau = least;
-    const unsigned long long c = pool_n;
-    ASCI_TRY_CUDA(cudaMemcpyAsync(dcount, &c, sizeof(c), cudaMemcpyHostToDevice, stream));
+    k_set_count<<<1, 1, 0, stream>>>(dcount, pool_n);
+    ASCI_CHECK_LAUNCH();
     return ASCI_OK;
   };
   // The counters before a tile launch: when its values found no room (rare: a
@@ -915,10 +925,8 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
     if (he == kErrValues && !full) {
       ASCI_TRACE("%s: values found no room; again with room for all", what);
       values_full = *again = true;
-      hcount[0] = pool_n;
-      ASCI_TRY_CUDA(cudaMemsetAsync(derr2, 0, sizeof(unsigned), stream));
-      ASCI_TRY_CUDA(cudaMemcpyAsync(dcount, hcount, 3 * sizeof(hcount[0]), cudaMemcpyHostToDevice,
-                                    stream));
+      k_set_counts<<<1, 1, 0, stream>>>(dcount, make_ulonglong3(pool_n, hcount[1], hcount[2]), derr2);
+      ASCI_CHECK_LAUNCH();
       return ASCI_OK;
     }
     if (he) {
