@@ -554,7 +554,8 @@ struct EmitArgs {
   Stage st;
   uint32_t st_cap;            // st.cap (below 2^32)
   double eps;                 // Alg. 2 screen; 0 keeps every pair
-  float eps_f;                // eps as a float (the screen's float pre-test)
+  float eps_f;                // eps 2^eps_shift as a float (the screen's float pre-test)
+  int eps_shift;
   int64_t E0_x;
   double inv_scale;
   float scale32;              // a unit of the 32-bit denominator
@@ -649,14 +650,22 @@ __device__ __forceinline__ void write_record(const EmitArgs &A, uint32_t pos, bo
     // 2^-23 below its value, eps_f and the bounds within 2^-24 of theirs, the
     // product within 2^-24); the rest take the FP64 test on the exact
     // denominator, so every decision is that test's.  (FP64 instructions are
-    // scarce on this GPU.)
-    bool okv;
-    const float vf = abs_as_float(v, &okv);
+    // scarce on this GPU.)  Both sides are scaled by the power of two that
+    // brings eps to eps_f in [0.5, 1]: eps_f times a bound is then in
+    // [2^-32, 2^51] or zero, and a scaled |v| beyond the float range on either
+    // side is replaced by a float that is beyond that interval too.  A pair of
+    // value zero is never kept; with symmetry most pairs are such: summing their
+    // exact denominators made a (24e,30o) search with seven eighths of the
+    // integrals zero, C = 1e4, take 127 ms, against 18.3 (19.7 without a screen).
+    const uint64_t b = (uint64_t)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    const int be = (int)(b >> 52), e = min(max(be - 896 + A.eps_shift, 1), 254);
+    const float vf = __uint_as_float(((uint32_t)e << 23) | (uint32_t)((b >> 29) & 0x7fffffu));
+    const bool normal = be > 0 && be < 0x7ff;  // neither zero, subnormal, infinite nor NaN
     const float lo = A.eps_f * df, hi = A.eps_f * ((float)(mag + kDenSlack) * A.scale32);
     bool keep;
-    if (okv && hi > 1e-37f && hi < 1e37f && vf > hi * 1.000004f) {
+    if (normal && vf > hi * 1.000004f) {
       keep = true;
-    } else if (okv && lo > 1e-37f && lo < 1e37f && vf < lo * 0.999996f) {
+    } else if ((normal && vf < lo * 0.999996f) || b == 0) {
       keep = false;
     } else {
       const double d = __ll2double_rn(A.E0_x - fx_diag(A.X, talpha, tb)) * A.inv_scale;
@@ -2486,7 +2495,9 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   A.st = st;
   A.st_cap = (uint32_t)std::min<uint64_t>(st.cap, 0xffffffffull);
   A.eps = eps;
-  A.eps_f = (float)eps;
+  int eps_exp = 0;
+  A.eps_f = (float)frexp(eps, &eps_exp);
+  A.eps_shift = -eps_exp;
   A.E0_x = F.E0_x;
   A.inv_scale = ldexp(1.0, -F.X.s);
   A.scale32 = (float)ldexp(1.0, kDenShift - F.X.s);
