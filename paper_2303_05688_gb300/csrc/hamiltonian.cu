@@ -836,11 +836,19 @@ __global__ void k_normalize(double *v, size_t n, const double *norm2) {
 //      eigenbasis Q, L as the approximate inverse (its own component left
 //      out), normalised.  Each step shrinks the error by about the FP32
 //      eigenbasis's own (1e-4), until |r| is at FP64 rounding.
-//   3. Several eigenvectors are orthonormalised by two passes of Gram-Schmidt.
-// A pair whose residual stays above 1e-13 of the matrix (eigenvalues too close
-// for FP32 to tell apart) sends the whole matrix through FP64 Jacobi: FP32
-// eigenvectors orthonormalised in FP64, Q^T Hs Q, FP64 sweeps to an
-// off-diagonal norm of 1e-13 of the diagonal's.
+//   3. Several eigenvectors are orthonormalised by two passes of Gram-Schmidt
+//      and ordered by their FP64 eigenvalues.
+// A small residual shows an eigenpair, not which one.  The next FP32 eigenvalue d
+// is a lower bound of every eigenvalue that was not refined, up to: the
+// off-diagonal norm left (Weyl's bound); 4e-3 |d|, for an eigenbasis off
+// orthonormal by at most 2e-3 (Ostrowski's bound; each of up to 28 x 12 x 31
+// warm-started rotations of a column scales it by 1 + 2e-7 at most); and 1e-5 of the
+// matrix for the FP32 rounding.  Unless the lowest refined eigenvalue is below d by
+// that much, and when a pair's residual stays above 1e-13 of the matrix or two
+// pairs turned out to be the same (eigenvalues too close for FP32 to tell
+// apart), the whole matrix goes through FP64 Jacobi: FP32 eigenvectors
+// orthonormalised in FP64, Q^T Hs Q, FP64 sweeps to an off-diagonal norm of 1e-13
+// of the diagonal's.
 // m = 16: 15 us against 135 for the FP64 Jacobi that every product took.
 constexpr int kEigThreads = 256;
 
@@ -995,9 +1003,11 @@ __device__ __forceinline__ float2 rotation_fast(float app, float aqq, float apq)
 // rotated against each other, a block of A (or a row's pair of Q) per thread,
 // and the results written one place on in the round-robin into the other
 // buffer, so a round has one barrier; after the M - 1 rounds of a sweep every
-// index is back in its place.  Returns the buffer that holds the result.
+// index is back in its place.  Returns the buffer that holds the result; *off2
+// and *all2 get the squares of its off-diagonal norm (infinite when the sweeps
+// ran out) and of its norm.
 __device__ int jacobi_fast(float (*A)[kMaxSub][kMaxSub + 1], float (*Q)[kMaxSub][kMaxSub + 1],
-                           int m, float (*red)[kEigThreads / 32]) {
+                           int m, float (*red)[kEigThreads / 32], float *off2, float *all2) {
   const int tid = threadIdx.x, M = m + (m & 1), half = M / 2;
   constexpr int kItems = (kMaxSub * kMaxSub / 4 + kMaxSub * kMaxSub / 2) / kEigThreads;
   const int items = half * half + M * half;  // blocks of A, then (row, pair) of Q
@@ -1018,6 +1028,8 @@ __device__ int jacobi_fast(float (*A)[kMaxSub][kMaxSub + 1], float (*Q)[kMaxSub]
     to_k1[u] = next(2 * it_k[u] + 1);
   }
   int b = 0;
+  *off2 = m > 1 ? __int_as_float(0x7f800000) : 0.0f;
+  *all2 = 0.0f;
   for (int sweep = 0; sweep < 12 && m > 1; ++sweep) {
     float off = 0.0f, all = 0.0f;
     for (int e = tid; e < kMaxSub * M; e += kEigThreads) {
@@ -1043,7 +1055,11 @@ __device__ int jacobi_fast(float (*A)[kMaxSub][kMaxSub + 1], float (*Q)[kMaxSub]
       off += red[0][w];
       all += red[1][w];
     }
-    if (!(off > 1e-8f * all)) break;  // uniform
+    *all2 = all;
+    if (!(off > 1e-8f * all)) {  // uniform
+      *off2 = off;
+      break;
+    }
     for (int r = 0; r < M - 1; ++r, b ^= 1) {
       const float(*Ab)[kMaxSub + 1] = A[b];
       const float(*Qb)[kMaxSub + 1] = Q[b];
@@ -1085,7 +1101,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // want lowest eigenpairs: theta[0 .. want), eigenvector k in Ct[k * kMaxSub + j].
 // Qw keeps the FP32 eigenbasis; with `warm` it holds that of the leading
 // m - 1 rows and columns, and the sweeps start in its basis (an arrowhead).
-__global__ void __launch_bounds__(kEigThreads) k_small_eig(const double *Hs, int m, int want,
+__global__ void __launch_bounds__(kEigThreads, 1) k_small_eig(const double *Hs, int m, int want,
                                                            bool warm, float *Qw, double *theta,
                                                            double *Ct, const int *stop) {
   __shared__ double H[kMaxSub][kMaxSub + 1];
@@ -1095,7 +1111,7 @@ __global__ void __launch_bounds__(kEigThreads) k_small_eig(const double *Hs, int
   __shared__ float Q2[2][kMaxSub][kMaxSub + 1];
   __shared__ double X[kKeep][kMaxSub], th[kKeep];
   __shared__ float gv[kKeep][kMaxSub], redf[2][kEigThreads / 32];
-  __shared__ int of_rank[kMaxSub], failed;
+  __shared__ int of_rank[kMaxSub], failed, lowest;
   __shared__ double gsr[kMaxSub];
   __shared__ double nrm;
   __shared__ EigScratch E;
@@ -1113,7 +1129,10 @@ __global__ void __launch_bounds__(kEigThreads) k_small_eig(const double *Hs, int
     A2[0][i][k] = (float)(in && i == k ? h - shift : h);
     Q2[0][i][k] = q;
   }
-  if (tid == 0) failed = 0;
+  if (tid == 0) {
+    failed = 0;
+    lowest = want >= m ? 1 : 0;  // the lowest of all pairs is among the refined ones
+  }
   __syncthreads();
   if (warm) {  // A = Q^T A Q
     float p[kMaxSub * kMaxSub / kEigThreads];
@@ -1137,7 +1156,8 @@ __global__ void __launch_bounds__(kEigThreads) k_small_eig(const double *Hs, int
       __syncthreads();
     }
   }
-  const int buf = jacobi_fast(A2, Q2, m, redf);
+  float off2, all2;
+  const int buf = jacobi_fast(A2, Q2, m, redf, &off2, &all2);
   const float(*Af)[kMaxSub + 1] = A2[buf];
   const float(*Qf)[kMaxSub + 1] = Q2[buf];
 #pragma unroll
@@ -1160,6 +1180,8 @@ __global__ void __launch_bounds__(kEigThreads) k_small_eig(const double *Hs, int
     float scale = in ? fabsf(lam) : 0.0f;
     for (int o = 16; o; o >>= 1) scale = fmaxf(scale, __shfl_xor_sync(0xffffffffu, scale, o));
     scale += fabsf((float)shift);
+    const float d = want < m ? Af[of_rank[want]][of_rank[want]] : 0.0f;
+    const float bound = d - (sqrtf(2.0f * off2 + 2e-10f * all2) + 4e-3f * fabsf(d));
     double x = in ? (double)Qf[lane][own] : 0.0;
     x *= rsqrt_fast(warp_sum(x * x));
     double t = 0.0;
@@ -1209,10 +1231,13 @@ __global__ void __launch_bounds__(kEigThreads) k_small_eig(const double *Hs, int
       x *= rsqrt_fast(warp_sum(x * x));
     }
     X[w][lane] = x;
-    if (lane == 0) th[w] = t;
+    if (lane == 0) {
+      th[w] = t;
+      if ((float)(t - shift) < bound) lowest = 1;
+    }
   }
   __syncthreads();
-  if (!failed) {
+  if (!failed && lowest) {
     if (want > 1 && w == 0) {  // orthonormal: two passes of Gram-Schmidt, one vector after another
       for (int k = 0; k < want; ++k) {
         double x = X[k][lane];
@@ -1224,15 +1249,26 @@ __global__ void __launch_bounds__(kEigThreads) k_small_eig(const double *Hs, int
           for (int j = 0; j < kKeep; ++j)
             if (j < k) x = fma(-dots[j], X[j][lane], x);
         }
-        x *= rsqrt_fast(warp_sum(x * x));
+        const double x2 = warp_sum(x * x);
+        if (!(x2 > 0.25) && lane == 0) failed = 1;  // found before
+        x *= rsqrt_fast(x2);
         X[k][lane] = x;
         __syncwarp();
       }
     }
     __syncthreads();
-    for (int e = tid; e < want * m; e += kEigThreads)
-      Ct[(size_t)(e / m) * kMaxSub + (e - (e / m) * m)] = X[e / m][e - (e / m) * m];
-    if (tid < want) theta[tid] = th[tid];
+  }
+  if (!failed && lowest) {
+    auto place = [&](int k) {  // rank of pair k (ties by number)
+      int rk = 0;
+      for (int j = 0; j < want; ++j) rk += (th[j] < th[k]) || (th[j] == th[k] && j < k);
+      return rk;
+    };
+    for (int k = w; k < want; k += kEigThreads / 32) {
+      const int rk = want > 1 ? place(k) : 0;
+      if (lane < m) Ct[(size_t)rk * kMaxSub + lane] = X[k][lane];
+      if (lane == 0) theta[rk] = th[k];
+    }
     return;
   }
   for (int e = tid; e < m * m; e += kEigThreads) {
