@@ -2998,7 +2998,7 @@ __global__ void __launch_bounds__(256) k_pt2_terms(const uint64_t *key, const do
     const double r = (fabs(den) >= 1e-30 && fabs(den) <= 1e30) ? recip_fast(den) : 1.0 / den;
     pt2_add(v * v * r, acc, &bad);
   }
-  if (bad) atomicOr(err, kErrAccum);
+  if (bad) atomicOr(err, kErrTerm);
   __syncthreads();
   const int k = threadIdx.x >> 5;  // a warp per limb
   long long t = 0;

@@ -57,6 +57,8 @@ struct Spill {
 // Bit of the device error word: the values of the targets to be summed found
 // no room (the launch is run again with room for all of them).
 constexpr unsigned kErrValues = 32u;
+// Bit: an ASCI-PT2 term that is not finite or is too large for the sum.
+constexpr unsigned kErrTerm = 64u;
 
 // Everything the batch kernels read that stays fixed during one search.
 struct FusedCore {

@@ -916,6 +916,11 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   // those after it, run with room for every record, fewer tiles at a time.
   unsigned long long hcount[4] = {0, 0, 0, 0};
   bool values_full = false;
+  auto bad_term = []() -> int {
+    record_error("a PT2 term is not finite or exceeds 2^40 (E0 equals or nearly equals a "
+                 "target's H_ii)", __FILE__, __LINE__);
+    return ASCI_EINVAL;
+  };
   auto read_counts = [&](bool full, const char *what, bool *again) -> int {
     unsigned long long c[5];
     *again = false;
@@ -929,6 +934,7 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
       ASCI_CHECK_LAUNCH();
       return ASCI_OK;
     }
+    if (he == kErrTerm) return bad_term();  // of an earlier launch's targets
     if (he) {
       char msg[96];
       snprintf(msg, sizeof(msg), "%s check failed (flags 0x%x)", what, he);
@@ -1078,11 +1084,7 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
       ASCI_TRY_CUDA(cudaMemcpyAsync(&he, derr2, sizeof(he), cudaMemcpyDeviceToHost, stream));
       ASCI_TRY_CUDA(cudaStreamSynchronize(stream));
     }
-    if (he) {
-      record_error("a PT2 term is not finite or exceeds 2^40 (E0 equals or nearly equals a "
-                   "target's H_ii)", __FILE__, __LINE__);
-      return ASCI_EINVAL;
-    }
+    if (he) return bad_term();
     *pt2_out = v;
     *out_n = 0;
     if (st) {
