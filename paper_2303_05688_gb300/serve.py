@@ -12,6 +12,7 @@ on what else is running (the batch size does not change any output).
 from __future__ import annotations
 
 import collections
+import math
 import threading
 import time
 from concurrent.futures import Future
@@ -23,17 +24,71 @@ from . import search as _search, FP64
 __all__ = ["Server", "footprint"]
 
 
-def footprint(norb: int, ndets: int, C: int, N: int, batch_pairs: int) -> int:
-    """Upper estimate of one search's device bytes beyond its resident inputs:
-    the staging of one constraint batch (16-byte pairs, 1.5 slots each, and the
-    alpha word), item lists, the candidate pool (two buffers of N + 2^29 entries
-    at most, 16 bytes each), the psi hash and routing, and the integral tables."""
-    staging = 28 * batch_pairs
-    pool = 32 * (N + min(batch_pairs, 1 << 29))
-    psi = 48 * ndets
-    tables = 40 * norb ** 4
-    items = 64 * C * (1 + norb * norb)
-    return int(staging + pool + psi + tables + items + (64 << 20))
+def footprint(norb: int, ndets: int, C: int, N: int, batch_pairs: int, *, na: int | None = None,
+              nb: int | None = None, alphas: int | None = None, group: int | None = None) -> int:
+    """Upper estimate of one search's device bytes beyond its resident inputs (N = 0: of
+    ASCI-PT2's), from the sizes of its allocations.  ``alphas`` is the number of distinct
+    alpha strings of psi and ``group`` the most determinants of one of them (both C by
+    default).  Without the electron counts half of the orbitals are taken, the counts of
+    most pairs, and a batch is taken to fill its cap."""
+    def pairs2(k):
+        return k * (k - 1) // 2
+
+    known = na is not None and nb is not None
+    na, nb = (na, nb) if known else (norb // 2, norb // 2)
+    C = min(C, ndets)
+    alphas = min(C, C if alphas is None else alphas)
+    group = min(C, C if group is None else group)
+    # operations on an alpha string, and pairs of a determinant: o = 0, an alpha single
+    singles, doubles = na * (norb - na), pairs2(na) * pairs2(norb - na)
+    beta = nb * (norb - nb)
+    npd0, npd1 = beta + pairs2(nb) * pairs2(norb - nb), 1 + beta
+    P = C * (npd0 + singles * npd1 + doubles)
+    items = alphas * (1 + singles + doubles)
+    # pairs of a batch: the cap, or one target alpha string's, which no cap divides
+    cap = batch_pairs or 1 << 31
+    b = max(min(P, cap) if known else cap, min(P, group * npd0 + C * npd1))
+    it = min(items, b)                                # items of a batch
+    strings = min(it, math.comb(norb, na))            # and their target alpha strings
+    runs = b // npd1 + b // 64 + (b // npd0 if npd0 else 0)
+    tiles = b // 256 + 2
+    cells = b // 400 + 1
+    appended = N + max(1024 * 152 * 16, min(b, 1 << 29))  # candidate pool
+    psi = (24 + 1 + 8 + 64) * ndets + 8192            # keys, sort, selection, hash table
+    core = (8 * norb + 120) * C
+    tables = 28 * norb ** 4 + 64 * norb ** 3 + (13 << 20)
+    plan = 29 * items + 60 * min(items, math.comb(norb, na))
+    staging = 20 * (b + b // 2 + (1 << 16))
+    pool = 32 * appended
+    lists = 40 * it + 60 * strings + 8 * runs + 32 * tiles + 16 * cells + 16 * ndets + b // 64
+    # records beyond their bucket's slots: the list, and one as long as it takes with its
+    # sort; then the oversized buckets' records gathered (on chip with their value
+    # buffers, or sorted)
+    big = b if b > 1024 else 0
+    spilled = 20 * max(1 << 20, b // 32) + 37 * big + 41 * big
+    # value buffers of a launch: 48 lists and 512 values a tile, or room for every record
+    # of a quarter of the tiles
+    launch = min(tiles, appended // 1024 + 1)
+    values = max(4864 * launch + (4 << 20), 16384 * min(launch, max(tiles // 4, 8192), 131072))
+    selected = 8 * appended + 48 * N
+    return int(psi + core + tables + plan + staging + pool + lists + spilled + values + selected
+               + (64 << 20))
+
+
+def _least(norb, ndets, C, N, batch_pairs):
+    """What a request must fit the budget with: the staging of a batch that fills its cap,
+    the candidate pool, the psi tables, the item lists and the integral tables."""
+    return int(28 * batch_pairs + 32 * (N + min(batch_pairs, 1 << 29)) + 48 * ndets
+               + 40 * norb ** 4 + 64 * C * (1 + norb * norb) + (64 << 20))
+
+
+def _shape(torch, dets):
+    """What footprint() can know of a determinant list beside its length."""
+    a, b = (bin(int(x)).count("1") for x in dets[0])
+    if a + b == 0:
+        return {}
+    count = torch.unique(dets[:, 0], return_counts=True)[1]
+    return dict(na=a, nb=b, alphas=int(count.numel()), group=int(count.max()))
 
 
 class Server:
@@ -80,7 +135,8 @@ class Server:
         h = dv(h1, torch.float64)
         self._systems[name] = dict(dets=d.to(dev), coeffs=dv(coeffs, torch.float64), E0=float(E0),
                                    h1=h, eri=dv(eri, torch.float64), ecore=float(ecore),
-                                   norb=int(round(h.numel() ** 0.5)), ndets=int(d.shape[0]))
+                                   norb=int(round(h.numel() ** 0.5)), ndets=int(d.shape[0]),
+                                   shape=_shape(torch, d))
 
     # ------------------------------------------------------------- requests ---
     def submit(self, name, C: int, N: int, precision: int = FP64, batch_pairs: int = 1 << 26):
@@ -89,9 +145,11 @@ class Server:
         request still in the queue is withdrawn by the future's cancel()
         (which then returns True); one already admitted runs to its end."""
         sy = self._systems[name]
-        fp = footprint(sy["norb"], sy["ndets"], C, N, batch_pairs)
-        if fp > self.budget:
-            raise ValueError(f"request needs {fp} bytes, more than the budget {self.budget}")
+        fp = footprint(sy["norb"], sy["ndets"], C, N, batch_pairs, **sy["shape"])
+        need = _least(sy["norb"], sy["ndets"], C, N, batch_pairs)
+        if need > self.budget:
+            raise ValueError(f"request needs {need} bytes, more than the budget {self.budget}")
+        fp = min(fp, self.budget)  # an upper estimate beyond the budget: it runs alone
         fut = Future()
         fut.add_done_callback(self._on_done)
         with self._cv:
