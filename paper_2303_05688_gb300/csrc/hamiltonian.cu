@@ -7,7 +7,8 @@
 //    visits the groups whose beta string is within one excitation (a group
 //    graph built by a tiled double loop over the beta strings), where it tests
 //    the alpha distance against 4 - popc(beta_i ^ beta_j), and, merged with
-//    them, the determinants of its own alpha string a beta double away.
+//    them, the determinants of its own alpha string a beta double away (listed, or
+//    searched where they are fewer than the alpha string's).
 //    Connected pairs get H_ij by the Slater-Condon rules, evaluated 32 at a
 //    time from a per-warp queue; nonzero elements are stored, each row's
 //    columns ascending.  A counting pass and a scan give the row pointers, the
@@ -129,10 +130,11 @@ __device__ double offdiag_element(const DevInts &I, uint32_t ai, uint32_t bi, ui
 // so a row has to visit the groups whose beta string is equal or a single
 // excitation away (the group graph, built once per list by a tiled double loop
 // over the G group strings), where only the alpha test remains, and the
-// determinants of its own alpha string whose beta string is a double away (from
-// the list in alpha order).  A warp takes a row and walks both, merged in
-// ascending order, 32 columns at a time; a ballot places the hits, so each
-// row's columns come out ascending.  A counting pass gives the row lengths, a scan the row
+// determinants of its own alpha string whose beta string is a double away: from
+// the list in alpha order, or, where an alpha string has many determinants,
+// searched in the groups a double away (mates_are_fewer).  A warp takes a row and
+// walks both, merged in ascending order, 32 columns at a time; a ballot places the
+// hits, so each row's columns come out ascending.  A counting pass gives the row lengths, a scan the row
 // pointers, and the filling pass writes (never past a row's counted end).
 
 // head[i] = 1 where a new beta string starts (keys sorted)
@@ -157,13 +159,14 @@ __global__ void k_beta_groups(const uint64_t *keys, uint32_t n, const uint32_t *
 }
 
 // Group graph: count (kFill false) or list (kFill true) the groups g2 with
-// popc(beta_g1 ^ beta_g2) <= 2, for the groups g1 = [blockIdx.x * 256, +256)
+// popc(beta_g1 ^ beta_g2) <= reach, for the groups g1 = [blockIdx.x * 256, +256)
 // (one per thread) against the groups [blockIdx.y * chunk, +chunk) staged in
 // shared memory.
 template <bool kFill>
 __global__ void __launch_bounds__(kRowThreads) k_beta_pairs(const uint32_t *gbeta, uint32_t G,
                                                             uint32_t chunk, uint32_t nchunks,
-                                                            uint64_t *cnt_off, uint32_t *nbr) {
+                                                            int reach, uint64_t *cnt_off,
+                                                            uint32_t *nbr) {
   __shared__ uint32_t sb[kColStage];
   const uint32_t g1 = blockIdx.x * kRowThreads + threadIdx.x;
   const bool live = g1 < G;
@@ -184,7 +187,7 @@ __global__ void __launch_bounds__(kRowThreads) k_beta_pairs(const uint32_t *gbet
     if (!live) continue;
 #pragma unroll 4
     for (uint32_t t = 0; t < m; ++t) {
-      if (__popc(b1 ^ sb[t]) > 2) continue;
+      if (__popc(b1 ^ sb[t]) > reach) continue;
       if (kFill) {
         if (pos < end) nbr[pos] = s + t;
         ++pos;
@@ -203,9 +206,12 @@ __global__ void k_alpha_keys(const uint64_t *keys, uint32_t n, uint64_t *akey) {
     akey[i] = ((uint64_t)key_alpha(keys[i]) << 32) | i;
 }
 // mates[t] = (row, its beta string) in alpha order; span[row] = the row's
-// [first, end) there, the rows of its own alpha string.
-__global__ void k_alpha_mates(const uint64_t *keys, const uint64_t *akey, uint32_t n, uint2 *mates,
-                              uint2 *span) {
+// [first, end) there, the rows of its own alpha string.  out (zero before): their
+// number over all rows, and the groups.
+__global__ void k_alpha_mates(const uint64_t *keys, const uint64_t *akey, uint32_t n,
+                              const uint32_t *head, const uint32_t *gid, uint2 *mates, uint2 *span,
+                              unsigned long long *out) {
+  unsigned long long all = 0;
   for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
     const uint32_t r = (uint32_t)akey[t], a = (uint32_t)(akey[t] >> 32);
     mates[t] = make_uint2(r, key_beta(keys[r]));
@@ -222,7 +228,11 @@ __global__ void k_alpha_mates(const uint64_t *keys, const uint64_t *akey, uint32
       else hi2 = mid;
     }
     span[r] = make_uint2(lo, lo2);
+    all += lo2 - lo;
+    if (t == n - 1) out[1] = gid[t] + head[t];
   }
+  for (int o = 16; o; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
+  if ((threadIdx.x & 31u) == 0 && all) atomicAdd(out, all);
 }
 
 // Row lengths (kFill false: rp[r] = count) or elements (kFill true: rp holds
@@ -232,14 +242,13 @@ __global__ void k_alpha_mates(const uint64_t *keys, const uint64_t *akey, uint32
 // evaluated 32 at a time, one per lane, so that the Slater-Condon work runs
 // on full warps rather than on the one or two lanes that hit in a step.
 //
-// Bound: latency of the gathers (integrals, columns' keys).  Looking the row's own
-// alpha string up in every group a beta double away (some 700 binary searches a
-// row at 16 orbitals) took 1.75 ms a counting pass over 1e5 random-walk
-// determinants; its mates, merged, take 1.34 (build 6.5 -> 5.2 ms).  Products of
-// whole string sets gain nothing, their rows having more mates than doubles: 320 x
-// 320 neighbouring strings 21.1 ms before and now, 300 x 300 random ones 2.2 and
-// 2.3, 8 x 12870 16.7 and 18.5 (20.4 with 48 registers instead of 32: the gathers
-// want warps).
+// Bound: latency of the gathers (integrals, columns' keys).  kMates: the doubles of
+// the row's own alpha string from its mates, merged; else by searching that string
+// in every group a beta double away.  A counting pass over 1e5 random-walk
+// determinants (117 mates a row against some 700 searches) takes 1.34 ms by mates,
+// 1.75 by searches; lists on either side of the choice are at mates_are_fewer.
+// (32 registers a thread by mates: with 48, 8 x 12870 strings took 20.4 instead of
+// 18.5 ms; the gathers want warps.)
 constexpr int kRowWarps = 8;
 
 template <bool kFill>
@@ -277,18 +286,18 @@ __device__ __forceinline__ void flush_queue(const DevInts &I, const uint64_t *ke
   }
 }
 
-template <bool kFill>
-__global__ void __launch_bounds__(kRowWarps * 32, 8) k_ham_rows(
+template <bool kFill, bool kMates>
+__global__ void __launch_bounds__(kRowWarps * 32, kMates ? 8 : 6) k_ham_rows(
     DevInts I, const uint64_t *__restrict__ keys, uint32_t n, const uint32_t *__restrict__ of_row,
     const uint32_t *__restrict__ gstart, const uint32_t *__restrict__ gbeta,
     const int64_t *__restrict__ nbr_ptr, const uint32_t *__restrict__ nbr,
     const uint2 *__restrict__ mates, const uint2 *__restrict__ span,
     const double *__restrict__ diag, int64_t *rp, int32_t *col, double *val) {
   __shared__ uint32_t queue[kRowWarps][64];
-  __shared__ uint2 place[kRowWarps][32];
-  __shared__ uint32_t found[kRowWarps][64];
-  uint2 *pl = place[threadIdx.x >> 5];
-  uint32_t *yq = found[threadIdx.x >> 5];
+  __shared__ uint2 place[kMates ? kRowWarps : 1][32];
+  __shared__ uint32_t found[kMates ? kRowWarps : 1][64];
+  uint2 *pl = place[kMates ? threadIdx.x >> 5 : 0];
+  uint32_t *yq = found[kMates ? threadIdx.x >> 5 : 0];
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t below = (1u << lane) - 1u;
   uint32_t *q = queue[threadIdx.x >> 5];
@@ -308,72 +317,93 @@ __global__ void __launch_bounds__(kRowWarps * 32, 8) k_ham_rows(
     // one column each); lane k then holds entry k's first column, length and
     // alpha threshold, and the columns are walked as one concatenated range, 32
     // per step, each lane finding its entry by a binary search over the lanes'
-    // offsets
+    // offsets.  Without the mates, the groups a beta double away are among x, and
+    // the row's alpha string is searched in each.
     int64_t x0 = nbr_ptr[g];
     const int64_t x1 = nbr_ptr[g + 1];
-    const uint2 ys = span[r];
+    const uint2 ys = kMates ? span[r] : make_uint2(0u, 0u);
     constexpr uint32_t kNone = 0xffffffffu;  // n < 2^31
     uint32_t y0 = ys.x;
     int yn = 0;  // mates in hand (warp-uniform, < 64)
-    while (true) {
-      for (; yn < 32 && y0 < ys.y; y0 += 32) {
-        uint2 m = make_uint2(0u, bi);
-        if (ys.y - y0 > lane) m = mates[y0 + lane];
-        const bool hit = __popc(bi ^ m.y) == 4;
-        const uint32_t bal = __ballot_sync(0xffffffffu, hit);
-        if (!bal) continue;
-        if (hit) yq[yn + __popc(bal & below)] = m.x;
-        yn += __popc(bal);
-      }
-      __syncwarp();
-      if (x0 >= x1 && yn == 0) break;
-      // groups that start past the mates seen so far wait for the next mates
-      const uint32_t lim = y0 < ys.y ? mates[y0 - 1u].x : kNone;
-      const uint32_t yj = (int)lane < yn ? yq[lane] : kNone;
-      uint32_t xs = kNone, xl = 0, xt = 0;
-      if (x1 - x0 > (int64_t)lane) {
-        const uint32_t g2 = nbr[x0 + lane];
-        xs = gstart[g2];
-        xl = gstart[g2 + 1] - xs;
-        xt = 4u - (uint32_t)__popc(bi ^ gbeta[g2]);  // 4 or 2
-      }
-      uint32_t nx = 0, ny = 0;  // groups up to this lane's mate, mates before its group
-      for (int step = 16; step; step >>= 1) {
-        const uint32_t a = __shfl_sync(0xffffffffu, xs, nx + step - 1);
-        const uint32_t b = __shfl_sync(0xffffffffu, yj, ny + step - 1);
-        if (a <= yj) nx += step;
-        if (b < xs) ny += step;
-      }
-      const uint32_t xlast = __shfl_sync(0xffffffffu, xs, 31);
-      if (nx == 31 && xlast <= yj) nx = 32;
-      const uint32_t y32 = __shfl_sync(0xffffffffu, yj, 31);
-      if (ny == 31 && y32 < xs) ny = 32;
-      const uint32_t rx = lane + ny, ry = lane + nx;
-      const bool take_x = xs != kNone && xs <= lim && rx < 32u, take_y = yj != kNone && ry < 32u;
-      // the threshold's two bits (0, 2 or 4) above the column and the length
-      if (take_x) pl[rx] = make_uint2(xs | ((xt & 2u) << 30), xl | ((xt & 4u) << 29));
-      if (take_y) pl[ry] = make_uint2(yj, 1u);
-      const uint32_t tx = __ballot_sync(0xffffffffu, take_x), ty = __ballot_sync(0xffffffffu, take_y);
-      __syncwarp();
+    while (kMates || x0 < x1) {
       uint32_t gs = 0, len = 0;
       int thr = -1;
-      if ((int)lane < __popc(tx) + __popc(ty)) {
-        const uint2 e = pl[lane];
-        gs = e.x & 0x7fffffffu;
-        len = e.y & 0x7fffffffu;
-        thr = (int)(((e.x >> 30) & 2u) | ((e.y >> 29) & 4u));
-      }
-      __syncwarp();
-      x0 += __popc(tx);
-      if (ty) {
-        const int k = __popc(ty);
-        const uint32_t a = (int)lane + k < yn ? yq[lane + k] : 0u;
-        const uint32_t b = (int)lane + 32 + k < yn ? yq[lane + 32 + k] : 0u;
+      if constexpr (!kMates) {
+        if (x1 - x0 > (int64_t)lane) {
+          const uint32_t g2 = nbr[x0 + lane];
+          gs = gstart[g2];
+          len = gstart[g2 + 1] - gs;
+          thr = 4 - __popc(bi ^ gbeta[g2]);
+          if (thr == 0) {  // the group (in alpha order) is that one column, or nothing
+            uint32_t lo = gs, hi = gs + len;
+            while (lo < hi) {
+              const uint32_t mid = (lo + hi) >> 1;
+              if (key_alpha(keys[mid]) < ai) lo = mid + 1;
+              else hi = mid;
+            }
+            len = lo < gs + len && key_alpha(keys[lo]) == ai ? 1u : 0u;
+            gs = lo;
+          }
+        }
+        x0 += 32;
+      } else {
+        for (; yn < 32 && y0 < ys.y; y0 += 32) {
+          uint2 m = make_uint2(0u, bi);
+          if (ys.y - y0 > lane) m = mates[y0 + lane];
+          const bool hit = __popc(bi ^ m.y) == 4;
+          const uint32_t bal = __ballot_sync(0xffffffffu, hit);
+          if (!bal) continue;
+          if (hit) yq[yn + __popc(bal & below)] = m.x;
+          yn += __popc(bal);
+        }
         __syncwarp();
-        yn -= k;
-        if ((int)lane < yn) yq[lane] = a;
-        if ((int)lane + 32 < yn) yq[lane + 32] = b;
+        if (x0 >= x1 && yn == 0) break;
+        // groups that start past the mates seen so far wait for the next mates
+        const uint32_t lim = y0 < ys.y ? mates[y0 - 1u].x : kNone;
+        const uint32_t yj = (int)lane < yn ? yq[lane] : kNone;
+        uint32_t xs = kNone, xl = 0, xt = 0;
+        if (x1 - x0 > (int64_t)lane) {
+          const uint32_t g2 = nbr[x0 + lane];
+          xs = gstart[g2];
+          xl = gstart[g2 + 1] - xs;
+          xt = 4u - (uint32_t)__popc(bi ^ gbeta[g2]);  // 4 or 2
+        }
+        uint32_t nx = 0, ny = 0;  // groups up to this lane's mate, mates before its group
+        for (int step = 16; step; step >>= 1) {
+          const uint32_t a = __shfl_sync(0xffffffffu, xs, nx + step - 1);
+          const uint32_t b = __shfl_sync(0xffffffffu, yj, ny + step - 1);
+          if (a <= yj) nx += step;
+          if (b < xs) ny += step;
+        }
+        const uint32_t xlast = __shfl_sync(0xffffffffu, xs, 31);
+        if (nx == 31 && xlast <= yj) nx = 32;
+        const uint32_t y32 = __shfl_sync(0xffffffffu, yj, 31);
+        if (ny == 31 && y32 < xs) ny = 32;
+        const uint32_t rx = lane + ny, ry = lane + nx;
+        const bool take_x = xs != kNone && xs <= lim && rx < 32u, take_y = yj != kNone && ry < 32u;
+        // the threshold's two bits (0, 2 or 4) above the column and the length
+        if (take_x) pl[rx] = make_uint2(xs | ((xt & 2u) << 30), xl | ((xt & 4u) << 29));
+        if (take_y) pl[ry] = make_uint2(yj, 1u);
+        const uint32_t tx = __ballot_sync(0xffffffffu, take_x), ty = __ballot_sync(0xffffffffu, take_y);
         __syncwarp();
+        if ((int)lane < __popc(tx) + __popc(ty)) {
+          const uint2 e = pl[lane];
+          gs = e.x & 0x7fffffffu;
+          len = e.y & 0x7fffffffu;
+          thr = (int)(((e.x >> 30) & 2u) | ((e.y >> 29) & 4u));
+        }
+        __syncwarp();
+        x0 += __popc(tx);
+        if (ty) {
+          const int k = __popc(ty);
+          const uint32_t a = (int)lane + k < yn ? yq[lane + k] : 0u;
+          const uint32_t b = (int)lane + 32 + k < yn ? yq[lane + 32 + k] : 0u;
+          __syncwarp();
+          yn -= k;
+          if ((int)lane < yn) yq[lane] = a;
+          if ((int)lane + 32 < yn) yq[lane + 32] = b;
+          __syncwarp();
+        }
       }
       uint32_t off = len;  // inclusive scan of the lengths
       for (int o = 1; o < 32; o <<= 1) {
@@ -1505,9 +1535,25 @@ struct BetaGraph {
   uint32_t *of_row = nullptr, *gstart = nullptr, *gbeta = nullptr, *nbr = nullptr;
   int64_t *nbr_ptr = nullptr;
   uint2 *mates = nullptr, *span = nullptr;  // rows in alpha order
+  bool by_mates = true;                     // k_ham_rows: which of its two ways
 };
 
-static int beta_graph(const uint64_t *keys, uint32_t n, int norb, BetaGraph *bg, Arena &arena) {
+// The row kernel looks at each of a row's mates (32 a step, loads that do not wait
+// for one another), or searches its alpha string in the `doubles` groups a beta
+// double away (32 at a time, ceil(log2 of a group's length) loads that do).  Build of
+// n determinants (two calls, mates / searches): 16 orbitals, random walk of 1e5, 117
+// mates against 705 groups of 11, 5.1 / 6.8 ms; 3335 mates, 784 groups of 8, 6.1 / 6.4;
+// products 300 x 300 and 3432 x 8, 1.8 to 2.6 mates a group and load, equal; 2500 x
+// 40, 152 groups of 40, 3.65 / 3.40; 12870 x 8, 16.8 / 15.7; 40000 of 20 orbitals x
+// 4, 26.4 / 13.2.
+static bool mates_are_fewer(double mates, double doubles, uint32_t n, uint32_t G) {
+  int loads = 1;
+  while (((uint64_t)G << loads) < (uint64_t)n) ++loads;
+  return mates <= 2.0 * loads * doubles;
+}
+
+static int beta_graph(const uint64_t *keys, uint32_t n, const DevInts &I, BetaGraph *bg,
+                      Arena &arena) {
   cudaStream_t s = arena.stream();
   uint32_t *head, *gid;
   ASCI_TRY(arena.alloc(&head, n));
@@ -1515,47 +1561,64 @@ static int beta_graph(const uint64_t *keys, uint32_t n, int norb, BetaGraph *bg,
   k_beta_heads<<<blocks_for(n, 256), 256, 0, s>>>(keys, n, head);
   ASCI_CHECK_LAUNCH();
   ASCI_TRY(scan_exclusive_u32(head, gid, n, arena));
-  uint32_t last[2];
-  ASCI_TRY_CUDA(cudaMemcpyAsync(&last[0], gid + n - 1, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-  ASCI_TRY_CUDA(cudaMemcpyAsync(&last[1], head + n - 1, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+  // rows in alpha order
+  uint64_t *akey, *akey_alt;
+  unsigned long long *d_tot, tot[2];
+  ASCI_TRY(arena.alloc(&akey, n));
+  ASCI_TRY(arena.alloc(&akey_alt, n));
+  ASCI_TRY(arena.alloc(&d_tot, 2));
+  ASCI_TRY(arena.alloc(&bg->mates, n));
+  ASCI_TRY(arena.alloc(&bg->span, n));
+  ASCI_TRY_CUDA(cudaMemsetAsync(d_tot, 0, sizeof(tot), s));
+  k_alpha_keys<<<blocks_for(n, 256), 256, 0, s>>>(keys, n, akey);
+  ASCI_CHECK_LAUNCH();
+  ASCI_TRY(radix_sort_u64_varying(&akey, &akey_alt, n, 32, 32 + I.n,
+                                  ((1ull << I.n) - 1ull) << 32, arena));
+  k_alpha_mates<<<blocks_for(n, 256), 256, 0, s>>>(keys, akey, n, head, gid, bg->mates, bg->span,
+                                                    d_tot);
+  ASCI_CHECK_LAUNCH();
+  ASCI_TRY_CUDA(cudaMemcpyAsync(tot, d_tot, sizeof(tot), cudaMemcpyDeviceToHost, s));
   ASCI_TRY_CUDA(cudaStreamSynchronize(s));
-  const uint32_t G = last[0] + last[1];
+  const uint32_t G = (uint32_t)tot[1];
   ASCI_TRY(arena.alloc(&bg->of_row, n));
   ASCI_TRY(arena.alloc(&bg->gstart, (size_t)G + 1));
   ASCI_TRY(arena.alloc(&bg->gbeta, G));
   k_beta_groups<<<blocks_for(n, 256), 256, 0, s>>>(keys, n, head, gid, bg->of_row, bg->gstart,
                                                     bg->gbeta);
   ASCI_CHECK_LAUNCH();
+  // which way: by the mates a row has and the beta doubles that G strings of all
+  // would have, then by the doubles they do have
+  const int nb = I.nb, nv = I.n - I.nb;
+  double strings = 1.0;
+  for (int k = 0; k < nb; ++k) strings *= (double)(I.n - k) / (k + 1);
+  const double per_row = (double)tot[0] / n;
+  bg->by_mates = mates_are_fewer(
+      per_row, G / strings * (0.25 * nb * (nb - 1) * nv * (nv - 1)), n, G);
   // the group graph: count, scan, list
   const HamGeom g = ham_geom(G);
   const size_t slots = (size_t)G * g.gy;
-  uint64_t *off;
+  uint64_t *off, total = 0;
   ASCI_TRY(arena.alloc(&off, slots + 1));
-  ASCI_TRY_CUDA(cudaMemsetAsync(off + slots, 0, sizeof(uint64_t), s));
-  k_beta_pairs<false><<<dim3(g.gx, g.gy), kRowThreads, 0, s>>>(bg->gbeta, G, g.chunk, g.gy, off,
-                                                                nullptr);
-  ASCI_CHECK_LAUNCH();
-  ASCI_TRY(scan_exclusive_u64(off, off, slots + 1, arena));
+  for (bool counted = false; !counted;) {
+    const int reach = bg->by_mates ? 2 : 4;
+    ASCI_TRY_CUDA(cudaMemsetAsync(off + slots, 0, sizeof(uint64_t), s));
+    k_beta_pairs<false><<<dim3(g.gx, g.gy), kRowThreads, 0, s>>>(bg->gbeta, G, g.chunk, g.gy,
+                                                                  reach, off, nullptr);
+    ASCI_CHECK_LAUNCH();
+    ASCI_TRY(scan_exclusive_u64(off, off, slots + 1, arena));
+    ASCI_TRY_CUDA(cudaMemcpyAsync(&total, off + slots, sizeof(total), cudaMemcpyDeviceToHost, s));
+    ASCI_TRY_CUDA(cudaStreamSynchronize(s));
+    counted = bg->by_mates || !mates_are_fewer(per_row, (double)total / G, n, G);
+    if (!counted) bg->by_mates = true;
+  }
+  ASCI_TRACE("hamiltonian rows: n=%u groups=%u mates=%llu pairs=%llu by %s", n, G, tot[0],
+             (unsigned long long)total, bg->by_mates ? "mates" : "searches");
   ASCI_TRY(arena.alloc(&bg->nbr_ptr, (size_t)G + 1));
   k_row_ptr<<<blocks_for((size_t)G + 1, 256), 256, 0, s>>>(off, G, g.gy, bg->nbr_ptr);
   ASCI_CHECK_LAUNCH();
-  uint64_t total = 0;
-  ASCI_TRY_CUDA(cudaMemcpyAsync(&total, off + slots, sizeof(total), cudaMemcpyDeviceToHost, s));
-  ASCI_TRY_CUDA(cudaStreamSynchronize(s));
   ASCI_TRY(arena.alloc(&bg->nbr, total));
-  k_beta_pairs<true><<<dim3(g.gx, g.gy), kRowThreads, 0, s>>>(bg->gbeta, G, g.chunk, g.gy, off,
-                                                               bg->nbr);
-  ASCI_CHECK_LAUNCH();
-  uint64_t *akey, *akey_alt;
-  ASCI_TRY(arena.alloc(&akey, n));
-  ASCI_TRY(arena.alloc(&akey_alt, n));
-  ASCI_TRY(arena.alloc(&bg->mates, n));
-  ASCI_TRY(arena.alloc(&bg->span, n));
-  k_alpha_keys<<<blocks_for(n, 256), 256, 0, s>>>(keys, n, akey);
-  ASCI_CHECK_LAUNCH();
-  ASCI_TRY(radix_sort_u64_varying(&akey, &akey_alt, n, 32, 32 + norb,
-                                  ((1ull << norb) - 1ull) << 32, arena));
-  k_alpha_mates<<<blocks_for(n, 256), 256, 0, s>>>(keys, akey, n, bg->mates, bg->span);
+  k_beta_pairs<true><<<dim3(g.gx, g.gy), kRowThreads, 0, s>>>(bg->gbeta, G, g.chunk, g.gy,
+                                                               bg->by_mates ? 2 : 4, off, bg->nbr);
   ASCI_CHECK_LAUNCH();
   bg->G = G;
   return ASCI_OK;
@@ -1570,9 +1633,9 @@ static int ham_count(const DevInts &I, const uint64_t *keys, uint32_t n, const d
                      const BetaGraph &bg, int64_t *rp, size_t *nnz, Arena &arena) {
   cudaStream_t s = arena.stream();
   ASCI_TRY_CUDA(cudaMemsetAsync(rp + n, 0, sizeof(int64_t), s));
-  k_ham_rows<false><<<row_blocks(n), kRowWarps * 32, 0, s>>>(I, keys, n, bg.of_row, bg.gstart, bg.gbeta,
-                                                   bg.nbr_ptr, bg.nbr, bg.mates, bg.span, diag, rp, nullptr,
-                                                   nullptr);
+  auto *k = bg.by_mates ? k_ham_rows<false, true> : k_ham_rows<false, false>;
+  k<<<row_blocks(n), kRowWarps * 32, 0, s>>>(I, keys, n, bg.of_row, bg.gstart, bg.gbeta, bg.nbr_ptr,
+                                             bg.nbr, bg.mates, bg.span, diag, rp, nullptr, nullptr);
   ASCI_CHECK_LAUNCH();
   ASCI_TRY(scan_exclusive_u64(reinterpret_cast<uint64_t *>(rp), reinterpret_cast<uint64_t *>(rp),
                               (size_t)n + 1, arena));
@@ -1585,9 +1648,10 @@ static int ham_count(const DevInts &I, const uint64_t *keys, uint32_t n, const d
 
 static int ham_fill(const DevInts &I, const uint64_t *keys, uint32_t n, const double *diag,
                     const BetaGraph &bg, int64_t *rp, int32_t *col, double *val, Arena &arena) {
-  k_ham_rows<true><<<row_blocks(n), kRowWarps * 32, 0, arena.stream()>>>(I, keys, n, bg.of_row, bg.gstart,
-                                                              bg.gbeta, bg.nbr_ptr, bg.nbr, bg.mates, bg.span, diag,
-                                                              rp, col, val);
+  auto *k = bg.by_mates ? k_ham_rows<true, true> : k_ham_rows<true, false>;
+  k<<<row_blocks(n), kRowWarps * 32, 0, arena.stream()>>>(I, keys, n, bg.of_row, bg.gstart, bg.gbeta,
+                                                          bg.nbr_ptr, bg.nbr, bg.mates, bg.span,
+                                                          diag, rp, col, val);
   ASCI_CHECK_LAUNCH();
   return ASCI_OK;
 }
@@ -1868,7 +1932,7 @@ static int ham_build(const DevInts &I, const uint64_t *keys, size_t n, Arena &ar
   ASCI_TRY(arena.alloc(&rp, n + 1));
   ASCI_TRY(diagonal_packed(I, keys, n, diag, arena));
   BetaGraph bg;
-  ASCI_TRY(beta_graph(keys, (uint32_t)n, I.n, &bg, arena));
+  ASCI_TRY(beta_graph(keys, (uint32_t)n, I, &bg, arena));
   size_t nnz = 0;
   ASCI_TRY(ham_count(I, keys, (uint32_t)n, diag, bg, rp, &nnz, arena));
   int32_t *col;
@@ -2142,7 +2206,7 @@ int asci_hamiltonian(const asci_det *dets, size_t n, const asci_ints *ints, int6
   ASCI_TRY(arena.alloc(&diag, n));
   ASCI_TRY(diagonal_packed(I, keys, n, diag, arena));
   BetaGraph bg;
-  ASCI_TRY(beta_graph(keys, (uint32_t)n, I.n, &bg, arena));
+  ASCI_TRY(beta_graph(keys, (uint32_t)n, I, &bg, arena));
   const bool same_order = hflag == 0;
   int64_t *rp, *urp;
   ASCI_TRY(out_buffer(row_ptr, n + 1, &urp, arena));
