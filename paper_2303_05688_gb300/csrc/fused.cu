@@ -429,8 +429,7 @@ __global__ void k_tile_write(uint32_t gb0, uint32_t ng, const uint64_t *soff, ui
 // owns kCap staging slots; its record count is known after emission.
 __global__ void k_cell_write(uint32_t gb0, uint32_t ng, uint32_t ncells, const uint64_t *soff,
                              const uint32_t *g_alpha, const uint32_t *tile_base,
-                             const uint32_t *cellbase, TileDesc *tiles, uint32_t *cell_pos0,
-                             uint32_t *cell_tile) {
+                             const uint32_t *cellbase, TileDesc *tiles, uint32_t *cell_tile) {
   for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells;
        c += gridDim.x * blockDim.x) {
     uint32_t lo = 0, hi = ng - 1;
@@ -448,7 +447,6 @@ __global__ void k_cell_write(uint32_t gb0, uint32_t ng, uint32_t ncells, const u
     d.alpha = g_alpha[g];
     d.psi_lo = d.psi_hi = 0;
     tiles[tile_base[lo] + b] = d;
-    cell_pos0[c] = d.start;
     cell_tile[c] = tile_base[lo] + b;
   }
 }
@@ -526,7 +524,7 @@ struct EmitArgs {
   uint32_t npieces;           // pieces of `piece` pairs a determinant's o = 0 run is cut into
   const uint64_t *items, *Wexcl;
   const uint32_t *item_group;
-  uint64_t t0, P0;
+  uint64_t t0;
   int opbits;
   const uint32_t *grp_alpha, *grp_start, *grp_count;
   // the core's records, its Fock-like diagonals and jk, jj in units of the
@@ -537,7 +535,6 @@ struct EmitArgs {
   const uint32_t *kind, *nb, *cellbase;
   const uint64_t *soff;       // first staging slot of each class of the batch
   const uint64_t *g_P0;       // first pair of each class
-  const uint32_t *cell_pos0;  // first staging slot of each bucket cell
   uint32_t *fill;             // records placed in each bucket cell
   StageRec *spill_rec;        // records beyond a cell's kCap slots
   uint32_t *spill_cell;
@@ -1268,9 +1265,6 @@ struct CellArgs {
   uint32_t ntiles;     // tiles [tile0, ntiles) are visited
   uint32_t tile0;
   Stage st;
-  FxInts X;          // exact diagonal of the targets that pass the screen
-  int64_t E0_x;
-  double inv_scale;  // 2^-s
   double tau;
   float tau_f;
   const uint64_t *psi_ht;
@@ -1420,8 +1414,8 @@ __device__ __forceinline__ bool tile_on_chip(const TileDesc &d, uint64_t stage_c
 // |v| / (tau |den|) in units of 1 / kThr, rounded up, at most kThr.  inv_tau is
 // kThr / tau_f, or infinity without a threshold.  An upper bound: |v| is
 // truncated to a float from its bits (no FP64 instruction; within 2^-23),
-// |den| was truncated when it was staged and tau_f rounded down, and the factor
-// 1.00001 covers those and the float operations.  A value above the normal
+// |den| was staged as a lower bound, rounded to a float, and tau_f rounded down,
+// and the factor 1.00001 covers those and the float operations.  A value above the normal
 // float range, a zero denominator and anything that is not a number count as
 // reaching the threshold; a |v| below the range counts as its smallest value.
 template <uint32_t kThr>
@@ -2403,7 +2397,7 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   // kCap slots from its class's first slot on
   TileDesc *tiles;
   unsigned *n_over, *n_spill;
-  uint32_t *over_list, *cell_pos0, *cell_tile, *fill, *spill_cell;
+  uint32_t *over_list, *cell_tile, *fill, *spill_cell;
   const uint32_t over_cap = (uint32_t)std::min<size_t>(ncells + 1, 1u << 20);
   uint32_t spill_cap = (uint32_t)std::min<uint64_t>(
       std::max<uint64_t>(1ull << 20, (P1 - P0) / 32), 1ull << 30);
@@ -2412,7 +2406,6 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   ASCI_TRY(arena.alloc(&n_over, 3));  // overfilled cells, spilled records, psi determinants routed
   n_spill = n_over + 1;
   ASCI_TRY(arena.alloc(&over_list, over_cap));
-  ASCI_TRY(arena.alloc(&cell_pos0, ncells + 1));
   ASCI_TRY(arena.alloc(&cell_tile, ncells + 1));
   ASCI_TRY(arena.alloc(&fill, ncells + 1));
   ASCI_TRY(arena.alloc(&spill_rec, spill_cap));
@@ -2425,8 +2418,7 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   ASCI_CHECK_LAUNCH();
   if (ncells) {
     k_cell_write<<<grid_for(ncells), 256, 0, s>>>(gb0, ng, (uint32_t)ncells, soff, F.g_alpha,
-                                                  tile_base, cellbase, tiles, cell_pos0,
-                                                  cell_tile);
+                                                  tile_base, cellbase, tiles, cell_tile);
     ASCI_CHECK_LAUNCH();
   }
   ASCI_TRACE("stage: tiles written");
@@ -2462,7 +2454,6 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   A.Wexcl = F.Wexcl;
   A.item_group = F.item_group;
   A.t0 = t0;
-  A.P0 = P0;
   A.opbits = F.opbits;
   A.grp_alpha = F.grp_alpha;
   A.grp_start = F.grp_start;
@@ -2478,7 +2469,6 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   A.cellbase = cellbase;
   A.soff = soff;
   A.g_P0 = F.g_P0;
-  A.cell_pos0 = cell_pos0;
   A.fill = fill;
   A.spill_rec = spill_rec;
   A.spill_cell = spill_cell;
@@ -2598,9 +2588,6 @@ static CellArgs cell_args(const FusedCore &F, const Stage &st,
   CellArgs CA;
   memset(&CA, 0, sizeof(CA));
   CA.st = st;
-  CA.X = F.X;
-  CA.E0_x = F.E0_x;
-  CA.inv_scale = ldexp(1.0, -F.X.s);
   CA.tau = tau;
   CA.tau_f = (float)tau;
   if ((double)CA.tau_f > tau) CA.tau_f = nextafterf(CA.tau_f, 0.0f);

@@ -28,8 +28,8 @@ namespace {
 
 constexpr size_t kNoAllocMaxPairs = ASCI_NOALLOC_MAX_PAIRS;
 // Per pair: keys (3 x 8 B), values (2 x 8 B), sums (8 B), unpacked keys (16 B),
-// staged inputs (24 B), run flags and positions (12 B); plus radix histograms,
-// scan partials, the error word and alignment slack.
+// staged inputs (24 B), run flags and positions (12 B); plus the words of the sort's
+// and the scans' tiles, the digit counts, the error word and alignment slack.
 constexpr size_t kNoAllocBytes = kNoAllocMaxPairs * 104 + (2u << 20);
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];

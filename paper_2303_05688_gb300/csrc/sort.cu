@@ -104,7 +104,8 @@ __device__ __forceinline__ uint64_t warp_sum(uint64_t v) {
   return v;
 }
 
-// Exclusive scan in one pass, a tile per CTA.  words[0] numbers the tiles in the
+// Exclusive scan in one pass, a tile per CTA: the single-pass scan with decoupled look
+// back of Merrill and Garland (2016).  words[0] numbers the tiles in the
 // order in which CTAs start; words[1 + t] is tile t's sum (below 2^62) under a
 // state: 0 unknown, 1 the tile's own sum, 2 the sum of it and all before.  A tile
 // publishes its sum, then its first warp adds up the tiles before it, 32 at a
@@ -281,7 +282,8 @@ constexpr size_t scatter_smem() {
          (size_t)(kSortWarps + 1) * kRadix * sizeof(uint32_t);
 }
 
-// Stable scatter by one digit, a tile per CTA.  Warp w owns elements
+// Stable scatter by one digit, a tile per CTA, the digits' starts by decoupled look back
+// (as in the Onesweep sort of Adinets and Merrill, 2022).  Warp w owns elements
 // [w*32*kSortItems, ...) of the tile in rounds of 32 consecutive elements, so tile
 // order is preserved.  Tiles are numbered in the order in which CTAs start, so a
 // tile's predecessors are running or done; each publishes its digit counts before
@@ -420,10 +422,9 @@ __global__ void __launch_bounds__(kSortThreads, 4)
 
 // The whole sort of at most one tile (4096 keys) in one CTA: 16 warps of 256
 // consecutive elements each, the digits that vary one after another in shared
-// memory (the ranks as in the scatter above, so just as stable).  A sort of a
-// small list through the tile kernels takes four or more launches a digit and a
-// host round trip for the varying bits: 2000 (key, index) pairs 95 us in 8
-// digits, against 20 here.
+// memory (the ranks as in the scatter above, so just as stable).  Through the tile
+// kernels a list of one tile would take a launch a digit, the counts' launch and,
+// where the varying bits are not given, a wait for them.
 constexpr int kSmallThreads = 512;
 constexpr int kSmallItems = kSortTile / kSmallThreads;
 constexpr int kSmallWarps = kSmallThreads / 32;
