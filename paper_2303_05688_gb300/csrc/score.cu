@@ -126,8 +126,11 @@ __host__ __device__ inline int sel_shift(int round) {
   return d == 5 ? 0 : 64 - kSelBits * (d + 1);
 }
 
-// The state before the first round, for the n largest.
-__global__ void k_select_init(SelState *st, uint64_t n) {
+// The state and the bins before the first round, for the n largest.
+__global__ void k_select_init(SelState *st, uint32_t *hist, uint64_t n) {
+  const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (i < kSelBins) hist[i] = 0;
+  if (i > 0) return;
   SelState s{};
   s.remaining = n;
   *st = s;
@@ -448,8 +451,7 @@ int select_topn_packed(const uint64_t *keys, const double *scores, size_t n, siz
     ASCI_TRY(arena.alloc(&flag, n));
     ASCI_TRY(arena.alloc(&pos, n));
     ASCI_TRY(arena.alloc(&hist, (size_t)kSelBins));
-    ASCI_TRY_CUDA(cudaMemsetAsync(hist, 0, kSelBins * sizeof(uint32_t), s));
-    k_select_init<<<1, 1, 0, s>>>(st, N);
+    k_select_init<<<kSelBins / 256, 256, 0, s>>>(st, hist, N);
     ASCI_CHECK_LAUNCH();
     for (int round = 0; round < kSelRounds; ++round) {
       k_select_round<<<grid_for(n, 152 * 4), 256, 0, s>>>(keys, scores, n, round, st, hist);
