@@ -612,10 +612,10 @@ constexpr int kPassBlocks = 304;  // at most: two per SM
 // at 50,000 determinants) with all loads of an element in flight, and takes up
 // to 3 m FP64 operations per element; 8 to 17 us at 50,000 elements, half of it
 // the launch and the tail of the sums.  With the subspace solve below, a
-// product costs 6 launches instead of 12: a solve at 50,000 determinants 39.0
-// -> 16.7 ms, a loop of two steps at 20,000 67.9 -> 35.3.  The sums of a warp's lanes are folded
-// value against value (half of the values kept by each half of the lanes, and
-// so on): M + 1 FP64 additions per warp for M values instead of 5 M.
+// product costs 6 launches instead of 12: a solve at 50,000 determinants 34.8
+// -> 15.4 ms.  The sums of a warp's lanes are folded value against value (half of
+// the values kept by each half of the lanes, and so on): M + 1 FP64 additions per
+// warp for M values instead of 5 M.
 enum : int { kProject, kRitz, kRestart, kOrth1, kOrth2 };
 
 struct PassArgs {
