@@ -199,16 +199,15 @@ __device__ __forceinline__ int64_t fx_diag(const FxInts &X, uint32_t A, uint32_t
 namespace {
 
 // The staged denominator E0 - H_ii serves screens only, so it is summed in
-// 32-bit fixed point: multiples of 2^29 units of the 64-bit grid (|E0 - H_ii| <
-// 2^59 of those), each term rounded to nearest; a sum of at most 15 such terms
-// is within 8 units of the exact value, and what is stored is a lower bound of
-// the magnitude.  A test that these 8 units could decide forms the exact value.
+// 32-bit fixed point: multiples of 2^ds units of the 64-bit grid (|E0 - H_ii| <
+// 2^30 of those: build_fx), each term rounded to nearest; a sum of at most 15 such
+// terms is within 8 units of the exact value, and what is stored is a lower bound
+// of the magnitude.  A test that these 8 units could decide forms the exact value.
 // Half the registers, shuffles, table bytes and additions of 64 bits.  (Unsigned:
 // sums may wrap on the way.)
-constexpr int kDenShift = 29;
 constexpr int32_t kDenSlack = 8;
-__host__ __device__ __forceinline__ uint32_t den_round(int64_t x) {
-  return (uint32_t)((x + (1ll << (kDenShift - 1))) >> kDenShift);
+__device__ __forceinline__ uint32_t den_round(int64_t x, int ds) {
+  return (uint32_t)((x + (1ll << (ds - 1))) >> ds);
 }
 
 // A core determinant as the emission reads it: one 16-byte load.
@@ -234,7 +233,7 @@ __global__ void k_core_fock(FxInts X, int64_t E0_x, const uint32_t *core_alpha,
     if (p == n) {
       CoreRec r;
       r.beta = B;
-      r.den = den_round(E0_x - fx_diag(X, A, B));
+      r.den = den_round(E0_x - fx_diag(X, A, B), X.ds);
       r.c = core_c[j];
       rec[j] = r;
       continue;
@@ -250,15 +249,15 @@ __global__ void k_core_fock(FxInts X, int64_t E0_x, const uint32_t *core_alpha,
       fb += X.jk[p * n + q];
       fa += X.jj[p * n + q];
     }
-    Fa[(size_t)p * m + j] = den_round(fa);
-    Fb[j * n + p] = den_round(fb);
+    Fa[(size_t)p * m + j] = den_round(fa, X.ds);
+    Fb[j * n + p] = den_round(fb, X.ds);
   }
 }
 
 __global__ void k_den_tables(FxInts X, uint32_t *jk, uint32_t *jj) {
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < X.n * X.n; t += gridDim.x * blockDim.x) {
-    jk[t] = den_round(X.jk[t]);
-    jj[t] = den_round(X.jj[t]);
+    jk[t] = den_round(X.jk[t], X.ds);
+    jj[t] = den_round(X.jj[t], X.ds);
   }
 }
 
@@ -2133,8 +2132,8 @@ int build_fx(const double *h1, const double *eri, int n, int na, int nb, double 
   // pair terms.  With s = 58 - log2(B) a sum of up to 32 such values cannot
   // overflow 64 bits.
   const double nn = (double)(na + nb), pairs_same = 0.5 * (na * (na - 1) + nb * (nb - 1));
-  const double B = fabs(ecore) + fabs(E0) + nn * h3[0] + (pairs_same + n) * h3[1] +
-                   ((double)na * nb + n) * h3[2] + 1.0;
+  const double terms = nn * h3[0] + (pairs_same + n) * h3[1] + ((double)na * nb + n) * h3[2] + 1.0;
+  const double B = fabs(ecore) + fabs(E0) + terms;
   int e = 0;
   frexp(B, &e);  // B < 2^e
   int sc = 58 - e;
@@ -2164,9 +2163,15 @@ int build_fx(const double *h1, const double *eri, int n, int na, int nb, double 
   k_fx_single_tables<<<(unsigned)std::min<size_t>((n3 + 255) / 256, 4096), 256, 0, s>>>(
       h1, eri, n, s1, h1x, ssx, sox);
   ASCI_CHECK_LAUNCH();
+  // the 32-bit denominators: |E0 - H_ii| is bounded without the core energy, which
+  // E0 contains as well (with it, ecore = 1e9 left so few bits that a (24e,30o) search
+  // with eps = 1e-6, C = 3000, took 43 ms instead of 7.2)
+  int ed = 0;
+  frexp(fabs(E0 - ecore) + terms, &ed);
   FxInts X;
   X.n = n;
   X.s = sc;
+  X.ds = std::max(1, ed + sc - 30);
   X.s1 = s1;
   X.h1x = h1x;
   X.ssx = ssx;
@@ -2490,7 +2495,7 @@ int fused_stage(const FusedCore &F, uint64_t t0, uint64_t t1, uint64_t P0, uint6
   A.eps_shift = -eps_exp;
   A.E0_x = F.E0_x;
   A.inv_scale = ldexp(1.0, -F.X.s);
-  A.scale32 = (float)ldexp(1.0, kDenShift - F.X.s);
+  A.scale32 = (float)ldexp(1.0, F.X.ds - F.X.s);
   A.survivors = survivors;
   A.ncore = F.ncore;
   A.err = err;

@@ -10,6 +10,7 @@ namespace asci {
 struct FxInts {
   int n;
   int s;              // values are multiples of 2^-s
+  int ds;             // the emission's denominators are multiples of 2^(ds-s)
   int64_t ecore_x;
   const int64_t *hh;  // n      h_pp
   const int64_t *jk;  // n*n    (pp|qq) - (pq|qp), zero diagonal
