@@ -2975,7 +2975,9 @@ template <int NC>
 __global__ void __launch_bounds__(256) k_pt2_terms(const uint64_t *key, const double *num,
                                                    size_t n, FxInts X, int64_t E0_x,
                                                    double inv_scale, long long *limbs,
-                                                   unsigned *err) {
+                                                   unsigned long long *count,
+                                                   unsigned long long left, unsigned *err) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *count = left;  // these candidates are dropped
   // limb sums of each thread, thread-contiguous so that any limbs are free of
   // bank conflicts
   __shared__ long long acc[kPt2Limbs][256];
@@ -3010,11 +3012,14 @@ __global__ void k_pt2_value(const long long *limbs, double *out) {
 
 }  // namespace
 
+// Adds the terms of n candidates and sets *count to the `left` that stay.
 int pt2_terms(const FusedCore &F, const uint64_t *key, const double *num, size_t n,
-              long long *limbs, unsigned *err, cudaStream_t s) {
+              long long *limbs, unsigned long long *count, unsigned long long left, unsigned *err,
+              cudaStream_t s) {
   if (!n) return ASCI_OK;
   auto *k = F.X.nc == 2 ? k_pt2_terms<2> : (F.X.nc == 3 ? k_pt2_terms<3> : k_pt2_terms<4>);
-  k<<<grid_for(n, 152 * 8), 256, 0, s>>>(key, num, n, F.X, F.E0_x, ldexp(1.0, -F.X.s), limbs, err);
+  k<<<grid_for(n, 152 * 8), 256, 0, s>>>(key, num, n, F.X, F.E0_x, ldexp(1.0, -F.X.s), limbs, count,
+                                         left, err);
   ASCI_CHECK_LAUNCH();
   return ASCI_OK;
 }

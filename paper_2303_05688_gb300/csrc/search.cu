@@ -81,7 +81,8 @@ size_t big_tile_capacity();
 int exact_scores(const FusedCore &F, const uint64_t *key, double *score, size_t n,
                  cudaStream_t s);
 int pt2_terms(const FusedCore &F, const uint64_t *key, const double *num, size_t n,
-              long long *limbs, unsigned *err, cudaStream_t s);
+              long long *limbs, unsigned long long *count, unsigned long long left, unsigned *err,
+              cudaStream_t s);
 int pt2_value(const long long *limbs, double *out, cudaStream_t s);
 
 static thread_local char g_last_error[512] = "";
@@ -886,11 +887,8 @@ static int search_impl(const asci_det *dets_in, const double *coeffs_in, size_t 
   // exact scores, or (PT2) add their terms and drop them.
   auto consume = [&](unsigned long long c) -> int {
     if (pt2_out) {
-      ASCI_TRY(pt2_terms(F, pool_k[pcur] + pool_n, pool_s[pcur] + pool_n, (size_t)c - pool_n,
-                         pt2_limbs, derr2, stream));
-      k_set_count<<<1, 1, 0, stream>>>(dcount, pool_n);
-      ASCI_CHECK_LAUNCH();
-      return ASCI_OK;
+      return pt2_terms(F, pool_k[pcur] + pool_n, pool_s[pcur] + pool_n, (size_t)c - pool_n,
+                       pt2_limbs, dcount, pool_n, derr2, stream);
     }
     ASCI_TRY(exact_scores(F, pool_k[pcur] + pool_n, pool_s[pcur] + pool_n, (size_t)c - pool_n,
                           stream));
